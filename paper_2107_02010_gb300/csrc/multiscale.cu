@@ -543,9 +543,24 @@ void Multiscale::setup_tcc(Solver &s) {
     const int D4 = s.X.stride;
     const int nwords = (std::max(ncl_x, ncl_y) + 31) / 32;
     s.launch.use_tcc = 0;
-    if (!s.use_tc || s.D <= 3 || D4 > 60 || nwords > kTccMaxWords) return;
+    const int np = s.tcc_pieces;
+    if (!np || D4 > 60 || nwords > kTccMaxWords) return;
     cudaStream_t st = s.st;
     Workspace &ws = *s.ws;
+    // The float32 form has the CUDA-core kernel to go back to, which needs no tiles: it stays in charge where the
+    // tiles would take more than half of the memory that is free (0.77 KB per point of 60 coordinates and copy).
+    // Asked only above 8 GB of new memory (some 5 million points per side), so that ordinary solves pay nothing.
+    if (np == 3) {
+        size_t need = 0, have = 0, free_b = 0, total_b = 0;
+        for (const std::vector<int> *off : {&s.X_off, &s.Y_off})
+            for (size_t J = 0; J + 1 < off->size(); ++J)
+                need += 2 * (size_t)(((*off)[J + 1] - (*off)[J] + 127) / 128) * tcc_tile_bytes(np, D4);
+        for (const char *nm : {"tcc:tiles0x", "tcc:tiles1x", "tcc:tiles0y", "tcc:tiles1y"}) have += ws.held(nm);
+        if (need > have + (size_t(8) << 30)) {
+            OTGB_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+            if (need - have > free_b / 2) return;
+        }
+    }
     struct Side {
         int *tile0, *tile_cl;
         int ntiles;
@@ -571,11 +586,11 @@ void Multiscale::setup_tcc(Solver &s) {
         OTGB_CUDA_TRY(cudaMemcpyAsync(S.tile0, t0.data(), sizeof(int) * (ncl + 1), cudaMemcpyHostToDevice, st));
         if (S.ntiles)
             OTGB_CUDA_TRY(cudaMemcpyAsync(S.tile_cl, tcl.data(), sizeof(int) * S.ntiles, cudaMemcpyHostToDevice, st));
-        const size_t bytes = (size_t)std::max(S.ntiles, 1) * tcc_tile_bytes();
+        const size_t bytes = (size_t)std::max(S.ntiles, 1) * tcc_tile_bytes(np, D4);
         S.copy[0] = static_cast<unsigned char *>(ws.get(std::string("tcc:tiles0") + tag[k], bytes));
         S.copy[1] = static_cast<unsigned char *>(ws.get(std::string("tcc:tiles1") + tag[k], bytes));
         S.half_norm = ws.get<float>(std::string("tcc:hn") + tag[k], (size_t)std::max(S.ntiles, 1) * 128);
-        tcc_build_side(k == 0 ? s.X.pts : s.Y.pts, D4, k == 0 ? d_off_x : d_off_y, S.tile0, S.tile_cl, S.ntiles,
+        tcc_build_side(np, k == 0 ? s.X.pts : s.Y.pts, D4, k == 0 ? d_off_x : d_off_y, S.tile0, S.tile_cl, S.ntiles,
                        k == 0 ? cen_x : cen_y, S.copy[0], S.copy[1], S.half_norm, st);
         OTGB_CUDA_TRY(cudaStreamSynchronize(st));  // host vectors go out of scope
     }
@@ -596,7 +611,7 @@ void Multiscale::setup_tcc(Solver &s) {
         I.tcc_blk_cl = blk_cl[q];
     }
     s.launch.tcc_nwords = nwords;
-    s.launch.use_tcc = 1;
+    s.launch.use_tcc = np;
 }
 
 }  // namespace otgb

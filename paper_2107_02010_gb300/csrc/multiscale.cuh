@@ -59,6 +59,7 @@ struct Solver {
     bool translation = false;
     bool use_tc = false;
     bool use_tc3 = false;
+    int tcc_pieces = 0;  // BF16 pieces of the cluster-tiled form where it applies (2: reduced precision, 3: float32)
     std::vector<cudaEvent_t> ev_pool;
     int ev_used = 0;
     double softmin_ms = 0.0;
@@ -130,8 +131,8 @@ struct Multiscale {
                  const std::vector<float> &hiy, float *d_box);
     int run_schedule(Solver &s, const otgb_params &P, const std::vector<double> &sched, int block_rows);
     void before_fine_step(Solver &s, double sigma);
-    // the column tiles of the cluster-tiled tensor-core form, when it applies (tensor-core precision,
-    // D4 <= 60, at most 32 x kTccMaxWords clusters per side)
+    // the column tiles of the cluster-tiled tensor-core form, when it applies (3 < D, D4 <= 60, at most
+    // 32 x kTccMaxWords clusters per side, and room for the tiles)
     void setup_tcc(Solver &s);
 };
 

@@ -105,6 +105,7 @@ struct Workspace {
     std::vector<Buf> bufs;
     cudaStream_t stream = nullptr;
     void *get(const std::string &name, size_t bytes);
+    size_t held(const std::string &name) const;  // bytes of a buffer already there (0: none)
     template <class T> T *get(const std::string &name, size_t count) {
         return static_cast<T *>(get(name, count * sizeof(T) + 16));
     }
@@ -141,8 +142,8 @@ struct SoftminInst {
     const int *rng_ptr;
     const int2 *col_rng;
     // Cluster-tiled tensor-core form (softmin_tcc.cu, coarse-to-fine solves): the column side's points
-    // centred at their cluster's centre and split into BF16 tiles of 128 columns (tcc_tiles, 32 KiB per
-    // tile: hi then lo, with H_j in K slots 60..63 rewritten every step); tile0[J] .. tile0[J+1] are the
+    // centred at their cluster's centre and split into BF16 tiles of 128 columns (tcc_tiles, the pieces one
+    // after the other, with H_j in the last K slots rewritten every step); tile0[J] .. tile0[J+1] are the
     // tiles of column cluster J (tile_cl: the cluster of each tile); half_norm: |y_j - c_J|^2 / 2 per tile
     // column; coff / ccen: column cluster offsets and centres; bits / blk_cl: keep bits of the row clusters
     // (tcc_nwords words each) and the row clusters of each block.
@@ -240,7 +241,8 @@ struct SoftminLaunch {
     int exact_max;           // 1: take each row's shift from an exact maximum pass even when old values exist
     int use_tc;              // 1: D >= 16 cross term on the tensor cores (BF16 hi/lo split, FP32 accumulate)
     int use_tc3;             // 1: D <= 3 exponent on the tensor cores (three-piece BF16, float32 accuracy)
-    int use_tcc;             // 1 (with use_tc): the cluster-tiled tensor-core form (tcc_* fields of the instances)
+    int use_tcc;             // 2 or 3: the cluster-tiled tensor-core form with that many BF16 pieces per operand
+                             // (tcc_* fields of the instances); 0: not used
     int cost_p1;             // 1: cost |x - y| (p = 1, direct form, softmin_direct.cu); 0: |x - y|^2 / 2
     int direct;              // 1: the direct difference form for p = 2 as well (softmin_direct.cu)
     int tcc_nwords;          // words of keep bits per row cluster
@@ -277,15 +279,15 @@ void softmin3_tc_launch(const SoftminLaunch &L, cudaStream_t st);
 size_t softmin_tc_smem_bytes();
 // Cluster-tiled tensor-core softmin (softmin_tcc.cu): D4 <= 60, old values required, one item per block.
 void softmin_tcc_launch(const SoftminLaunch &L, int D, cudaStream_t st);
-// Bytes of one column tile of the cluster-tiled form (128 columns, hi and lo pieces).
-size_t tcc_tile_bytes();
+// Bytes of one column tile of the cluster-tiled form (128 columns, np BF16 pieces of points of width D4).
+size_t tcc_tile_bytes(int np, int D4);
 // Column tiles of one side (points pts with stride D4, cluster offsets / first tiles / tile clusters and
 // centres on the device), written into two copies (one per instance that uses this side as columns).
-void tcc_build_side(const float *pts, int D4, const int *d_off, const int *d_tile0, const int *d_tile_cl,
+void tcc_build_side(int np, const float *pts, int D4, const int *d_off, const int *d_tile0, const int *d_tile_cl,
                     int ntiles, const float *cen, unsigned char *dst0, unsigned char *dst1, float *half_norm,
                     cudaStream_t st);
 // H_j of the current step into the column tiles of every instance of L (uses col_pot, col_logw, s, eps).
-void tcc_update(const SoftminLaunch &L, cudaStream_t st);
+void tcc_update(const SoftminLaunch &L, int D, cudaStream_t st);
 
 // Build uniform row blocks of `block_rows` rows for an instance of n rows:
 // writes blk_row0 (n_blocks+1) on the device.  Returns n_blocks.

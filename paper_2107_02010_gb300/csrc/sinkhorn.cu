@@ -129,7 +129,7 @@ void Solver::step(double sigma, bool count_pairs) {
         harvest_timing();
     }
     if (timing) OTGB_CUDA_TRY(cudaEventRecord(ev_pool[2 * ev_used], st));
-    if (L.use_tcc) tcc_update(L, st);
+    if (L.use_tcc) tcc_update(L, D, st);
     softmin_run(L, D, rows_per_thread, st);
     if (timing) {
         OTGB_CUDA_TRY(cudaEventRecord(ev_pool[2 * ev_used + 1], st));
@@ -514,6 +514,7 @@ int otgb::solve_divergence(otgb_ctx *ctx, const float *x, const float *a, int N,
         s.translation = P.translation != 0;
         s.use_tc = P.precision == OTGB_TC_BF16X3 && D >= 16 && P.p == 2;
         s.use_tc3 = P.precision == OTGB_FP32 && D <= 3 && P.p == 2;
+        s.tcc_pieces = P.p != 2 || D <= 3 ? 0 : (s.use_tc ? 2 : (P.precision == OTGB_FP32 ? 3 : 0));
         cudaStream_t st = s.st;
         OTGB_CUDA_TRY(cudaEventRecord(ctx_event(ctx, 0), st));
 

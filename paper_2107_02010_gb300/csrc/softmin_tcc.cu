@@ -1,101 +1,62 @@
-// Cluster-tiled tensor-core form of the softmin sweep (16 <= D, D4 <= 60, coarse-to-fine solves): the
-// reduced-precision cross term of the tensor-core form, with the column operand prepared once per solve.
+// Cluster-tiled tensor-core form of the softmin sweep (D4 <= 60, coarse-to-fine solves): the column operand is
+// prepared once per solve and the CUDA cores evaluate only ex2 and the sum.
 //
 // In the kernel truncation of Section 2 every row block walks the columns of its kept column clusters J.
 // Centring the pair at the column cluster's centre c_J instead of at the row block's centre,
 //   -|x_i - y_j|^2 / 2 = (x_i - c_J) . yh_j - |x_i - c_J|^2 / 2 - |yh_j|^2 / 2,   yh_j = y_j - c_J,
-// makes the column operand yh_j independent of the row block: it is split into BF16 hi + lo once per solve
-// and stored in global memory as ready tiles of 128 columns in the canonical K-major layout of the tensor
-// core (tcc_build), so the kernel copies each tile with one bulk TMA copy and the CUDA cores do no column
-// work at all.  The rest of the exponent rides in the free K slots 60..63 (D4 <= 60):
-//   column slots: 60 = (H1 | H2 in the lo piece), 61 = H3, 62 = 1, 63 = 1,
-//                 H_j = s (eps log w_j + pot_j - |yh_j|^2 / 2) in three BF16 pieces (rewritten every step
-//                 by tcc_update);
-//   row slots:    60 = 1, 61 = 1, 62 = (R1 | R2 in the lo piece), 63 = R3,
-//                 R_iJ = -s |x_i - c_J|^2 / 2 - M_i in three pieces, M_i = -s old_i / lam,
-// so that the three products hi.hi + hi.lo + lo.hi of every K step leave in the accumulator
-//   e_ij = s (x_i - c_J) . yh_j + H_j + R_iJ = (exponent of the pair in base 2) - M_i,
-// and the finish takes M_i + log2 sum_j 2^e_ij in double.  The row operand s (x_i - c_J) (hi + lo, with
-// the R slots) is restaged once per kept cluster of the block.
+// makes the column operand yh_j independent of the row block: it is split into BF16 pieces once per solve and
+// stored in global memory as ready tiles of 128 columns (tcc_build), so the kernel brings each tile with one bulk
+// TMA copy.  The rest of the exponent rides in the last K slots (xtile.cuh):
+//   H_j  = s (eps log w_j + pot_j - |yh_j|^2 / 2) on the column side (rewritten every step by tcc_update),
+//   R_iJ = -s |x_i - c_J|^2 / 2 - M_i on the row side, M_i = -s old_i / lam,
+// so that the accumulator holds e_ij = (exponent of the pair in base 2) - M_i, and the finish takes
+// M_i + log2 sum_j 2^e_ij in double.  The row operand is restaged once per kept cluster of the block.
 //
-// One CTA (4 warps, one tensor-memory lane per row) owns a block of at most 128 rows.  Thread 0 issues the
-// bulk copies (two shared-memory stages of a 32 KiB tile: hi then lo) and the MMAs (two 128-column
-// accumulators), so that the MMA of tile k+1 runs while the CTA sums tile k; the threads hand an
-// accumulator back through an mbarrier, so the only CTA barriers are the restagings of the row operand.
-// Every wait is bounded; a timeout sets an error word and the kernel still releases its tensor memory.
+// Two pieces per operand (NP = 2) are the reduced-precision form (OTGB_TC_BF16X3); three (NP = 3) hold 24 bits and
+// are the float32 form of coarse-to-fine solves with k-means clusters: 6 x 2 K tensor flops per pair, where the
+// CUDA-core form (softmin_gen_kernel) needs D + 2 FP32 operations at a fiftieth of the rate.
+// Bound: the tensor pipe, 1910.7 TFLOP/s (measured) / (2 K x products) = 2.49e12 (NP = 3) and 4.98e12 (NP = 2)
+// pairs/s at K = 64.  Measured on the 60-D fiber bundles (300k and 1M per side): NP = 3 2.30e12 pairs/s = 92 %, where
+// softmin_gen_kernel has 3.9e11 (a solve of 300k per side 379 -> 76 ms); NP = 2 3.76e12 = 75 %, where the form with
+// the row operand in shared memory, one warp group for everything and two accumulators had 2.9e12.  Error of one
+// step of NP = 3 against FP64, geometric mean over D = 5 .. 60: 1.07e-7 of the duals, softmin_gen_kernel 1.28e-7.
+//
+// One CTA owns a block of at most 128 rows; two CTAs share an SM (256 tensor-memory columns and about 97 KB of
+// shared memory each), so that the MMAs of one run while the other sums.  Warps 0-3: one row per thread -- the row
+// operand into tensor memory, the sums; warp 4: one lane issues the bulk copies; warp 5: one lane issues the MMAs.
+// No CTA barrier after the setup: the roles hand tiles over through mbarriers.  Every wait is bounded; a timeout
+// sets an error word and the kernel still releases its tensor memory.
 #include <cfloat>
 #include <cmath>
 
-#include <cuda_bf16.h>
-
 #include "otgb_internal.cuh"
-#include "tcgen05.cuh"
+#include "xtile.cuh"
 
 namespace otgb {
 namespace {
 
-constexpr int kM = 128, kN = 128, kK = 64;
-constexpr int kPiece = kN * kK * 2;    // 16 KiB: one BF16 piece of a tile
-constexpr int kTile = 2 * kPiece;      // hi, then lo
-constexpr uint32_t kTmemCols = 256;    // two 128-column FP32 accumulators
+constexpr int kN = xt::kCols;
 constexpr int kMaxWords = kTccMaxWords;
+constexpr int kThreads = 192;
+constexpr int kStageBudget = 96 * 1024;  // shared memory for column tiles: two CTAs per SM
 
-struct TccSmem {
-    unsigned char a[2][kPiece];        // row operand: hi, lo
-    unsigned char b[2][kTile];         // two stages of column tiles
-    unsigned words[kMaxWords];         // kept column clusters of this block
-    unsigned long long mb_tma[2], mb_mma[2], mb_free[2];
-    uint32_t tslot;
-    int ncols;
+template <int NP, int K> struct Geom {
+    static constexpr int tile = xt::tile_bytes(NP, K);
+    static constexpr int st = kStageBudget / tile;
+    static constexpr int stages = st > 6 ? 6 : st;
+    // a second row operand where 256 tensor-memory columns hold it: the next cluster's rows are then staged while
+    // the MMAs of the current one run
+    static constexpr int abuf = kN + 2 * NP * (K / 2) <= (int)xt::kTmemCols ? 2 : 1;
+    static_assert(kN + NP * (K / 2) <= (int)xt::kTmemCols && stages >= 2, "tile does not fit");
 };
 
-__device__ __forceinline__ uint16_t bfbits(float v) { return __bfloat16_as_ushort(__float2bfloat16_rn(v)); }
-__device__ __forceinline__ float bfval(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
-__device__ __forceinline__ uint32_t pk(uint16_t lo, uint16_t hi) { return (uint32_t)lo | ((uint32_t)hi << 16); }
-constexpr uint16_t kOne = 0x3F80;  // 1.0 in BF16
-
-// v ~ h + m + l in BF16 (about 24 significant bits)
-__device__ __forceinline__ void split3(float v, uint16_t &h, uint16_t &m, uint16_t &l) {
-    h = bfbits(v);
-    const float r = v - bfval(h);
-    m = bfbits(r);
-    l = bfbits(r - bfval(m));
-}
-
-// Two values rounded to BF16 by one packed conversion (its own pipe, not the MUFU unit's): `hi` in the high
-// half, `lo` in the low half, each to nearest even as the scalar conversion rounds.
-__device__ __forceinline__ uint32_t bf2(float hi, float lo) {
-    uint32_t d;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-    return d;
-}
-
-// 8 consecutive values -> BF16 hi and lo parts as two 16-byte vectors (value 2q in the low half of word q)
-__device__ __forceinline__ void split8(const float (&v)[8], uint4 &hi, uint4 &lo) {
-    uint32_t h[4], l[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        h[q] = bf2(v[2 * q + 1], v[2 * q]);
-        l[q] = bf2(v[2 * q + 1] - __uint_as_float(h[q] & 0xFFFF0000u), v[2 * q] - __uint_as_float(h[q] << 16));
-    }
-    hi = make_uint4(h[0], h[1], h[2], h[3]);
-    lo = make_uint4(l[0], l[1], l[2], l[3]);
-}
-
-__device__ __forceinline__ float ex2f(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-__device__ __forceinline__ void tma_tile(void *dst, const void *src, unsigned long long *bar) {
-    const uint32_t b = tc::smem_u32(bar);
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(kTile) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     tc::smem_u32(dst)),
-                 "l"(src), "r"(kTile), "r"(b)
-                 : "memory");
-}
+struct TccCtl {
+    unsigned words[kMaxWords];  // kept column clusters of this block
+    unsigned long long full[6], empty[6], acc_full, acc_free, a_ready[2], drain;
+    uint32_t tslot;
+    int ncols;
+    int abort;
+};
 
 // Walks the tiles of the kept column clusters of a block in cluster order.
 struct TileIt {
@@ -122,36 +83,45 @@ __device__ __forceinline__ bool tile_next(TileIt &it, const unsigned *words, int
     }
 }
 
-__global__ void __launch_bounds__(128, 2) softmin_tcc_kernel(const __grid_constant__ SoftminLaunch L, int D4) {
+template <int NP, int K>
+__global__ void __launch_bounds__(kThreads, 2) softmin_tcc_kernel(const __grid_constant__ SoftminLaunch L, int D4) {
+    using G = Geom<NP, K>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    TccSmem &S = *reinterpret_cast<TccSmem *>(smem_raw);
-    const int t = threadIdx.x, warp = t >> 5;
+    unsigned char *tiles_s = smem_raw;  // stages
+    TccCtl &S = *reinterpret_cast<TccCtl *>(smem_raw + G::stages * G::tile);
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     int4 item = L.items[blockIdx.x];
     OTGB_DCLAMP(item.x, 0, L.n_inst);
     const SoftminInst &I = L.inst[item.x];
     const int blk = item.y;
     int r0 = I.blk_row0[blk], r1 = I.blk_row0[blk + 1];
     OTGB_DCLAMP(r0, 0, I.n_rows + 1);
-    OTGB_DCLAMP(r1, r0, min(I.n_rows, r0 + kM) + 1);
+    OTGB_DCLAMP(r1, r0, min(I.n_rows, r0 + xt::kRows) + 1);
     const int nr = r1 - r0;
     const float s = L.s;
     const int nwords = L.tcc_nwords;
+    volatile int *abort = &S.abort;
 
     // ---- kept column clusters of this block: union of its row clusters' keep bits
     const int cl0 = I.tcc_blk_cl[2 * blk], cl1 = I.tcc_blk_cl[2 * blk + 1];
     if (t == 0) {
         S.ncols = 0;
-        tc::mbar_init(&S.mb_tma[0], 1);
-        tc::mbar_init(&S.mb_tma[1], 1);
-        tc::mbar_init(&S.mb_mma[0], 1);
-        tc::mbar_init(&S.mb_mma[1], 1);
-        tc::mbar_init(&S.mb_free[0], kM);
-        tc::mbar_init(&S.mb_free[1], kM);
+        S.abort = 0;
+        for (int q = 0; q < G::stages; ++q) {
+            tc::mbar_init(&S.full[q], 1);
+            tc::mbar_init(&S.empty[q], 1);
+        }
+        tc::mbar_init(&S.acc_full, 1);
+        tc::mbar_init(&S.acc_free, 128);
+        tc::mbar_init(&S.a_ready[0], 128);
+        tc::mbar_init(&S.a_ready[1], 128);
+        tc::mbar_init(&S.drain, 1);
         tc::mbar_init_fence();
     }
+    if (warp == 5) tc::tmem_alloc(&S.tslot, xt::kTmemCols);
     __syncthreads();
     int ncols = 0;
-    for (int w = t; w < nwords; w += kM) {
+    for (int w = t; w < nwords; w += kThreads) {
         unsigned u = 0u;
         for (int c = cl0; c < cl1; ++c) u |= I.tcc_bits[(size_t)c * nwords + w];
         S.words[w] = u;
@@ -163,174 +133,129 @@ __global__ void __launch_bounds__(128, 2) softmin_tcc_kernel(const __grid_consta
     }
     if (ncols) atomicAdd(&S.ncols, ncols);
 
-    // ---- this thread's row: M_i = -s old_i / lam
+    // ---- this thread's row (its coordinates stay in registers): M_i = -s old_i / lam
     const bool valid = t < nr;
-    const float *xr = I.rows + (size_t)(r0 + (valid ? t : 0)) * D4;
     float Mi = 0.f;
-    if (valid) Mi = (float)(-(double)s * (double)I.row_old[r0 + t] / (double)I.lam);
-
-    // row operand for column cluster J: s (x - c_J) split hi / lo, R_iJ in slots 62, 63
-    const float4 *xr4 = reinterpret_cast<const float4 *>(xr);
-    auto stage_rows = [&](int J) {
-        const float4 *cj4 = reinterpret_cast<const float4 *>(I.tcc_ccen + (size_t)J * D4);
-        float sq = 0.f;
+    float x[K - 4];
+    if (warp < 4) {
+        const float4 *xr4 = reinterpret_cast<const float4 *>(I.rows + (size_t)(r0 + (valid ? t : 0)) * D4);
 #pragma unroll
-        for (int ch = 0; ch < 8; ++ch) {
-            float v[8];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int k4 = 2 * ch + h;
-                float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (valid && 4 * k4 < D4) {
-                    const float4 a = xr4[k4], c = cj4[k4];
-                    d = make_float4(a.x - c.x, a.y - c.y, a.z - c.z, a.w - c.w);
-                }
-                sq = fmaf(d.x, d.x, fmaf(d.y, d.y, fmaf(d.z, d.z, fmaf(d.w, d.w, sq))));
-                v[4 * h] = s * d.x;
-                v[4 * h + 1] = s * d.y;
-                v[4 * h + 2] = s * d.z;
-                v[4 * h + 3] = s * d.w;
-            }
-            uint4 hi, lo;
-            split8(v, hi, lo);
-            if (ch == 7) {
-                const float R = valid ? -0.5f * s * sq - Mi : 0.f;
-                uint16_t R1, R2, R3;
-                split3(R, R1, R2, R3);
-                hi.z = pk(kOne, kOne);
-                hi.w = pk(R1, R3);
-                lo.z = 0u;
-                lo.w = pk(R2, 0);
-            }
-            *reinterpret_cast<uint4 *>(S.a[0] + tc::core_off(t, 8 * ch)) = hi;
-            *reinterpret_cast<uint4 *>(S.a[1] + tc::core_off(t, 8 * ch)) = lo;
+        for (int q = 0; q < K / 4 - 1; ++q) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (valid && 4 * q < D4) v = xr4[q];
+            x[4 * q] = v.x;
+            x[4 * q + 1] = v.y;
+            x[4 * q + 2] = v.z;
+            x[4 * q + 3] = v.w;
         }
-    };
-
-    if (warp == 0) tc::tmem_alloc(&S.tslot, kTmemCols);
+        if (valid) Mi = (float)(-(double)s * (double)I.row_old[r0 + t] / (double)I.lam);
+    }
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
     const uint32_t tmem = S.tslot;
-    const uint32_t idesc = tc::idesc_bf16(kM, kN);
-    auto issue = [&](int buf) {  // tile in stage buf -> accumulator buf
-        const uint32_t d = tmem + (uint32_t)(buf * kN);
-        const uint32_t ah = tc::smem_u32(S.a[0]), al = tc::smem_u32(S.a[1]);
-        const uint32_t bh = tc::smem_u32(S.b[buf]), bl = bh + kPiece;
-#pragma unroll
-        for (int kk = 0; kk < kK / 16; ++kk) {
-            const uint32_t off = kk * 256;
-            tc::mma_bf16(d, tc::sdesc(ah + off), tc::sdesc(bh + off), idesc, kk > 0 ? 1u : 0u);
-            tc::mma_bf16(d, tc::sdesc(ah + off), tc::sdesc(bl + off), idesc, 1u);
-            tc::mma_bf16(d, tc::sdesc(al + off), tc::sdesc(bh + off), idesc, 1u);
-        }
-        tc::commit(&S.mb_mma[buf]);
-    };
-
     const int *tile0 = I.tcc_tile0;
-    const unsigned char *tiles = I.tcc_tiles;
-    bool ok = true;
     float tot = 0.f;
-    // bit b: parity of the next completion of stage b's copy / accumulator b's MMA / accumulator b's release
-    uint32_t ph_tma = 0u, ph_mma = 0u, ph_free = 0u;
-    TileIt itL, itM;
-    bool have = tile_next(itM, S.words, nwords, tile0);
-    if (t == 0) {
-        for (int q = 0; q < 2; ++q)
-            if (tile_next(itL, S.words, nwords, tile0)) tma_tile(S.b[q], tiles + (size_t)itL.g * kTile, &S.mb_tma[q]);
-    }
-    int aJ = -1;
-    if (have) {
-        stage_rows(itM.J);
-        aJ = itM.J;
-        tc::fence_proxy_async();
-        tc::fence_before();
-        __syncthreads();
-        tc::fence_after();
-        if (t == 0) {
-            if (!tc::mbar_wait(&S.mb_tma[0], ph_tma & 1u)) ok = false;
-            ph_tma ^= 1u;
+    bool ok = true;
+
+    if (warp == 4) {
+        // ---------------------------------------------------------- column tiles
+        if (lane == 0) {
+            TileIt it;
+            int k = 0;
+            while (tile_next(it, S.words, nwords, tile0)) {
+                const int st = k % G::stages;
+                if (k >= G::stages && !xt::wait(&S.empty[st], (uint32_t)((k / G::stages - 1) & 1), abort)) {
+                    *abort = 1;
+                    break;
+                }
+                xt::tma_load(tiles_s + st * G::tile, I.tcc_tiles + (size_t)it.g * G::tile, (uint32_t)G::tile, &S.full[st]);
+                ++k;
+            }
+            // nothing in flight at exit: the last copy into each stage has landed
+            for (int q = max(0, k - G::stages); q < k; ++q)
+                if (!tc::mbar_wait(&S.full[q % G::stages], (uint32_t)((q / G::stages) & 1))) *abort = 1;
+        }
+        __syncwarp();
+    } else if (warp == 5) {
+        // ------------------------------------------------------------------ MMAs
+        if (lane == 0) {
+            TileIt it;
+            int k = 0, aJ = -1, na = 0;  // na: row operands taken so far
+            while (tile_next(it, S.words, nwords, tile0)) {
+                const int st = k % G::stages;
+                if (it.J != aJ) {
+                    const int ab = na % G::abuf;
+                    if (!xt::wait(&S.a_ready[ab], (uint32_t)((na / G::abuf) & 1), abort)) {
+                        ok = false;
+                        break;
+                    }
+                    aJ = it.J;
+                    ++na;
+                }
+                if (!xt::wait(&S.full[st], (uint32_t)((k / G::stages) & 1), abort) ||
+                    (k >= 1 && !xt::wait(&S.acc_free, (uint32_t)((k - 1) & 1), abort))) {
+                    ok = false;
+                    break;
+                }
+                tc::fence_after();
+                const uint32_t a = tmem + kN + (uint32_t)(((na - 1) % G::abuf) * NP * (K / 2));
+                xt::issue<NP, K>(tmem, a, tc::smem_u32(tiles_s + st * G::tile), k & 1);
+                tc::commit(&S.empty[st]);
+                tc::commit(&S.acc_full);
+                ++k;
+            }
+            // nothing in flight at exit: every MMA issued completed
+            tc::commit(&S.drain);
+            if (!tc::mbar_wait(&S.drain, 0)) ok = false;
+            if (!ok) *abort = 1;
+        }
+        __syncwarp();
+    } else {
+        // --------------------------------------------------- row operands and sums
+        const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);
+        int na = 0;  // row operands staged so far
+        auto stage = [&](int J) {
+            const uint32_t a = lanes + kN + (uint32_t)((na % G::abuf) * NP * (K / 2));
+            xt::stage_row<NP, K>(x, D4, I.tcc_ccen + (size_t)J * D4, s, Mi, valid, a);
+            xt::st_wait();
+            tc::fence_before();
+            xt::arrive(&S.a_ready[na % G::abuf]);
+            ++na;
+        };
+        TileIt it;
+        bool have = tile_next(it, S.words, nwords, tile0);
+        if (have) stage(it.J);
+        for (int k = 0; have; ++k) {
+            TileIt nx = it;
+            const bool more = tile_next(nx, S.words, nwords, tile0);
+            const bool fresh = more && nx.J != it.J;
+            // the other row operand belongs to an earlier cluster, whose MMAs are complete: tile k - 1's are
+            if (G::abuf == 2 && fresh) stage(nx.J);
+            ok = __all_sync(0xffffffffu, xt::wait(&S.acc_full, (uint32_t)(k & 1), abort));
+            if (!ok) {  // tensor-memory loads are warp-collective
+                *abort = 1;
+                break;
+            }
             tc::fence_after();
-            issue(0);
-        }
-    }
-    int k = 0;
-    while (have) {
-        const int buf = k & 1, nb = buf ^ 1;
-        TileIt itN = itM;
-        const bool haveN = tile_next(itN, S.words, nwords, tile0);
-        if (haveN) {
-            if (itN.J != aJ) {
-                // the row operand changes: the MMA of tile k (the last one issued) must be done with it
-                if (!tc::mbar_wait(&S.mb_mma[buf], (ph_mma >> buf) & 1u)) ok = false;
-                tc::fence_after();
-                stage_rows(itN.J);
-                aJ = itN.J;
-                tc::fence_proxy_async();
+            tot = xt::sum_row(lanes, tot, [&] {
                 tc::fence_before();
-                __syncthreads();
-                tc::fence_after();
-            }
-            if (t == 0) {
-                if (k >= 1) {  // every thread has read accumulator nb (tile k-1)
-                    if (!tc::mbar_wait(&S.mb_free[nb], (ph_free >> nb) & 1u)) ok = false;
-                    ph_free ^= 1u << nb;
-                }
-                if (!tc::mbar_wait(&S.mb_tma[nb], (ph_tma >> nb) & 1u)) ok = false;
-                ph_tma ^= 1u << nb;
-                tc::fence_after();
-                issue(nb);
-            }
+                xt::arrive(&S.acc_free);
+            });
+            if (G::abuf == 1 && fresh) stage(nx.J);  // tile k was the cluster's last: its MMAs are complete
+            it = nx;
+            have = more;
         }
-        // sums of tile k
-        if (!tc::mbar_wait(&S.mb_mma[buf], (ph_mma >> buf) & 1u)) ok = false;
-        ph_mma ^= 1u << buf;
-        // stage buf is free (MMA k completed): the copy of tile k+2 starts before the sums
-        if (t == 0 && tile_next(itL, S.words, nwords, tile0))
-            tma_tile(S.b[buf], tiles + (size_t)itL.g * kTile, &S.mb_tma[buf]);
-        ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld below is warp-collective
-        tc::fence_after();
-        if (ok) {
-            const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * kN);
-            uint32_t va[32], vb[32];
-            auto sum32 = [&](const uint32_t (&v)[32]) {
-                float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll
-                for (int q = 0; q < 32; q += 4) {
-                    a0 += ex2f(__uint_as_float(v[q]));
-                    a1 += ex2f(__uint_as_float(v[q + 1]));
-                    a2 += ex2f(__uint_as_float(v[q + 2]));
-                    a3 += ex2f(__uint_as_float(v[q + 3]));
-                }
-                tot += (a0 + a1) + (a2 + a3);
-            };
-            tc::ld32_async(base, va);
-            tc::ld_wait(va);
-            tc::ld32_async(base + 32, vb);
-            sum32(va);
-            tc::ld_wait(vb);
-            tc::ld32_async(base + 64, va);
-            sum32(vb);
-            tc::ld_wait(va);
-            tc::ld32_async(base + 96, vb);
-            sum32(va);
-            tc::ld_wait(vb);
-            sum32(vb);
-        }
-        // accumulator buf is read: released to the MMA issuer without a CTA barrier
-        tc::fence_before();
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(&S.mb_free[buf])) : "memory");
-        itM = itN;
-        have = haveN;
-        ++k;
     }
-    // copies issued past the last tile: none (the loads walk the same sequence, two ahead, and stop at its end)
-    ok = __syncthreads_and(ok) != 0;
-    if (!ok && t == 0 && L.tc_err) atomicOr(L.tc_err, 1u);
+    tc::fence_before();
+    __syncthreads();
     tc::fence_after();
-    if (warp == 0) tc::tmem_dealloc(tmem, kTmemCols);
+    ok = S.abort == 0;
+    if (!ok && t == 0 && L.tc_err) atomicOr(L.tc_err, 1u);
+    if (warp == 5) tc::tmem_dealloc(tmem, xt::kTmemCols);
 
     if (t == 0 && L.pairs) atomicAdd(L.pairs, (unsigned long long)nr * (unsigned long long)S.ncols);
+    if (warp >= 4) return;
     float dmax = 0.f;
     if (valid && ok) {
         const int r = r0 + t;
@@ -349,42 +274,27 @@ __global__ void __launch_bounds__(128, 2) softmin_tcc_kernel(const __grid_consta
         }
     }
     for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-    if ((t & 31) == 0 && L.delta_max) atomicMax(L.delta_max, __float_as_uint(dmax));
+    if (lane == 0 && L.delta_max) atomicMax(L.delta_max, __float_as_uint(dmax));
 }
 
 // Column tiles of one side: tile g of cluster J = tile_cl[g] holds columns off[J] + 128 (g - tile0[J]) + c,
-// c < 128 (past the cluster's end: zero), centred at c_J and split hi / lo; half_norm = |yh|^2 / 2.
-// Written into `copies` buffers at once.
-__global__ void tcc_build_kernel(const float *pts, int D4, const int *off, const int *tile0, const int *tile_cl,
-                                 const float *cen, unsigned char *dst0, unsigned char *dst1, float *half_norm) {
+// c < 128 (past the cluster's end: zero), centred at c_J and split; half_norm = |yh|^2 / 2.  Written into both
+// copies (one per instance that uses the side as columns) at once.
+template <int NP, int K>
+__global__ void __launch_bounds__(kN) tcc_build_kernel(const float *pts, int D4, const int *off, const int *tile0,
+                                                       const int *tile_cl, const float *cen, unsigned char *dst0,
+                                                       unsigned char *dst1, float *half_norm) {
     const int g = blockIdx.x, c = threadIdx.x;
     const int J = tile_cl[g];
     const int j = off[J] + (g - tile0[J]) * kN + c;
     const bool ok = j < off[J + 1];
-    const float *y = pts + (size_t)(ok ? j : 0) * D4;
-    const float *cj = cen + (size_t)J * D4;
-    float sq = 0.f;
-    for (int ch = 0; ch < 8; ++ch) {
-        float v[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int k = 8 * ch + e;
-            v[e] = (ok && k < D4) ? y[k] - cj[k] : 0.f;
-            sq = fmaf(v[e], v[e], sq);
-        }
-        uint4 hi, lo;
-        split8(v, hi, lo);
-        unsigned char *t0 = dst0 + (size_t)g * kTile, *t1 = dst1 + (size_t)g * kTile;
-        *reinterpret_cast<uint4 *>(t0 + tc::core_off(c, 8 * ch)) = hi;
-        *reinterpret_cast<uint4 *>(t0 + kPiece + tc::core_off(c, 8 * ch)) = lo;
-        *reinterpret_cast<uint4 *>(t1 + tc::core_off(c, 8 * ch)) = hi;
-        *reinterpret_cast<uint4 *>(t1 + kPiece + tc::core_off(c, 8 * ch)) = lo;
-    }
-    half_norm[(size_t)g * kN + c] = 0.5f * sq;
+    const size_t o = (size_t)g * xt::tile_bytes(NP, K);
+    half_norm[(size_t)g * kN + c] = xt::build_col<NP, K>(pts + (size_t)(ok ? j : 0) * D4, cen + (size_t)J * D4, D4, ok, c,
+                                                         dst0 + o, dst1 + o);
 }
 
-// Per step: H_j = s (eps log w_j + pot_j - |yh_j|^2 / 2) in three BF16 pieces into slots 60..63 of the
-// column tiles of every instance (past a cluster's end, or for w_j = 0: a large negative H).
+// Per step: H_j = s (eps log w_j + pot_j - |yh_j|^2 / 2) into the column tiles of every instance (past a cluster's
+// end, or for w_j = 0: a large negative H).
 struct TccUpdate {
     unsigned char *tiles[kMaxInst];
     const float *half_norm[kMaxInst];
@@ -395,37 +305,81 @@ struct TccUpdate {
     float s, eps;
 };
 
-__global__ void tcc_update_kernel(const __grid_constant__ TccUpdate U) {
+template <int NP, int K> __global__ void tcc_update_kernel(const __grid_constant__ TccUpdate U) {
     const int q = blockIdx.y, c = threadIdx.x;
     for (int g = blockIdx.x; g < U.ntiles[q]; g += gridDim.x) {
         const int J = U.tile_cl[q][g];
         const int j = U.off[q][J] + (g - U.tile0[q][J]) * kN + c;
-        float H = -1e30f;
+        double H = -1e30;  // in double: three terms that cancel, once per column and step
         if (j < U.off[q][J + 1])
-            H = U.s * (fmaf(U.eps, U.logw[q][j], U.pot[q][j]) - U.half_norm[q][(size_t)g * kN + c]);
-        if (!(H > -1e30f)) H = -1e30f;  // zero weight (log w = -inf) or past the end
-        uint16_t h1, h2, h3;
-        split3(H, h1, h2, h3);
-        unsigned char *t0 = U.tiles[q] + (size_t)g * kTile;
-        *reinterpret_cast<uint2 *>(t0 + tc::core_off(c, 60)) = make_uint2(pk(h1, h3), pk(kOne, kOne));
-        *reinterpret_cast<uint2 *>(t0 + kPiece + tc::core_off(c, 60)) = make_uint2(pk(h2, 0), 0u);
+            H = (double)U.s * ((double)U.eps * U.logw[q][j] + (double)U.pot[q][j] - U.half_norm[q][(size_t)g * kN + c]);
+        xt::put_h<NP, K>(U.tiles[q] + (size_t)g * xt::tile_bytes(NP, K), c, H);
     }
 }
 
+// f.template operator()<NP, K>() for the run-time pieces and slots
+template <class F> void dispatch(int np, int K, F &&f) {
+    switch (np * 100 + K) {
+        case 232: f.template operator()<2, 32>(); break;
+        case 248: f.template operator()<2, 48>(); break;
+        case 264: f.template operator()<2, 64>(); break;
+        case 316: f.template operator()<3, 16>(); break;
+        case 332: f.template operator()<3, 32>(); break;
+        case 348: f.template operator()<3, 48>(); break;
+        case 364: f.template operator()<3, 64>(); break;
+        default: throw Error{OTGB_EINTERNAL, "cluster-tiled form: unsupported pieces or width"};
+    }
+}
+
+struct BuildFn {
+    const float *pts;
+    int D4;
+    const int *off, *tile0, *tile_cl;
+    int ntiles;
+    const float *cen;
+    unsigned char *dst0, *dst1;
+    float *half_norm;
+    cudaStream_t st;
+    template <int NP, int K> void operator()() const {
+        tcc_build_kernel<NP, K><<<ntiles, kN, 0, st>>>(pts, D4, off, tile0, tile_cl, cen, dst0, dst1, half_norm);
+    }
+};
+struct UpdateFn {
+    const TccUpdate &U;
+    dim3 grid;
+    cudaStream_t st;
+    template <int NP, int K> void operator()() const { tcc_update_kernel<NP, K><<<grid, kN, 0, st>>>(U); }
+};
+struct SweepFn {
+    const SoftminLaunch &L;
+    int D4;
+    cudaStream_t st;
+    template <int NP, int K> void operator()() const {
+        constexpr int bytes = Geom<NP, K>::stages * Geom<NP, K>::tile + (int)sizeof(TccCtl);
+        static_assert(2 * (bytes + 1024) <= 227 * 1024, "two CTAs per SM");
+        static PerDevice<int> attr;
+        attr.get([] {
+            OTGB_CUDA_TRY(cudaFuncSetAttribute(softmin_tcc_kernel<NP, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+            return 1;
+        });
+        softmin_tcc_kernel<NP, K><<<L.n_items, kThreads, bytes, st>>>(L, D4);
+    }
+};
+
 }  // namespace
 
-size_t tcc_tile_bytes() { return (size_t)kTile; }
+size_t tcc_tile_bytes(int np, int D4) { return (size_t)xt::tile_bytes(np, xt::k_slots(D4)); }
 
-void tcc_build_side(const float *pts, int D4, const int *d_off, const int *d_tile0, const int *d_tile_cl,
+void tcc_build_side(int np, const float *pts, int D4, const int *d_off, const int *d_tile0, const int *d_tile_cl,
                     int ntiles, const float *cen, unsigned char *dst0, unsigned char *dst1, float *half_norm,
                     cudaStream_t st) {
     require(D4 <= 60, "tcc_build_side: D4 must be <= 60", OTGB_EINTERNAL);
     if (ntiles <= 0) return;
-    tcc_build_kernel<<<ntiles, kN, 0, st>>>(pts, D4, d_off, d_tile0, d_tile_cl, cen, dst0, dst1, half_norm);
+    dispatch(np, xt::k_slots(D4), BuildFn{pts, D4, d_off, d_tile0, d_tile_cl, ntiles, cen, dst0, dst1, half_norm, st});
     OTGB_CHECK_LAUNCH();
 }
 
-void tcc_update(const SoftminLaunch &L, cudaStream_t st) {
+void tcc_update(const SoftminLaunch &L, int D, cudaStream_t st) {
     TccUpdate U;
     int mx = 0;
     for (int q = 0; q < kMaxInst; ++q) {
@@ -443,20 +397,14 @@ void tcc_update(const SoftminLaunch &L, cudaStream_t st) {
     U.s = L.s;
     U.eps = L.eps;
     if (mx <= 0) return;
-    tcc_update_kernel<<<dim3(std::min(mx, 65535), L.n_inst), kN, 0, st>>>(U);
+    dispatch(L.use_tcc, xt::k_slots((D + 3) & ~3), UpdateFn{U, dim3(std::min(mx, 65535), L.n_inst), st});
     OTGB_CHECK_LAUNCH();
 }
 
 void softmin_tcc_launch(const SoftminLaunch &L, int D, cudaStream_t st) {
     const int D4 = (D + 3) & ~3;
     require(D4 <= 60 && L.tcc_nwords <= kMaxWords, "softmin_tcc_launch: unsupported shape", OTGB_EINTERNAL);
-    static PerDevice<int> attr;
-    attr.get([] {
-        OTGB_CUDA_TRY(cudaFuncSetAttribute(softmin_tcc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)sizeof(TccSmem)));
-        return 1;
-    });
-    softmin_tcc_kernel<<<L.n_items, kM, sizeof(TccSmem), st>>>(L, D4);
+    dispatch(L.use_tcc, xt::k_slots(D4), SweepFn{L, D4, st});
     OTGB_CHECK_LAUNCH();
 }
 

@@ -49,7 +49,7 @@ void *Workspace::get(const std::string &name, size_t bytes) {
     for (auto &b : bufs)
         if (b.name == name) {
             if (b.bytes >= bytes) return b.ptr;
-            OTGB_CUDA_TRY(cudaFreeAsync(b.ptr, stream));
+            if (b.ptr) OTGB_CUDA_TRY(cudaFreeAsync(b.ptr, stream));  // null after a growth that failed
             b.ptr = nullptr;
             b.bytes = 0;
             const cudaError_t e = cudaMallocAsync(&b.ptr, bytes, stream);
@@ -64,6 +64,12 @@ void *Workspace::get(const std::string &name, size_t bytes) {
     b.bytes = bytes;
     bufs.push_back(b);
     return b.ptr;
+}
+
+size_t Workspace::held(const std::string &name) const {
+    for (auto &b : bufs)
+        if (b.name == name) return b.bytes;
+    return 0;
 }
 
 void Workspace::release() {

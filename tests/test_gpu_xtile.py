@@ -1,0 +1,57 @@
+"""One coarse-to-fine step of the cluster-tiled tensor-core form against the FP64 oracle's softmin, at the edges of
+its tiles: point widths around the K steps (4 .. 60 coordinates), clusters of one point, of a tile and one more, of
+less than a tile, and sizes that are no multiple of anything."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2107_02010_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+# the bars of the library: 1e-5 of the duals' scale in float32 (precision 0), 1e-3 in the reduced form (precision 1)
+BAR = {0: 1e-5, 1: 1e-3}
+
+
+def T(v):
+    return torch.from_numpy(np.ascontiguousarray(v)).cuda()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("D,n,m,K", [(4, 129, 257, 1), (5, 300, 260, 2), (12, 333, 290, 3), (13, 257, 128, 2),
+                                     (16, 128, 129, 1), (28, 400, 301, 3), (29, 333, 290, 40), (44, 300, 517, 4),
+                                     (45, 290, 333, 3), (60, 641, 500, 5), (60, 40, 37, 37), (60, 1, 200, 1)])
+def test_one_step_matches_the_oracle(D, n, m, K, prec):
+    from paper_2107_02010_gb300 import otgb
+
+    if prec == 1 and D < 16:
+        pytest.skip("the reduced-precision form needs D >= 16")
+    x = synth.fiber_bundles(n, seed=4, perturb=3.0)[0][:, :D].copy()
+    y = synth.fiber_bundles(m, seed=5)[0][:, :D].copy()
+    rng = np.random.default_rng(6)
+    a, b = (rng.uniform(0.5, 1.5, k).astype(np.float32) for k in (n, m))
+    a, b = a / a.sum(), b / b.sum()
+    b[0] = 0.0  # a column without weight
+    blur, reach = 2.0, 20.0
+    eps, lam = blur ** 2, 1.0 / (1.0 + blur ** 2 / reach ** 2)
+    # duals near a solution: the row shift is an estimate of the result, not the result
+    f, g, s, t = (np.zeros(k) for k in (n, m, n, m))
+    for _ in range(3):
+        f, g = oracle.softmin(x, y, b, g, eps, lam), oracle.softmin(y, x, a, f, eps, lam)
+        s, t = 0.5 * (s + oracle.softmin(x, x, a, s, eps, lam)), 0.5 * (t + oracle.softmin(y, y, b, t, eps, lam))
+    f, g, s, t = (v.astype(np.float32) for v in (f, g, s, t))
+    want = {"f": 0.5 * (f + oracle.softmin(x, y, b, g.astype(np.float64), eps, lam)),
+            "g": 0.5 * (g + oracle.softmin(y, x, a, f.astype(np.float64), eps, lam)),
+            "a_self": 0.5 * (s + oracle.softmin(x, x, a, s.astype(np.float64), eps, lam)),
+            "b_self": 0.5 * (t + oracle.softmin(y, y, b, t.astype(np.float64), eps, lam))}
+    ctx = otgb.Context()
+    dev = [T(v) for v in (f, g, s, t)]
+    p = otgb.default_params(blur=blur, reach=reach, multiscale=1, cluster=1, k_clusters=K, precision=prec,
+                            fixed_iters=1, max_iters=1, sigma_start=blur, translation=0, anderson=0,
+                            f_init=dev[0].data_ptr(), g_init=dev[1].data_ptr(), a_init=dev[2].data_ptr(),
+                            b_init=dev[3].data_ptr())
+    out = otgb.sinkhorn_divergence(ctx, T(x), T(a), T(y), T(b), p, want_self=True)
+    for k, w in want.items():
+        err = np.max(np.abs(out[k].cpu().numpy() - w)) / (np.max(np.abs(w)) + eps)
+        assert err < BAR[prec], (k, err)
+    ctx.close()
