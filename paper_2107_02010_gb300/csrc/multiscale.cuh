@@ -59,6 +59,7 @@ struct Solver {
     bool translation = false;
     bool use_tc = false;
     bool use_tc3 = false;
+    bool use_xd = false;
     int tcc_pieces = 0;  // BF16 pieces of the cluster-tiled form where it applies (2: reduced precision, 3: float32)
     std::vector<cudaEvent_t> ev_pool;
     int ev_used = 0;

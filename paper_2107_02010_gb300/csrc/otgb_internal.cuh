@@ -229,7 +229,8 @@ constexpr int kTccMaxWords = 256;  // column clusters of the cluster-tiled form:
 // partial sums (same per-row shift in every item) to
 // part[item * kPartRows + local row] and a finalize warp per block, listed in
 // fin as (inst, blk, first item, item count), sums them in a fixed order and
-// finishes the rows.  Only the D <= 3 kernel splits.
+// finishes the rows.  The D <= 3 kernels split, and softmin_xd_kernel (shift and sum per row: 2 kPartRows floats
+// per item).
 constexpr int kPartRows = 128;
 
 struct SoftminLaunch {
@@ -243,6 +244,7 @@ struct SoftminLaunch {
     int use_tc3;             // 1: D <= 3 exponent on the tensor cores (three-piece BF16, float32 accuracy)
     int use_tcc;             // 2 or 3: the cluster-tiled tensor-core form with that many BF16 pieces per operand
                              // (tcc_* fields of the instances); 0: not used
+    int use_xd;              // 1: 3 < D, D4 <= 60, dense columns: float32 on the tensor cores (softmin_xd.cu)
     int cost_p1;             // 1: cost |x - y| (p = 1, direct form, softmin_direct.cu); 0: |x - y|^2 / 2
     int direct;              // 1: the direct difference form for p = 2 as well (softmin_direct.cu)
     int tcc_nwords;          // words of keep bits per row cluster
@@ -273,6 +275,13 @@ void softmin_run(const SoftminLaunch &L, int D, int rows_per_thread, cudaStream_
 void softmin_direct_launch(const SoftminLaunch &L, int D, cudaStream_t st);
 // Tensor-core softmin (softmin_tc.cu), D >= 16, old values required, blocks <= 128 rows.
 void softmin_tc_launch(const SoftminLaunch &L, int D, cudaStream_t st);
+// Dense float32 softmin on the tensor cores (softmin_xd.cu), 3 < D, D4 <= 60, blocks <= 128 rows.  maxp: no old
+// values (or they are no estimate of the result); split blocks with item_fin / fin_count, part holding 2 kPartRows
+// floats per item.
+void softmin_xd_launch(const SoftminLaunch &L, int D, bool maxp, cudaStream_t st);
+// Columns per item for a launch over (number of blocks, columns of each) groups on a GPU of `sms` SMs.
+int xd_chunk(const std::vector<std::pair<long long, long long>> &blocks_cols, int sms);
+inline bool xd_width(int D) { return D > 3 && ((D + 3) & ~3) <= 60; }
 // Tensor-core D <= 3 softmin at float32 accuracy (softmin3_tc.cu): old values required,
 // blocks <= 128 rows, split blocks only with item_fin / fin_count.
 void softmin3_tc_launch(const SoftminLaunch &L, cudaStream_t st);

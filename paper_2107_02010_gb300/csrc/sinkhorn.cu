@@ -89,6 +89,16 @@ int *spatial_sort(otgb_ctx *ctx, const std::string &tag, const float *x, int n, 
     return perm;
 }
 
+// Work items of a one-instance sweep: block k's columns in `parts` pieces of `chunk` columns.
+__global__ void split_items_kernel(int4 *items, int *item_fin, int4 *fin, int nb, int n_in, int chunk, int parts) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= nb * parts) return;
+    const int k = e / parts, q = e - k * parts;
+    items[e] = make_int4(0, k, q * chunk, q + 1 < parts ? (q + 1) * chunk : n_in);
+    if (item_fin) item_fin[e] = k;
+    if (fin && q == 0) fin[k] = make_int4(0, k, e, parts);
+}
+
 // The bounded-wait error path, exercised on purpose (params.debug_wait_probe):
 // one thread polls a device word that nothing writes, pausing between polls,
 // and gives up after `polls` polls by flagging the error word that the
@@ -221,7 +231,7 @@ void Solver::setup_dense_instances(int block_rows) {
     std::vector<std::vector<int>> ncols(4);
     const int rows_x[4] = {1, 0, 0, 1};
     for (int k = 0; k < 4; ++k) ncols[k].assign(rows_x[k] ? nblk_x : nblk_y, launch.inst[k].n_cols);
-    set_work(ncols, D <= 3 && p == 2);
+    set_work(ncols, p == 2 && (D <= 3 || launch.use_xd));
 }
 
 // Items (inst, blk, cb, ce): a block's columns are cut into chunks of CH
@@ -241,7 +251,12 @@ void Solver::set_work(const std::vector<std::vector<int>> &ncols, bool allow_spl
     // tensor-core form: one CTA per item, fewer and longer items
     const double target = use_tc3 ? OTGB_TC3_ITEMS_PER_SM * sms : 3.0 * 5.0 * 4.0 * sms;
     int CH = 1 << 30;
-    if (allow_split) {
+    if (allow_split && D > 3) {  // softmin_xd_kernel
+        std::vector<std::pair<long long, long long>> groups;
+        for (auto &v : ncols)
+            if (!v.empty()) groups.push_back({(long long)v.size(), v[0]});  // dense: the same for every block
+        CH = xd_chunk(groups, sms);
+    } else if (allow_split) {
         CH = (int)std::ceil(W / target);
         CH = std::max(512, (CH + 127) / 128 * 128);
     }
@@ -276,7 +291,7 @@ void Solver::set_work(const std::vector<std::vector<int>> &ncols, bool allow_spl
     if (split) {
         int4 *d_fin = ws->get<int4>(nm("fin"), fin.size() + 1);
         OTGB_CUDA_TRY(cudaMemcpyAsync(d_fin, fin.data(), fin.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-        launch.part = ws->get<float>(nm("part"), items.size() * (size_t)kPartRows);
+        launch.part = ws->get<float>(nm("part"), items.size() * (size_t)kPartRows * (D > 3 ? 2 : 1));
         launch.fin = d_fin;
         launch.n_fin = (int)fin.size();
         int *d_ifin = ws->get<int>(nm("itemfin"), items.size() + 1);
@@ -302,6 +317,7 @@ void Solver::alloc_common() {
     OTGB_CUDA_TRY(cudaMemsetAsync(launch.tc_err, 0, sizeof(unsigned), st));
     launch.use_tc = use_tc ? 1 : 0;
     launch.use_tc3 = use_tc3 ? 1 : 0;
+    launch.use_xd = use_xd ? 1 : 0;
     launch.cost_p1 = p == 1 ? 1 : 0;
     OTGB_CUDA_TRY(cudaMemsetAsync(d_fb_total, 0, sizeof(unsigned long long), st));
     OTGB_CUDA_TRY(cudaMemsetAsync(d_pairs, 0, sizeof(unsigned long long), st));
@@ -514,6 +530,7 @@ int otgb::solve_divergence(otgb_ctx *ctx, const float *x, const float *a, int N,
         s.translation = P.translation != 0;
         s.use_tc = P.precision == OTGB_TC_BF16X3 && D >= 16 && P.p == 2;
         s.use_tc3 = P.precision == OTGB_FP32 && D <= 3 && P.p == 2;
+        s.use_xd = P.precision == OTGB_FP32 && P.p == 2 && xd_width(D);
         s.tcc_pieces = P.p != 2 || D <= 3 ? 0 : (s.use_tc ? 2 : (P.precision == OTGB_FP32 ? 3 : 0));
         cudaStream_t st = s.st;
         OTGB_CUDA_TRY(cudaEventRecord(ctx_event(ctx, 0), st));
@@ -621,6 +638,10 @@ int otgb::solve_divergence(otgb_ctx *ctx, const float *x, const float *a, int N,
             // polish: the same loop on the direct difference form of the cost (see otgb_params.polish)
             s.launch.direct = 1;
             s.launch.use_tcc = 0;
+            if (s.launch.part) {  // the direct form takes whole blocks
+                const std::vector<std::vector<int>> nc = s.work_ncols;
+                s.set_work(nc, false);
+            }
             s.no_progress = 0;
             s.floor_hits = 0;
             s.delta_best = 1e300;
@@ -757,10 +778,14 @@ extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const floa
         const int block_rows = D <= 3 ? 32 * rpt : 128;
         int *blk = ws.get<int>("sm:blk", n_out / block_rows + 2);
         const int nb = uniform_blocks(blk, n_out, block_rows, st);
-        std::vector<int4> items(nb);
-        for (int k = 0; k < nb; ++k) items[k] = make_int4(0, k, 0, n_in);
-        int4 *d_items = ws.get<int4>("sm:items", nb);
-        OTGB_CUDA_TRY(cudaMemcpyAsync(d_items, items.data(), nb * sizeof(int4), cudaMemcpyHostToDevice, st));
+        const bool xd = xd_width(D);
+        const int chunk = xd ? xd_chunk({{nb, n_in}}, ctx_sm_count(ctx)) : n_in;
+        const int parts = (n_in - 1) / chunk + 1, n_items = nb * parts;
+        int4 *d_items = ws.get<int4>("sm:items", n_items);
+        int4 *d_fin = parts > 1 ? ws.get<int4>("sm:fin", nb) : nullptr;
+        int *d_ifin = parts > 1 ? ws.get<int>("sm:ifin", n_items) : nullptr;
+        split_items_kernel<<<(n_items + 255) / 256, 256, 0, st>>>(d_items, d_ifin, d_fin, nb, n_in, chunk, parts);
+        OTGB_CHECK_LAUNCH();
         SoftminLaunch L;
         std::memset(&L, 0, sizeof(L));
         L.n_inst = 1;
@@ -769,7 +794,15 @@ extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const floa
         I.n_rows = n_out; I.n_cols = n_in; I.lam = (float)lam; I.omega = (float)omega;
         I.blk_row0 = blk;
         L.items = d_items;
-        L.n_items = nb;
+        L.n_items = n_items;
+        L.use_xd = xd ? 1 : 0;
+        if (parts > 1) {
+            L.part = ws.get<float>("sm:part", (size_t)n_items * kPartRows * 2);
+            L.fin = d_fin;
+            L.n_fin = nb;
+            L.item_fin = d_ifin;
+            L.fin_count = ws.get<int>("sm:fincnt", nb);
+        }
         L.exact_max = 1;  // `old` is a blend target here, not an estimate of the result
         L.eps = (float)eps;
         L.s = (float)(1.4426950408889634 / eps);
@@ -779,7 +812,7 @@ extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const floa
         L.n_fallback = ws.get<int>("sm:nfb", 1);
         L.fallback_cap = cap;
         softmin_run(L, D, rpt, st);
-        OTGB_CUDA_TRY(cudaStreamSynchronize(st));  // the host item vector is released here
+        OTGB_CUDA_TRY(cudaStreamSynchronize(st));
         return OTGB_OK;
     } catch (const Error &e) {
         return fail(ctx, e);

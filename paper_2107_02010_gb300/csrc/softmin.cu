@@ -960,8 +960,11 @@ void softmin_run(const SoftminLaunch &L, int D, int rows_per_thread, cudaStream_
     // the first-pass maximum is needed when some instance has no old value
     bool two = L.exact_max != 0;
     for (int k = 0; k < L.n_inst; ++k) two = two || (L.inst[k].row_old == nullptr);
-    require(!(two && L.part), "softmin_run: split blocks need old values", OTGB_EINTERNAL);
-    require(!(D > 3 && L.part), "softmin_run: split blocks are D <= 3 only", OTGB_EINTERNAL);
+    // the float32 form of dense sweeps in more than 3 dimensions
+    bool xd = L.use_xd && xd_width(D) && !L.use_tcc;
+    for (int k = 0; k < L.n_inst; ++k) xd = xd && L.inst[k].col_rng == nullptr;
+    require(!(two && L.part && !xd), "softmin_run: split blocks need old values", OTGB_EINTERNAL);
+    require(!(D > 3 && L.part && !xd), "softmin_run: split blocks are D <= 3 only", OTGB_EINTERNAL);
     if (D <= 3 && L.use_tc3 && !two && rows_per_thread <= 4 && (!L.part || L.fin_count)) {
         if (L.part) OTGB_CUDA_TRY(cudaMemsetAsync(L.fin_count, 0, sizeof(int) * L.n_fin, st));
         softmin3_tc_launch(L, st);
@@ -997,7 +1000,10 @@ void softmin_run(const SoftminLaunch &L, int D, int rows_per_thread, cudaStream_
             OTGB_CUDA_TRY(cudaFuncSetAttribute(softmin_gen_kernel<true, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
             return 1;
         });
-        if (two) {
+        if (xd) {
+            if (L.part) OTGB_CUDA_TRY(cudaMemsetAsync(L.fin_count, 0, sizeof(int) * L.n_fin, st));
+            softmin_xd_launch(L, D, two, st);
+        } else if (two) {
             softmin_gen_kernel<true, 0><<<L.n_items, kNTg, sizeof(GenSmem), st>>>(L, D, D4);
             OTGB_CHECK_LAUNCH();
         } else if (L.use_tcc) {

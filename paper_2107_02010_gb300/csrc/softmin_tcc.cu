@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kN) tcc_build_kernel(const float *pts, int D4,
     const int j = off[J] + (g - tile0[J]) * kN + c;
     const bool ok = j < off[J + 1];
     const size_t o = (size_t)g * xt::tile_bytes(NP, K);
-    half_norm[(size_t)g * kN + c] = xt::build_col<NP, K>(pts + (size_t)(ok ? j : 0) * D4, cen + (size_t)J * D4, D4, ok, c,
+    half_norm[(size_t)g * kN + c] = xt::build_col<NP, K, double>(pts + (size_t)(ok ? j : 0) * D4, cen + (size_t)J * D4, D4, ok, c,
                                                          dst0 + o, dst1 + o);
 }
 
@@ -313,7 +313,7 @@ template <int NP, int K> __global__ void tcc_update_kernel(const __grid_constant
         double H = -1e30;  // in double: three terms that cancel, once per column and step
         if (j < U.off[q][J + 1])
             H = (double)U.s * ((double)U.eps * U.logw[q][j] + (double)U.pot[q][j] - U.half_norm[q][(size_t)g * kN + c]);
-        xt::put_h<NP, K>(U.tiles[q] + (size_t)g * xt::tile_bytes(NP, K), c, H);
+        xt::put_h<NP, K>(U.tiles[q] + (size_t)g * xt::tile_bytes(NP, K), c, (float)H, (float)(H - (double)(float)H));
     }
 }
 

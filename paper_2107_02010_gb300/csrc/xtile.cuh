@@ -195,24 +195,27 @@ __device__ __forceinline__ void stage_row(const float (&x)[K - 4], int D4, const
 }
 
 // Column c of a tile: the point y centred at `cen` in NP pieces into `dst` (and `dst2` when non-null); the folded
-// H slots are left 0 (put_h writes them), the ones are set.  Returns |y - cen|^2 / 2 (summed in double, once per
-// solve: it enters every exponent of the column).
-template <int NP, int K>
+// H slots are left 0 (put_h writes them), the ones are set.  Returns |y - cen|^2 / 2, summed in Acc: double where a
+// tile is built once per solve, float (four short chains) where it is built per row block.
+template <int NP, int K, class Acc>
 __device__ __forceinline__ float build_col(const float *y, const float *cen, int D4, bool ok, int c, unsigned char *dst,
                                            unsigned char *dst2) {
     const float4 *y4 = reinterpret_cast<const float4 *>(y), *c4 = reinterpret_cast<const float4 *>(cen);
-    double sq = 0.0;
+    Acc s0 = 0, s1 = 0, s2 = 0, s3 = 0;
 #pragma unroll
     for (int ch = 0; ch < K / 8; ++ch) {
         uint32_t w[NP][4];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (ok && 8 * ch + 4 * h < D4) {
+            if (8 * ch + 4 * h < K - 4 && ok && 8 * ch + 4 * h < D4) {
                 const float4 u = y4[2 * ch + h], cc = c4[2 * ch + h];
                 d = make_float4(u.x - cc.x, u.y - cc.y, u.z - cc.z, u.w - cc.w);
             }
-            sq += ((double)d.x * d.x + (double)d.y * d.y) + ((double)d.z * d.z + (double)d.w * d.w);
+            s0 += (Acc)d.x * d.x;
+            s1 += (Acc)d.y * d.y;
+            s2 += (Acc)d.z * d.z;
+            s3 += (Acc)d.w * d.w;
             uint32_t p[NP], r[NP];
             split2<NP>(d.x, d.y, p);
             split2<NP>(d.z, d.w, r);
@@ -233,14 +236,17 @@ __device__ __forceinline__ float build_col(const float *y, const float *cen, int
             if (dst2) *reinterpret_cast<uint4 *>(dst2 + q * piece_bytes(K) + off(K, c, 8 * ch)) = u;
         }
     }
-    return (float)(0.5 * sq);
+    return (float)((Acc)0.5 * ((s0 + s1) + (s2 + s3)));
 }
 
-// H of column c of a tile (three BF16 pieces)
-template <int NP, int K> __device__ __forceinline__ void put_h(unsigned char *tile, int c, double H) {
-    if (!(H > -1e30)) H = -1e30;  // zero weight (log w = -inf), NaN, or past the end
+// H + rest of column c of a tile (three BF16 pieces)
+template <int NP, int K> __device__ __forceinline__ void put_h(unsigned char *tile, int c, float H, float rest) {
+    if (H <= -1e30f) {  // zero weight (log w = -inf) or past the end; NaN and +inf go on and make the row's sum NaN
+        H = -1e30f;
+        rest = 0.f;
+    }
     uint16_t h1, h2, h3;
-    split3((float)H, (float)(H - (double)(float)H), h1, h2, h3);
+    split3(H, rest, h1, h2, h3);
     if constexpr (NP == 3) {
         *reinterpret_cast<uint32_t *>(tile + off(K, c, K - 2)) = pk(h1, kOne);
         *reinterpret_cast<uint32_t *>(tile + piece_bytes(K) + off(K, c, K - 2)) = pk(h2, 0);
@@ -249,6 +255,16 @@ template <int NP, int K> __device__ __forceinline__ void put_h(unsigned char *ti
         *reinterpret_cast<uint2 *>(tile + off(K, c, K - 4)) = make_uint2(pk(h1, h3), pk(kOne, kOne));
         *reinterpret_cast<uint2 *>(tile + piece_bytes(K) + off(K, c, K - 4)) = make_uint2(pk(h2, 0), 0u);
     }
+}
+
+// H = s (eps lw + pot - hn) with what its three roundings lose (products and sums with their exact errors)
+template <int NP, int K>
+__device__ __forceinline__ void put_h_sum(unsigned char *tile, int c, float s, float eps, float lw, float pot, float hn) {
+    const float p = eps * lw, pe = fmaf(eps, lw, -p);
+    const float a = p + pot, ab = a - p, ae = (p - (a - ab)) + (pot - ab);
+    const float u = a - hn, ub = u - a, ue = (a - (u - ub)) - (hn + ub);
+    const float H = s * u;
+    put_h<NP, K>(tile, c, H, fmaf(s, u, -H) + s * ((pe + ae) + ue));
 }
 
 // ---- bulk copies and bounded waits
@@ -308,6 +324,47 @@ template <class F> __device__ __forceinline__ float sum_row(uint32_t base, float
     freed();
     sum32(vb);
     return tot;
+}
+
+// The same without a known shift: the row's sum is tot 2^sh.  Per 32 columns the maximum; where it passes the shift by
+// 30 binades the sum is rescaled to it (rare after the first columns, so the branch is cheap).
+template <class F> __device__ __forceinline__ void sum_row_max(uint32_t base, float &tot, float &sh, F &&freed) {
+    uint32_t va[32], vb[32];
+    auto sum32 = [&](const uint32_t (&v)[32]) {
+        float m0 = __uint_as_float(v[0]), m1 = __uint_as_float(v[1]);
+#pragma unroll
+        for (int q = 2; q < 32; q += 2) {
+            m0 = fmaxf(m0, __uint_as_float(v[q]));
+            m1 = fmaxf(m1, __uint_as_float(v[q + 1]));
+        }
+        m0 = fmaxf(m0, m1);
+        if (m0 > sh + 30.f) {
+            tot *= ex2(sh - m0);
+            sh = m0;
+        }
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+        for (int q = 0; q < 32; q += 4) {
+            a0 += ex2(__uint_as_float(v[q]) - sh);
+            a1 += ex2(__uint_as_float(v[q + 1]) - sh);
+            a2 += ex2(__uint_as_float(v[q + 2]) - sh);
+            a3 += ex2(__uint_as_float(v[q + 3]) - sh);
+        }
+        tot += (a0 + a1) + (a2 + a3);
+    };
+    tc::ld32_async(base, va);
+    tc::ld_wait(va);
+    tc::ld32_async(base + 32, vb);
+    sum32(va);
+    tc::ld_wait(vb);
+    tc::ld32_async(base + 64, va);
+    sum32(vb);
+    tc::ld_wait(va);
+    tc::ld32_async(base + 96, vb);
+    sum32(va);
+    tc::ld_wait(vb);
+    freed();
+    sum32(vb);
 }
 
 }  // namespace xt

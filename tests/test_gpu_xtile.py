@@ -1,6 +1,6 @@
-"""One coarse-to-fine step of the cluster-tiled tensor-core form against the FP64 oracle's softmin, at the edges of
-its tiles: point widths around the K steps (4 .. 60 coordinates), clusters of one point, of a tile and one more, of
-less than a tile, and sizes that are no multiple of anything."""
+"""The tensor-core tiles of D > 3 against the FP64 oracle's softmin, at the edges of the tiles: point widths around the
+K steps (4 .. 60 coordinates), sizes of one point, of a tile and one more, of less than a tile, of no multiple of
+anything.  One coarse-to-fine step of the cluster-tiled form, and the dense sweep with its running shift."""
 import numpy as np
 import pytest
 import torch
@@ -54,4 +54,37 @@ def test_one_step_matches_the_oracle(D, n, m, K, prec):
     for k, w in want.items():
         err = np.max(np.abs(out[k].cpu().numpy() - w)) / (np.max(np.abs(w)) + eps)
         assert err < BAR[prec], (k, err)
+    ctx.close()
+
+
+@pytest.mark.parametrize("D,n,m", [(4, 1, 129), (5, 300, 1), (12, 129, 4000), (13, 257, 128), (16, 128, 127),
+                                   (29, 130, 1025), (44, 64, 3001), (45, 290, 333), (60, 641, 2500), (60, 3000, 37)])
+def test_dense_sweep_matches_the_oracle(D, n, m):
+    from paper_2107_02010_gb300 import otgb
+
+    q = synth.fiber_bundles(n, seed=4, perturb=3.0)[0][:, :D].copy()
+    p = synth.fiber_bundles(m, seed=5)[0][:, :D].copy()
+    rng = np.random.default_rng(7)
+    w = rng.uniform(0.5, 1.5, m).astype(np.float32) / m
+    if m > 1:
+        w[rng.integers(0, m)] = 0.0
+    eps, lam = 4.0, 1.0 / 1.01
+    ctx = otgb.Context()
+    # potentials of a few eps, and potentials that climb by 600 binades over the columns (the shift has to follow)
+    for pot in (rng.normal(0.0, 12.0, m), np.linspace(-2000.0, 0.0, m)):
+        pot = pot.astype(np.float32)
+        old = rng.normal(0.0, 12.0, n).astype(np.float32)
+        tilde = oracle.softmin(q, p, w, pot.astype(np.float64), eps, lam)
+        for o, want in ((None, tilde), (old, 0.5 * (old + tilde))):
+            got = otgb.softmin(ctx, T(q), T(p), T(w), T(pot), eps, lam=lam, old=None if o is None else T(o))
+            err = np.max(np.abs(got.cpu().numpy() - want)) / (np.max(np.abs(want)) + eps)
+            assert err < BAR[0], (err, o is None)
+    # nothing but one column carries weight; and no finite answer where a potential is not finite
+    w1 = np.zeros(m, np.float32)
+    w1[m // 2] = 1.0
+    want = oracle.softmin(q, p, w1, pot.astype(np.float64), eps, lam)
+    got = otgb.softmin(ctx, T(q), T(p), T(w1), T(pot), eps, lam=lam).cpu().numpy()
+    assert np.max(np.abs(got - want)) < BAR[0] * (np.max(np.abs(want)) + eps)
+    pot[m // 2] = np.nan
+    assert not np.any(np.isfinite(otgb.softmin(ctx, T(q), T(p), T(w1), T(pot), eps, lam=lam).cpu().numpy()))
     ctx.close()
