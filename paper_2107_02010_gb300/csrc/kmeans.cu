@@ -19,69 +19,117 @@ constexpr int kAT = 256;   // threads
 constexpr int kAR = 128;   // points per CTA
 constexpr int kAC = 64;    // centroids per tile
 
-// Nearest centroid by argmin_k (|c_k|^2 - 2 x.c_k): each thread keeps 8 points
-// x 4 centroids of dot products, register-tiled like a GEMM.
+// Nearest centroid by argmin_k (|c_k|^2 - 2 x.c_k): each thread keeps 8 points x 4 centroids of dot products,
+// register-tiled like a GEMM.  The four centroids go in pairs through packed f32x2 FMAs (each half is the scalar chain
+// over the coordinates, so the result does not change), the point operand is stored twice per value so that one
+// 16-byte load feeds two packed operands; the next centroid tile is fetched into registers while this one is
+// multiplied, and |c_k|^2 comes from a launch of its own (64 threads computing it per tile left the others waiting).
+// Bound: FP32 FMA, n K D lane operations.
 struct AssignSmem {
-    float xs[64][kAR];
-    float cs[64][kAC];
-    float cn[kAC];
+    float2 xs[64][kAR];         // (v, v)
+    float cs[2][64][kAC];
+    float cn[2][kAC];
     float bd[16][kAR];
     int bk[16][kAR];
 };
 
-__global__ void __launch_bounds__(kAT) kmeans_assign_kernel(const float *x, int n, int D, int D4, const float *cent,
-                                                            int K, int *labels) {
+__device__ __forceinline__ unsigned long long fma2k(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+__global__ void centroid_norm_kernel(const float *cent, int K, int D4, float *cn) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= K) return;
+    const float4 *c4 = reinterpret_cast<const float4 *>(cent + (size_t)k * D4);
+    float acc = 0.f;
+#pragma unroll 8
+    for (int q = 0; q < D4 / 4; ++q) {
+        const float4 v = c4[q];
+        acc = fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.y, v.y, fmaf(v.x, v.x, acc))));
+    }
+    cn[k] = acc;
+}
+
+__global__ void __launch_bounds__(kAT, 2) kmeans_assign_kernel(const float *x, int n, int D, int D4, const float *cent,
+                                                               const float *cnorm, int K, int *labels) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     AssignSmem &S = *reinterpret_cast<AssignSmem *>(smem_raw);
     const int t = threadIdx.x, r0 = blockIdx.x * kAR;
     for (int e = t; e < kAR * D4; e += kAT) {
         const int r = e / D4, k = e - r * D4;
-        S.xs[k][r] = (r0 + r < n && k < D) ? x[(size_t)(r0 + r) * D + k] : 0.f;
+        const float v = (r0 + r < n && k < D) ? x[(size_t)(r0 + r) * D + k] : 0.f;
+        S.xs[k][r] = make_float2(v, v);
     }
+    // centroid tile: thread (centroid t % 64, quads t / 64, + 4, ..) moves up to four 16-byte pieces
+    const int cc = t & 63, q0 = t >> 6, Q = D4 >> 2;
+    float4 pre[4];
+    float pn = INFINITY;
+    auto fetch = [&](int c0) {
+        const bool in = c0 + cc < K;
+        const float4 *src = reinterpret_cast<const float4 *>(cent + (size_t)(in ? c0 + cc : 0) * D4);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int q = q0 + 4 * u;
+            pre[u] = in && q < Q ? src[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        if (q0 == 0) pn = in ? cnorm[c0 + cc] : INFINITY;
+    };
+    auto store = [&](int buf) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int q = q0 + 4 * u;
+            if (q < Q) {
+                S.cs[buf][4 * q][cc] = pre[u].x;
+                S.cs[buf][4 * q + 1][cc] = pre[u].y;
+                S.cs[buf][4 * q + 2][cc] = pre[u].z;
+                S.cs[buf][4 * q + 3][cc] = pre[u].w;
+            }
+        }
+        if (q0 == 0) S.cn[buf][cc] = pn;
+    };
     const int tr = t >> 4, tc = t & 15;
     float best[8];
     int bidx[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) { best[i] = INFINITY; bidx[i] = 0x7fffffff; }
-    for (int c0 = 0; c0 < K; c0 += kAC) {
-        __syncthreads();
-        for (int e = t; e < kAC * D4; e += kAT) {
-            const int c = e / D4, k = e - c * D4;
-            S.cs[k][c] = (c0 + c < K && k < D) ? cent[(size_t)(c0 + c) * D4 + k] : 0.f;
-        }
-        __syncthreads();
-        if (t < kAC) {
-            float acc = 0.f;
-            for (int k = 0; k < D4; ++k) acc = fmaf(S.cs[k][t], S.cs[k][t], acc);
-            S.cn[t] = (c0 + t < K) ? acc : INFINITY;
-        }
-        __syncthreads();
-        float acc[8][4];
+    fetch(0);
+    store(0);
+    __syncthreads();
+    int buf = 0;
+    for (int c0 = 0; c0 < K; c0 += kAC, buf ^= 1) {
+        if (c0 + kAC < K) fetch(c0 + kAC);
+        unsigned long long acc[8][2];
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+        for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = 0ull;
+#pragma unroll 4
         for (int k = 0; k < D4; ++k) {
-            const float4 xa = *reinterpret_cast<const float4 *>(&S.xs[k][tr * 8]);
-            const float4 xb = *reinterpret_cast<const float4 *>(&S.xs[k][tr * 8 + 4]);
-            const float4 cv = *reinterpret_cast<const float4 *>(&S.cs[k][tc * 4]);
-            const float xv[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
-            const float cc[4] = {cv.x, cv.y, cv.z, cv.w};
+            const ulonglong2 cv = *reinterpret_cast<const ulonglong2 *>(&S.cs[buf][k][tc * 4]);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xv[i], cc[j], acc[i][j]);
+            for (int h = 0; h < 4; ++h) {
+                const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(&S.xs[k][tr * 8 + 2 * h]);
+                acc[2 * h][0] = fma2k(xv.x, cv.x, acc[2 * h][0]);
+                acc[2 * h][1] = fma2k(xv.x, cv.y, acc[2 * h][1]);
+                acc[2 * h + 1][0] = fma2k(xv.y, cv.x, acc[2 * h + 1][0]);
+                acc[2 * h + 1][1] = fma2k(xv.y, cv.y, acc[2 * h + 1][1]);
+            }
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int c = c0 + tc * 4 + j;
-            const float cn = S.cn[tc * 4 + j];
+            const float cn = S.cn[buf][tc * 4 + j];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const float d = fmaf(-2.f, acc[i][j], cn);
+                const unsigned long long w = acc[i][j >> 1];
+                const float dot = __uint_as_float((j & 1) ? (unsigned)(w >> 32) : (unsigned)w);
+                const float d = fmaf(-2.f, dot, cn);
                 if (d < best[i] || (d == best[i] && c < bidx[i])) { best[i] = d; bidx[i] = c; }
             }
         }
+        // the other buffer was read before the last barrier
+        if (c0 + kAC < K) store(buf ^ 1);
+        __syncthreads();
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) { S.bd[tc][tr * 8 + i] = best[i]; S.bk[tc][tr * 8 + i] = bidx[i]; }
@@ -118,11 +166,23 @@ __global__ void kmeans_segment_mean_kernel(const float *x, const float *w, int D
     const int k = blockIdx.x, t = threadIdx.x, d = t & 63, g = t >> 6;
     const int a = off[k], b = off[k + 1];
     float s = 0.f, m = 0.f;
-    for (int i = a + g; i < b; i += 4) {
-        const int src = perm[i];
-        const float wi = w ? w[src] : 1.f;
-        if (d < D) s = fmaf(wi, x[(size_t)src * D + d], s);
-        m += wi;
+    // eight rows' indices, then their values, in flight at once; summed in order
+    for (int i = a + g; i < b; i += 32) {
+        int src[8];
+        float wi[8], v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) src[u] = i + 4 * u < b ? perm[i + 4 * u] : -1;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            wi[u] = src[u] >= 0 ? (w ? w[src[u]] : 1.f) : 0.f;
+            v[u] = src[u] >= 0 && d < D ? x[(size_t)src[u] * D + d] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (src[u] >= 0) {
+                s = fmaf(wi[u], v[u], s);
+                m += wi[u];
+            }
     }
     ps[g][d] = s;
     if (d == 0) pm[g] = m;
@@ -148,19 +208,33 @@ __global__ void copy_rows_kernel(const float *src, int D, int K, float *out, int
     out[e] = d < D ? src[(size_t)k * D + d] : 0.f;
 }
 
-__global__ void label_keys_kernel(const int *labels, int n, uint32_t *keys, int *counts) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        keys[i] = (uint32_t)labels[i];
-        atomicAdd(&counts[labels[i]], 1);
-    }
+// offsets[k] = first sorted position with cluster >= k, k <= K
+__global__ void offsets_kernel(const uint32_t *keys, int m, int K, int *offsets) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= m) return;
+    const int cur = (int)keys[j], prev = j > 0 ? (int)keys[j - 1] : -1;
+    for (int k = prev + 1; k <= cur; ++k) offsets[k] = j;
+    if (j == m - 1)
+        for (int k = cur + 1; k <= K; ++k) offsets[k] = m;
 }
 
-__global__ void offsets_finish_kernel(const int *excl, const int *counts, int K, int *offsets) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < K) offsets[k] = excl[k];
-    if (k == K - 1) offsets[K] = excl[k] + counts[k];
-}
+// Stable sort by cluster and offsets of all K clusters (empty ones included) of the first m points of the buffers.
+struct LabelSort {
+    uint32_t *keys;
+    void *scr;
+    int K, bits = 0;
+    LabelSort(otgb_ctx *ctx, const std::string &tag, int n, int K_) : K(K_) {
+        Workspace &ws = ctx_ws(ctx);
+        keys = ws.get<uint32_t>(tag + ":keys", n);
+        while ((1 << bits) < K) ++bits;
+        scr = ws.get("sort:scratch", radix_sort_scratch_bytes(n));
+    }
+    void run(const int *labels, int m, int *perm, int *offsets, cudaStream_t st) {
+        radix_sort_pairs_from(reinterpret_cast<const uint32_t *>(labels), keys, perm, m, bits, scr, st);
+        offsets_kernel<<<(m + 255) / 256, 256, 0, st>>>(keys, m, K, offsets);
+        OTGB_CHECK_LAUNCH();
+    }
+};
 
 uint64_t splitmix64(uint64_t &s) {
     uint64_t z = (s += 0x9e3779b97f4a7c15ull);
@@ -184,15 +258,17 @@ std::vector<int> sample_distinct(int n, int K, unsigned long long seed) {
     return out;
 }
 
-void kmeans_assign(const float *x, int n, int D, const float *cent, int K, int *labels, cudaStream_t st) {
+void kmeans_assign(const float *x, int n, int D, const float *cent, float *cnorm, int K, int *labels, cudaStream_t st) {
     const int D4 = (D + 3) & ~3;
+    centroid_norm_kernel<<<(K + 127) / 128, 128, 0, st>>>(cent, K, D4, cnorm);
+    OTGB_CHECK_LAUNCH();
     static PerDevice<int> attr;
     attr.get([] {
         OTGB_CUDA_TRY(cudaFuncSetAttribute(kmeans_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)sizeof(AssignSmem)));
         return 1;
     });
-    kmeans_assign_kernel<<<(n + kAR - 1) / kAR, kAT, sizeof(AssignSmem), st>>>(x, n, D, D4, cent, K, labels);
+    kmeans_assign_kernel<<<(n + kAR - 1) / kAR, kAT, sizeof(AssignSmem), st>>>(x, n, D, D4, cent, cnorm, K, labels);
     OTGB_CHECK_LAUNCH();
 }
 
@@ -208,6 +284,7 @@ KmeansResult kmeans(otgb_ctx *ctx, const std::string &tag, const float *x, const
     r.labels = ws.get<int>(tag + ":lab", n);
     r.perm = ws.get<int>(tag + ":perm", n);
     r.offsets = ws.get<int>(tag + ":off", K + 1);
+    float *cnorm = ws.get<float>(tag + ":cn", K);
     // the points the Lloyd iterations run on: all of them, or every s-th
     const float *xi = x, *wi = w;
     int ni = n;
@@ -232,33 +309,17 @@ KmeansResult kmeans(otgb_ctx *ctx, const std::string &tag, const float *x, const
         OTGB_CHECK_LAUNCH();
         OTGB_CUDA_TRY(cudaStreamSynchronize(st));  // idx is host memory about to go out of scope
     }
-    // stable sort by cluster and offsets of all K clusters (empty ones included)
-    uint32_t *keys = ws.get<uint32_t>(tag + ":keys", n);
-    int *counts = ws.get<int>(tag + ":cnt", K + 1);
-    int *excl = ws.get<int>(tag + ":excl", K + 1);
-    int bits = 0;
-    while ((1 << bits) < K) ++bits;
-    void *scr = ws.get("sort:scratch", radix_sort_scratch_bytes(n));
-    int *sscr = ws.get<int>("scan:scratch", scan_scratch_ints(K + 1) + 64);
-    // labels, order and offsets of the first m points of the buffers (m = ni during the iterations, n at the end)
-    auto sort_by_label = [&](int m) {
-        OTGB_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(int) * (K + 1), st));
-        label_keys_kernel<<<(m + 255) / 256, 256, 0, st>>>(r.labels, m, keys, counts);
-        OTGB_CHECK_LAUNCH();
-        radix_sort_pairs(keys, r.perm, m, bits, scr, st);
-        exclusive_scan(counts, excl, K, sscr, st);
-        offsets_finish_kernel<<<(K + 255) / 256, 256, 0, st>>>(excl, counts, K, r.offsets);
-        OTGB_CHECK_LAUNCH();
-    };
+    LabelSort sorter(ctx, tag, n, K);
+    auto sort_by_label = [&](int m) { sorter.run(r.labels, m, r.perm, r.offsets, st); };
     for (int it = 0; it < iters; ++it) {
-        kmeans_assign(xi, ni, D, r.centroids, K, r.labels, st);
+        kmeans_assign(xi, ni, D, r.centroids, cnorm, K, r.labels, st);
         sort_by_label(ni);
         kmeans_segment_mean_kernel<<<K, 256, 0, st>>>(xi, wi, D, D4, r.perm, r.offsets, r.centroids);
         OTGB_CHECK_LAUNCH();
     }
-    kmeans_assign(x, n, D, r.centroids, K, r.labels, st);
+    kmeans_assign(x, n, D, r.centroids, cnorm, K, r.labels, st);
     sort_by_label(n);
-    r.sorted_keys = keys;
+    r.sorted_keys = sorter.keys;
     return r;
 }
 

@@ -33,11 +33,6 @@ void *scratch_address() {
     return g_noalloc_ptr[dev];
 }
 
-__global__ void centre_kernel(const float *lo, const float *hi, int D, float *c) {
-    const int d = threadIdx.x;
-    if (d < 64) c[d] = d < D ? 0.5f * (lo[d] + hi[d]) : 0.f;
-}
-
 __global__ void dense_items_kernel(int4 *items, int nb, int n_in) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < nb) items[k] = make_int4(0, k, 0, n_in);
@@ -109,8 +104,7 @@ extern "C" int otgb_softmin_noalloc(const float *q, int n_out, const float *p, c
         int *nfb = c.take<int>(1);
 
         bbox(p, n_in, D, D, lohi, lohi + 64, bpart, st);
-        centre_kernel<<<1, 64, 0, st>>>(lohi, lohi + 64, D, cen);
-        OTGB_CHECK_LAUNCH();
+        box_centre(lohi, lohi + 64, D, cen, st);
         pack_points(q, nullptr, nullptr, n_out, D, cen, R, nullptr, nullptr, st);
         pack_points(p, w, nullptr, n_in, D, cen, Cc, Clw, nullptr, st);
         uniform_blocks(blk, n_out, block_rows, st);

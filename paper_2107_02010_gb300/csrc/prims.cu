@@ -12,29 +12,56 @@ namespace {
 constexpr int kRB = 256;  // threads per block for the reductions
 
 // ------------------------------------------------------------------ bbox --
-__global__ void bbox_partial_kernel(const float *x, int n, int D, int stride, float *part, int nblk) {
-    // part: [nblk][2*D]: lo then hi of this block
-    __shared__ float s_lo[kRB], s_hi[kRB];
-    for (int d = 0; d < D; ++d) {
-        float lo = FLT_MAX, hi = -FLT_MAX;
-        for (int i = blockIdx.x * kRB + threadIdx.x; i < n; i += gridDim.x * kRB) {
-            const float v = x[(size_t)i * stride + d];
-            lo = fminf(lo, v);
-            hi = fmaxf(hi, v);
-        }
-        s_lo[threadIdx.x] = lo;
-        s_hi[threadIdx.x] = hi;
-        __syncthreads();
-        for (int o = kRB / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) {
-                s_lo[threadIdx.x] = fminf(s_lo[threadIdx.x], s_lo[threadIdx.x + o]);
-                s_hi[threadIdx.x] = fmaxf(s_hi[threadIdx.x], s_hi[threadIdx.x + o]);
+// V floats per load (4 when rows are whole 16-byte groups): a CTA of kBoxT threads holds kBoxT / (D / V) rows at a time, so
+// consecutive threads read consecutive addresses whatever D is (one pass over the points; a pass per coordinate read
+// 300k x 60 points in 329 us).  bad (optional): bit 2 when a coordinate is not finite.
+constexpr int kBoxT = 1024, kBoxBlocks = 64;
+template <int V>
+__global__ void __launch_bounds__(kBoxT) bbox_partial_kernel(const float *x, int n, int D, int stride, float *part, int *bad) {
+    // part: [gridDim.x][2*D]: lo then hi of this block
+    __shared__ float red[kBoxT * V];
+    const int Q = D / V, G = kBoxT / Q;  // loads per row, rows per sweep of the CTA
+    const int t = threadIdx.x, g = t / Q, q = t - g * Q;
+    float lo[V], hi[V];
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+        lo[e] = FLT_MAX;
+        hi[e] = -FLT_MAX;
+    }
+    bool fine = true;
+    if (g < G) {
+        const size_t step = (size_t)gridDim.x * G;
+#pragma unroll 4
+        for (size_t i = (size_t)blockIdx.x * G + g; i < (size_t)n; i += step) {
+            float v[V];
+            if constexpr (V == 4) {
+                const float4 u = *reinterpret_cast<const float4 *>(x + i * stride + 4 * q);
+                v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
+            } else {
+                v[0] = x[i * stride + q];
             }
-            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                lo[e] = fminf(lo[e], v[e]);
+                hi[e] = fmaxf(hi[e], v[e]);
+                fine = fine && isfinite(v[e]);
+            }
         }
-        if (threadIdx.x == 0) {
-            part[(size_t)blockIdx.x * 2 * D + d] = s_lo[0];
-            part[(size_t)blockIdx.x * 2 * D + D + d] = s_hi[0];
+    }
+    if (bad && !fine) atomicOr(bad, 2);
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) red[t * V + e] = h ? hi[e] : lo[e];
+        __syncthreads();
+        // a warp per coordinate combines the G groups: groups lie D floats apart
+        for (int d = t >> 5; d < D; d += kBoxT / 32) {
+            float v = h ? -FLT_MAX : FLT_MAX;
+            for (int k = t & 31; k < G; k += 32) v = h ? fmaxf(v, red[k * D + d]) : fminf(v, red[k * D + d]);
+            for (int o = 16; o > 0; o >>= 1) {
+                const float u = __shfl_xor_sync(0xffffffffu, v, o);
+                v = h ? fmaxf(v, u) : fminf(v, u);
+            }
+            if ((t & 31) == 0) part[(size_t)blockIdx.x * 2 * D + h * D + d] = v;
         }
         __syncthreads();
     }
@@ -44,12 +71,18 @@ __global__ void bbox_final_kernel(const float *part, int nblk, int D, float *lo,
     const int d = threadIdx.x;
     if (d >= D) return;
     float l = FLT_MAX, h = -FLT_MAX;
+#pragma unroll 16
     for (int b = 0; b < nblk; ++b) {
         l = fminf(l, part[(size_t)b * 2 * D + d]);
         h = fmaxf(h, part[(size_t)b * 2 * D + D + d]);
     }
     lo[d] = l;
     hi[d] = h;
+}
+
+__global__ void box_centre_kernel(const float *lo, const float *hi, int D, float *c) {
+    const int d = threadIdx.x;
+    if (d < 64) c[d] = d < D ? 0.5f * (lo[d] + hi[d]) : 0.f;
 }
 
 // ------------------------------------------------------- FP64 sums (Eq. 6) --
@@ -79,9 +112,13 @@ __global__ void divsum_partial_kernel(const float *wa, const float *f, const flo
 
 __global__ void divsum_final_kernel(const double *part, int nblk, double rho, double eps, int balanced,
                                     double *out) {
+    __shared__ double s[128];
+    if (threadIdx.x < nblk) s[threadIdx.x] = part[threadIdx.x];
+    __syncthreads();
     if (threadIdx.x != 0) return;
     double acc = 0.0;
-    for (int b = 0; b < nblk; ++b) acc += part[b];  // fixed order: deterministic
+#pragma unroll 16
+    for (int b = 0; b < nblk; ++b) acc += s[b];  // fixed order: deterministic
     *out = balanced ? acc : -(rho + 0.5 * eps) * acc;
 }
 
@@ -155,6 +192,43 @@ __global__ void scan_block_kernel(const int *in, int *out, int n, int *block_sum
     if (threadIdx.x == kScanB - 1) block_sums[blockIdx.x] = s[kScanB - 1];
 }
 
+// Up to kScanOne values in one launch: every thread sums kScanV consecutive values, one scan over the threads.
+constexpr int kScanV = 32, kScanOne = kScanB * kScanV;
+__global__ void __launch_bounds__(kScanB) scan_one_kernel(const int *in, int *out, int n) {
+    __shared__ int ws[32];
+    const int per = (n + kScanB - 1) / kScanB, i0 = threadIdx.x * per, i1 = min(n, i0 + per);
+    int v[kScanV], sum = 0;
+#pragma unroll
+    for (int q = 0; q < kScanV; ++q) {
+        v[q] = q < per && i0 + q < i1 ? in[i0 + q] : 0;
+        sum += v[q];
+    }
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int x = sum;  // inclusive scan over the threads
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += u;
+    }
+    if (lane == 31) ws[w] = x;
+    __syncthreads();
+    if (w == 0) {
+        int y = ws[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) y += u;
+        }
+        ws[lane] = y;
+    }
+    __syncthreads();
+    int run = x - sum + (w > 0 ? ws[w - 1] : 0);
+#pragma unroll
+    for (int q = 0; q < kScanV; ++q)
+        if (q < per && i0 + q < i1) {
+            out[i0 + q] = run;
+            run += v[q];
+        }
+}
+
 __global__ void scan_add_kernel(int *out, int n, const int *block_off) {
     const int i = blockIdx.x * kScanB + threadIdx.x;
     if (i < n) out[i] += block_off[blockIdx.x];
@@ -166,7 +240,7 @@ __global__ void scan_add_kernel(int *out, int n, const int *block_off) {
 // an exclusive scan in digit-major order, then a stable scatter where each
 // element's rank among equal digits of its chunk follows input order.
 constexpr int kSortT = 256;
-constexpr int kPerT = 8;
+constexpr int kPerT = 4;  // 1024 keys per CTA: sorts of 16k to 131k keys then fill the GPU (8 left most of it idle)
 constexpr int kChunk = kSortT * kPerT;
 
 __global__ void radix_hist_kernel(const uint32_t *keys, int n, int shift, int *counts, int nchunks) {
@@ -217,24 +291,47 @@ __global__ void radix_scatter_kernel(const uint32_t *keys, const int *vals, int 
 
 // ------------------------------------------------------------- packing ---
 // D <= 3: out[k] = (x - c, log w) as float4 (zero-padded coordinates).
-// D >  3: out row k = x - c padded with zeros to D4 floats; logw[k] = log w.
-__global__ void pack_kernel(const float *x, const float *w, const int *perm, int n, int D, int D4,
-                            const float *center, float *out, float *logw, float *w_sorted) {
+// D >  3 (pack_rows_kernel): out row k = x - c padded with zeros to D4 floats; logw[k] = log w.
+__global__ void pack_kernel(const float *x, const float *w, const int *perm, int n, int D, const float *center,
+                            float *out, float *logw, float *w_sorted) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     int i = perm ? perm[k] : k;
     OTGB_DCLAMP(i, 0, n);
     const float wi = w ? w[i] : 1.0f;
     const float lw = wi > 0.f ? logf(wi) : -INFINITY;
-    if (D <= 3) {
-        float v[3] = {0.f, 0.f, 0.f};
-        for (int d = 0; d < D; ++d) v[d] = x[(size_t)i * D + d] - center[d];
-        reinterpret_cast<float4 *>(out)[k] = make_float4(v[0], v[1], v[2], lw);
-    } else {
-        for (int d = 0; d < D4; ++d) out[(size_t)k * D4 + d] = d < D ? x[(size_t)i * D + d] - center[d] : 0.f;
-    }
+    float v[3] = {0.f, 0.f, 0.f};
+    for (int d = 0; d < D; ++d) v[d] = x[(size_t)i * D + d] - center[d];
+    reinterpret_cast<float4 *>(out)[k] = make_float4(v[0], v[1], v[2], lw);
     if (logw) logw[k] = lw;
     if (w_sorted) w_sorted[k] = wi;
+}
+
+// D > 3: one thread per point and four coordinates, so that reads and writes run along the rows.
+__global__ void pack_rows_kernel(const float *x, const float *w, const int *perm, int n, int D, int D4, int vec,
+                                 const float *center, float *out, float *logw, float *w_sorted) {
+    const int Q = D4 >> 2;
+    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t k = e / Q;
+    const int q = (int)(e - k * Q);
+    if (k >= (size_t)n) return;
+    int i = perm ? perm[k] : (int)k;
+    OTGB_DCLAMP(i, 0, n);
+    float v[4];
+    if (vec) {
+        const float4 u = *reinterpret_cast<const float4 *>(x + (size_t)i * D + 4 * q);
+        const float4 c = *reinterpret_cast<const float4 *>(center + 4 * q);
+        v[0] = u.x - c.x; v[1] = u.y - c.y; v[2] = u.z - c.z; v[3] = u.w - c.w;
+    } else {
+#pragma unroll
+        for (int d = 0; d < 4; ++d) v[d] = 4 * q + d < D ? x[(size_t)i * D + 4 * q + d] - center[4 * q + d] : 0.f;
+    }
+    reinterpret_cast<float4 *>(out)[e] = make_float4(v[0], v[1], v[2], v[3]);
+    if (q == 0) {
+        const float wi = w ? w[i] : 1.0f;
+        if (logw) logw[k] = wi > 0.f ? logf(wi) : -INFINITY;
+        if (w_sorted) w_sorted[k] = wi;
+    }
 }
 
 __global__ void iota_kernel(int *v, int n) {
@@ -280,9 +377,10 @@ __global__ void check_points_kernel(const float *x, size_t n, int *bad) {
         if (!isfinite(x[i])) atomicOr(bad, 2);
 }
 
-__global__ void absmax_kernel(const float *v, int n, unsigned *out) {
+__global__ void absmax_kernel(const float *v, size_t n, unsigned *out) {
     float m = 0.f;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) m = fmaxf(m, fabsf(v[i]));
+#pragma unroll 4
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) m = fmaxf(m, fabsf(v[i]));
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));
 }
@@ -293,82 +391,166 @@ __global__ void finite_kernel(const float *v, int n, int *bad) {
 }
 
 // ------------------------------------------------------ cluster statistics --
-// One CTA per cluster k over sorted positions [off[k], off[k+1]) of the packed
-// points (stride floats per point): mass = sum w, centroid = weighted mean
-// (plain mean when the mass is 0), radius = max distance to the centroid.
-__global__ void cluster_stats_kernel(const float *pts, int stride, int D, const float *w_sorted, const int *off,
-                                     int ncl, float *cent, int cstride, float *mass, float *radius, float *ssq) {
-    __shared__ double red[128];
+// A sum in two floats (about 48 bits: Knuth's two-sum, Dekker's product by FMA).  The FP64 units of this GPU do two
+// operations per clock and SM, so double sums over all coordinates bounded the kernel (290 us for 100 clusters of 512
+// points); a two-float step is ten FP32 operations.
+struct DF {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v, float e = 0.f) {
+        const float s = __fadd_rn(hi, v), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(e, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b))));
+        hi = s;
+    }
+    __device__ __forceinline__ void add_product(float a, float b) {
+        const float p = __fmul_rn(a, b);
+        add(p, fmaf(a, b, -p));
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
+// Over sorted positions [off[k], off[k+1]) of the packed points (stride floats per point): mass = sum w, centroid =
+// weighted mean (plain mean when the mass is 0), radius = max distance to the centroid, ssq = sum w |x - c|^2.  Sums to
+// about 48 bits, in a fixed order.
+// D > 3: one CTA per cluster, thread (group g, coordinate d): a warp reads along the rows, and the points pass twice (a
+// pass per coordinate with a reduction each took 380 us for 300 clusters of 1000 points).
+constexpr int kStT = 1024, kStG = kStT / 64, kStW = kStT / 32;
+__global__ void __launch_bounds__(kStT) cluster_stats_kernel(const float *pts, int stride, int D, const float *w_sorted,
+                                                            const int *off, int ncl, float *cent, int cstride, float *mass,
+                                                            float *radius, float *ssq) {
+    __shared__ double red[kStG][64], mred[kStG];
     __shared__ float c_s[64];
+    __shared__ float rmax[kStW];
+    __shared__ double wsum[kStW];
     const int k = blockIdx.x;
     if (k >= ncl) return;
     const int a = off[k], b = off[k + 1];
-    const int t = threadIdx.x;
-    double m = 0.0;
-    for (int i = a + t; i < b; i += 128) m += w_sorted[i];
-    red[t] = m;
-    __syncthreads();
-    for (int o = 64; o > 0; o >>= 1) {
-        if (t < o) red[t] += red[t + o];
-        __syncthreads();
+    const int t = threadIdx.x, g = t >> 6, d = t & 63;
+    DF acc, m;
+#pragma unroll 4
+    for (int i = a + g; i < b; i += kStG) {
+        const float w = w_sorted[i], v = d < D ? pts[(size_t)i * stride + d] : 0.f;
+        m.add(w);
+        acc.add_product(w, v);
     }
-    const double mass_k = red[0];
-    __syncthreads();
-    for (int d = 0; d < D; ++d) {
-        double acc = 0.0;
-        for (int i = a + t; i < b; i += 128)
-            acc += (mass_k > 0.0 ? (double)w_sorted[i] : 1.0) * pts[(size_t)i * stride + d];
-        red[t] = acc;
-        __syncthreads();
-        for (int o = 64; o > 0; o >>= 1) {
-            if (t < o) red[t] += red[t + o];
-            __syncthreads();
+    double accd = acc.value(), md = m.value();
+    if (__syncthreads_or(!isfinite(accd) || !isfinite(md))) {  // beyond the float range: in double
+        accd = md = 0.0;
+        for (int i = a + g; i < b; i += kStG) {
+            const double w = w_sorted[i];
+            md += w;
+            accd += w * (d < D ? pts[(size_t)i * stride + d] : 0.f);
         }
-        if (t == 0) c_s[d] = (float)(red[0] / (mass_k > 0.0 ? mass_k : (double)(b - a)));
+    }
+    red[g][d] = accd;
+    if (d == 0) mred[g] = md;
+    __syncthreads();
+    double mass_k = 0.0;
+    for (int q = 0; q < kStG; ++q) mass_k += mred[q];
+    if (!(mass_k > 0.0)) {  // uniform
+        DF plain;
+        for (int i = a + g; i < b; i += kStG) plain.add(d < D ? pts[(size_t)i * stride + d] : 0.f);
+        __syncthreads();
+        red[g][d] = plain.value();
         __syncthreads();
     }
+    if (g == 0) {
+        double v = 0.0;
+        for (int q = 0; q < kStG; ++q) v += red[q][d];
+        c_s[d] = (float)(v / (mass_k > 0.0 ? mass_k : (double)(b - a)));
+    }
+    __syncthreads();
+    // distances: a warp per point
+    const int warp = t >> 5, lane = t & 31;
+    const float c0 = lane < D ? c_s[lane] : 0.f, c1 = lane + 32 < D ? c_s[lane + 32] : 0.f;
+    float r2 = 0.f;
+    DF wss;
+#pragma unroll 4
+    for (int i = a + warp; i < b; i += kStW) {
+        const float u = lane < D ? pts[(size_t)i * stride + lane] - c0 : 0.f;
+        const float v = lane + 32 < D ? pts[(size_t)i * stride + lane + 32] - c1 : 0.f;
+        float s2 = fmaf(u, u, v * v);
+        for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        r2 = fmaxf(r2, s2);
+        wss.add_product(w_sorted[i], s2);
+    }
+    if (lane == 0) {
+        rmax[warp] = r2;
+        wsum[warp] = wss.value();
+    }
+    __syncthreads();
+    if (t == 0) {
+        double ws = 0.0;
+        for (int q = 0; q < kStW; ++q) {
+            r2 = fmaxf(r2, rmax[q]);
+            ws += wsum[q];
+        }
+        mass[k] = (float)mass_k;
+        radius[k] = sqrtf(r2) * (1.0f + 1e-6f) + 1e-30f;
+        if (ssq) ssq[k] = (float)ws;
+    }
+    if (t < cstride) cent[(size_t)k * cstride + t] = t < D ? c_s[t] : 0.f;
+}
+
+// D <= 3 (float4 points): one warp per cluster.  The coarse measure is packed like the points: (centroid, log mass).
+__global__ void cluster_stats3_kernel(const float4 *pts, int D, const float *w_sorted, const int *off, int ncl, float *cent,
+                                      int cstride, float *mass, float *radius, float *ssq) {
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (k >= ncl) return;
+    const int a = off[k], b = off[k + 1];
+    double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // mass, weighted sums, plain sums
+    for (int i = a + lane; i < b; i += 32) {
+        const float4 p = pts[i];
+        const double w = w_sorted[i];
+        v[0] += w;
+        v[1] += w * p.x; v[2] += w * p.y; v[3] += w * p.z;
+        v[4] += p.x; v[5] += p.y; v[6] += p.z;
+    }
+#pragma unroll
+    for (int q = 0; q < 7; ++q)
+        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+    const bool pos = v[0] > 0.0;
+    const double den = pos ? v[0] : (double)(b - a);
+    float c[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) c[q] = q < D ? (float)((pos ? v[1 + q] : v[4 + q]) / den) : 0.f;
     float r2 = 0.f;
     double wss = 0.0;
-    for (int i = a + t; i < b; i += 128) {
-        float s2 = 0.f;
-        for (int d = 0; d < D; ++d) { const float u = pts[(size_t)i * stride + d] - c_s[d]; s2 = fmaf(u, u, s2); }
+    for (int i = a + lane; i < b; i += 32) {
+        const float4 p = pts[i];
+        const float u0 = p.x - c[0], u1 = p.y - c[1], u2 = p.z - c[2];
+        const float s2 = fmaf(u2, u2, fmaf(u1, u1, u0 * u0));
         r2 = fmaxf(r2, s2);
         wss += (double)w_sorted[i] * s2;
     }
-    red[t] = r2;
-    __syncthreads();
-    for (int o = 64; o > 0; o >>= 1) {
-        if (t < o) red[t] = fmax(red[t], red[t + o]);
-        __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) {
+        r2 = fmaxf(r2, __shfl_xor_sync(0xffffffffu, r2, o));
+        wss += __shfl_xor_sync(0xffffffffu, wss, o);
     }
-    if (t == 0) {
-        mass[k] = (float)mass_k;
-        radius[k] = sqrtf((float)red[0]) * (1.0f + 1e-6f) + 1e-30f;
-    }
-    __syncthreads();
-    red[t] = wss;
-    __syncthreads();
-    for (int o = 64; o > 0; o >>= 1) {
-        if (t < o) red[t] += red[t + o];
-        __syncthreads();
-    }
-    if (t == 0 && ssq) ssq[k] = (float)red[0];
-    // D <= 3 packs the coarse measure like the points: (centroid, log mass)
-    if (t < cstride) {
-        float v = t < D ? c_s[t] : 0.f;
-        if (D <= 3 && cstride == 4 && t == 3) v = mass_k > 0.0 ? (float)log(mass_k) : -INFINITY;
-        cent[(size_t)k * cstride + t] = v;
+    if (lane == 0) {
+        mass[k] = (float)v[0];
+        radius[k] = sqrtf(r2) * (1.0f + 1e-6f) + 1e-30f;
+        if (ssq) ssq[k] = (float)wss;
+        for (int q = 0; q < cstride; ++q)
+            cent[(size_t)k * cstride + q] = q < D ? (q == 0 ? c[0] : (q == 1 ? c[1] : c[2]))
+                                                  : (q == 3 ? (pos ? (float)log(v[0]) : -INFINITY) : 0.f);
     }
 }
 
 }  // namespace
 
 // =================================================================== host ==
-void bbox(const float *x, int n, int D, int stride, float *d_lo, float *d_hi, float *d_part, cudaStream_t st) {
-    const int nblk = 64;
-    bbox_partial_kernel<<<nblk, kRB, 0, st>>>(x, n, D, stride, d_part, nblk);
+void bbox(const float *x, int n, int D, int stride, float *d_lo, float *d_hi, float *d_part, cudaStream_t st, int *d_bad) {
+    if (D % 4 == 0 && stride % 4 == 0 && ((uintptr_t)x & 15) == 0)
+        bbox_partial_kernel<4><<<kBoxBlocks, kBoxT, 0, st>>>(x, n, D, stride, d_part, d_bad);
+    else
+        bbox_partial_kernel<1><<<kBoxBlocks, kBoxT, 0, st>>>(x, n, D, stride, d_part, d_bad);
     OTGB_CHECK_LAUNCH();
-    bbox_final_kernel<<<1, 64, 0, st>>>(d_part, nblk, D, d_lo, d_hi);
+    bbox_final_kernel<<<1, 64, 0, st>>>(d_part, kBoxBlocks, D, d_lo, d_hi);
+    OTGB_CHECK_LAUNCH();
+}
+
+void box_centre(const float *lo, const float *hi, int D, float *c, cudaStream_t st) {
+    box_centre_kernel<<<1, 64, 0, st>>>(lo, hi, D, c);
     OTGB_CHECK_LAUNCH();
 }
 
@@ -379,7 +561,7 @@ void divergence_sum(const float *wa, const float *f, const float *aa, int N, con
     const int balanced = std::isinf(rho) ? 1 : 0;
     divsum_partial_kernel<<<nblk, kRB, 0, st>>>(wa, f, aa, N, wb, g, bb, M, rho, balanced, d_part);
     OTGB_CHECK_LAUNCH();
-    divsum_final_kernel<<<1, 32, 0, st>>>(d_part, nblk, rho, eps, balanced, d_out);
+    divsum_final_kernel<<<1, 128, 0, st>>>(d_part, nblk, rho, eps, balanced, d_out);
     OTGB_CHECK_LAUNCH();
 }
 
@@ -403,6 +585,11 @@ size_t scan_scratch_ints_level(int nb) {
 
 void exclusive_scan(const int *in, int *out, int n, int *scratch, cudaStream_t st) {
     if (n <= 0) return;
+    if (n <= kScanOne) {
+        scan_one_kernel<<<1, kScanB, 0, st>>>(in, out, n);
+        OTGB_CHECK_LAUNCH();
+        return;
+    }
     const int nb = (n + kScanB - 1) / kScanB;
     int *bsum = scratch;
     scan_block_kernel<<<nb, kScanB, 0, st>>>(in, out, n, bsum);
@@ -422,13 +609,10 @@ size_t radix_sort_scratch_bytes(int n) {
            256;
 }
 
-void radix_sort_pairs(uint32_t *keys, int *vals, int n, int nbits, void *scratch, cudaStream_t st) {
-    if (n <= 1 || nbits <= 0) {
-        if (n == 1) OTGB_CUDA_TRY(cudaMemsetAsync(vals, 0, sizeof(int), st));
-        if (n > 1 && nbits <= 0) {
-            // keys all equal: identity permutation
-            iota(vals, n, st);
-        }
+void radix_sort_pairs_from(const uint32_t *src, uint32_t *keys, int *vals, int n, int nbits, void *scratch, cudaStream_t st) {
+    if (n <= 1 || nbits <= 0) {  // one key, or keys all equal: identity permutation
+        if (n >= 1 && src != keys) OTGB_CUDA_TRY(cudaMemcpyAsync(keys, src, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st));
+        if (n >= 1) iota(vals, n, st);
         return;
     }
     const int nchunks = (n + kChunk - 1) / kChunk;
@@ -439,27 +623,32 @@ void radix_sort_pairs(uint32_t *keys, int *vals, int n, int nbits, void *scratch
     uint8_t *p = reinterpret_cast<uint8_t *>(scan_scr + scan_scratch_ints((int)cnt) + 64);
     uint32_t *k2 = reinterpret_cast<uint32_t *>(p);
     int *v2 = reinterpret_cast<int *>(k2 + n);
-    uint32_t *kin = keys, *kout = k2;
-    int *vin = nullptr, *vout = v2;  // first pass: values are the input positions
     const int passes = (nbits + 7) / 8;
+    // the passes alternate between (keys, vals) and the scratch pair so that the last one writes (keys, vals); the first
+    // reads src, which must not be what it writes
+    const uint32_t *kin = src;
+    const int *vin = nullptr;  // first pass: values are the input positions
+    bool to_keys = passes % 2 == 1;
+    if (to_keys && src == keys) {
+        OTGB_CUDA_TRY(cudaMemcpyAsync(k2, src, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st));
+        kin = k2;
+    }
     for (int ps = 0; ps < passes; ++ps) {
+        uint32_t *kout = to_keys ? keys : k2;
+        int *vout = to_keys ? vals : v2;
         radix_hist_kernel<<<nchunks, kSortT, 0, st>>>(kin, n, 8 * ps, counts, nchunks);
         OTGB_CHECK_LAUNCH();
         exclusive_scan(counts, offs, (int)cnt, scan_scr, st);
         radix_scatter_kernel<<<nchunks, kSortT, 0, st>>>(kin, vin, n, 8 * ps, offs, nchunks, kout, vout);
         OTGB_CHECK_LAUNCH();
-        // the next pass reads what this one wrote and overwrites the other buffer
-        uint32_t *tk = kin;
         kin = kout;
-        kout = tk;
-        int *tv = vin ? vin : vals;
         vin = vout;
-        vout = tv;
+        to_keys = !to_keys;
     }
-    if (kin != keys) {
-        OTGB_CUDA_TRY(cudaMemcpyAsync(keys, kin, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st));
-        OTGB_CUDA_TRY(cudaMemcpyAsync(vals, vin, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
-    }
+}
+
+void radix_sort_pairs(uint32_t *keys, int *vals, int n, int nbits, void *scratch, cudaStream_t st) {
+    radix_sort_pairs_from(keys, keys, vals, n, nbits, scratch, st);
 }
 
 void iota(int *v, int n, cudaStream_t st) {
@@ -469,8 +658,14 @@ void iota(int *v, int n, cudaStream_t st) {
 
 void pack_points(const float *x, const float *w, const int *perm, int n, int D, const float *d_center, float *out,
                  float *logw, float *w_sorted, cudaStream_t st) {
-    const int D4 = D <= 3 ? 4 : ((D + 3) & ~3);
-    pack_kernel<<<(n + 255) / 256, 256, 0, st>>>(x, w, perm, n, D, D4, d_center, out, logw, w_sorted);
+    if (D > 3) {
+        const int D4 = (D + 3) & ~3;
+        const int vec = D % 4 == 0 && ((uintptr_t)x & 15) == 0 && ((uintptr_t)d_center & 15) == 0;
+        const size_t tot = (size_t)n * (D4 >> 2);
+        pack_rows_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(x, w, perm, n, D, D4, vec, d_center, out, logw, w_sorted);
+    } else {
+        pack_kernel<<<(n + 255) / 256, 256, 0, st>>>(x, w, perm, n, D, d_center, out, logw, w_sorted);
+    }
     OTGB_CHECK_LAUNCH();
 }
 
@@ -494,8 +689,8 @@ void check_points(const float *x, size_t n, int *d_bad, cudaStream_t st) {
     OTGB_CHECK_LAUNCH();
 }
 
-void absmax(const float *v, int n, unsigned *d_out, cudaStream_t st) {
-    absmax_kernel<<<64, 256, 0, st>>>(v, n, d_out);
+void absmax(const float *v, size_t n, unsigned *d_out, cudaStream_t st) {
+    absmax_kernel<<<152, 256, 0, st>>>(v, n, d_out);
     OTGB_CHECK_LAUNCH();
 }
 
@@ -507,7 +702,13 @@ void check_finite(const float *v, int n, int *d_bad, cudaStream_t st) {
 void cluster_stats(const float *pts, int stride, int D, const float *w_sorted, const int *off, int ncl, float *cent,
                    int cstride, float *mass, float *radius, float *ssq, cudaStream_t st) {
     if (ncl <= 0) return;
-    cluster_stats_kernel<<<ncl, 128, 0, st>>>(pts, stride, D, w_sorted, off, ncl, cent, cstride, mass, radius, ssq);
+    if (D <= 3) {
+        require(stride == 4, "cluster_stats: D <= 3 points are float4", OTGB_EINTERNAL);
+        cluster_stats3_kernel<<<(ncl + 7) / 8, 256, 0, st>>>(reinterpret_cast<const float4 *>(pts), D, w_sorted, off, ncl,
+                                                             cent, cstride, mass, radius, ssq);
+    } else {
+        cluster_stats_kernel<<<ncl, kStT, 0, st>>>(pts, stride, D, w_sorted, off, ncl, cent, cstride, mass, radius, ssq);
+    }
     OTGB_CHECK_LAUNCH();
 }
 

@@ -6,8 +6,12 @@
 namespace otgb {
 
 // Bounding box of the first D coordinates of n points (stride floats apart).
-// d_part: scratch of 64 * 2 * D floats.
-void bbox(const float *x, int n, int D, int stride, float *d_lo, float *d_hi, float *d_part, cudaStream_t st);
+// d_part: scratch of 64 * 2 * D floats.  d_bad (optional): bit 2 is set when a coordinate is not finite.
+void bbox(const float *x, int n, int D, int stride, float *d_lo, float *d_hi, float *d_part, cudaStream_t st,
+          int *d_bad = nullptr);
+
+// c (64 floats) = middle of the box, 0 beyond D.
+void box_centre(const float *lo, const float *hi, int D, float *c, cudaStream_t st);
 
 // S of Eq. (6) in double from the four duals (internal order) and the weights;
 // rho = +inf selects the balanced form.  d_part: scratch of 128 doubles.
@@ -30,6 +34,9 @@ size_t radix_sort_scratch_bytes(int n);
 // position of each sorted key.  keys are sorted in place.
 void radix_sort_pairs(uint32_t *keys, int *vals, int n, int nbits, void *scratch, cudaStream_t st);
 
+// The same with the keys read from src (unchanged unless src == keys); keys receives them sorted.
+void radix_sort_pairs_from(const uint32_t *src, uint32_t *keys, int *vals, int n, int nbits, void *scratch, cudaStream_t st);
+
 void iota(int *v, int n, cudaStream_t st);
 
 // Internal layout: D <= 3 -> float4 (x - c, log w); D > 3 -> D4 floats (x - c, 0-padded)
@@ -44,7 +51,7 @@ void check_weights(const float *w, int n, int *d_bad, double *d_mass_part, cudaS
 void check_points(const float *x, size_t n, int *d_bad, cudaStream_t st);
 void check_finite(const float *v, int n, int *d_bad, cudaStream_t st);
 // *d_out = max(*d_out, max_i |v_i|) as the bits of a non-negative float (zero it first).
-void absmax(const float *v, int n, unsigned *d_out, cudaStream_t st);
+void absmax(const float *v, size_t n, unsigned *d_out, cudaStream_t st);
 
 // Per-cluster mass, weighted centroid (cstride floats per centroid; for D <= 3 and
 // cstride = 4 the 4th float is log mass), radius (max distance to the centroid)

@@ -46,10 +46,8 @@ DeviceChecks validate_and_bound(otgb_ctx *ctx, const float *x, const float *a, i
     OTGB_CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(int), st));
     check_weights(a, N, bad, mpart, st);
     check_weights(b, M, bad, mpart + 64, st);
-    check_points(x, (size_t)N * D, bad, st);
-    check_points(y, (size_t)M * D, bad, st);
-    bbox(x, N, D, D, box, box + 64, bpart, st);
-    bbox(y, M, D, D, box + 128, box + 192, bpart, st);
+    bbox(x, N, D, D, box, box + 64, bpart, st, bad);
+    bbox(y, M, D, D, box + 128, box + 192, bpart, st, bad);
     char *mb = static_cast<char *>(ctx_pinned(ctx));
     OTGB_CUDA_TRY(cudaMemcpyAsync(mb + kMbBad, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
     OTGB_CUDA_TRY(cudaMemcpyAsync(mb + kMbMass, mpart, 128 * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -166,10 +164,7 @@ double Solver::divergence(double eps) {
     unsigned *dmax = ws->get<unsigned>(nm("potmax"), 1);
     divergence_sum(X.w, pf[cur], pa[cur], X.n, Y.w, pg[cur], pb[cur], Y.n, eps, rho, dS, dpart, st);
     OTGB_CUDA_TRY(cudaMemsetAsync(dmax, 0, sizeof(unsigned), st));
-    absmax(pf[cur], X.n, dmax, st);
-    absmax(pa[cur], X.n, dmax, st);
-    absmax(pg[cur], Y.n, dmax, st);
-    absmax(pb[cur], Y.n, dmax, st);
+    absmax(Z[cur], 2 * (size_t)X.n + 2 * (size_t)Y.n, dmax, st);  // the four duals lie one after the other
     char *mb = static_cast<char *>(ctx_pinned(ctx));
     OTGB_CUDA_TRY(cudaMemcpyAsync(mb + kMbS, dS, sizeof(double), cudaMemcpyDeviceToHost, st));
     OTGB_CUDA_TRY(cudaMemcpyAsync(mb + kMbDelta, launch.delta_max, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
