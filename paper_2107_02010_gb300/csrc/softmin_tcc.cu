@@ -38,54 +38,17 @@ namespace {
 constexpr int kN = xt::kCols;
 constexpr int kMaxWords = kTccMaxWords;
 constexpr int kThreads = 192;
-constexpr int kStageBudget = 96 * 1024;  // shared memory for column tiles: two CTAs per SM
-
-template <int NP, int K> struct Geom {
-    static constexpr int tile = xt::tile_bytes(NP, K);
-    static constexpr int st = kStageBudget / tile;
-    static constexpr int stages = st > 6 ? 6 : st;
-    // a second row operand where 256 tensor-memory columns hold it: the next cluster's rows are then staged while
-    // the MMAs of the current one run
-    static constexpr int abuf = kN + 2 * NP * (K / 2) <= (int)xt::kTmemCols ? 2 : 1;
-    static_assert(kN + NP * (K / 2) <= (int)xt::kTmemCols && stages >= 2, "tile does not fit");
-};
-
 struct TccCtl {
     unsigned words[kMaxWords];  // kept column clusters of this block
-    unsigned long long full[6], empty[6], acc_full, acc_free, a_ready[2], drain;
+    unsigned long long full[xt::kMaxStages], empty[xt::kMaxStages], acc_full, acc_free, a_ready[2], drain;
     uint32_t tslot;
     int ncols;
     int abort;
 };
 
-// Walks the tiles of the kept column clusters of a block in cluster order.
-struct TileIt {
-    int w = -1;
-    unsigned u = 0u;
-    int J = -1, g = 0, gend = 0;
-};
-__device__ __forceinline__ bool tile_next(TileIt &it, const unsigned *words, int nwords, const int *tile0) {
-    if (it.g + 1 < it.gend) {
-        ++it.g;
-        return true;
-    }
-    for (;;) {
-        while (it.u == 0u) {
-            if (++it.w >= nwords) return false;
-            it.u = words[it.w];
-        }
-        const int bit = __ffs(it.u) - 1;
-        it.u &= it.u - 1u;
-        it.J = it.w * 32 + bit;
-        it.g = tile0[it.J];
-        it.gend = tile0[it.J + 1];
-        if (it.g < it.gend) return true;
-    }
-}
-
 template <int NP, int K>
 __global__ void __launch_bounds__(kThreads, 2) softmin_tcc_kernel(const __grid_constant__ SoftminLaunch L, int D4) {
-    using G = Geom<NP, K>;
+    using G = xt::Geom<NP, K>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *tiles_s = smem_raw;  // stages
     TccCtl &S = *reinterpret_cast<TccCtl *>(smem_raw + G::stages * G::tile);
@@ -161,9 +124,9 @@ __global__ void __launch_bounds__(kThreads, 2) softmin_tcc_kernel(const __grid_c
     if (warp == 4) {
         // ---------------------------------------------------------- column tiles
         if (lane == 0) {
-            TileIt it;
+            xt::TileIt it;
             int k = 0;
-            while (tile_next(it, S.words, nwords, tile0)) {
+            while (xt::tile_next(it, S.words, nwords, tile0)) {
                 const int st = k % G::stages;
                 if (k >= G::stages && !xt::wait(&S.empty[st], (uint32_t)((k / G::stages - 1) & 1), abort)) {
                     *abort = 1;
@@ -180,9 +143,9 @@ __global__ void __launch_bounds__(kThreads, 2) softmin_tcc_kernel(const __grid_c
     } else if (warp == 5) {
         // ------------------------------------------------------------------ MMAs
         if (lane == 0) {
-            TileIt it;
+            xt::TileIt it;
             int k = 0, aJ = -1, na = 0;  // na: row operands taken so far
-            while (tile_next(it, S.words, nwords, tile0)) {
+            while (xt::tile_next(it, S.words, nwords, tile0)) {
                 const int st = k % G::stages;
                 if (it.J != aJ) {
                     const int ab = na % G::abuf;
@@ -223,12 +186,12 @@ __global__ void __launch_bounds__(kThreads, 2) softmin_tcc_kernel(const __grid_c
             xt::arrive(&S.a_ready[na % G::abuf]);
             ++na;
         };
-        TileIt it;
-        bool have = tile_next(it, S.words, nwords, tile0);
+        xt::TileIt it;
+        bool have = xt::tile_next(it, S.words, nwords, tile0);
         if (have) stage(it.J);
         for (int k = 0; have; ++k) {
-            TileIt nx = it;
-            const bool more = tile_next(nx, S.words, nwords, tile0);
+            xt::TileIt nx = it;
+            const bool more = xt::tile_next(nx, S.words, nwords, tile0);
             const bool fresh = more && nx.J != it.J;
             // the other row operand belongs to an earlier cluster, whose MMAs are complete: tile k - 1's are
             if (G::abuf == 2 && fresh) stage(nx.J);
@@ -279,7 +242,7 @@ __global__ void __launch_bounds__(kThreads, 2) softmin_tcc_kernel(const __grid_c
 
 // Column tiles of one side: tile g of cluster J = tile_cl[g] holds columns off[J] + 128 (g - tile0[J]) + c,
 // c < 128 (past the cluster's end: zero), centred at c_J and split; half_norm = |yh|^2 / 2.  Written into both
-// copies (one per instance that uses the side as columns) at once.
+// copies (one per instance that uses the side as columns) at once; a null dst1 means one copy.
 template <int NP, int K>
 __global__ void __launch_bounds__(kN) tcc_build_kernel(const float *pts, int D4, const int *off, const int *tile0,
                                                        const int *tile_cl, const float *cen, unsigned char *dst0,
@@ -290,7 +253,7 @@ __global__ void __launch_bounds__(kN) tcc_build_kernel(const float *pts, int D4,
     const bool ok = j < off[J + 1];
     const size_t o = (size_t)g * xt::tile_bytes(NP, K);
     half_norm[(size_t)g * kN + c] = xt::build_col<NP, K, double>(pts + (size_t)(ok ? j : 0) * D4, cen + (size_t)J * D4, D4, ok, c,
-                                                         dst0 + o, dst1 + o);
+                                                         dst0 + o, dst1 ? dst1 + o : nullptr);
 }
 
 // Per step: H_j = s (eps log w_j + pot_j - |yh_j|^2 / 2) into the column tiles of every instance (past a cluster's
@@ -355,7 +318,7 @@ struct SweepFn {
     int D4;
     cudaStream_t st;
     template <int NP, int K> void operator()() const {
-        constexpr int bytes = Geom<NP, K>::stages * Geom<NP, K>::tile + (int)sizeof(TccCtl);
+        constexpr int bytes = xt::Geom<NP, K>::stages * xt::Geom<NP, K>::tile + (int)sizeof(TccCtl);
         static_assert(2 * (bytes + 1024) <= 227 * 1024, "two CTAs per SM");
         static PerDevice<int> attr;
         attr.get([] {

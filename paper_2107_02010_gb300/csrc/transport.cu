@@ -12,6 +12,7 @@
 #include "multiscale.cuh"
 #include "prims.cuh"
 #include "solver.cuh"
+#include "transport.cuh"
 
 namespace otgb {
 namespace {
@@ -34,6 +35,7 @@ struct TransportArgs {
     float *mass;
     int4 *fallback;
     int *n_fallback;
+    const int *out_perm;   // safe kernel: row -> place in scores / argmax / mass (null: the row itself)
 };
 
 __device__ __forceinline__ float ex2f_(float x) {
@@ -286,7 +288,7 @@ __global__ void transport_fallback_kernel(const __grid_constant__ TransportArgs 
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < count; w += nw) {
-        const int r = A.fallback[w].x;
+        const int r = A.fallback[w].x, o = A.out_perm ? A.out_perm[r] : r;
         const float *xi = A.rows + (size_t)r * A.stride;
         double mass = 0.0, best = -1.0;
         int bestl = -1;
@@ -313,13 +315,13 @@ __global__ void transport_fallback_kernel(const __grid_constant__ TransportArgs 
                 }
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             const double v = (m > -INFINITY) ? exp2((double)A.s * A.f[r] + m + log2(acc)) : 0.0;
-            if (lane == 0 && A.scores) A.scores[(size_t)r * A.L + l] = (float)v;
+            if (lane == 0 && A.scores) A.scores[(size_t)o * A.L + l] = (float)v;
             mass += v;
             if (v > best) { best = v; bestl = l; }
         }
         if (lane == 0) {
-            A.argmax[r] = bestl;
-            if (A.mass) A.mass[r] = (float)mass;
+            A.argmax[o] = bestl;
+            if (A.mass) A.mass[o] = (float)mass;
         }
     }
 }
@@ -355,6 +357,19 @@ __global__ void unpermute_rows_kernel(const float *sc, const int *am, const floa
 }
 
 }  // namespace
+
+void label_order(otgb_ctx *ctx, const int *labels, int M, int L, uint32_t *keys, int *perm, int *lab_off) {
+    cudaStream_t st = ctx_stream(ctx);
+    label_sort_keys_kernel<<<(M + 255) / 256, 256, 0, st>>>(labels, M, L, keys);
+    OTGB_CHECK_LAUNCH();
+    int bits = 0;
+    while ((1 << bits) < L + 1) ++bits;
+    void *scr = ctx_ws(ctx).get("sort:scratch", radix_sort_scratch_bytes(M));
+    radix_sort_pairs(keys, perm, M, bits, scr, st);
+    label_hist_kernel<<<(M + 255) / 256, 256, 0, st>>>(keys, M, L, lab_off);
+    OTGB_CHECK_LAUNCH();
+}
+
 }  // namespace otgb
 
 using namespace otgb;
@@ -376,22 +391,29 @@ extern "C" int transport_apply(otgb_ctx *ctx, const otgb_plan *plan, const float
         float *box = ws.get<float>("box", 4 * 64);
         float *bpart = ws.get<float>("bpart", 64 * 2 * 64);
         bbox(plan->y, M, D, D, box, box + 64, bpart, st);
-        std::vector<float> h(128);
-        OTGB_CUDA_TRY(cudaMemcpyAsync(h.data(), box, 128 * sizeof(float), cudaMemcpyDeviceToHost, st));
-        OTGB_CUDA_TRY(cudaStreamSynchronize(st));
-        std::vector<float> cen(64, 0.f);
-        for (int d = 0; d < D; ++d) cen[d] = 0.5f * (h[d] + h[64 + d]);
         float *d_cen = ws.get<float>("cen", 64);
-        OTGB_CUDA_TRY(cudaMemcpyAsync(d_cen, cen.data(), 64 * sizeof(float), cudaMemcpyHostToDevice, st));
+        box_centre(box, box + 64, D, d_cen, st);
+        if (xd_width(D)) {
+            const TransportCall c{plan->x, plan->y, plan->b, N, M, D, L, plan->eps, f, g, labels, d_cen, scores, argmax, row_mass};
+            const TransportFallback r = transport_xt_apply(ctx, c);
+            TransportArgs A;
+            std::memset(&A, 0, sizeof(A));
+            A.rows = r.rows; A.f = r.f; A.cols = r.cols; A.col_logw = r.col_logw; A.g = r.g; A.col_lab = r.col_lab;
+            A.n = N; A.m = M; A.D = D; A.stride = stride; A.L = L;
+            A.eps = (float)plan->eps;
+            A.s = (float)(1.4426950408889634 / plan->eps);
+            A.scores = scores; A.argmax = argmax; A.mass = row_mass;
+            A.fallback = r.fallback; A.n_fallback = r.n_fallback; A.out_perm = r.row_perm;
+            transport_fallback_kernel<<<64, 256, 0, st>>>(A);
+            OTGB_CHECK_LAUNCH();
+            OTGB_CUDA_TRY(cudaStreamSynchronize(st));
+            return OTGB_OK;
+        }
         // columns sorted by label
         uint32_t *keys = ws.get<uint32_t>("ta:keys", M);
         int *cperm = ws.get<int>("ta:cperm", M);
-        label_sort_keys_kernel<<<(M + 255) / 256, 256, 0, st>>>(labels, M, L, keys);
-        OTGB_CHECK_LAUNCH();
-        int bits = 0;
-        while ((1 << bits) < L + 1) ++bits;
-        void *scr = ws.get("sort:scratch", radix_sort_scratch_bytes(std::max(N, M)));
-        radix_sort_pairs(keys, cperm, M, bits, scr, st);
+        int *lab_off = ws.get<int>("ta:laboff", L + 1);
+        label_order(ctx, labels, M, L, keys, cperm, lab_off);
         float *C = ws.get<float>("ta:C", (size_t)M * stride);
         float *Clw = D > 3 ? ws.get<float>("ta:Clw", M) : nullptr;
         float *gs = ws.get<float>("ta:g", M);
@@ -442,9 +464,6 @@ extern "C" int transport_apply(otgb_ctx *ctx, const otgb_plan *plan, const float
             std::vector<int> hb = make_row_blocks(N, 128, &off);
             int *d_blk = ws.get<int>("ta:blk", hb.size());
             OTGB_CUDA_TRY(cudaMemcpyAsync(d_blk, hb.data(), sizeof(int) * hb.size(), cudaMemcpyHostToDevice, st));
-            int *lab_off = ws.get<int>("ta:laboff", L + 1);
-            label_hist_kernel<<<(M + 255) / 256, 256, 0, st>>>(keys, M, L, lab_off);
-            OTGB_CHECK_LAUNCH();
             row_perm = kr.perm;
             pack_points(plan->x, nullptr, kr.perm, N, D, d_cen, Rw, nullptr, nullptr, st);
             permute(f, kr.perm, N, fs, st);

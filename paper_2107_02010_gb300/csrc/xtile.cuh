@@ -136,10 +136,10 @@ template <int NP, int K> __device__ __forceinline__ void issue(uint32_t d, uint3
 }
 
 // The row operand of this thread's row for centre c: s (x - c) in NP pieces, the folded slots, R = -s |x - c|^2 / 2
-// - M.  `a`: tensor-memory column of the row pieces, with the warp's lane quadrant.  Warp-collective.
+// - (M + Mlo).  `a`: tensor-memory column of the row pieces, with the warp's lane quadrant.  Warp-collective.
 template <int NP, int K>
 __device__ __forceinline__ void stage_row(const float (&x)[K - 4], int D4, const float *c, float s, float M, bool valid,
-                                          uint32_t a) {
+                                          uint32_t a, float Mlo = 0.f) {
     const float4 *c4 = reinterpret_cast<const float4 *>(c);
     float4 sq = make_float4(0.f, 0.f, 0.f, 0.f);  // four short chains: less rounding than one long one
 #pragma unroll
@@ -171,11 +171,11 @@ __device__ __forceinline__ void stage_row(const float (&x)[K - 4], int D4, const
             for (int q = 0; q < NP; ++q) w[q][j] = p[q];
         }
         if (kk == K / 16 - 1) {
-            // R = P - M with what the product and the difference lose to rounding (M's own rounding cancels: the
-            // finish adds the same M back)
+            // R = P - M with what the product and the difference lose to rounding (where the finish adds M back its
+            // own rounding cancels and Mlo is 0)
             const float hq = 0.5f * ((sq.x + sq.y) + (sq.z + sq.w)), P = -s * hq;
             const float R = P - M, bb = P - R;  // two-difference (Knuth)
-            const float rest = fmaf(-s, hq, -P) + ((P - (R + bb)) + (bb - M));
+            const float rest = (fmaf(-s, hq, -P) + ((P - (R + bb)) + (bb - M))) - Mlo;
             uint16_t r1, r2, r3;
             split3(valid ? R : 0.f, valid ? rest : 0.f, r1, r2, r3);
             if constexpr (NP == 3) {
@@ -365,6 +365,45 @@ template <class F> __device__ __forceinline__ void sum_row_max(uint32_t base, fl
     tc::ld_wait(vb);
     freed();
     sum32(vb);
+}
+
+// ---- the cluster-tiled kernels: column tiles prepared in global memory, walked cluster by cluster
+constexpr int kStageBudget = 96 * 1024;  // shared memory for column tiles: two CTAs per SM
+constexpr int kMaxStages = 6;
+
+template <int NP, int K> struct Geom {
+    static constexpr int tile = tile_bytes(NP, K);
+    static constexpr int st = kStageBudget / tile;
+    static constexpr int stages = st > kMaxStages ? kMaxStages : st;
+    // a second row operand where 256 tensor-memory columns hold it: the next cluster's rows are then staged while
+    // the MMAs of the current one run
+    static constexpr int abuf = kCols + 2 * NP * (K / 2) <= (int)kTmemCols ? 2 : 1;
+    static_assert(kCols + NP * (K / 2) <= (int)kTmemCols && stages >= 2, "tile does not fit");
+};
+
+// Walks the tiles of the kept column clusters of a block in cluster order.
+struct TileIt {
+    int w = -1;
+    unsigned u = 0u;
+    int J = -1, g = 0, gend = 0;
+};
+__device__ __forceinline__ bool tile_next(TileIt &it, const unsigned *words, int nwords, const int *tile0) {
+    if (it.g + 1 < it.gend) {
+        ++it.g;
+        return true;
+    }
+    for (;;) {
+        while (it.u == 0u) {
+            if (++it.w >= nwords) return false;
+            it.u = words[it.w];
+        }
+        const int bit = __ffs(it.u) - 1;
+        it.u &= it.u - 1u;
+        it.J = it.w * 32 + bit;
+        it.g = tile0[it.J];
+        it.gend = tile0[it.J + 1];
+        if (it.g < it.gend) return true;
+    }
 }
 
 }  // namespace xt

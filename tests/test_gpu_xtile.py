@@ -1,4 +1,4 @@
-"""The tensor-core tiles of D > 3 against the FP64 oracle's softmin, at the edges of the tiles: point widths around the
+"""The tensor-core tiles against the FP64 oracle's softmin, at the edges of the tiles: point widths around the
 K steps (4 .. 60 coordinates), sizes of one point, of a tile and one more, of less than a tile, of no multiple of
 anything.  One coarse-to-fine step of the cluster-tiled form, and the dense sweep with its running shift."""
 import numpy as np
@@ -57,7 +57,7 @@ def test_one_step_matches_the_oracle(D, n, m, K, prec):
     ctx.close()
 
 
-@pytest.mark.parametrize("D,n,m", [(4, 1, 129), (5, 300, 1), (12, 129, 4000), (13, 257, 128), (16, 128, 127),
+@pytest.mark.parametrize("D,n,m", [(1, 129, 300), (2, 1, 40000), (3, 128, 1), (3, 4000, 2049), (3, 257, 128), (4, 1, 129), (5, 300, 1), (12, 129, 4000), (13, 257, 128), (16, 128, 127),
                                    (29, 130, 1025), (44, 64, 3001), (45, 290, 333), (60, 641, 2500), (60, 3000, 37)])
 def test_dense_sweep_matches_the_oracle(D, n, m):
     from paper_2107_02010_gb300 import otgb
@@ -87,4 +87,47 @@ def test_dense_sweep_matches_the_oracle(D, n, m):
     assert np.max(np.abs(got - want)) < BAR[0] * (np.max(np.abs(want)) + eps)
     pot[m // 2] = np.nan
     assert not np.any(np.isfinite(otgb.softmin(ctx, T(q), T(p), T(w1), T(pot), eps, lam=lam).cpu().numpy()))
+    ctx.close()
+
+
+@pytest.mark.parametrize("D,n,m,L,how", [(4, 1, 1, 1, "bundle"), (9, 129, 40, 3, "random"), (16, 200, 700, 20, "bundle"),
+                                         (29, 300, 129, 5, "random"), (45, 131, 650, 40, "ignored"),
+                                         (60, 1500, 1300, 20, "bundle"), (60, 257, 2000, 7, "random")])
+def test_label_transfer_matches_the_oracle(D, n, m, L, how):
+    """Labels along the bundles, labels that change from column to column, ignored labels, columns without weight, and
+    rows so far away that they take the safe path."""
+    from paper_2107_02010_gb300 import otgb
+
+    x = synth.fiber_bundles(n, seed=4, perturb=3.0)[0][:, :D].copy()
+    y, b, lab = synth.fiber_bundles(m, seed=5)
+    y = y[:, :D].copy()
+    rng = np.random.default_rng(8)
+    if how != "bundle":
+        lab = rng.integers(-1 if how == "ignored" else 0, L + (2 if how == "ignored" else 0), m).astype(np.int32)
+    lab = lab.astype(np.int32)
+    if m > 2:
+        b[rng.integers(0, m)] = 0.0
+    if n > 2:
+        x[n // 2] += 40.0
+    blur, eps, lam = 2.0, 4.0, 1.0 / 1.01
+    a = np.full(n, 1.0 / n, np.float32)
+    g = np.zeros(m)
+    for _ in range(3):
+        f = oracle.softmin(x, y, b, g, eps, lam)
+        g = oracle.softmin(y, x, a, f, eps, lam)
+    f, g = f.astype(np.float32), g.astype(np.float32)
+    if n > 2:
+        f[n // 2] = 0.0  # an outlier: its exponents are far below the float32 range
+    ctx = otgb.Context()
+    p = otgb.default_params(blur=blur, reach=20.0, fixed_iters=1)
+    plan = otgb.sinkhorn_divergence(ctx, T(x), T(a), T(y), T(b), p, want_plan=True)["plan"]
+    rsc, ram, rrm = oracle.transport_apply(x, y, b, eps, f.astype(np.float64), g.astype(np.float64), lab, L)
+    for want_scores in (True, False):
+        sc, am, rm = otgb.transport_apply(ctx, plan, T(f), T(g), T(lab), L, want_scores=want_scores)
+        if want_scores:
+            np.testing.assert_allclose(sc.cpu().numpy(), rsc, rtol=1e-4, atol=1e-5 * rsc.max())
+        np.testing.assert_allclose(rm.cpu().numpy(), rrm, rtol=1e-4, atol=1e-30)
+        top2 = np.sort(np.concatenate([rsc, np.zeros((n, 1))], axis=1), axis=1)[:, -2:]
+        clear = (top2[:, 1] - top2[:, 0] >= 1e-4 * top2[:, 1]) & (rrm > 1e-30)
+        assert np.all(am.cpu().numpy()[clear] == ram[clear])
     ctx.close()
