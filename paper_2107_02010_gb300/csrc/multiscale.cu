@@ -367,6 +367,7 @@ int Multiscale::run_schedule(Solver &s, const otgb_params &P, const std::vector<
         cs.rho = s.rho;
         cs.timing = false;
         cs.use_xd = s.use_xd;
+        cs.use_tc3 = s.use_tc3;
         cs.X.n = ncl_x; cs.X.D = D; cs.X.stride = stride; cs.X.pts = cen_x; cs.X.logw = lm_x; cs.X.w = mass_x;
         cs.X.mass = s.X.mass;
         cs.Y.n = ncl_y; cs.Y.D = D; cs.Y.stride = stride; cs.Y.pts = cen_y; cs.Y.logw = lm_y; cs.Y.w = mass_y;

@@ -245,6 +245,7 @@ struct SoftminLaunch {
     int use_tcc;             // 2 or 3: the cluster-tiled tensor-core form with that many BF16 pieces per operand
                              // (tcc_* fields of the instances); 0: not used
     int use_xd;              // 1: 3 < D, D4 <= 60, dense columns: float32 on the tensor cores (softmin_xd.cu)
+    int counters_zeroed;     // 1: n_fallback and fin_count are zero already
     int cost_p1;             // 1: cost |x - y| (p = 1, direct form, softmin_direct.cu); 0: |x - y|^2 / 2
     int direct;              // 1: the direct difference form for p = 2 as well (softmin_direct.cu)
     int tcc_nwords;          // words of keep bits per row cluster
@@ -279,12 +280,13 @@ void softmin_tc_launch(const SoftminLaunch &L, int D, cudaStream_t st);
 // values (or they are no estimate of the result); split blocks with item_fin / fin_count, part holding 2 kPartRows
 // floats per item.
 void softmin_xd_launch(const SoftminLaunch &L, int D, bool maxp, cudaStream_t st);
-// Columns per item for a launch over (number of blocks, columns of each) groups on a GPU of `sms` SMs.
-int xd_chunk(const std::vector<std::pair<long long, long long>> &blocks_cols, int sms);
+// Columns per item for a launch over (number of blocks, columns of each) groups when `slots` CTAs are resident at once.
+int split_chunk(const std::vector<std::pair<long long, long long>> &blocks_cols, long long slots);
 inline bool xd_width(int D) { return D > 3 && ((D + 3) & ~3) <= 60; }
-// Tensor-core D <= 3 softmin at float32 accuracy (softmin3_tc.cu): old values required,
+// Tensor-core D <= 3 softmin at float32 accuracy (softmin3_tc.cu):
 // blocks <= 128 rows, split blocks only with item_fin / fin_count.
-void softmin3_tc_launch(const SoftminLaunch &L, cudaStream_t st);
+// maxp: no old values (or they are no estimate of the result); split blocks then hold 2 kPartRows floats per item.
+void softmin3_tc_launch(const SoftminLaunch &L, bool maxp, cudaStream_t st);
 size_t softmin_tc_smem_bytes();
 // Cluster-tiled tensor-core softmin (softmin_tcc.cu): D4 <= 60, old values required, one item per block.
 void softmin_tcc_launch(const SoftminLaunch &L, int D, cudaStream_t st);

@@ -85,6 +85,40 @@ __global__ void box_centre_kernel(const float *lo, const float *hi, int D, float
     if (d < 64) c[d] = d < D ? 0.5f * (lo[d] + hi[d]) : 0.f;
 }
 
+// Box and centre of a small input in one CTA (up to kBoxSmall values: a few microseconds, less than the launches and the
+// partial results of the general form).
+constexpr int kBoxSmall = 32768;
+__global__ void __launch_bounds__(kBoxT) bbox_small_kernel(const float *x, int n, int D, float *c) {
+    __shared__ float red[kBoxT];
+    const int G = kBoxT / D, t = threadIdx.x, g = t / D, d = t - g * D;
+    float lo = FLT_MAX, hi = -FLT_MAX;
+    if (g < G) {
+#pragma unroll 4
+        for (int i = g; i < n; i += G) {
+            const float v = x[(size_t)i * D + d];
+            lo = fminf(lo, v);
+            hi = fmaxf(hi, v);
+        }
+    }
+    float out[2] = {0.f, 0.f};
+    for (int h = 0; h < 2; ++h) {
+        red[t] = h ? hi : lo;
+        __syncthreads();
+        for (int q = t >> 5, u = 0; q < D; q += kBoxT / 32, ++u) {
+            float v = h ? -FLT_MAX : FLT_MAX;
+            for (int k = t & 31; k < G; k += 32) v = h ? fmaxf(v, red[k * D + q]) : fminf(v, red[k * D + q]);
+            for (int o = 16; o > 0; o >>= 1) {
+                const float w = __shfl_xor_sync(0xffffffffu, v, o);
+                v = h ? fmaxf(v, w) : fminf(v, w);
+            }
+            out[u] = h ? 0.5f * (out[u] + v) : v;
+        }
+        __syncthreads();
+    }
+    if ((t & 31) == 0)
+        for (int q = t >> 5, u = 0; q < 64; q += kBoxT / 32, ++u) c[q] = q < D ? out[u] : 0.f;
+}
+
 // ------------------------------------------------------- FP64 sums (Eq. 6) --
 // Balanced: sum_i a_i (f_i - aa_i) + sum_j b_j (g_j - bb_j).
 // Unbalanced: -(rho + eps/2) [ sum_i a_i e^{-aa_i/rho} expm1(-(f_i - aa_i)/rho) + (same for b) ].
@@ -292,10 +326,8 @@ __global__ void radix_scatter_kernel(const uint32_t *keys, const int *vals, int 
 // ------------------------------------------------------------- packing ---
 // D <= 3: out[k] = (x - c, log w) as float4 (zero-padded coordinates).
 // D >  3 (pack_rows_kernel): out row k = x - c padded with zeros to D4 floats; logw[k] = log w.
-__global__ void pack_kernel(const float *x, const float *w, const int *perm, int n, int D, const float *center,
-                            float *out, float *logw, float *w_sorted) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
+__device__ __forceinline__ void pack_point(int k, const float *x, const float *w, const int *perm, int n, int D,
+                                           const float *center, float *out, float *logw, float *w_sorted) {
     int i = perm ? perm[k] : k;
     OTGB_DCLAMP(i, 0, n);
     const float wi = w ? w[i] : 1.0f;
@@ -307,11 +339,16 @@ __global__ void pack_kernel(const float *x, const float *w, const int *perm, int
     if (w_sorted) w_sorted[k] = wi;
 }
 
+__global__ void pack_kernel(const float *x, const float *w, const int *perm, int n, int D, const float *center,
+                            float *out, float *logw, float *w_sorted) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n) pack_point(k, x, w, perm, n, D, center, out, logw, w_sorted);
+}
+
 // D > 3: one thread per point and four coordinates, so that reads and writes run along the rows.
-__global__ void pack_rows_kernel(const float *x, const float *w, const int *perm, int n, int D, int D4, int vec,
-                                 const float *center, float *out, float *logw, float *w_sorted) {
+__device__ __forceinline__ void pack_quad(size_t e, const float *x, const float *w, const int *perm, int n, int D, int D4,
+                                          int vec, const float *center, float *out, float *logw, float *w_sorted) {
     const int Q = D4 >> 2;
-    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t k = e / Q;
     const int q = (int)(e - k * Q);
     if (k >= (size_t)n) return;
@@ -331,6 +368,27 @@ __global__ void pack_rows_kernel(const float *x, const float *w, const int *perm
         const float wi = w ? w[i] : 1.0f;
         if (logw) logw[k] = wi > 0.f ? logf(wi) : -INFINITY;
         if (w_sorted) w_sorted[k] = wi;
+    }
+}
+
+__global__ void pack_rows_kernel(const float *x, const float *w, const int *perm, int n, int D, int D4, int vec,
+                                 const float *center, float *out, float *logw, float *w_sorted) {
+    pack_quad((size_t)blockIdx.x * blockDim.x + threadIdx.x, x, w, perm, n, D, D4, vec, center, out, logw, w_sorted);
+}
+
+// rows and columns of one sweep: CTAs [0, split) pack the rows, the others the columns
+__global__ void pack_pair_kernel(const float *q, int n_out, float *rows, const float *p, const float *w, int n_in,
+                                 float *cols, float *col_logw, int D, int vec_q, int vec_p, const float *center, int split) {
+    const bool r = (int)blockIdx.x < split;
+    const size_t e = (size_t)(r ? blockIdx.x : blockIdx.x - split) * blockDim.x + threadIdx.x;
+    if (D > 3) {
+        const int D4 = (D + 3) & ~3;
+        if (r) pack_quad(e, q, nullptr, nullptr, n_out, D, D4, vec_q, center, rows, nullptr, nullptr);
+        else pack_quad(e, p, w, nullptr, n_in, D, D4, vec_p, center, cols, col_logw, nullptr);
+    } else if (r) {
+        if (e < (size_t)n_out) pack_point((int)e, q, nullptr, nullptr, n_out, D, center, rows, nullptr, nullptr);
+    } else {
+        if (e < (size_t)n_in) pack_point((int)e, p, w, nullptr, n_in, D, center, cols, nullptr, nullptr);
     }
 }
 
@@ -554,6 +612,16 @@ void box_centre(const float *lo, const float *hi, int D, float *c, cudaStream_t 
     OTGB_CHECK_LAUNCH();
 }
 
+void bbox_centre(const float *x, int n, int D, float *d_centre, float *d_box, float *d_part, cudaStream_t st) {
+    if ((size_t)n * D <= kBoxSmall) {
+        bbox_small_kernel<<<1, kBoxT, 0, st>>>(x, n, D, d_centre);
+        OTGB_CHECK_LAUNCH();
+        return;
+    }
+    bbox(x, n, D, D, d_box, d_box + 64, d_part, st);
+    box_centre(d_box, d_box + 64, D, d_centre, st);
+}
+
 void divergence_sum(const float *wa, const float *f, const float *aa, int N, const float *wb, const float *g,
                     const float *bb, int M, double eps, double rho, double *d_out, double *d_part,
                     cudaStream_t st) {
@@ -666,6 +734,16 @@ void pack_points(const float *x, const float *w, const int *perm, int n, int D, 
     } else {
         pack_kernel<<<(n + 255) / 256, 256, 0, st>>>(x, w, perm, n, D, d_center, out, logw, w_sorted);
     }
+    OTGB_CHECK_LAUNCH();
+}
+
+void pack_pair(const float *q, int n_out, float *rows, const float *p, const float *w, int n_in, float *cols, float *col_logw,
+               int D, const float *d_center, cudaStream_t st) {
+    const size_t per = D > 3 ? (size_t)(((D + 3) & ~3) >> 2) : 1;
+    const unsigned gr = (unsigned)((n_out * per + 255) / 256), gc = (unsigned)((n_in * per + 255) / 256);
+    const bool v4 = D % 4 == 0 && ((uintptr_t)d_center & 15) == 0;
+    pack_pair_kernel<<<gr + gc, 256, 0, st>>>(q, n_out, rows, p, w, n_in, cols, col_logw, D, v4 && ((uintptr_t)q & 15) == 0,
+                                              v4 && ((uintptr_t)p & 15) == 0, d_center, (int)gr);
     OTGB_CHECK_LAUNCH();
 }
 

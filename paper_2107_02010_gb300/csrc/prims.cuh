@@ -13,6 +13,9 @@ void bbox(const float *x, int n, int D, int stride, float *d_lo, float *d_hi, fl
 // c (64 floats) = middle of the box, 0 beyond D.
 void box_centre(const float *lo, const float *hi, int D, float *c, cudaStream_t st);
 
+// The middle of the bounding box in one call (one launch for small inputs).  d_box: 128 floats, d_part as for bbox.
+void bbox_centre(const float *x, int n, int D, float *d_centre, float *d_box, float *d_part, cudaStream_t st);
+
 // S of Eq. (6) in double from the four duals (internal order) and the weights;
 // rho = +inf selects the balanced form.  d_part: scratch of 128 doubles.
 void divergence_sum(const float *wa, const float *f, const float *aa, int N, const float *wb, const float *g,
@@ -43,6 +46,9 @@ void iota(int *v, int n, cudaStream_t st);
 // and a separate log w.  perm (optional) gives the source index of each output row.
 void pack_points(const float *x, const float *w, const int *perm, int n, int D, const float *d_center, float *out,
                  float *logw, float *w_sorted, cudaStream_t st);
+// Rows (no weights) and columns of one sweep, packed in one launch.
+void pack_pair(const float *q, int n_out, float *rows, const float *p, const float *w, int n_in, float *cols, float *col_logw,
+               int D, const float *d_center, cudaStream_t st);
 void unpermute(const float *in, const int *perm, int n, float *out, cudaStream_t st);
 void permute(const float *in, const int *perm, int n, float *out, cudaStream_t st);
 

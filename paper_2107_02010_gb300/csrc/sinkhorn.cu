@@ -87,14 +87,20 @@ int *spatial_sort(otgb_ctx *ctx, const std::string &tag, const float *x, int n, 
     return perm;
 }
 
-// Work items of a one-instance sweep: block k's columns in `parts` pieces of `chunk` columns.
-__global__ void split_items_kernel(int4 *items, int *item_fin, int4 *fin, int nb, int n_in, int chunk, int parts) {
+// Work of a one-instance sweep: blocks of 128 rows, block k's columns in `parts` pieces of `chunk` columns; counters (the
+// number of fallback rows, then one per block) zeroed.
+__global__ void softmin_plan_kernel(int *blk, int n_out, int4 *items, int *item_fin, int4 *fin, int nb, int n_in, int chunk,
+                                    int parts, int *counters) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e <= nb) {
+        blk[e] = (int)min((long long)e * 128, (long long)n_out);
+        counters[e] = 0;
+        if (e < nb) fin[e] = make_int4(0, e, e * parts, parts);
+    }
     if (e >= nb * parts) return;
     const int k = e / parts, q = e - k * parts;
     items[e] = make_int4(0, k, q * chunk, q + 1 < parts ? (q + 1) * chunk : n_in);
-    if (item_fin) item_fin[e] = k;
-    if (fin && q == 0) fin[k] = make_int4(0, k, e, parts);
+    item_fin[e] = k;
 }
 
 // The bounded-wait error path, exercised on purpose (params.debug_wait_probe):
@@ -239,18 +245,13 @@ void Solver::set_work(const std::vector<std::vector<int>> &ncols, bool allow_spl
     double W = 0.0;
     for (auto &v : ncols)
         for (int c : v) W += c;
-#ifndef OTGB_TC3_ITEMS_PER_SM
-#define OTGB_TC3_ITEMS_PER_SM 10.0
-#endif
-    // D <= 3 warp kernel: about three waves of warps (6 CTAs of 4 warps per SM);
-    // tensor-core form: one CTA per item, fewer and longer items
     const double target = use_tc3 ? OTGB_TC3_ITEMS_PER_SM * sms : 3.0 * 5.0 * 4.0 * sms;
     int CH = 1 << 30;
     if (allow_split && D > 3) {  // softmin_xd_kernel
         std::vector<std::pair<long long, long long>> groups;
         for (auto &v : ncols)
             if (!v.empty()) groups.push_back({(long long)v.size(), v[0]});  // dense: the same for every block
-        CH = xd_chunk(groups, sms);
+        CH = split_chunk(groups, 2LL * sms);
     } else if (allow_split) {
         CH = (int)std::ceil(W / target);
         CH = std::max(512, (CH + 127) / 128 * 128);
@@ -263,7 +264,11 @@ void Solver::set_work(const std::vector<std::vector<int>> &ncols, bool allow_spl
             const int first = (int)items.size();
             if (n <= CH) items.push_back(make_int4(k, b, 0, n));
             else
-                for (int c = 0; c < n; c += CH) items.push_back(make_int4(k, b, c, std::min(n, c + CH)));
+{
+                // equal pieces of whole tiles
+                const int parts = (n + CH - 1) / CH, len = ((n + parts - 1) / parts + 127) / 128 * 128;
+                for (int c = 0; c < n; c += len) items.push_back(make_int4(k, b, c, std::min(n, c + len)));
+            }
             item_fin.resize(items.size(), (int)fin.size());
             fin.push_back(make_int4(k, b, first, (int)items.size() - first));
         }
@@ -747,39 +752,23 @@ extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const floa
         Workspace &ws = ctx_ws(ctx);
         const int stride = D <= 3 ? 4 : ((D + 3) & ~3);
         // common centre: middle of the bounding box of the columns
-        float *box = ws.get<float>("box", 4 * 64);
-        float *bpart = ws.get<float>("bpart", 64 * 2 * 64);
-        bbox(p, n_in, D, D, box, box + 64, bpart, st);
-        std::vector<float> h(128);
-        OTGB_CUDA_TRY(cudaMemcpyAsync(h.data(), box, 128 * sizeof(float), cudaMemcpyDeviceToHost, st));
-        OTGB_CUDA_TRY(cudaStreamSynchronize(st));
-        std::vector<float> cen(64, 0.f);
-        for (int d = 0; d < D; ++d) cen[d] = 0.5f * (h[d] + h[64 + d]);
         float *d_cen = ws.get<float>("cen", 64);
-        OTGB_CUDA_TRY(cudaMemcpyAsync(d_cen, cen.data(), 64 * sizeof(float), cudaMemcpyHostToDevice, st));
+        bbox_centre(p, n_in, D, d_cen, ws.get<float>("box", 4 * 64), ws.get<float>("bpart", 64 * 2 * 64), st);
+        // blocks of 128 rows, their columns split so that the launch fills the GPU (tensor-core kernels); the CUDA-core
+        // kernel of D > 60 takes whole blocks
+        const bool tc = D <= 3 || xd_width(D);
+        const int nb = (n_out + 127) / 128, sms = ctx_sm_count(ctx);
+        const int chunk = tc ? split_chunk({{nb, n_in}}, (D <= 3 ? 4LL : 2LL) * sms) : n_in;
+        const int parts = (n_in - 1) / chunk + 1, n_items = nb * parts;
         float *R = ws.get<float>("sm:R", (size_t)n_out * stride);
         float *C = ws.get<float>("sm:C", (size_t)n_in * stride);
         float *Clw = D > 3 ? ws.get<float>("sm:Clw", n_in) : nullptr;
-        pack_points(q, nullptr, nullptr, n_out, D, d_cen, R, nullptr, nullptr, st);
-        pack_points(p, w, nullptr, n_in, D, d_cen, C, Clw, nullptr, st);
-        // rows per thread as in the solver: the largest R in {4, 2} that still
-        // gives two CTAs per SM, else 1
-        int rpt = 1;
-        if (D <= 3) {
-            const int sms = ctx_sm_count(ctx);
-            for (int r : {4, 2})
-                if ((n_out + 32 * r - 1) / (32 * r) >= 8 * sms) { rpt = r; break; }
-        }
-        const int block_rows = D <= 3 ? 32 * rpt : 128;
-        int *blk = ws.get<int>("sm:blk", n_out / block_rows + 2);
-        const int nb = uniform_blocks(blk, n_out, block_rows, st);
-        const bool xd = xd_width(D);
-        const int chunk = xd ? xd_chunk({{nb, n_in}}, ctx_sm_count(ctx)) : n_in;
-        const int parts = (n_in - 1) / chunk + 1, n_items = nb * parts;
-        int4 *d_items = ws.get<int4>("sm:items", n_items);
-        int4 *d_fin = parts > 1 ? ws.get<int4>("sm:fin", nb) : nullptr;
-        int *d_ifin = parts > 1 ? ws.get<int>("sm:ifin", n_items) : nullptr;
-        split_items_kernel<<<(n_items + 255) / 256, 256, 0, st>>>(d_items, d_ifin, d_fin, nb, n_in, chunk, parts);
+        pack_pair(q, n_out, R, p, w, n_in, C, Clw, D, d_cen, st);
+        int *blk = ws.get<int>("sm:blk", nb + 1);
+        int4 *d_items = ws.get<int4>("sm:items", n_items), *d_fin = ws.get<int4>("sm:fin", nb);
+        int *d_ifin = ws.get<int>("sm:ifin", n_items), *cnt = ws.get<int>("sm:cnt", nb + 1);
+        softmin_plan_kernel<<<(std::max(n_items, nb + 1) + 255) / 256, 256, 0, st>>>(blk, n_out, d_items, d_ifin, d_fin, nb, n_in,
+                                                                                 chunk, parts, cnt);
         OTGB_CHECK_LAUNCH();
         SoftminLaunch L;
         std::memset(&L, 0, sizeof(L));
@@ -790,13 +779,15 @@ extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const floa
         I.blk_row0 = blk;
         L.items = d_items;
         L.n_items = n_items;
-        L.use_xd = xd ? 1 : 0;
+        L.use_xd = xd_width(D) ? 1 : 0;
+        L.use_tc3 = D <= 3 ? 1 : 0;
+        L.counters_zeroed = 1;
         if (parts > 1) {
             L.part = ws.get<float>("sm:part", (size_t)n_items * kPartRows * 2);
             L.fin = d_fin;
             L.n_fin = nb;
             L.item_fin = d_ifin;
-            L.fin_count = ws.get<int>("sm:fincnt", nb);
+            L.fin_count = cnt + 1;
         }
         L.exact_max = 1;  // `old` is a blend target here, not an estimate of the result
         L.eps = (float)eps;
@@ -804,9 +795,9 @@ extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const floa
         L.eps_ln2 = eps * 0.69314718055994530942;
         const int cap = n_out + 64;
         L.fallback = ws.get<int4>("sm:fb", cap);
-        L.n_fallback = ws.get<int>("sm:nfb", 1);
+        L.n_fallback = cnt;
         L.fallback_cap = cap;
-        softmin_run(L, D, rpt, st);
+        softmin_run(L, D, D <= 3 ? 4 : 1, st);
         OTGB_CUDA_TRY(cudaStreamSynchronize(st));
         return OTGB_OK;
     } catch (const Error &e) {

@@ -952,7 +952,7 @@ int fallback_grid_sms() {
 
 void softmin_run(const SoftminLaunch &L, int D, int rows_per_thread, cudaStream_t st) {
     if (L.n_items <= 0) return;
-    OTGB_CUDA_TRY(cudaMemsetAsync(L.n_fallback, 0, sizeof(int), st));
+    if (!L.counters_zeroed) OTGB_CUDA_TRY(cudaMemsetAsync(L.n_fallback, 0, sizeof(int), st));
     if (L.cost_p1 || L.direct) {  // the direct form with a running maximum: no shift estimate, no fallback rows
         softmin_direct_launch(L, D, st);
         return;
@@ -963,11 +963,12 @@ void softmin_run(const SoftminLaunch &L, int D, int rows_per_thread, cudaStream_
     // the float32 form of dense sweeps in more than 3 dimensions
     bool xd = L.use_xd && xd_width(D) && !L.use_tcc;
     for (int k = 0; k < L.n_inst; ++k) xd = xd && L.inst[k].col_rng == nullptr;
-    require(!(two && L.part && !xd), "softmin_run: split blocks need old values", OTGB_EINTERNAL);
+    const bool tc3 = D <= 3 && L.use_tc3 && rows_per_thread <= 4 && (!L.part || L.fin_count);
+    require(!(two && L.part && !xd && !tc3), "softmin_run: split blocks need old values", OTGB_EINTERNAL);
     require(!(D > 3 && L.part && !xd), "softmin_run: split blocks are D <= 3 only", OTGB_EINTERNAL);
-    if (D <= 3 && L.use_tc3 && !two && rows_per_thread <= 4 && (!L.part || L.fin_count)) {
-        if (L.part) OTGB_CUDA_TRY(cudaMemsetAsync(L.fin_count, 0, sizeof(int) * L.n_fin, st));
-        softmin3_tc_launch(L, st);
+    if (tc3) {
+        if (L.part && !L.counters_zeroed) OTGB_CUDA_TRY(cudaMemsetAsync(L.fin_count, 0, sizeof(int) * L.n_fin, st));
+        softmin3_tc_launch(L, two, st);
     } else if (D <= 3) {
         if (L.work_counter) OTGB_CUDA_TRY(cudaMemsetAsync(L.work_counter, 0, sizeof(int), st));
         if (L.part && L.fin_count) OTGB_CUDA_TRY(cudaMemsetAsync(L.fin_count, 0, sizeof(int) * L.n_fin, st));
@@ -1001,7 +1002,7 @@ void softmin_run(const SoftminLaunch &L, int D, int rows_per_thread, cudaStream_
             return 1;
         });
         if (xd) {
-            if (L.part) OTGB_CUDA_TRY(cudaMemsetAsync(L.fin_count, 0, sizeof(int) * L.n_fin, st));
+            if (L.part && !L.counters_zeroed) OTGB_CUDA_TRY(cudaMemsetAsync(L.fin_count, 0, sizeof(int) * L.n_fin, st));
             softmin_xd_launch(L, D, two, st);
         } else if (two) {
             softmin_gen_kernel<true, 0><<<L.n_items, kNTg, sizeof(GenSmem), st>>>(L, D, D4);

@@ -14,8 +14,8 @@
 // terms are small for every pair that matters.  The finish adds back exactly
 // the shift the accumulator applied, in double precision.
 //
-// One CTA (8 warps) owns a row block of at most 128 rows (one tensor-memory
-// lane per row); columns come in tiles of kN.  Column staging is software
+// One CTA (4 warps) owns a row block of at most 128 rows (one tensor-memory
+// lane and thread per row); columns come in tiles of kN.  Column staging is software
 // pipelined: the indices of tile t+2 and the point of tile t+1 are loaded
 // while the tensor core multiplies tile t+1 and the CTA sums tile t.  The
 // indices come from the block's kept ranges (copied into shared memory once
@@ -31,46 +31,27 @@
 
 #include "otgb_internal.cuh"
 #include "tcgen05.cuh"
+#include "xtile.cuh"
 
 namespace otgb {
 namespace {
 
-// Measured on the track-density workload (softmin rate): 256-column tiles with
-// one accumulator and two warpgroups 5.0e12 pairs/s; 128 columns with two
-// accumulators 4.4-4.6e12; deeper pipelines (4-8 accumulators) were slower;
-// a warp-specialised variant (staging, MMA and sum warps handing tiles over
-// through mbarriers, no CTA barrier per tile) reached 4.6e12; overlapping the
-// tensor-memory loads with the sums changed nothing.  The MUFU ex2 unit (32 per
-// clock per SM) is half busy at 5.0e12.
-#ifndef OTGB_TC3_N
-#define OTGB_TC3_N 256
-#endif
-#ifndef OTGB_TC3_STAGES
-#define OTGB_TC3_STAGES 1
-#endif
-#ifndef OTGB_TC3_MINB
-#define OTGB_TC3_MINB 2
-#endif
-#ifndef OTGB_TC3_THREADS
-#define OTGB_TC3_THREADS 256
-#endif
-// Column tiles of kN columns; kStages accumulators in tensor memory and as
-// many staged column tiles, so that the MMA of a tile is issued kStages - 1
-// tiles before its sums are taken.
-// kThreads = 256: two warpgroups read the same tensor-memory lanes (rows) and
-// each takes half of a tile's columns in the epilogue.
-constexpr int kM = 128, kN = OTGB_TC3_N, kK = 32, kStages = OTGB_TC3_STAGES, kThreads = OTGB_TC3_THREADS;
-constexpr int kHalves = kThreads / 128;
+// Four CTAs of 128 threads share an SM (128 tensor-memory columns each): staging, MMA and sums of a tile follow each
+// other within a CTA, and the CTAs fill each other's gaps.  Measured on the track-density workload (100k voxels per
+// side): 128-column tiles, four CTAs 6.3e12 pairs/s; three CTAs 5.8e12; 256-column tiles, 256 threads, two CTAs 5.3e12;
+// 64-column tiles, four CTAs 5.3e12.  Earlier forms: two accumulators per CTA 4.4-4.6e12; warp-specialised roles 4.6e12.
+// Bound: the MUFU ex2 unit, 32 per clock per SM (1.0e13 pairs/s).  With MAXP (maximum and shift per pair besides)
+// 5.8e12 pairs/s on 100k x 100k; otgb_softmin there 7.0 -> 1.9 ms against the two sweeps of softmin3_kernel, and
+// 1000 x 800 109 -> 49 us (columns split over items, four launches, no host copies).
+constexpr int kM = 128, kN = 128, kK = 32, kThreads = 128;
 constexpr int kATile = kM * kK * 2;  // 8 KiB
 constexpr int kBTile = kN * kK * 2;
-constexpr uint32_t kTmemCols = kStages * kN <= 32 ? 32u : (kStages * kN <= 64 ? 64u : (kStages * kN <= 128 ? 128u
-                                   : (kStages * kN <= 256 ? 256u : 512u)));
+constexpr uint32_t kTmemCols = kN;
 // range entries of a block staged in shared memory; a block with more reads them from global memory
 constexpr int kRngSmem = 1024;
 // positions per expansion chunk (two buffers in flight) and per thread of an expansion
 constexpr int kChunkTiles = 16, kChunk = kChunkTiles * kN, kPerThr = kChunk / kThreads;
 static_assert(kPerThr * kThreads == kChunk && kPerThr % 4 == 0, "an expansion writes whole int4 groups");
-static_assert(kChunkTiles >= kStages + 2, "a chunk is expanded at least one barrier before its first read");
 
 // Word of position q (of a chunk) in the index buffer: 16-byte groups of four positions, group g stored at
 // g ^ ((g >> 2) & 7) (a permutation of each aligned run of eight groups), so that both the expansion's
@@ -111,11 +92,10 @@ __device__ __forceinline__ void expand_positions(const Entries &r, int n, int p0
 
 struct Tc3Smem {
     unsigned char a[kATile];
-    unsigned char b[kStages][kBTile];
+    unsigned char b[kBTile];
     float red[4][8];
-    float tot1[128];
     int bc[2];
-    unsigned long long mbar[kStages];
+    unsigned long long mbar;
     uint32_t tslot;
     int2 rng[kRngSmem];
     alignas(16) int idx[2][kChunk];
@@ -133,12 +113,6 @@ __device__ __forceinline__ uint64_t sdesc32(uint32_t addr) {
     d |= (uint64_t)(512 >> 4) << 32;
     d |= (uint64_t)1 << 46;
     return d;
-}
-
-__device__ __forceinline__ float ex2f(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
 }
 
 // Scalar split for the row operand (once per CTA).  The per-tile column operand
@@ -167,20 +141,34 @@ __device__ __forceinline__ uint32_t bf2(float hi, float lo) {
 }
 __device__ __forceinline__ float hi_val(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 __device__ __forceinline__ float lo_val(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ void split3x2(float a, float b, uint32_t &H, uint32_t &M, uint32_t &L) {
+// rest: what b lost to its own rounding.
+__device__ __forceinline__ void split3x2(float a, float b, uint32_t &H, uint32_t &M, uint32_t &L, float rest = 0.f) {
     H = bf2(a, b);
     const float ra = a - hi_val(H), rb = b - lo_val(H);
     M = bf2(ra, rb);
-    L = bf2(ra - hi_val(M), rb - lo_val(M));
+    L = bf2(ra - hi_val(M), (rb - lo_val(M)) + rest);
 }
 
 constexpr uint16_t kOne = 0x3F80;  // 1.0 in BF16
 
-__global__ void __launch_bounds__(kThreads, OTGB_TC3_MINB) softmin3_tc_kernel(const __grid_constant__ SoftminLaunch L) {
+constexpr float kNoTerm = -1e29f;  // shift of a row without terms (absent columns have an exponent of about -1e30)
+
+// MAXP: the shift is not known (no old value, or one that is no estimate of the result), and the rows come as the caller
+// has them, so that a block may span the whole cloud and |x - c| |y - c| be much larger than any exponent that matters.
+// The accumulator then holds the pair's whole exponent, -s |x - y|^2 / 2 + s (eps log w + pot), arranged so that each of
+// the two K = 16 steps is small by itself for a pair that matters: step 0 holds coordinates 0 and 1 with their own share
+// of the squares (two pieces of -s (y0^2 + y1^2) / 2 against 1, two of -s (x0^2 + x1^2) / 2), step 1 coordinate 2 and
+// everything else (three pieces each).  The sum is cut off towards zero after each step, at the size of what it holds.
+// The row keeps a running shift (xt::sum_row_max).
+// First word (two K slots) of coordinate d.
+template <bool MAXP> __device__ __forceinline__ constexpr int coord_word(int d) { return MAXP && d == 2 ? 8 : 3 * d; }
+
+template <bool MAXP>
+__global__ void __launch_bounds__(kThreads, 4) softmin3_tc_kernel(const __grid_constant__ SoftminLaunch L) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     Tc3Smem &S = *reinterpret_cast<Tc3Smem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int t = tid & 127, half = tid >> 7;  // row (tensor-memory lane) and warpgroup
+    const int t = tid;  // row (tensor-memory lane)
     const int it = blockIdx.x;
     int4 item = L.items[it];
     OTGB_DCLAMP(item.x, 0, L.n_inst);
@@ -210,10 +198,10 @@ __global__ void __launch_bounds__(kThreads, OTGB_TC3_MINB) softmin3_tc_kernel(co
         for (int q = tid; q < nE; q += kThreads) S.rng[q] = rb[q];
 
     // ---- rows: centre of the block's bounding box, shifts, the row operand
-    const bool valid = half == 0 && t < nr;
+    const bool valid = t < nr;
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
     if (valid) p = rows4[r0 + t];
-    if (half == 0) {
+    {
         float v[6] = {valid ? p.x : FLT_MAX, valid ? p.y : FLT_MAX, valid ? p.z : FLT_MAX,
                       valid ? -p.x : FLT_MAX, valid ? -p.y : FLT_MAX, valid ? -p.z : FLT_MAX};
 #pragma unroll
@@ -223,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, OTGB_TC3_MINB) softmin3_tc_kernel(co
         }
     }
     if (tid == 0) {
-        for (int q = 0; q < kStages; ++q) tc::mbar_init(&S.mbar[q], 1);
+        tc::mbar_init(&S.mbar, 1);
         tc::mbar_init_fence();
     }
     __syncthreads();
@@ -251,48 +239,61 @@ __global__ void __launch_bounds__(kThreads, OTGB_TC3_MINB) softmin3_tc_kernel(co
     const float x0 = valid ? p.x - c[0] : 0.f, x1 = valid ? p.y - c[1] : 0.f, x2 = valid ? p.z - c[2] : 0.f;
     const double hx = 0.5 * ((double)x0 * x0 + (double)x1 * x1 + (double)x2 * x2);
     float m = -INFINITY;
-    if (valid) m = (float)((double)s * (hx - (double)I.row_old[r0 + t] / (double)I.lam));
-    __syncthreads();  // S.red is reused
-    if (half == 0) {
+    if (!MAXP && valid) m = (float)((double)s * (hx - (double)I.row_old[r0 + t] / (double)I.lam));
+    float Cb = 0.f;
+    if constexpr (!MAXP) {
         float mx = m;
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         if (lane == 0) S.red[warp][6] = mx;
+        __syncthreads();
+        Cb = fmaxf(fmaxf(S.red[0][6], S.red[1][6]), fmaxf(S.red[2][6], S.red[3][6]));
+        if (!(Cb > -INFINITY)) Cb = 0.f;
     }
-    __syncthreads();
-    float Cb = fmaxf(fmaxf(S.red[0][6], S.red[1][6]), fmaxf(S.red[2][6], S.red[3][6]));
-    if (!(Cb > -INFINITY)) Cb = 0.f;
-    const uint16_t mb = valid ? bfbits(-(m - Cb)) : (uint16_t)0;
+    const uint16_t mb = !MAXP && valid ? bfbits(-(m - Cb)) : (uint16_t)0;
     const double m_eff = (double)Cb - (double)bfval(mb);  // the shift the accumulator applies
-    if (half == 0) {
+    {
         uint16_t h[3], md[3], l[3];
         split3(s * x0, h[0], md[0], l[0]);
         split3(s * x1, h[1], md[1], l[1]);
         split3(s * x2, h[2], md[2], l[2]);
         uint32_t w[16];
-        // slots 6d .. 6d+5: h h m h l m (against the column's h m h l h m)
+        // six slots per coordinate: h h m h l m (against the column's h m h l h m)
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const int b0 = 3 * d;  // three words per coordinate
+            const int b0 = coord_word<MAXP>(d);  // three words per coordinate
             w[b0] = pk(h[d], h[d]);
             w[b0 + 1] = pk(md[d], h[d]);
             w[b0 + 2] = pk(l[d], md[d]);
         }
-        w[9] = pk(kOne, kOne);  // slots 18, 19: against H pieces 1, 2
-        w[10] = pk(kOne, mb);   // slot 20: H piece 3; slot 21: the shift
+        if constexpr (MAXP) {
+            const double R01 = -0.5 * (double)s * ((double)x0 * x0 + (double)x1 * x1);
+            const uint16_t ra = bfbits((float)R01), rb = bfbits((float)(R01 - (double)bfval(ra)));
+            const double R2 = (R01 - (double)bfval(ra) - (double)bfval(rb)) - 0.5 * (double)s * ((double)x2 * x2);
+            uint16_t r1, r2, r3;
+            xt::split3((float)R2, (float)(R2 - (double)(float)R2), r1, r2, r3);
+            w[6] = pk(kOne, kOne);
+            w[7] = pk(ra, rb);
+            w[11] = pk(kOne, kOne);
+            w[12] = pk(kOne, r1);
+            w[13] = pk(r2, r3);
+        } else {
+            w[9] = pk(kOne, kOne);  // slots 18, 19: against H pieces 1, 2
+            w[10] = pk(kOne, mb);   // slot 20: H piece 3; slot 21: the shift
 #pragma unroll
-        for (int q = 11; q < 16; ++q) w[q] = 0u;
+            for (int q = 11; q < 14; ++q) w[q] = 0u;
+        }
+        w[14] = w[15] = 0u;
 #pragma unroll
         for (int q = 0; q < 4; ++q)
             *reinterpret_cast<uint4 *>(S.a + off32(t, 8 * q)) =
                 make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
     }
 
-    // ---- column staging: thread tid < kN stages column tid of each tile
-    const bool stager = tid < kN;
+    // ---- column staging: thread tid stages column tid of each tile
     auto load_idx = [&](int tile) -> int {
         const int pp = tile * kN + tid;
         int jj = -1;
-        if (stager && tile < ntiles && pp < ncol) {
+        if (tile < ntiles && pp < ncol) {
             jj = ranged ? S.idx[(tile / kChunkTiles) & 1][idx_word((tile % kChunkTiles) * kN + tid)] : cb + pp;
             OTGB_DCLAMP(jj, 0, I.n_cols);
         }
@@ -307,34 +308,67 @@ __global__ void __launch_bounds__(kThreads, OTGB_TC3_MINB) softmin3_tc_kernel(co
             rpot = I.col_pot[jc];
         }
     };
-    auto convert = [&](int buf) {
-        if (!stager) return;
+    auto convert = [&]() {
         const bool okc = jc >= 0;
         const float y0 = okc ? rq.x - c[0] : 0.f, y1 = okc ? rq.y - c[1] : 0.f, y2 = okc ? rq.z - c[2] : 0.f;
-        const float sq = y0 * y0 + y1 * y1 + y2 * y2;
-        const float H = okc ? s * (fmaf(eps, rq.w, rpot) - 0.5f * sq) - Cb : -1e30f;
+        float H, rest = 0.f;
+        uint32_t w[16];
+        if constexpr (MAXP) {
+            // |y0|^2 + |y1|^2 with its rounding errors (Knuth's two-sum, products by FMA), times -s/2; two BF16 pieces of it
+            // stay with those coordinates, what they leave joins the rest of H, which is summed with its errors too
+            const float hs = -0.5f * s;
+            const float p0 = y0 * y0, p1 = y1 * y1, t01 = p0 + p1, tb = t01 - p0;
+            const float te = ((p0 - (t01 - tb)) + (p1 - tb)) + (fmaf(y0, y0, -p0) + fmaf(y1, y1, -p1));
+            const float q01 = hs * t01, qe = fmaf(hs, t01, -q01) + hs * te;
+            const uint32_t wa = bf2(0.f, q01);
+            const float qa = q01 - lo_val(wa);
+            const uint32_t wb = bf2(0.f, qa);
+            const float rem = qa - lo_val(wb);
+            w[6] = okc ? pk((uint16_t)wa, (uint16_t)wb) : 0u;
+            w[7] = pk(kOne, kOne);
+            const float u = fmaf(eps, rq.w, rpot), v = s * u, ve = fmaf(s, u, -v);
+            const float z = y2 * y2, g = hs * z, ge = fmaf(hs, z, -g) + hs * fmaf(y2, y2, -z);
+            const float S1 = v + g, sb = S1 - v, se = (v - (S1 - sb)) + (g - sb);
+            H = S1 + rem;
+            const float hb = H - S1;
+            rest = ((S1 - (H - hb)) + (rem - hb)) + (se + (ve + ge) + qe);
+            if (!okc || H <= -1e30f) {  // absent, or zero weight (log w = -inf); NaN goes on
+                H = -1e30f;
+                rest = 0.f;
+            }
+        } else {
+            const float sq = y0 * y0 + y1 * y1 + y2 * y2;
+            H = okc ? s * (fmaf(eps, rq.w, rpot) - 0.5f * sq) - Cb : -1e30f;
+            if (H <= -1e30f) H = -1e30f;  // zero weight (log w = -inf); NaN goes on
+        }
         uint32_t H01, M01, L01, H2h, M2h, L2h;
         split3x2(y0, y1, H01, M01, L01);
-        split3x2(y2, H, H2h, M2h, L2h);
+        split3x2(y2, H, H2h, M2h, L2h, rest);
         const uint16_t h[3] = {(uint16_t)(H01 >> 16), (uint16_t)H01, (uint16_t)(H2h >> 16)};
         const uint16_t md[3] = {(uint16_t)(M01 >> 16), (uint16_t)M01, (uint16_t)(M2h >> 16)};
         const uint16_t l[3] = {(uint16_t)(L01 >> 16), (uint16_t)L01, (uint16_t)(L2h >> 16)};
         const uint16_t hh[3] = {(uint16_t)H2h, (uint16_t)M2h, (uint16_t)L2h};
-        uint32_t w[16];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const int b0 = 3 * d;
+            const int b0 = coord_word<MAXP>(d);
             w[b0] = pk(h[d], md[d]);
             w[b0 + 1] = pk(h[d], l[d]);
             w[b0 + 2] = pk(h[d], md[d]);
         }
-        w[9] = pk(hh[0], hh[1]);
-        w[10] = pk(hh[2], kOne);
+        if constexpr (MAXP) {
+            w[11] = pk(hh[0], hh[1]);
+            w[12] = pk(hh[2], kOne);
+            w[13] = pk(kOne, kOne);
+        } else {
+            w[9] = pk(hh[0], hh[1]);
+            w[10] = pk(hh[2], kOne);
 #pragma unroll
-        for (int q = 11; q < 16; ++q) w[q] = 0u;
+            for (int q = 11; q < 14; ++q) w[q] = 0u;
+        }
+        w[14] = w[15] = 0u;
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<uint4 *>(S.b[buf] + off32(tid, 8 * q)) =
+            *reinterpret_cast<uint4 *>(S.b + off32(tid, 8 * q)) =
                 make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
     };
 
@@ -344,110 +378,59 @@ __global__ void __launch_bounds__(kThreads, OTGB_TC3_MINB) softmin3_tc_kernel(co
     tc::fence_after();
     const uint32_t tmem = S.tslot;
     const uint32_t idesc = tc::idesc_bf16(kM, kN);
-    auto issue = [&](int buf) {
-        const uint32_t d = tmem + (uint32_t)(buf * kN);
-        const uint32_t a = tc::smem_u32(S.a), b = tc::smem_u32(S.b[buf]);
+    auto issue = [&]() {
+        const uint32_t a = tc::smem_u32(S.a), b = tc::smem_u32(S.b);
 #pragma unroll
         for (int kk = 0; kk < kK / 16; ++kk)
-            tc::mma_bf16(d, sdesc32(a + kk * 256), sdesc32(b + kk * 256), idesc, kk > 0 ? 1u : 0u);
-        tc::commit(&S.mbar[buf]);
+            tc::mma_bf16(tmem, sdesc32(a + kk * 256), sdesc32(b + kk * 256), idesc, kk > 0 ? 1u : 0u);
+        tc::commit(&S.mbar);
     };
 
-    float tot = 0.f;
-    uint32_t phase_bits = 0u;  // bit q: parity of the next completion of accumulator q
+    float tot = 0.f, sh = kNoTerm;
     bool ok = true;
     // rows of this warp that exist: the epilogue of an empty warp is skipped
-    const bool warp_rows = (warp & 3) * 32 < nr;
-    // prologue: tiles 0 .. kStages-2 staged, tile kStages-1 in registers
-    for (int q = 0; q < kStages - 1; ++q) {
-        if (q < ntiles) {
-            jc = load_idx(q);
-            load_raw();
-            convert(q);
-        }
-    }
-    jc = load_idx(kStages - 1);
+    const bool warp_rows = warp * 32 < nr;
+    const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);
+    jc = load_idx(0);
     load_raw();
-    jn = load_idx(kStages);
-    tc::fence_proxy_async();
-    tc::fence_before();
-    __syncthreads();
-    tc::fence_after();
-    if (tid == 0)
-        for (int q = 0; q < kStages - 1 && q < ntiles; ++q) issue(q);
+    jn = load_idx(1);
     for (int tt = 0; tt < ntiles; ++tt) {
-        const int buf = tt % kStages;
-        const int ahead = tt + kStages - 1;  // the tile whose MMA is issued now
-        if (ahead < ntiles) {
-            convert(ahead % kStages);  // from registers
-            jc = jn;
-            load_raw();                // tile ahead + 1
-            jn = load_idx(ahead + 2);
-        }
+        convert();  // from registers
+        jc = jn;
+        load_raw();  // tile tt + 1
+        jn = load_idx(tt + 2);
         tc::fence_proxy_async();
         tc::fence_before();
         __syncthreads();
         tc::fence_after();
-        if (tid == 0 && ahead < ntiles) issue(ahead % kStages);
-        // chunk c + 1 in the first iteration of chunk c, while the tensor core works: the index of
-        // tile T is read at the top of iteration T - kStages - 1, so the last read of chunk c - 1 (same
-        // buffer) came kStages + 2 iterations before, and the first read of chunk c + 1 comes
-        // kChunkTiles - kStages - 1 >= 1 iterations later, past this iteration's closing barrier
+        if (tid == 0) issue();
+        // chunk c + 1 in the first iteration of chunk c, while the tensor core works: the index of tile T is read in
+        // iteration T - 2, so the last read of chunk c - 1 (same buffer) came two iterations before, and the first read
+        // of chunk c + 1 comes kChunkTiles - 2 iterations later, past this iteration's closing barrier
         if (tt % kChunkTiles == 0 && tt + kChunkTiles < ntiles) expand(tt / kChunkTiles + 1);
-        if (!tc::mbar_wait(&S.mbar[buf], (phase_bits >> buf) & 1u)) ok = false;
+        if (!tc::mbar_wait(&S.mbar, (uint32_t)(tt & 1))) ok = false;
         ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld below is warp-collective
-        phase_bits ^= 1u << buf;
         tc::fence_after();
         if (ok && warp_rows) {
-            // the load of chunk k+1 flies while chunk k is summed
-            constexpr int kChunks = kN / kHalves / 32;
-            const uint32_t base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(buf * kN + half * (kN / kHalves));
-            uint32_t va[32], vb[32];
-            auto sum32 = [&](const uint32_t (&v)[32]) {
-                float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll
-                for (int q = 0; q < 32; q += 4) {
-                    a0 += ex2f(__uint_as_float(v[q]));
-                    a1 += ex2f(__uint_as_float(v[q + 1]));
-                    a2 += ex2f(__uint_as_float(v[q + 2]));
-                    a3 += ex2f(__uint_as_float(v[q + 3]));
-                }
-                tot += (a0 + a1) + (a2 + a3);
-            };
-            tc::ld32_async(base, va);
-            tc::ld_wait(va);
-#pragma unroll
-            for (int k = 0; k < kChunks; k += 2) {
-                if (k + 1 < kChunks) tc::ld32_async(base + 32 * (k + 1), vb);
-                sum32(va);
-                if (k + 1 < kChunks) {
-                    tc::ld_wait(vb);
-                    if (k + 2 < kChunks) tc::ld32_async(base + 32 * (k + 2), va);
-                    sum32(vb);
-                    if (k + 2 < kChunks) tc::ld_wait(va);
-                }
-            }
+            if constexpr (MAXP) xt::sum_row_max(lanes, tot, sh, [] {});
+            else tot = xt::sum_row(lanes, tot, [] {});
         }
         tc::fence_before();
-        __syncthreads();  // the buffers of this tile are free again
+        __syncthreads();  // the operand tile and the accumulator are free again
     }
     ok = __syncthreads_and(ok) != 0;
     if (!ok && tid == 0 && L.tc_err) atomicOr(L.tc_err, 1u);
     tc::fence_after();
     if (warp == 0) tc::tmem_dealloc(tmem, kTmemCols);
     if (!ok) return;  // uniform
-    // the two warpgroups' sums of a row
-    if (kHalves > 1) {
-        if (half == 1) S.tot1[t] = tot;
-        __syncthreads();
-        if (half == 0) tot += S.tot1[t];
-    }
-
     if (tid == 0 && L.pairs) atomicAdd(L.pairs, (unsigned long long)nr * (unsigned long long)ncol);
 
     if (L.part) {
-        // split block: partial sums; the CTA that completes the block's last item finishes it
-        if (half == 0) L.part[(size_t)it * kPartRows + t] = tot;
+        // split block: partial sums (MAXP: with their shifts); the CTA that completes the block's last item combines
+        // them in item order
+        float2 *part2 = reinterpret_cast<float2 *>(L.part);
+        if constexpr (MAXP) part2[(size_t)it * kPartRows + t] = make_float2(sh, tot);
+        else L.part[(size_t)it * kPartRows + t] = tot;
         __threadfence();
         __syncthreads();
         if (tid == 0) {
@@ -461,12 +444,21 @@ __global__ void __launch_bounds__(kThreads, OTGB_TC3_MINB) softmin3_tc_kernel(co
         if (S.bc[1] != fe.w) return;  // uniform
         __threadfence();
         tot = 0.f;
-        if (half == 0)
+        if constexpr (MAXP) {
+            const float2 *p = part2 + (size_t)fe.z * kPartRows + t;
+            sh = kNoTerm;
+            for (int q = 0; q < fe.w; ++q) sh = fmaxf(sh, __ldcg(&p[(size_t)q * kPartRows]).x);
+            for (int q = 0; q < fe.w; ++q) {
+                const float2 v = __ldcg(&p[(size_t)q * kPartRows]);
+                tot += v.y * xt::ex2(v.x - sh);
+            }
+        } else {
             for (int q = 0; q < fe.w; ++q) {
                 int iq = fe.z + q;
                 OTGB_DCLAMP(iq, 0, L.n_items);
                 tot += __ldcg(L.part + (size_t)iq * kPartRows + t);
             }
+        }
     }
     float dmax = 0.f;
     if (valid) {
@@ -475,8 +467,8 @@ __global__ void __launch_bounds__(kThreads, OTGB_TC3_MINB) softmin3_tc_kernel(co
             const int k = atomicAdd(L.n_fallback, 1);
             if (k < L.fallback_cap) L.fallback[k] = make_int4(item.x, r, blk, 0);
         } else {
-            const double L2 = m_eff + log2((double)tot);
-            const double tilde = -(double)I.lam * (L.eps_ln2 * L2 - hx);
+            const double L2 = (MAXP ? (double)sh : m_eff) + log2((double)tot);
+            const double tilde = -(double)I.lam * (L.eps_ln2 * L2 - (MAXP ? 0.0 : hx));
             double nw = tilde;
             if (I.row_old) {
                 const double old = (double)I.row_old[r];
@@ -493,14 +485,17 @@ __global__ void __launch_bounds__(kThreads, OTGB_TC3_MINB) softmin3_tc_kernel(co
 
 }  // namespace
 
-void softmin3_tc_launch(const SoftminLaunch &L, cudaStream_t st) {
+void softmin3_tc_launch(const SoftminLaunch &L, bool maxp, cudaStream_t st) {
     static PerDevice<int> attr;
     attr.get([] {
-        OTGB_CUDA_TRY(cudaFuncSetAttribute(softmin3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        OTGB_CUDA_TRY(cudaFuncSetAttribute(softmin3_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)sizeof(Tc3Smem)));
+        OTGB_CUDA_TRY(cudaFuncSetAttribute(softmin3_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)sizeof(Tc3Smem)));
         return 1;
     });
-    softmin3_tc_kernel<<<L.n_items, kThreads, sizeof(Tc3Smem), st>>>(L);
+    if (maxp) softmin3_tc_kernel<true><<<L.n_items, kThreads, sizeof(Tc3Smem), st>>>(L);
+    else softmin3_tc_kernel<false><<<L.n_items, kThreads, sizeof(Tc3Smem), st>>>(L);
     OTGB_CHECK_LAUNCH();
 }
 

@@ -276,10 +276,9 @@ void softmin_xd_launch(const SoftminLaunch &L, int D, bool maxp, cudaStream_t st
     OTGB_CHECK_LAUNCH();
 }
 
-int xd_chunk(const std::vector<std::pair<long long, long long>> &blocks_cols, int sms) {
-    // One item per slot and wave: the split into chunks of c tiles that minimises waves x (c + 3), the set-up of an
-    // item (tensor memory, centre, row operand, first copies: about 4 us) counted as three tiles.
-    const long long slots = 2LL * sms;
+int split_chunk(const std::vector<std::pair<long long, long long>> &blocks_cols, long long slots) {
+    // The split into chunks of c tiles that minimises waves x (c + 3), the set-up of an item (tensor memory, centre, row
+    // operand, first copies: 3 to 4 us) counted as three tiles.
     long long tmax = 1;
     for (auto &bc : blocks_cols) tmax = std::max(tmax, (bc.second + kN - 1) / kN);
     long long best = tmax, cost = -1;
@@ -292,7 +291,7 @@ int xd_chunk(const std::vector<std::pair<long long, long long>> &blocks_cols, in
             cost = v;
             best = c;
         }
-        if (items > 64 * slots) break;
+        if (items > 16 * slots) break;
     }
     return (int)std::min<long long>(best * kN, 1 << 30);
 }
