@@ -245,7 +245,10 @@ void Solver::set_work(const std::vector<std::vector<int>> &ncols, bool allow_spl
     double W = 0.0;
     for (auto &v : ncols)
         for (int c : v) W += c;
-    const double target = use_tc3 ? OTGB_TC3_ITEMS_PER_SM * sms : 3.0 * 5.0 * 4.0 * sms;
+    // D <= 3 warp kernel: about three waves of warps (6 CTAs of 4 warps per SM); tensor-core form: one CTA per item, two
+    // waves of four CTAs per SM (density maps of 100k voxels: 3 to 8 items per SM 15.2 ms of sweeps, 12 items 16.4, as
+    // every item pays its set-up)
+    const double target = use_tc3 ? 8.0 * sms : 3.0 * 5.0 * 4.0 * sms;
     int CH = 1 << 30;
     if (allow_split && D > 3) {  // softmin_xd_kernel
         std::vector<std::pair<long long, long long>> groups;
