@@ -25,6 +25,7 @@
 
 #include "multiscale.cuh"
 #include "solver.cuh"
+#include "sorted3.cuh"
 
 namespace otgb {
 namespace {
@@ -281,6 +282,12 @@ __global__ void __launch_bounds__(kGR) grad_sparse_kernel(const __grid_constant_
 }
 
 void grad_sparse_run(const Solver &s, double eps, const GradRequest &gr, cudaStream_t st) {
+    if (s.D <= 3 && s.p == 2) {  // the solve's points are in spatial order: every pair that can matter, on the tensor cores
+        const float4 *X = reinterpret_cast<const float4 *>(s.X.pts), *Y = reinterpret_cast<const float4 *>(s.Y.pts);
+        const Grad3Part part[2] = {{Y, s.pg[s.cur], s.Y.n, 1.f, s.pf[s.cur]}, {X, s.pa[s.cur], s.X.n, -1.f, s.pa[s.cur]}};
+        grad3_run(s.ctx, X, s.X.n, s.D, part, eps, s.X.w, gr.scale, gr.accumulate, s.X.perm, gr.grad, st);
+        return;
+    }
     SpGradArgs A;
     std::memset(&A, 0, sizeof(A));
     A.inst[0] = s.launch.inst[3];  // rows x against (y, beta, g)
@@ -348,6 +355,12 @@ extern "C" int sinkhorn_grad_x(otgb_ctx *ctx, const float *x, const float *alpha
         require(p == 1 || p == 2, "sinkhorn_grad_x: p must be 1 or 2");
         require(eps > 0.0 && std::isfinite(eps), "sinkhorn_grad_x: eps must be > 0");
         cudaStream_t st = ctx_stream(ctx);
+        // p = 2 in up to three dimensions: sorted, on the tensor cores (sorted3.cu), from about 4,000 points on; below, the
+        // sorts cost more than the pairs
+        if (D <= 3 && p == 2 && (double)N * ((double)N + M) >= 2e7) {
+            grad3_apply(ctx, x, alpha, N, y, beta, M, D, eps, f, g, a_self, grad);
+            return OTGB_OK;
+        }
         grad_launch(grad_args(x, alpha, N, y, beta, M, D, p, eps, a_self, f, g, grad, 1.f, 0), st);
         OTGB_CUDA_TRY(cudaStreamSynchronize(st));
         return OTGB_OK;

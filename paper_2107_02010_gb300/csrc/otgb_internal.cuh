@@ -271,6 +271,9 @@ struct SoftminLaunch {
 // D selects the specialisation.  Errors throw otgb::Error.
 void softmin_run(const SoftminLaunch &L, int D, int rows_per_thread, cudaStream_t st);
 
+// The safe two-pass kernel over the rows listed in L.fallback.
+void softmin_fallback_launch(const SoftminLaunch &L, int D, cudaStream_t st);
+
 // Softmin in the direct difference form (softmin_direct.cu), cost |x - y| (cost_p1) or
 // |x - y|^2 / 2: any D, blocks <= 128 rows, no split blocks.
 void softmin_direct_launch(const SoftminLaunch &L, int D, cudaStream_t st);

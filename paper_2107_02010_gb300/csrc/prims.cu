@@ -226,17 +226,18 @@ __global__ void scan_block_kernel(const int *in, int *out, int n, int *block_sum
     if (threadIdx.x == kScanB - 1) block_sums[blockIdx.x] = s[kScanB - 1];
 }
 
-// Up to kScanOne values in one launch: every thread sums kScanV consecutive values, one scan over the threads.
-constexpr int kScanV = 32, kScanOne = kScanB * kScanV;
+// Up to kScanOne values in one launch, held in shared memory: every thread sums consecutive values (an odd number of them:
+// no bank conflicts), one scan over the threads, reads and writes along the array.
+constexpr int kScanV = 31, kScanOne = kScanB * kScanV;
 __global__ void __launch_bounds__(kScanB) scan_one_kernel(const int *in, int *out, int n) {
+    extern __shared__ int sv[];
     __shared__ int ws[32];
-    const int per = (n + kScanB - 1) / kScanB, i0 = threadIdx.x * per, i1 = min(n, i0 + per);
-    int v[kScanV], sum = 0;
-#pragma unroll
-    for (int q = 0; q < kScanV; ++q) {
-        v[q] = q < per && i0 + q < i1 ? in[i0 + q] : 0;
-        sum += v[q];
-    }
+    const int per = ((n + kScanB - 1) / kScanB) | 1, i0 = min(n, (int)threadIdx.x * per), i1 = min(n, i0 + per);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += kScanB) sv[i] = in[i];
+    __syncthreads();
+    int sum = 0;
+    for (int i = i0; i < i1; ++i) sum += sv[i];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int x = sum;  // inclusive scan over the threads
     for (int o = 1; o < 32; o <<= 1) {
@@ -255,12 +256,14 @@ __global__ void __launch_bounds__(kScanB) scan_one_kernel(const int *in, int *ou
     }
     __syncthreads();
     int run = x - sum + (w > 0 ? ws[w - 1] : 0);
-#pragma unroll
-    for (int q = 0; q < kScanV; ++q)
-        if (q < per && i0 + q < i1) {
-            out[i0 + q] = run;
-            run += v[q];
-        }
+    for (int i = i0; i < i1; ++i) {
+        const int v = sv[i];
+        sv[i] = run;
+        run += v;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += kScanB) out[i] = sv[i];
 }
 
 __global__ void scan_add_kernel(int *out, int n, const int *block_off) {
@@ -654,7 +657,13 @@ size_t scan_scratch_ints_level(int nb) {
 void exclusive_scan(const int *in, int *out, int n, int *scratch, cudaStream_t st) {
     if (n <= 0) return;
     if (n <= kScanOne) {
-        scan_one_kernel<<<1, kScanB, 0, st>>>(in, out, n);
+        static PerDevice<int> attr;
+        attr.get([] {
+            OTGB_CUDA_TRY(cudaFuncSetAttribute(scan_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               kScanOne * (int)sizeof(int)));
+            return 1;
+        });
+        scan_one_kernel<<<1, kScanB, n * sizeof(int), st>>>(in, out, n);
         OTGB_CHECK_LAUNCH();
         return;
     }

@@ -950,6 +950,12 @@ int fallback_grid_sms() {
 }
 }  // namespace
 
+void softmin_fallback_launch(const SoftminLaunch &L, int D, cudaStream_t st) {
+    const int stride = D <= 3 ? 4 : ((D + 3) & ~3);
+    softmin_fallback_kernel<<<2 * fallback_grid_sms(), kFbThreads, 0, st>>>(L, D, stride);
+    OTGB_CHECK_LAUNCH();
+}
+
 void softmin_run(const SoftminLaunch &L, int D, int rows_per_thread, cudaStream_t st) {
     if (L.n_items <= 0) return;
     if (!L.counters_zeroed) OTGB_CUDA_TRY(cudaMemsetAsync(L.n_fallback, 0, sizeof(int), st));
@@ -1019,9 +1025,7 @@ void softmin_run(const SoftminLaunch &L, int D, int rows_per_thread, cudaStream_
             OTGB_CHECK_LAUNCH();
         }
     }
-    const int stride = D <= 3 ? 4 : ((D + 3) & ~3);
-    softmin_fallback_kernel<<<2 * fallback_grid_sms(), kFbThreads, 0, st>>>(L, D, stride);
-    OTGB_CHECK_LAUNCH();
+    softmin_fallback_launch(L, D, st);
 }
 
 }  // namespace otgb

@@ -31,6 +31,7 @@
 
 #include "otgb_internal.cuh"
 #include "tcgen05.cuh"
+#include "tile3.cuh"
 #include "xtile.cuh"
 
 namespace otgb {
@@ -101,68 +102,26 @@ struct Tc3Smem {
     alignas(16) int idx[2][kChunk];
 };
 
-// K-major canonical layout of a tile with 32 K-columns: 8-row x 16-byte core
-// matrices, 4 along K (leading byte offset 128), 8-row groups 512 bytes apart
-__device__ __forceinline__ int off32(int r, int k) {
-    return (r >> 3) * 512 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2;
-}
+using t3::bf2;
+using t3::bfbits;
+using t3::bfval;
+using t3::hi_val;
+using t3::kOne;
+using t3::lo_val;
+using t3::off32;
+using t3::pk;
+using t3::sdesc32;
+using t3::split3x2;
 
-__device__ __forceinline__ uint64_t sdesc32(uint32_t addr) {
-    uint64_t d = (uint64_t)((addr & 0x3FFFF) >> 4);
-    d |= (uint64_t)(128 >> 4) << 16;
-    d |= (uint64_t)(512 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    return d;
-}
-
-// Scalar split for the row operand (once per CTA).  The per-tile column operand
-// uses the packed form below.  (Rounding with integer operations instead, which
-// also frees the MUFU unit, measured 2 % slower: it costs issue slots.)
-__device__ __forceinline__ uint16_t bfbits(float v) { return __bfloat16_as_ushort(__float2bfloat16_rn(v)); }
-__device__ __forceinline__ float bfval(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
-
-// v ~ h + m + l in BF16 (about 24 significant bits)
-__device__ __forceinline__ void split3(float v, uint16_t &h, uint16_t &m, uint16_t &l) {
-    h = bfbits(v);
-    const float r = v - bfval(h);
-    m = bfbits(r);
-    l = bfbits(r - bfval(m));
-}
-
-__device__ __forceinline__ uint32_t pk(uint16_t lo, uint16_t hi) { return (uint32_t)lo | ((uint32_t)hi << 16); }
-
-// Two values split at once: H, M, L hold the h, m, l pieces of a in their high halves and of b in their low
-// halves.  The packed conversion rounds each half to nearest even, as the scalar one does, so the pieces are
-// those of split3; it runs on its own pipe, leaving the MUFU unit to ex2.
-__device__ __forceinline__ uint32_t bf2(float hi, float lo) {
-    uint32_t d;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-    return d;
-}
-__device__ __forceinline__ float hi_val(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
-__device__ __forceinline__ float lo_val(uint32_t w) { return __uint_as_float(w << 16); }
-// rest: what b lost to its own rounding.
-__device__ __forceinline__ void split3x2(float a, float b, uint32_t &H, uint32_t &M, uint32_t &L, float rest = 0.f) {
-    H = bf2(a, b);
-    const float ra = a - hi_val(H), rb = b - lo_val(H);
-    M = bf2(ra, rb);
-    L = bf2(ra - hi_val(M), (rb - lo_val(M)) + rest);
-}
-
-constexpr uint16_t kOne = 0x3F80;  // 1.0 in BF16
+// Scalar split for the row operand (once per CTA): v ~ h + m + l in BF16 (about 24 significant bits).  The per-tile
+// column operand uses the packed form (t3::split3x2).  (Rounding with integer operations instead, which also frees the
+// MUFU unit, measured 2 % slower: it costs issue slots.)
+__device__ __forceinline__ void split3(float v, uint16_t &h, uint16_t &m, uint16_t &l) { xt::split3(v, 0.f, h, m, l); }
 
 constexpr float kNoTerm = -1e29f;  // shift of a row without terms (absent columns have an exponent of about -1e30)
 
-// MAXP: the shift is not known (no old value, or one that is no estimate of the result), and the rows come as the caller
-// has them, so that a block may span the whole cloud and |x - c| |y - c| be much larger than any exponent that matters.
-// The accumulator then holds the pair's whole exponent, -s |x - y|^2 / 2 + s (eps log w + pot), arranged so that each of
-// the two K = 16 steps is small by itself for a pair that matters: step 0 holds coordinates 0 and 1 with their own share
-// of the squares (two pieces of -s (y0^2 + y1^2) / 2 against 1, two of -s (x0^2 + x1^2) / 2), step 1 coordinate 2 and
-// everything else (three pieces each).  The sum is cut off towards zero after each step, at the size of what it holds.
-// The row keeps a running shift (xt::sum_row_max).
-// First word (two K slots) of coordinate d.
-template <bool MAXP> __device__ __forceinline__ constexpr int coord_word(int d) { return MAXP && d == 2 ? 8 : 3 * d; }
-
+// MAXP: the shift is not known (no old value, or one that is no estimate of the result).  The accumulator then holds the
+// pair's whole exponent (tile3.cuh) and the row keeps a running shift (xt::sum_row_max).
 template <bool MAXP>
 __global__ void __launch_bounds__(kThreads, 4) softmin3_tc_kernel(const __grid_constant__ SoftminLaunch L) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -252,41 +211,28 @@ __global__ void __launch_bounds__(kThreads, 4) softmin3_tc_kernel(const __grid_c
     const uint16_t mb = !MAXP && valid ? bfbits(-(m - Cb)) : (uint16_t)0;
     const double m_eff = (double)Cb - (double)bfval(mb);  // the shift the accumulator applies
     {
-        uint16_t h[3], md[3], l[3];
-        split3(s * x0, h[0], md[0], l[0]);
-        split3(s * x1, h[1], md[1], l[1]);
-        split3(s * x2, h[2], md[2], l[2]);
         uint32_t w[16];
-        // six slots per coordinate: h h m h l m (against the column's h m h l h m)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const int b0 = coord_word<MAXP>(d);  // three words per coordinate
-            w[b0] = pk(h[d], h[d]);
-            w[b0 + 1] = pk(md[d], h[d]);
-            w[b0 + 2] = pk(l[d], md[d]);
-        }
         if constexpr (MAXP) {
-            const double R01 = -0.5 * (double)s * ((double)x0 * x0 + (double)x1 * x1);
-            const uint16_t ra = bfbits((float)R01), rb = bfbits((float)(R01 - (double)bfval(ra)));
-            const double R2 = (R01 - (double)bfval(ra) - (double)bfval(rb)) - 0.5 * (double)s * ((double)x2 * x2);
-            uint16_t r1, r2, r3;
-            xt::split3((float)R2, (float)(R2 - (double)(float)R2), r1, r2, r3);
-            w[6] = pk(kOne, kOne);
-            w[7] = pk(ra, rb);
-            w[11] = pk(kOne, kOne);
-            w[12] = pk(kOne, r1);
-            w[13] = pk(r2, r3);
+            t3::row_words(x0, x1, x2, s, w);
         } else {
+            uint16_t h[3], md[3], l[3];
+            split3(s * x0, h[0], md[0], l[0]);
+            split3(s * x1, h[1], md[1], l[1]);
+            split3(s * x2, h[2], md[2], l[2]);
+            // slots 6d .. 6d+5: h h m h l m (against the column's h m h l h m)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int b0 = 3 * d;  // three words per coordinate
+                w[b0] = pk(h[d], h[d]);
+                w[b0 + 1] = pk(md[d], h[d]);
+                w[b0 + 2] = pk(l[d], md[d]);
+            }
             w[9] = pk(kOne, kOne);  // slots 18, 19: against H pieces 1, 2
             w[10] = pk(kOne, mb);   // slot 20: H piece 3; slot 21: the shift
 #pragma unroll
-            for (int q = 11; q < 14; ++q) w[q] = 0u;
+            for (int q = 11; q < 16; ++q) w[q] = 0u;
         }
-        w[14] = w[15] = 0u;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<uint4 *>(S.a + off32(t, 8 * q)) =
-                make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+        t3::store_words(S.a, t, w);
     }
 
     // ---- column staging: thread tid stages column tid of each tile
@@ -311,65 +257,33 @@ __global__ void __launch_bounds__(kThreads, 4) softmin3_tc_kernel(const __grid_c
     auto convert = [&]() {
         const bool okc = jc >= 0;
         const float y0 = okc ? rq.x - c[0] : 0.f, y1 = okc ? rq.y - c[1] : 0.f, y2 = okc ? rq.z - c[2] : 0.f;
-        float H, rest = 0.f;
         uint32_t w[16];
         if constexpr (MAXP) {
-            // |y0|^2 + |y1|^2 with its rounding errors (Knuth's two-sum, products by FMA), times -s/2; two BF16 pieces of it
-            // stay with those coordinates, what they leave joins the rest of H, which is summed with its errors too
-            const float hs = -0.5f * s;
-            const float p0 = y0 * y0, p1 = y1 * y1, t01 = p0 + p1, tb = t01 - p0;
-            const float te = ((p0 - (t01 - tb)) + (p1 - tb)) + (fmaf(y0, y0, -p0) + fmaf(y1, y1, -p1));
-            const float q01 = hs * t01, qe = fmaf(hs, t01, -q01) + hs * te;
-            const uint32_t wa = bf2(0.f, q01);
-            const float qa = q01 - lo_val(wa);
-            const uint32_t wb = bf2(0.f, qa);
-            const float rem = qa - lo_val(wb);
-            w[6] = okc ? pk((uint16_t)wa, (uint16_t)wb) : 0u;
-            w[7] = pk(kOne, kOne);
-            const float u = fmaf(eps, rq.w, rpot), v = s * u, ve = fmaf(s, u, -v);
-            const float z = y2 * y2, g = hs * z, ge = fmaf(hs, z, -g) + hs * fmaf(y2, y2, -z);
-            const float S1 = v + g, sb = S1 - v, se = (v - (S1 - sb)) + (g - sb);
-            H = S1 + rem;
-            const float hb = H - S1;
-            rest = ((S1 - (H - hb)) + (rem - hb)) + (se + (ve + ge) + qe);
-            if (!okc || H <= -1e30f) {  // absent, or zero weight (log w = -inf); NaN goes on
-                H = -1e30f;
-                rest = 0.f;
-            }
+            t3::col_words(y0, y1, y2, rq.w, rpot, s, eps, okc, w);
         } else {
             const float sq = y0 * y0 + y1 * y1 + y2 * y2;
-            H = okc ? s * (fmaf(eps, rq.w, rpot) - 0.5f * sq) - Cb : -1e30f;
+            float H = okc ? s * (fmaf(eps, rq.w, rpot) - 0.5f * sq) - Cb : -1e30f;
             if (H <= -1e30f) H = -1e30f;  // zero weight (log w = -inf); NaN goes on
-        }
-        uint32_t H01, M01, L01, H2h, M2h, L2h;
-        split3x2(y0, y1, H01, M01, L01);
-        split3x2(y2, H, H2h, M2h, L2h, rest);
-        const uint16_t h[3] = {(uint16_t)(H01 >> 16), (uint16_t)H01, (uint16_t)(H2h >> 16)};
-        const uint16_t md[3] = {(uint16_t)(M01 >> 16), (uint16_t)M01, (uint16_t)(M2h >> 16)};
-        const uint16_t l[3] = {(uint16_t)(L01 >> 16), (uint16_t)L01, (uint16_t)(L2h >> 16)};
-        const uint16_t hh[3] = {(uint16_t)H2h, (uint16_t)M2h, (uint16_t)L2h};
+            uint32_t H01, M01, L01, H2h, M2h, L2h;
+            split3x2(y0, y1, H01, M01, L01);
+            split3x2(y2, H, H2h, M2h, L2h);
+            const uint16_t h[3] = {(uint16_t)(H01 >> 16), (uint16_t)H01, (uint16_t)(H2h >> 16)};
+            const uint16_t md[3] = {(uint16_t)(M01 >> 16), (uint16_t)M01, (uint16_t)(M2h >> 16)};
+            const uint16_t l[3] = {(uint16_t)(L01 >> 16), (uint16_t)L01, (uint16_t)(L2h >> 16)};
+            const uint16_t hh[3] = {(uint16_t)H2h, (uint16_t)M2h, (uint16_t)L2h};
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const int b0 = coord_word<MAXP>(d);
-            w[b0] = pk(h[d], md[d]);
-            w[b0 + 1] = pk(h[d], l[d]);
-            w[b0 + 2] = pk(h[d], md[d]);
-        }
-        if constexpr (MAXP) {
-            w[11] = pk(hh[0], hh[1]);
-            w[12] = pk(hh[2], kOne);
-            w[13] = pk(kOne, kOne);
-        } else {
+            for (int d = 0; d < 3; ++d) {
+                const int b0 = 3 * d;
+                w[b0] = pk(h[d], md[d]);
+                w[b0 + 1] = pk(h[d], l[d]);
+                w[b0 + 2] = pk(h[d], md[d]);
+            }
             w[9] = pk(hh[0], hh[1]);
             w[10] = pk(hh[2], kOne);
 #pragma unroll
-            for (int q = 11; q < 14; ++q) w[q] = 0u;
+            for (int q = 11; q < 16; ++q) w[q] = 0u;
         }
-        w[14] = w[15] = 0u;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<uint4 *>(S.b + off32(tid, 8 * q)) =
-                make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+        t3::store_words(S.b, tid, w);
     };
 
     if (warp == 0) tc::tmem_alloc(&S.tslot, kTmemCols);
@@ -377,15 +291,6 @@ __global__ void __launch_bounds__(kThreads, 4) softmin3_tc_kernel(const __grid_c
     __syncthreads();
     tc::fence_after();
     const uint32_t tmem = S.tslot;
-    const uint32_t idesc = tc::idesc_bf16(kM, kN);
-    auto issue = [&]() {
-        const uint32_t a = tc::smem_u32(S.a), b = tc::smem_u32(S.b);
-#pragma unroll
-        for (int kk = 0; kk < kK / 16; ++kk)
-            tc::mma_bf16(tmem, sdesc32(a + kk * 256), sdesc32(b + kk * 256), idesc, kk > 0 ? 1u : 0u);
-        tc::commit(&S.mbar);
-    };
-
     float tot = 0.f, sh = kNoTerm;
     bool ok = true;
     // rows of this warp that exist: the epilogue of an empty warp is skipped
@@ -403,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, 4) softmin3_tc_kernel(const __grid_c
         tc::fence_before();
         __syncthreads();
         tc::fence_after();
-        if (tid == 0) issue();
+        if (tid == 0) t3::issue(tmem, tc::smem_u32(S.a), tc::smem_u32(S.b), &S.mbar);
         // chunk c + 1 in the first iteration of chunk c, while the tensor core works: the index of tile T is read in
         // iteration T - 2, so the last read of chunk c - 1 (same buffer) came two iterations before, and the first read
         // of chunk c + 1 comes kChunkTiles - 2 iterations later, past this iteration's closing barrier

@@ -1,0 +1,716 @@
+// Large dense D <= 3 sums on the tensor cores over spatially sorted points: otgb_softmin and the gradient in the points.
+//
+// Rows and columns come in the order of a Hilbert curve, so that a block of 128 rows and a tile of 128 columns are compact
+// (on the Morton curve the blocks that straddle one of its jumps have boxes as large as the cloud).  A CTA bounds
+// the exponents of every tile from the boxes of the block and the tile and the tile's largest s (eps log w + pot), visits
+// the best tile first, and then only the tiles whose bound reaches to 60 binades below the smallest running shift of its
+// rows: a term below 2^-60 of the row's largest one changes neither a float32 sum of fewer than 2^31 terms nor a weighted
+// mean of it (the exponents in between are visited, whatever the potentials are, so nothing depends on their being near a
+// solution).  On voxels at blur 1 that leaves about one pair in eight.
+//
+// The exponent of a pair is one K = 32 tensor-core dot product (tile3.cuh).  One thread per row keeps a running shift, the
+// sum of the terms, and for the gradient the sums of the terms times the coordinate differences x - y (two columns per
+// packed f32x2 operation; ys: the tile's coordinates, read as broadcasts).  The differences are formed from the
+// coordinates as they came: sums of w y, subtracted from x once, lose the digits that x and y share.
+// The curve jumps where the points leave gaps.  A block is therefore cut into runs whose box stays compact (s times its
+// squared half diagonal at most kCompact): groups of 16 rows, each cut once more at its longest step, are merged in order
+// while their box allows it.  The runs take their turns on the CTA, each with its own centre and its own tiles: a block
+// across a jump costs two short passes instead of one that visits everything between.  A single part above kSpread
+// (outliers: the dot product's terms would dwarf the exponents) is summed from coordinate differences alone.
+// Bound: issue, about 7.5 instructions per pair for the gradient (ex2, two subtractions, maximum, the differences and FMAs
+// and an add for two columns, 0.75 shared loads) = 17 pairs per clock and SM; MUFU (32) for the softmin.
+// Measured: otgb_softmin on 100k x 100k points 7.0 -> 0.85 ms (the dense tensor-core sweep: 1.89), of it 0.56 the sums;
+// sinkhorn_grad_x on 50k + 50k points 8.6 -> 1.05 ms, of it 0.79 the sums (on the Morton curve, uncut blocks: 1.11 and
+// 1.20 ms).
+//
+// Each (block, split, part) writes its shift and sums; a finish kernel combines the splits in order, so the result does
+// not depend on scheduling.
+#include <cfloat>
+#include <cmath>
+#include <cstring>
+
+#include "prims.cuh"
+#include "solver.cuh"
+#include "sorted3.cuh"
+#include "tile3.cuh"
+
+namespace otgb {
+namespace {
+
+constexpr int kT = 128;           // threads, rows of a block, columns of a tile
+constexpr int kMaxTiles = 4096;   // tiles bounded at once (524,288 columns)
+constexpr float kNoTerm = -1e29f;
+constexpr float kReach = 60.f;    // binades below the row's largest term that are visited
+constexpr float kCompact = 96.f;
+constexpr float kSpread = 256.f;  // terms of this size are rounded at 8e-6, as s f + s g - s C is at |s f| = 128
+
+struct S3Part {
+    const float4 *cols;
+    const float *pot;
+    const float4 *box;  // per tile: (lo, largest s (eps log w + pot)), (hi, 0)
+    int n;
+};
+struct S3Args {
+    const float4 *rows;
+    int n_rows, splits;
+    S3Part part[2];
+    float eps, s;
+    float4 *out;  // [part][split][row]: shift, then S (softmin) or the three sums
+    unsigned *err;
+};
+
+struct S3Smem {
+    unsigned char a[t3::kBytes], b[t3::kBytes];
+    alignas(16) float ys[3][kT];
+    float ct[kT];  // s (eps log w + pot), for a spread block
+    float bnd[kMaxTiles];
+    unsigned short list[kMaxTiles];
+    float red[4][8];
+    float sub[16][6];  // boxes of the two parts of each group of 16 rows: lo, -hi
+    int start[17];     // their first rows
+    int ired[4], wsum[4];
+    unsigned long long mbar;
+    uint32_t tslot;
+};
+
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float sum2(unsigned long long v) {
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+    return lo + hi;
+}
+
+template <bool GRAD>
+__global__ void __launch_bounds__(kT, 4) sorted3_kernel(const __grid_constant__ S3Args A) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    S3Smem &S = *reinterpret_cast<S3Smem *>(smem_raw);
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int r0 = blockIdx.x * kT, nr = min(kT, A.n_rows - r0);
+    const S3Part &P = A.part[blockIdx.z];
+    const float s = A.s;
+    const bool valid = t < nr;
+    const int ntiles = (P.n + kT - 1) / kT;
+
+    // ---- the groups of 16 rows, cut at their longest step, and the boxes of the parts
+    const float4 mine = A.rows[r0 + (valid ? t : 0)];
+    {
+        const int u = t & 15;
+        const float px = __shfl_up_sync(0xffffffffu, mine.x, 1), py = __shfl_up_sync(0xffffffffu, mine.y, 1),
+                    pz = __shfl_up_sync(0xffffffffu, mine.z, 1);
+        const float e0 = mine.x - px, e1 = mine.y - py, e2 = mine.z - pz;
+        float len = fmaf(e0, e0, fmaf(e1, e1, e2 * e2));
+        if (!(len >= 0.f)) len = INFINITY;  // a row that is no number: all lanes agree on the cut
+        if (u == 0 || !valid) len = -1.f;
+        int cut = u;
+        for (int o = 8; o > 0; o >>= 1) {
+            const float ol = __shfl_xor_sync(0xffffffffu, len, o);
+            const int oc = __shfl_xor_sync(0xffffffffu, cut, o);
+            if (ol > len || (ol == len && oc < cut)) {
+                len = ol;
+                cut = oc;
+            }
+        }
+        if (len < 0.f) cut = 16;  // a group of at most one row
+        const int g = t >> 4;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const bool in = valid && (h ? u >= cut : u < cut);
+            float v[6] = {mine.x, mine.y, mine.z, -mine.x, -mine.y, -mine.z};
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                v[q] = in ? v[q] : FLT_MAX;
+                for (int o = 8; o > 0; o >>= 1) v[q] = fminf(v[q], __shfl_xor_sync(0xffffffffu, v[q], o));
+                if (u == 0) S.sub[2 * g + h][q] = v[q];
+            }
+            if (u == 0) S.start[2 * g + h] = min(nr, 16 * g + (h ? cut : 0));
+        }
+        if (t == 0) S.start[16] = nr;
+    }
+    if (t == 0) {
+        tc::mbar_init(&S.mbar, 1);
+        tc::mbar_init_fence();
+    }
+    if (warp == 0) tc::tmem_alloc(&S.tslot, kT);
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tmem = S.tslot, lanes = tmem + ((uint32_t)(warp * 32) << 16);
+    bool ok = true;
+    int phase = 0;
+    float4 rq = make_float4(0.f, 0.f, 0.f, 0.f);
+    float rpot = 0.f;
+    bool rin = false;
+    for (int ga = 0, gb; ok && ga < 16; ga = gb) {
+    // ---- the run of parts [ga, gb): box, centre, row operand
+    if (S.start[ga] >= S.start[ga + 1]) {  // an empty part (uniform)
+        gb = ga + 1;
+        continue;
+    }
+    float lo[3], hi[3], hd2 = 0.f;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        lo[d] = S.sub[ga][d];
+        hi[d] = -S.sub[ga][d + 3];
+        hd2 = fmaf(0.25f * (hi[d] - lo[d]), hi[d] - lo[d], hd2);
+    }
+    const bool spread = !(s * hd2 <= kSpread);  // uniform
+    for (gb = ga + 1; gb < 16 && !spread; ++gb) {
+        if (S.start[gb] >= S.start[gb + 1]) continue;
+        float l[3], h[3], u = 0.f;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            l[d] = fminf(lo[d], S.sub[gb][d]);
+            h[d] = fmaxf(hi[d], -S.sub[gb][d + 3]);
+            u = fmaf(0.25f * (h[d] - l[d]), h[d] - l[d], u);
+        }
+        if (!(s * u <= kCompact)) break;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            lo[d] = l[d];
+            hi[d] = h[d];
+        }
+    }
+    const int ra = S.start[ga], rb = S.start[gb];
+    const bool in_run = t >= ra && t < rb;
+    const bool warp_on = 32 * warp < rb && 32 * warp + 32 > ra;  // some of the warp's rows are in the run
+    const float4 p = in_run ? mine : A.rows[r0 + ra];  // the other threads repeat the run's first row
+    const float c[3] = {0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2])};
+    {
+        uint32_t w[16];
+        t3::row_words(p.x - c[0], p.y - c[1], p.z - c[2], s, w);
+        t3::store_words(S.a, t, w);
+    }
+    const unsigned long long X2[3] = {pack2(p.x, p.x), pack2(p.y, p.y), pack2(p.z, p.z)};
+
+    float sh = kNoTerm, tot = 0.f;
+    unsigned long long S2 = 0ull, V[3] = {0ull, 0ull, 0ull};
+    auto load_raw = [&](int tile) {
+        const int j = tile * kT + t;
+        rin = tile >= 0 && j < P.n;
+        if (rin) {
+            rq = P.cols[j];
+            rpot = P.pot[j];
+        }
+    };
+    auto chunk = [&](const uint32_t (&v)[32], int c0) {
+        float m0 = __uint_as_float(v[0]), m1 = __uint_as_float(v[1]);
+#pragma unroll
+        for (int q = 2; q < 32; q += 2) {
+            m0 = fmaxf(m0, __uint_as_float(v[q]));
+            m1 = fmaxf(m1, __uint_as_float(v[q + 1]));
+        }
+        m0 = fmaxf(m0, m1);
+        if (m0 > sh + 30.f) {
+            const float f = xt::ex2(sh - m0);
+            const unsigned long long ff = pack2(f, f);
+            S2 = mul2(S2, ff);
+            if constexpr (GRAD) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) V[d] = mul2(V[d], ff);
+            }
+            sh = m0;
+        }
+#pragma unroll
+        for (int q = 0; q < 32; q += 4) {
+            const unsigned long long wa = pack2(xt::ex2(__uint_as_float(v[q]) - sh), xt::ex2(__uint_as_float(v[q + 1]) - sh));
+            const unsigned long long wb = pack2(xt::ex2(__uint_as_float(v[q + 2]) - sh), xt::ex2(__uint_as_float(v[q + 3]) - sh));
+            S2 = add2(S2, wa);
+            S2 = add2(S2, wb);
+            if constexpr (GRAD) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(&S.ys[d][c0 + q]);  // -y
+                    V[d] = fma2(wa, add2(X2[d], y.x), V[d]);
+                    V[d] = fma2(wb, add2(X2[d], y.y), V[d]);
+                }
+            }
+        }
+    };
+    // one tile from registers: operand, MMA, sums; `next` is fetched meanwhile (-1: none).  Returns the smallest shift of
+    // the block's rows.
+    auto tile_step = [&](int next) -> float {
+        if (spread) {
+            S.ys[0][t] = -rq.x;
+            S.ys[1][t] = -rq.y;
+            S.ys[2][t] = -rq.z;
+            S.ct[t] = rin ? s * fmaf(A.eps, rq.w, rpot) : -INFINITY;
+            load_raw(next);
+            __syncthreads();
+            for (int q = 0; warp_on && q < kT; ++q) {
+                const float ct = S.ct[q];
+                if (ct == -INFINITY) continue;  // uniform
+                const float d0 = p.x + S.ys[0][q], d1 = p.y + S.ys[1][q], d2 = p.z + S.ys[2][q];
+                const float e = fmaf(-0.5f * s, fmaf(d0, d0, fmaf(d1, d1, d2 * d2)), ct);
+                if (e > sh + 30.f) {
+                    const float f = xt::ex2(sh - e);
+                    const unsigned long long ff = pack2(f, f);
+                    S2 = mul2(S2, ff);
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) V[d] = mul2(V[d], ff);
+                    sh = e;
+                }
+                const float w = xt::ex2(e - sh);
+                const unsigned long long w1 = pack2(w, 0.f);
+                S2 = add2(S2, w1);
+                if constexpr (GRAD) {
+                    V[0] = fma2(w1, pack2(d0, 0.f), V[0]);
+                    V[1] = fma2(w1, pack2(d1, 0.f), V[1]);
+                    V[2] = fma2(w1, pack2(d2, 0.f), V[2]);
+                }
+            }
+            float m = warp_on ? sh : INFINITY;
+            for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (lane == 0) S.red[warp][6] = m;
+            __syncthreads();
+            return fminf(fminf(S.red[0][6], S.red[1][6]), fminf(S.red[2][6], S.red[3][6]));
+        }
+        const float y0 = rin ? rq.x - c[0] : 0.f, y1 = rin ? rq.y - c[1] : 0.f, y2 = rin ? rq.z - c[2] : 0.f;
+        {
+            uint32_t w[16];
+            t3::col_words(y0, y1, y2, rq.w, rpot, s, A.eps, rin, w);
+            t3::store_words(S.b, t, w);
+        }
+        if constexpr (GRAD) {
+            S.ys[0][t] = -rq.x;  // of a column past the end: any finite value, its term is 0
+            S.ys[1][t] = -rq.y;
+            S.ys[2][t] = -rq.z;
+        }
+        load_raw(next);
+        tc::fence_proxy_async();
+        tc::fence_before();
+        __syncthreads();
+        tc::fence_after();
+        if (t == 0) t3::issue(tmem, tc::smem_u32(S.a), tc::smem_u32(S.b), &S.mbar);
+        if (!tc::mbar_wait(&S.mbar, (uint32_t)(phase & 1))) ok = false;
+        ++phase;
+        ok = __all_sync(0xffffffffu, ok);  // tensor-memory loads are warp-collective
+        tc::fence_after();
+        if (ok && warp_on) {
+            uint32_t va[32], vb[32];
+            tc::ld32_async(lanes, va);
+            tc::ld_wait(va);
+            tc::ld32_async(lanes + 32, vb);
+            chunk(va, 0);
+            tc::ld_wait(vb);
+            tc::ld32_async(lanes + 64, va);
+            chunk(vb, 32);
+            tc::ld_wait(va);
+            tc::ld32_async(lanes + 96, vb);
+            chunk(va, 64);
+            tc::ld_wait(vb);
+            chunk(vb, 96);
+        }
+        float m = warp_on ? sh : INFINITY;  // threads outside the run repeat one of its rows
+        for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane == 0) S.red[warp][6] = m;
+        tc::fence_before();
+        ok = __syncthreads_and(ok) != 0;  // operand, coordinates and accumulator are free again
+        return fminf(fminf(S.red[0][6], S.red[1][6]), fminf(S.red[2][6], S.red[3][6]));
+    };
+
+    // the tiles of this split (all of them are bounded, so that every split starts from the same best tile)
+    const int per = (ntiles + A.splits - 1) / A.splits, ta = blockIdx.y * per, tb = min(ntiles, ta + per);
+    float thr = -INFINITY;
+    for (int w0 = 0; ok && w0 < ntiles; w0 += kMaxTiles) {
+        if (w0 > 0 && (w0 >= tb || w0 + kMaxTiles <= ta)) continue;  // none of this split's tiles
+        const int nw = min(kMaxTiles, ntiles - w0);
+        float best = -INFINITY;
+        int bi = 0x7fffffff;
+        for (int q = t; q < nw; q += kT) {
+            const float4 l = P.box[2 * (w0 + q)], h = P.box[2 * (w0 + q) + 1];
+            const float g0 = fmaxf(fmaxf(l.x - hi[0], lo[0] - h.x), 0.f), g1 = fmaxf(fmaxf(l.y - hi[1], lo[1] - h.y), 0.f),
+                        g2 = fmaxf(fmaxf(l.z - hi[2], lo[2] - h.z), 0.f);
+            const float b = l.w - 0.49999f * s * fmaf(g0, g0, fmaf(g1, g1, g2 * g2));
+            S.bnd[q] = b;
+            if (b > best) {
+                best = b;
+                bi = q;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (ob > best || (ob == best && oi < bi)) {
+                best = ob;
+                bi = oi;
+            }
+        }
+        if (lane == 0) {
+            S.red[warp][7] = best;
+            S.ired[warp] = bi;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (q == 0) {
+                best = S.red[0][7];
+                bi = S.ired[0];
+            } else if (S.red[q][7] > best || (S.red[q][7] == best && S.ired[q] < bi)) {
+                best = S.red[q][7];
+                bi = S.ired[q];
+            }
+        }
+        if (bi == 0x7fffffff) bi = 0;  // every bound is -inf or NaN
+        const bool own = w0 + bi >= ta && w0 + bi < tb;
+        if (own || w0 == 0) {
+            load_raw(w0 + bi);
+            thr = tile_step(-1) - kReach;
+            if (!ok) break;
+            if (!own) {  // another split's tile: it only set the shift
+                S2 = 0ull;
+                V[0] = V[1] = V[2] = 0ull;
+            }
+        }
+        // the other tiles of this split that can matter, in order (a NaN bound is visited)
+        const int qa = max(ta - w0, 0), qb = min(tb - w0, nw), len = max(qb - qa, 0);
+        const int each = (len + kT - 1) / kT, i0 = min(qa + t * each, qb), i1 = min(i0 + each, qb);
+        int cnt = 0;
+        for (int q = i0; q < i1; ++q) cnt += q != bi && !(S.bnd[q] < thr);
+        int inc = cnt;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += u;
+        }
+        if (lane == 31) S.wsum[warp] = inc;
+        __syncthreads();
+        int pos = inc - cnt;
+        for (int q = 0; q < warp; ++q) pos += S.wsum[q];
+        const int n_list = S.wsum[0] + S.wsum[1] + S.wsum[2] + S.wsum[3];
+        for (int q = i0; q < i1; ++q)
+            if (q != bi && !(S.bnd[q] < thr)) S.list[pos++] = (unsigned short)q;
+        __syncthreads();
+        auto find = [&](int k) {  // first entry from k on that still reaches the shift
+            while (k < n_list && S.bnd[S.list[k]] < thr) ++k;
+            return k;
+        };
+        int k = find(0);
+        if (k < n_list) load_raw(w0 + S.list[k]);
+        while (ok && k < n_list) {
+            const int nx = find(k + 1);
+            thr = tile_step(nx < n_list ? w0 + S.list[nx] : -1) - kReach;
+            k = nx;
+        }
+        __syncthreads();  // the next window overwrites the bounds
+    }
+    if (in_run) {
+        tot = sum2(S2);
+        float4 o = make_float4(sh, tot, 0.f, 0.f);
+        if constexpr (GRAD) {
+            o.y = sum2(V[0]);
+            o.z = sum2(V[1]);
+            o.w = sum2(V[2]);
+        }
+        A.out[((size_t)blockIdx.z * A.splits + blockIdx.y) * A.n_rows + r0 + t] = o;
+    }
+    }
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    if (!ok && t == 0) atomicOr(A.err, 1u);
+    if (warp == 0) tc::tmem_dealloc(tmem, kT);
+}
+
+// Boxes of the column tiles of both parts (blockIdx.y), one warp per tile.
+__global__ void tile_box_kernel(const __grid_constant__ S3Args A, float4 *box0, float4 *box1) {
+    const S3Part &P = A.part[blockIdx.y];
+    float4 *box = blockIdx.y ? box1 : box0;
+    const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (g * kT >= P.n) return;
+    float v[6] = {FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX}, m = -INFINITY;
+    for (int j = g * kT + lane; j < min(P.n, g * kT + kT); j += 32) {
+        const float4 q = P.cols[j];
+        v[0] = fminf(v[0], q.x); v[1] = fminf(v[1], q.y); v[2] = fminf(v[2], q.z);
+        v[3] = fminf(v[3], -q.x); v[4] = fminf(v[4], -q.y); v[5] = fminf(v[5], -q.z);
+        const float u = A.s * fmaf(A.eps, q.w, P.pot[j]);
+        const bool num = u == u && q.x == q.x && q.y == q.y && q.z == q.z;
+        m = num ? fmaxf(m, u) : INFINITY;  // a column that is not a number is visited by every row
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+        for (int o = 16; o > 0; o >>= 1) v[q] = fminf(v[q], __shfl_xor_sync(0xffffffffu, v[q], o));
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) {
+        box[2 * g] = make_float4(v[0], v[1], v[2], m);
+        box[2 * g + 1] = make_float4(-v[3], -v[4], -v[5], 0.f);
+    }
+}
+
+struct GradFinish {
+    const float4 *part;
+    int n, D, splits;
+    const float *row_pot[2];
+    float sign[2];
+    const float *row_w;
+    const int *perm;
+    float s, scale;
+    int accumulate;
+    float *grad;
+};
+__global__ void grad3_finish_kernel(const __grid_constant__ GradFinish F) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= F.n) return;
+    float out[3] = {0.f, 0.f, 0.f};
+    for (int q = 0; q < 2; ++q) {
+        const float4 *p = F.part + (size_t)q * F.splits * F.n + r;
+        float m = kNoTerm;
+        for (int k = 0; k < F.splits; ++k) m = fmaxf(m, p[(size_t)k * F.n].x);
+        if (!(m > kNoTerm)) continue;  // no term
+        float v[3] = {0.f, 0.f, 0.f};
+        for (int k = 0; k < F.splits; ++k) {
+            const float4 u = p[(size_t)k * F.n];
+            const float f = xt::ex2(u.x - m);
+            v[0] = fmaf(f, u.y, v[0]);
+            v[1] = fmaf(f, u.z, v[1]);
+            v[2] = fmaf(f, u.w, v[2]);
+        }
+        const float em = F.sign[q] * exp2f((float)((double)m + (double)F.s * (double)F.row_pot[q][r]));
+        for (int d = 0; d < 3; ++d) out[d] = fmaf(em, v[d], out[d]);
+    }
+    const size_t i = F.perm ? F.perm[r] : r;
+    const float aw = F.row_w[r] * F.scale;
+    for (int d = 0; d < F.D; ++d) {
+        float v = aw * out[d];
+        if (F.accumulate) v += F.grad[i * F.D + d];
+        F.grad[i * F.D + d] = v;
+    }
+}
+
+struct SoftFinish {
+    const float4 *part;
+    int n, splits;
+    const float *row_old;
+    float *row_out;
+    float lam, omega;
+    double eps_ln2;
+    int4 *fallback;
+    int *n_fallback;
+};
+__global__ void softmin3_finish_kernel(const __grid_constant__ SoftFinish F) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= F.n) return;
+    const float4 *p = F.part + r;
+    float m = kNoTerm, tot = 0.f;
+    for (int k = 0; k < F.splits; ++k) m = fmaxf(m, p[(size_t)k * F.n].x);
+    for (int k = 0; k < F.splits; ++k) {
+        const float4 u = p[(size_t)k * F.n];
+        tot += u.y * xt::ex2(u.x - m);
+    }
+    if (!(tot >= 0x1p-60f && tot <= 0x1p60f)) {
+        F.fallback[atomicAdd(F.n_fallback, 1)] = make_int4(0, r, r / kT, 0);
+        return;
+    }
+    const double tilde = -(double)F.lam * F.eps_ln2 * ((double)m + log2((double)tot));
+    double nw = tilde;
+    if (F.row_old) {
+        const double old = (double)F.row_old[r];
+        nw = old + (double)F.omega * (tilde - old);
+    }
+    F.row_out[r] = (float)nw;
+}
+
+__device__ __forceinline__ uint32_t spread3(uint32_t v) {  // bit k -> bit 3 k, 10 bits
+    v &= 0x3ffu;
+    v = (v | (v << 16)) & 0x030000ffu;
+    v = (v | (v << 8)) & 0x0300f00fu;
+    v = (v | (v << 4)) & 0x030c30c3u;
+    v = (v | (v << 2)) & 0x09249249u;
+    return v;
+}
+// Position on the Hilbert curve of a 2^bits grid over the points' box (J. Skilling, Programming the Hilbert curve, AIP
+// Conf. Proc. 707, 2004: undo the rotations of every level from the top, then Gray-encode; the index interleaves the
+// three coordinates' bits).
+__global__ void hilbert_kernel(const float *x, int n, int D, const float *box, int bits, uint32_t *keys) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float ext = 0.f;
+    for (int d = 0; d < D; ++d) ext = fmaxf(ext, box[64 + d] - box[d]);
+    const float inv = ext > 0.f ? (float)(1 << bits) / ext : 0.f;
+    uint32_t c[3] = {0u, 0u, 0u};
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+        if (d < D) {
+            const float u = (x[(size_t)i * D + d] - box[d]) * inv;
+            c[d] = u > 0.f ? (uint32_t)min((int)fminf(u, 1e6f), (1 << bits) - 1) : 0u;  // also for a point that is not finite
+        }
+    for (uint32_t q = 1u << (bits - 1); q > 1u; q >>= 1) {
+        const uint32_t low = q - 1u;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            if (c[d] & q) {
+                c[0] ^= low;
+            } else {
+                const uint32_t u = (c[0] ^ c[d]) & low;
+                c[0] ^= u;
+                c[d] ^= u;
+            }
+        }
+    }
+    c[1] ^= c[0];
+    c[2] ^= c[1];
+    uint32_t g = 0u;
+    for (uint32_t q = 1u << (bits - 1); q > 1u; q >>= 1)
+        if (c[2] & q) g ^= q - 1u;
+    keys[i] = (spread3(c[0] ^ g) << 2) | (spread3(c[1] ^ g) << 1) | spread3(c[2] ^ g);
+}
+
+// Order of n points along the Hilbert curve of their box (lo at d_box, hi at d_box + 64).  Five bits per axis (two sort
+// passes) up to 32k points, eight (three passes) above.
+int *curve_order(otgb_ctx *ctx, const std::string &tag, const float *x, int n, int D, const float *d_box) {
+    cudaStream_t st = ctx_stream(ctx);
+    Workspace &ws = ctx_ws(ctx);
+    uint32_t *src = ws.get<uint32_t>(tag + ":k0", n), *keys = ws.get<uint32_t>(tag + ":k1", n);
+    int *perm = ws.get<int>(tag + ":perm", n);
+    const int bits = n <= 32768 ? 5 : 8;
+    hilbert_kernel<<<(n + 255) / 256, 256, 0, st>>>(x, n, D, d_box, bits, src);
+    OTGB_CHECK_LAUNCH();
+    radix_sort_pairs_from(src, keys, perm, n, 3 * bits, ws.get("sort:scratch", radix_sort_scratch_bytes(n)), st);
+    return perm;
+}
+
+// Fills boxes and splits, launches the sums over `parts` parts.
+template <bool GRAD> void run_sums(otgb_ctx *ctx, S3Args &A, int parts, cudaStream_t st) {
+    Workspace &ws = ctx_ws(ctx);
+    int mx = 0;
+    float4 *box[2] = {nullptr, nullptr};
+    for (int q = 0; q < parts; ++q) {
+        const int nt = (A.part[q].n + kT - 1) / kT;
+        mx = std::max(mx, nt);
+        box[q] = ws.get<float4>(q ? "s3:box1" : "s3:box0", 2 * (size_t)nt);
+        A.part[q].box = box[q];
+    }
+    const int nblk = (A.n_rows + kT - 1) / kT;
+    // about two waves of four CTAs per SM; a split visits the best tile for its shift only, so at least 16 tiles each
+    const int want = (8 * ctx_sm_count(ctx) + nblk * parts - 1) / (nblk * parts);
+    A.splits = std::max(1, std::min(want, mx / 16));
+    A.out = ws.get<float4>("s3:part", (size_t)parts * A.splits * A.n_rows);
+    A.err = ws.get<unsigned>("s3:err", 1);
+    OTGB_CUDA_TRY(cudaMemsetAsync(A.err, 0, sizeof(unsigned), st));
+    tile_box_kernel<<<dim3((mx + 7) / 8, parts), 256, 0, st>>>(A, box[0], box[1]);
+    OTGB_CHECK_LAUNCH();
+    static_assert(sizeof(S3Smem) * 4 + 4096 <= 228 * 1024, "four CTAs per SM");
+    static PerDevice<int> attr;
+    attr.get([] {
+        OTGB_CUDA_TRY(cudaFuncSetAttribute(sorted3_kernel<GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(S3Smem)));
+        return 1;
+    });
+    sorted3_kernel<GRAD><<<dim3(nblk, A.splits, parts), kT, sizeof(S3Smem), st>>>(A);
+    OTGB_CHECK_LAUNCH();
+}
+
+void check_timeout(otgb_ctx *ctx, const unsigned *err, const char *what, cudaStream_t st) {
+    unsigned *h = static_cast<unsigned *>(ctx_pinned(ctx));
+    OTGB_CUDA_TRY(cudaMemcpyAsync(h, err, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+    OTGB_CUDA_TRY(cudaStreamSynchronize(st));
+    require(*h == 0, std::string(what) + ": a bounded device wait gave up", OTGB_ETIMEOUT);
+}
+
+}  // namespace
+
+void grad3_run(otgb_ctx *ctx, const float4 *rows, int n, int D, const Grad3Part (&part)[2], double eps, const float *row_w,
+               float scale, int accumulate, const int *perm, float *grad, cudaStream_t st) {
+    S3Args A;
+    std::memset(&A, 0, sizeof(A));
+    GradFinish F;
+    std::memset(&F, 0, sizeof(F));
+    A.rows = rows;
+    A.n_rows = n;
+    A.eps = (float)eps;
+    A.s = (float)(1.4426950408889634 / eps);
+    for (int q = 0; q < 2; ++q) {
+        A.part[q] = S3Part{part[q].cols, part[q].pot, nullptr, part[q].n};
+        F.row_pot[q] = part[q].row_pot;
+        F.sign[q] = part[q].sign;
+    }
+    run_sums<true>(ctx, A, 2, st);
+    F.part = A.out; F.n = n; F.D = D; F.splits = A.splits; F.row_w = row_w; F.perm = perm; F.s = A.s; F.scale = scale;
+    F.accumulate = accumulate; F.grad = grad;
+    grad3_finish_kernel<<<(n + 127) / 128, 128, 0, st>>>(F);
+    OTGB_CHECK_LAUNCH();
+    check_timeout(ctx, A.err, "gradient", st);
+}
+
+void grad3_apply(otgb_ctx *ctx, const float *x, const float *alpha, int N, const float *y, const float *beta, int M, int D,
+                 double eps, const float *f, const float *g, const float *a_self, float *grad) {
+    cudaStream_t st = ctx_stream(ctx);
+    Workspace &ws = ctx_ws(ctx);
+    float *box = ws.get<float>("box", 4 * 64), *bpart = ws.get<float>("bpart", 64 * 2 * 64), *cen = ws.get<float>("cen", 64);
+    bbox(x, N, D, D, box, box + 64, bpart, st);
+    bbox(y, M, D, D, box + 128, box + 192, bpart, st);
+    OTGB_CUDA_TRY(cudaMemsetAsync(cen, 0, 64 * sizeof(float), st));  // the coordinates as they are
+    int *px = curve_order(ctx, "s3:x", x, N, D, box), *py = curve_order(ctx, "s3:y", y, M, D, box + 128);
+    float4 *X = ws.get<float4>("s3:X", N), *Y = ws.get<float4>("s3:Y", M);
+    float *xw = ws.get<float>("s3:xw", N), *fs = ws.get<float>("s3:f", N), *as = ws.get<float>("s3:a", N), *gs = ws.get<float>("s3:g", M);
+    pack_points(x, alpha, px, N, D, cen, reinterpret_cast<float *>(X), nullptr, xw, st);
+    pack_points(y, beta, py, M, D, cen, reinterpret_cast<float *>(Y), nullptr, nullptr, st);
+    permute(f, px, N, fs, st);
+    permute(a_self, px, N, as, st);
+    permute(g, py, M, gs, st);
+    const Grad3Part part[2] = {{Y, gs, M, 1.f, fs}, {X, as, N, -1.f, as}};
+    grad3_run(ctx, X, N, D, part, eps, xw, 1.f, 0, px, grad, st);
+}
+
+void softmin3_sorted(otgb_ctx *ctx, const float *q, int n_out, const float *p, const float *w, const float *pot, int n_in,
+                     int D, double eps, double lam, const float *old, double omega, float *out, const float *d_box,
+                     const float *d_cen) {
+    cudaStream_t st = ctx_stream(ctx);
+    Workspace &ws = ctx_ws(ctx);
+    float *qbox = ws.get<float>("s3:qbox", 128), *bpart = ws.get<float>("bpart", 64 * 2 * 64);
+    bbox(q, n_out, D, D, qbox, qbox + 64, bpart, st);
+    int *pq = curve_order(ctx, "s3:x", q, n_out, D, qbox), *pp = curve_order(ctx, "s3:y", p, n_in, D, d_box);
+    float4 *R = ws.get<float4>("s3:X", n_out), *C = ws.get<float4>("s3:Y", n_in);
+    float *ps = ws.get<float>("s3:g", n_in), *os = old ? ws.get<float>("s3:f", n_out) : nullptr, *res = ws.get<float>("s3:a", n_out);
+    pack_points(q, nullptr, pq, n_out, D, d_cen, reinterpret_cast<float *>(R), nullptr, nullptr, st);
+    pack_points(p, w, pp, n_in, D, d_cen, reinterpret_cast<float *>(C), nullptr, nullptr, st);
+    permute(pot, pp, n_in, ps, st);
+    if (old) permute(old, pq, n_out, os, st);
+    S3Args A;
+    std::memset(&A, 0, sizeof(A));
+    A.rows = R;
+    A.n_rows = n_out;
+    A.eps = (float)eps;
+    A.s = (float)(1.4426950408889634 / eps);
+    A.part[0] = S3Part{C, ps, nullptr, n_in};
+    run_sums<false>(ctx, A, 1, st);
+    // rows whose sums are no number take the safe kernel, over all columns
+    SoftminLaunch L;
+    std::memset(&L, 0, sizeof(L));
+    L.n_inst = 1;
+    SoftminInst &I = L.inst[0];
+    I.rows = reinterpret_cast<const float *>(R); I.cols = reinterpret_cast<const float *>(C);
+    I.col_pot = ps; I.row_old = os; I.row_out = res;
+    I.n_rows = n_out; I.n_cols = n_in; I.lam = (float)lam; I.omega = (float)omega;
+    L.eps = A.eps;
+    L.s = A.s;
+    L.eps_ln2 = eps * 0.69314718055994530942;
+    L.fallback = ws.get<int4>("sm:fb", n_out + 64);
+    L.n_fallback = ws.get<int>("s3:nfb", 1);
+    L.fallback_cap = n_out + 64;
+    OTGB_CUDA_TRY(cudaMemsetAsync(L.n_fallback, 0, sizeof(int), st));
+    const SoftFinish F{A.out, n_out, A.splits, os, res, I.lam, I.omega, L.eps_ln2, L.fallback, L.n_fallback};
+    softmin3_finish_kernel<<<(n_out + 127) / 128, 128, 0, st>>>(F);
+    OTGB_CHECK_LAUNCH();
+    softmin_fallback_launch(L, D, st);
+    unpermute(res, pq, n_out, out, st);
+    check_timeout(ctx, A.err, "otgb_softmin", st);
+}
+
+}  // namespace otgb
