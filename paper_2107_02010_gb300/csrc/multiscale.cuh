@@ -66,6 +66,7 @@ struct Solver {
     double softmin_ms = 0.0;
     long softmin_launches = 0;
     Multiscale *ms = nullptr;
+    bool warm = false;                        // started from given duals
     bool g_from_f = false;                    // before the first step: g = one plain softmin of f
     std::vector<std::vector<int>> work_ncols; // columns per (instance, block) of the current work
 

@@ -138,7 +138,13 @@ void Solver::step(double sigma, bool count_pairs) {
     L.inst[3].col_pot = pg[c]; L.inst[3].row_old = pf[c]; L.inst[3].row_out = pf[n];
     for (int k = 0; k < 4; ++k) { L.inst[k].lam = lam; L.inst[k].omega = 0.5f; }
     L.pairs = count_pairs ? d_pairs : nullptr;
-    OTGB_CUDA_TRY(cudaMemsetAsync(L.delta_max, 0, sizeof(unsigned), st));
+    // the largest step, the number of fallback rows and the per-block counters of split blocks lie together
+    OTGB_CUDA_TRY(cudaMemsetAsync(L.delta_max, 0, sizeof(int) * (2 + (L.part ? L.n_fin : 0)), st));
+    L.counters_zeroed = 1;
+    // A warm start's duals can be far from the softmin of these points (the barycenter's points have moved), and the
+    // averaged steps halve the distance: the first steps keep a running shift instead of trusting the old values, which
+    // sent most rows to the safe kernel (2.0 of 11 ms per barycenter step).
+    L.exact_max = warm && use_tc3 && fine_steps < 6 ? 1 : 0;
     if (timing && ev_used == kEvPool) {  // pool full: wait for the oldest window, then reuse it
         OTGB_CUDA_TRY(cudaEventSynchronize(ev_pool[2 * kEvPool - 1]));
         harvest_timing();
@@ -150,6 +156,7 @@ void Solver::step(double sigma, bool count_pairs) {
         OTGB_CUDA_TRY(cudaEventRecord(ev_pool[2 * ev_used + 1], st));
         ++ev_used;
     }
+    L.counters_zeroed = 0;
     cur = n;
     ++steps;
 }
@@ -292,26 +299,30 @@ void Solver::set_work(const std::vector<std::vector<int>> &ncols, bool allow_spl
     launch.n_fin = 0;
     launch.item_fin = nullptr;
     launch.fin_count = nullptr;
+    int *ctl = ws->get<int>(nm("ctl"), 2 + (split ? fin.size() : 0));
+    launch.delta_max = reinterpret_cast<unsigned *>(ctl);
+    launch.n_fallback = ctl + 1;
     if (split) {
         int4 *d_fin = ws->get<int4>(nm("fin"), fin.size() + 1);
         OTGB_CUDA_TRY(cudaMemcpyAsync(d_fin, fin.data(), fin.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-        launch.part = ws->get<float>(nm("part"), items.size() * (size_t)kPartRows * (D > 3 ? 2 : 1));
+        launch.part = ws->get<float>(nm("part"), items.size() * (size_t)kPartRows * 2);
         launch.fin = d_fin;
         launch.n_fin = (int)fin.size();
         int *d_ifin = ws->get<int>(nm("itemfin"), items.size() + 1);
         OTGB_CUDA_TRY(cudaMemcpyAsync(d_ifin, item_fin.data(), item_fin.size() * sizeof(int), cudaMemcpyHostToDevice, st));
         launch.item_fin = d_ifin;
-        launch.fin_count = ws->get<int>(nm("fincnt"), fin.size() + 1);
+        launch.fin_count = ctl + 2;
     }
     OTGB_CUDA_TRY(cudaStreamSynchronize(st));  // host vectors go out of scope
 }
 
 void Solver::alloc_common() {
     launch = SoftminLaunch();
-    launch.delta_max = ws->get<unsigned>(nm("delta"), 1);
     const int cap = 2 * (X.n + Y.n) + 64;
     launch.fallback = ws->get<int4>(nm("fb"), cap);
-    launch.n_fallback = ws->get<int>(nm("nfb"), 1);
+    int *ctl = ws->get<int>(nm("ctl"), 2);
+    launch.delta_max = reinterpret_cast<unsigned *>(ctl);
+    launch.n_fallback = ctl + 1;
     launch.work_counter = ws->get<int>(nm("wctr"), 1);
     launch.fallback_cap = cap;
     d_fb_total = ws->get<unsigned long long>(nm("fbtot"), 1);
@@ -605,6 +616,7 @@ int otgb::solve_divergence(otgb_ctx *ctx, const float *x, const float *a, int N,
             OTGB_CHECK_LAUNCH();
         }
         s.alloc_pots(P);
+        s.warm = P.f_init || P.g_init || P.a_init || P.b_init;
         s.g_from_f = P.init_g_from_f != 0 && P.f_init != nullptr && P.g_init == nullptr;
 
         // rows per CTA: enough CTAs to fill the GPU twice, else the smallest blocks
@@ -656,7 +668,7 @@ int otgb::solve_divergence(otgb_ctx *ctx, const float *x, const float *a, int N,
             rc = s.iterate_at_blur(Pp, P.max_iters);
         }
         OTGB_CUDA_TRY(cudaEventRecord(ctx_event(ctx, 4), st));
-        if (rc == OTGB_OK || rc == OTGB_ENOCONV) s.S = s.divergence(s.eps_of(P.blur));
+        // S is that of the last check or of the last fixed step: the duals have not changed since
         if (gr && (rc == OTGB_OK || rc == OTGB_ENOCONV)) grad_sparse_launch(s, s.eps_of(P.blur), *gr, st);
 
         // outputs in the caller's order
