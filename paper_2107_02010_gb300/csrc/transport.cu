@@ -393,7 +393,19 @@ extern "C" int transport_apply(otgb_ctx *ctx, const otgb_plan *plan, const float
         bbox(plan->y, M, D, D, box, box + 64, bpart, st);
         float *d_cen = ws.get<float>("cen", 64);
         box_centre(box, box + 64, D, d_cen, st);
-        if (xd_width(D)) {
+        // The tensor-core path keeps column tiles and the scores of every row (N x L).  The kernels below need neither: they
+        // stay in charge where both would take more than half of the memory that is free (asked only above 8 GB).
+        bool tc_path = xd_width(D) != 0;
+        if (tc_path) {
+            const size_t need = sizeof(float) * (size_t)N * L + ((size_t)M / 128 + 2049) * tcc_tile_bytes(3, stride);
+            const size_t have = ws.held("ta:sct") + ws.held("ta:tiles");
+            if (need > have + (size_t(8) << 30)) {
+                size_t free_b = 0, total_b = 0;
+                OTGB_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+                tc_path = need - have <= free_b / 2;
+            }
+        }
+        if (tc_path) {
             const TransportCall c{plan->x, plan->y, plan->b, N, M, D, L, plan->eps, f, g, labels, d_cen, scores, argmax, row_mass};
             const TransportFallback r = transport_xt_apply(ctx, c);
             TransportArgs A;
