@@ -48,27 +48,23 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # add per pair.
 SFU_EX2_PER_CLK_SM = 32
 FP32_LANES_PER_CLK_SM = 128
-# tensor flops per pair: D <= 3 float32-accuracy form (K = 32 BF16 slots), and
-# the 60-D BF16 hi/lo cross term (three K = 64 products)
+# tensor flops per pair: D <= 3 float32-accuracy form (K = 32 BF16 slots), the
+# 60-D BF16 hi/lo cross term (three K = 64 products), and its float32-accuracy
+# form (three pieces per operand, six products)
 TC3_TENSOR_FLOP_PER_PAIR = 2 * 32
 TC60_TENSOR_FLOP_PER_PAIR = 3 * 2 * 64
+FP32_60_TENSOR_FLOP_PER_PAIR = 6 * 2 * 64
 # DRAM bytes (ncu dram__bytes_read.sum + dram__bytes_write.sum) per launch of the
 # dominant kernel of each workload, from one capture of the current kernel
-# (null when the kernel has changed since).  softmin3_tc_kernel: a fine step of
-# the track-density workload (100k x 100k), 6,644,224 bytes read, 0 written.
+# (null when the kernel has changed since).
 TRAFFIC = {
-    "softmin3_tc_kernel": 6644224,
-    "softmin_gen_kernel": None,
+    "softmin3_tc_kernel": None,
+    "softmin_tcc_kernel": None,
 }
 
 
 def peaks():
     return json.load(open(PEAKS_FILE)) if os.path.exists(PEAKS_FILE) else {}
-
-
-def fp32_form_peak(D, clock_mhz, n_sm):
-    per_clk = min(SFU_EX2_PER_CLK_SM, FP32_LANES_PER_CLK_SM / (D + 2))
-    return per_clk * n_sm * clock_mhz * 1e6
 
 
 # ------------------------------------------------------------------ inputs --
@@ -352,8 +348,8 @@ def run_fibers(args):
     h2d = sum(v.nbytes for v in (x, a, y, b))
     d2h = 4 * (x.shape[0] + y.shape[0])
 
-    # roofline of the dominant kernel (softmin_gen_kernel: 60-D float32 dot-product form)
-    peak = fp32_form_peak(D, clk, n_sm)
+    # roofline of the dominant kernel (softmin_tcc_kernel, three BF16 pieces per operand: float32 accuracy)
+    peak = min(pk.get("bf16_tflops", 1910.7) * 1e12 / FP32_60_TENSOR_FLOP_PER_PAIR, SFU_EX2_PER_CLK_SM * n_sm * clk * 1e6)
     achieved = s32["pairs_per_solve"] / (s32["softmin_ms_per_solve"] / 1e3)
     line = {
         "metric": "softmin pairs/s", "value": value, "unit": "pairs/s", "n_gpus": world, "steps": args.steps,
@@ -373,12 +369,11 @@ def run_fibers(args):
         "converged": s32["converged"], "iters_per_solve": s32["iters_per_solve"],
         "pairs_per_solve": s32["pairs_per_solve"], "kept_fraction": s32["kept_fraction"],
         "softmin_ms_per_solve": s32["softmin_ms_per_solve"], "phases_ms": s32["phases_ms"],
-        "roofline": {"bound": "alu", "kernel": "softmin_gen_kernel (+ fallback), 60-D float32 dot-product form",
+        "roofline": {"bound": "tensor", "kernel": "softmin_tcc_kernel (three-piece BF16 operands, float32 accuracy)",
                      "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Gpairs/s", "frac": achieved / peak,
-                     "traffic": TRAFFIC["softmin_gen_kernel"],
-                     "peak_basis": "FP32: %d SMs x 128 lanes/clk / (D + 2) FP32 ops per pair x %.0f MHz "
-                                   "(sm_max_mhz of MEASURED_PEAKS.json); MUFU ex2 (32/clk) is not binding at "
-                                   "D = 60" % (n_sm, clk)},
+                     "traffic": TRAFFIC["softmin_tcc_kernel"],
+                     "peak_basis": "bf16 burst of measured / %d flop per pair; MUFU ex2 (32/clk) is not binding" %
+                                   FP32_60_TENSOR_FLOP_PER_PAIR},
         "e2e": {"value": e2e_val, "unit": "pairs/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "repeats": len(e2e_ms), "ms_per_step": statistics.mean(e2e_ms)},
         "gpu_launches": int(launches), "clocks": clocks,
