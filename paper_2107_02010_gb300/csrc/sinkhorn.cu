@@ -772,8 +772,10 @@ extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const floa
         float *box = ws.get<float>("box", 4 * 64);
         bbox_centre(p, n_in, D, d_cen, box, ws.get<float>("bpart", 64 * 2 * 64), st);
         // Large 3-D sweeps sort their points and visit the tiles that can matter (sorted3.cu); the sorts and permutations
-        // are some twenty launches (0.2 ms, a dense sweep over 1e9 pairs).  100k x 100k: 0.85 ms sorted, 1.89 dense.
-        if (D <= 3 && n_out >= 4096 && n_in >= 4096 && (double)n_out * n_in >= 2e9) {
+        // are some twenty launches.  Sorted against dense: 32k x 32k 0.33 / 0.27 ms, 45k x 45k 0.46 / 0.45, 64k x 64k
+        // 0.63 / 0.81, 100k x 100k 0.85 / 1.89.  Few rows or columns make large blocks or tiles, which reach everything:
+        // 4,200 x 500k 0.93 / 0.48, 500k x 4,200 0.52 / 0.45.
+        if (D <= 3 && n_out >= 32768 && n_in >= 32768 && (double)n_out * n_in >= 2e9) {
             softmin3_sorted(ctx, q, n_out, p, w, pot, n_in, D, eps, lam, old, omega, out, box, d_cen);
             return OTGB_OK;
         }

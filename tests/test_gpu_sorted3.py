@@ -22,7 +22,7 @@ def cloud(rng, n, D, scale):
 
 
 @pytest.mark.parametrize("D,n,m,how", [(3, 45_001, 44_999, "near"), (3, 4097, 500_000, "ramp"), (2, 60_000, 40_000, "near"),
-                                       (1, 50_000, 45_000, "ramp"), (3, 4096, 530_000, "near")])
+                                       (1, 50_000, 45_000, "ramp"), (3, 4096, 530_000, "near"), (3, 32_768, 530_000, "ramp")])
 def test_large_softmin_sampled_rows(D, n, m, how):
     from paper_2107_02010_gb300 import otgb
 
@@ -47,7 +47,8 @@ def test_large_softmin_sampled_rows(D, n, m, how):
     ctx.close()
 
 
-@pytest.mark.parametrize("D,n,m,shift", [(3, 5003, 4100, 0.0), (2, 4400, 777, 0.0), (1, 4500, 129, 0.0), (3, 4471, 3000, 30.0)])
+@pytest.mark.parametrize("D,n,m,shift", [(3, 5003, 4100, 0.0), (2, 4400, 777, 0.0), (1, 4500, 129, 0.0), (3, 4471, 3000, 30.0),
+                                         (3, 2000, 2001, 0.0)])
 def test_gradient_matches_oracle(D, n, m, shift):
     from paper_2107_02010_gb300 import otgb
 
