@@ -120,6 +120,7 @@ struct Multiscale {
     float *cen_x = nullptr, *cen_y = nullptr;    // ncl x stride (coarse points; D <= 3: (c, log mass))
     float *lm_x = nullptr, *lm_y = nullptr;      // D > 3: log mass
     float *mass_x = nullptr, *mass_y = nullptr, *rad_x = nullptr, *rad_y = nullptr;
+    float4 *box_x = nullptr, *box_y = nullptr;   // D <= 3: bounding boxes (lo, hi)
     // fine row blocks: host starts and cluster ranges
     std::vector<int> hbx, hby, hclx, hcly;       // hcl: 2 ints per block (cl0, cl1)
     int *d_clx = nullptr, *d_cly = nullptr;
