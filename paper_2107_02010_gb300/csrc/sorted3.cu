@@ -41,7 +41,9 @@ constexpr int kT = 128;           // threads, rows of a block, columns of a tile
 constexpr int kMaxTiles = 4096;   // tiles bounded at once (524,288 columns)
 constexpr float kNoTerm = -1e29f;
 constexpr float kReach = 60.f;    // binades below the row's largest term that are visited
-constexpr float kCompact = 96.f;
+// s (half diagonal)^2 of a run: what the products of the exponent are rounded at.  The softmin's error is 7e-8 at 96, far
+// below the CUDA cores'; the gradient, a small difference of two large sums, needs smaller runs (@FIG@).
+template <bool GRAD> constexpr float kCompact = GRAD ? 12.f : 96.f;
 constexpr float kSpread = 256.f;  // terms of this size are rounded at 8e-6, as s f + s g - s C is at |s f| = 128
 
 struct S3Part {
@@ -182,7 +184,7 @@ __global__ void __launch_bounds__(kT, 4) sorted3_kernel(const __grid_constant__ 
             h[d] = fmaxf(hi[d], -S.sub[gb][d + 3]);
             u = fmaf(0.25f * (h[d] - l[d]), h[d] - l[d], u);
         }
-        if (!(s * u <= kCompact)) break;
+        if (!(s * u <= kCompact<GRAD>)) break;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             lo[d] = l[d];
