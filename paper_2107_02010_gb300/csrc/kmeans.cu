@@ -93,7 +93,9 @@ __global__ void __launch_bounds__(kAT, 2) kmeans_assign_kernel(const float *x, i
     float best[8];
     int bidx[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) { best[i] = INFINITY; bidx[i] = 0x7fffffff; }
+    // cluster 0 until a distance is finite: a point that is not finite, or whose squares overflow, keeps it, so that every
+    // label indexes a cluster
+    for (int i = 0; i < 8; ++i) { best[i] = INFINITY; bidx[i] = 0; }
     fetch(0);
     store(0);
     __syncthreads();
