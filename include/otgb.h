@@ -105,8 +105,9 @@ typedef struct {
     int debug_wait_probe;  /* test hook of the bounded-wait error path: 1 = the solve also runs one device
                               wait on a word that nothing writes; it gives up after about a millisecond,
                               flags the error word that the tensor-core and tile waits use, and the solve
-                              (whose outputs are still written) returns OTGB_ETIMEOUT.  Nothing faults or
-                              hangs and the context stays usable.  0 = off (default). */
+                              (whose outputs are still written) returns OTGB_ETIMEOUT.  2 = the same, the wait
+                              belonging to the coarse phase of a coarse-to-fine solve where there is one.
+                              Nothing faults or hangs and the context stays usable.  0 = off (default). */
     int polish;            /* D > 3 only: 1 = once the stopping rule holds, run the loop at blur again, to the
                               same rule, with every softmin in the direct difference form of the cost
                               (sum of squared coordinate differences, FP32 CUDA cores, about twice the work

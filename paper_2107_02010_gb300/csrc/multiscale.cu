@@ -398,7 +398,9 @@ int Multiscale::run_schedule(Solver &s, const otgb_params &P, const std::vector<
     // coarse phase on the cluster measures while sigma > sigma_switch
     size_t k = 0;
     const bool warm = P.f_init || P.g_init || P.a_init || P.b_init;
-    if (!warm && !sched.empty() && sched[0] > sigma_switch) {
+    const bool coarse = !warm && !sched.empty() && sched[0] > sigma_switch;
+    if (P.debug_wait_probe == 2 && !coarse) wait_probe(s.ctx, s.launch.tc_err);
+    if (coarse) {
         Solver cs;
         cs.tag = "c:";
         cs.ctx = s.ctx;
@@ -416,6 +418,8 @@ int Multiscale::run_schedule(Solver &s, const otgb_params &P, const std::vector<
         cs.Y.n = ncl_y; cs.Y.D = D; cs.Y.stride = stride; cs.Y.pts = cen_y; cs.Y.logw = lm_y; cs.Y.w = mass_y;
         cs.Y.mass = s.Y.mass;
         cs.alloc_common();
+        cs.launch.tc_err = s.launch.tc_err;  // the word that the solve reads back
+        if (P.debug_wait_probe == 2) wait_probe(s.ctx, cs.launch.tc_err);
         otgb_params Pc = P;
         Pc.f_init = Pc.g_init = Pc.a_init = Pc.b_init = nullptr;
         cs.alloc_pots(Pc);

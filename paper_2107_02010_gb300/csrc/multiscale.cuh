@@ -139,4 +139,7 @@ struct Multiscale {
     void setup_tcc(Solver &s);
 };
 
+// Test hook of the bounded-wait error path: one wait that runs out, on a word that nothing writes, and flags *err.
+void wait_probe(otgb_ctx *ctx, unsigned *err);
+
 }  // namespace otgb

@@ -119,6 +119,14 @@ __global__ void wait_probe_kernel(const volatile unsigned *flag, unsigned *err, 
 
 }  // namespace
 
+void wait_probe(otgb_ctx *ctx, unsigned *err) {
+    cudaStream_t st = ctx_stream(ctx);
+    unsigned *flag = ctx_ws(ctx).get<unsigned>("probe", 1);
+    OTGB_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(unsigned), st));
+    wait_probe_kernel<<<1, 32, 0, st>>>(flag, err, 1000);
+    OTGB_CHECK_LAUNCH();
+}
+
 // One averaged step of the four instances at temperature eps.
 void Solver::step(double sigma, bool count_pairs) {
     const double eps = eps_of(sigma);
@@ -609,12 +617,7 @@ int otgb::solve_divergence(otgb_ctx *ctx, const float *x, const float *a, int N,
         pack_points(y, b, s.Y.perm, M, D, d_cen, s.Y.pts, s.Y.logw, s.Y.w, st);
 
         s.alloc_common();
-        if (P.debug_wait_probe) {
-            unsigned *flag = s.ws->get<unsigned>("probe", 1);
-            OTGB_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(unsigned), st));
-            wait_probe_kernel<<<1, 32, 0, st>>>(flag, s.launch.tc_err, 1000);
-            OTGB_CHECK_LAUNCH();
-        }
+        if (P.debug_wait_probe && !(P.debug_wait_probe == 2 && msp)) wait_probe(ctx, s.launch.tc_err);
         s.alloc_pots(P);
         s.warm = P.f_init || P.g_init || P.a_init || P.b_init;
         s.g_from_f = P.init_g_from_f != 0 && P.f_init != nullptr && P.g_init == nullptr;
