@@ -158,6 +158,10 @@ void otgb_default_params(otgb_params *p);
 int otgb_create(otgb_ctx **out, int device, void *cuda_stream);
 /* Release the context and all its scratch memory. */
 int otgb_destroy(otgb_ctx *ctx);
+/* Test hooks of a context, all 0 by default.  OTGB_DEBUG_WAIT_PROBE: 1 = an otgb_softmin over all pairs also runs one device
+   wait that runs out (as otgb_params.debug_wait_probe) and returns OTGB_ETIMEOUT. */
+typedef enum { OTGB_DEBUG_WAIT_PROBE = 0, OTGB_DEBUG_KEYS = 1 } otgb_debug_key;
+int otgb_debug_set(otgb_ctx *ctx, int key, long long value);
 /* Last error message of the context (static storage when ctx is NULL). */
 const char *otgb_last_error(const otgb_ctx *ctx);
 
@@ -312,7 +316,8 @@ int sinkhorn_barycenter(otgb_ctx *ctx, float *x, const float *alpha, int N, int 
  * for rows q (n_out x D) and columns p (n_in x D) with weights w (n_in) and
  * potential pot (n_in), dense.  When old is non-null the result is blended:
  *   out_i <- old_i + omega (out_i - old_i)   (omega = 1/2 is the paper's average).
- * Errors: EINVAL for sizes < 1, D outside [1, 64], eps <= 0.
+ * Errors: EINVAL for sizes < 1, D outside [1, 64], eps <= 0; ETIMEOUT when a bounded device wait gave up (out is
+ * then not complete).
  */
 int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const float *p, const float *w, const float *pot,
                  int n_in, int D, double eps, double lam, const float *old, double omega, float *out);

@@ -825,8 +825,13 @@ extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const floa
         L.fallback = ws.get<int4>("sm:fb", cap);
         L.n_fallback = cnt;
         L.fallback_cap = cap;
+        unsigned *err = ctx_error_word(ctx);  // nothing of this context is in flight: every call ends with a synchronise
+        *err = 0;
+        L.tc_err = err;
+        if (ctx_debug(ctx, OTGB_DEBUG_WAIT_PROBE)) wait_probe(ctx, err);
         softmin_run(L, D, D <= 3 ? 4 : 1, st);
         OTGB_CUDA_TRY(cudaStreamSynchronize(st));
+        require(*const_cast<volatile unsigned *>(err) == 0, "otgb_softmin: a bounded device wait gave up", OTGB_ETIMEOUT);
         return OTGB_OK;
     } catch (const Error &e) {
         return fail(ctx, e);

@@ -20,6 +20,7 @@ struct otgb_ctx {
     cudaEvent_t ev[8] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     // pinned host mailbox for small device->host reads
     void *pinned = nullptr;
+    long long debug[OTGB_DEBUG_KEYS] = {};  // test hooks
 };
 
 static thread_local std::string g_err;
@@ -164,6 +165,15 @@ int otgb_destroy(otgb_ctx *ctx) {
     return OTGB_OK;
 }
 
+int otgb_debug_set(otgb_ctx *ctx, int key, long long value) {
+    if (!ctx || key < 0 || key >= OTGB_DEBUG_KEYS) {
+        g_err = "otgb_debug_set: null context or unknown key";
+        return OTGB_EINVAL;
+    }
+    ctx->debug[key] = value;
+    return OTGB_OK;
+}
+
 const char *otgb_last_error(const otgb_ctx *ctx) { return ctx ? ctx->err.c_str() : g_err.c_str(); }
 
 unsigned long long otgb_kernel_launches(void) { return otgb::launch_count(); }
@@ -181,6 +191,8 @@ int fail(otgb_ctx *ctx, const Error &e) {
 cudaStream_t ctx_stream(otgb_ctx *ctx) { return ctx->stream; }
 Workspace &ctx_ws(otgb_ctx *ctx) { return ctx->ws; }
 void *ctx_pinned(otgb_ctx *ctx) { return ctx->pinned; }
+unsigned *ctx_error_word(otgb_ctx *ctx) { return reinterpret_cast<unsigned *>(static_cast<char *>(ctx->pinned) + 4032); }
+long long ctx_debug(otgb_ctx *ctx, int key) { return ctx->debug[key]; }
 cudaEvent_t ctx_event(otgb_ctx *ctx, int k) { return ctx->ev[k]; }
 void ctx_set_device(otgb_ctx *ctx) { OTGB_CUDA_TRY(cudaSetDevice(ctx->device)); }
 int ctx_sm_count(otgb_ctx *ctx) {

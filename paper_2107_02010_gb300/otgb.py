@@ -95,7 +95,7 @@ EXPORTS = ["otgb_default_params", "otgb_create", "otgb_destroy", "otgb_last_erro
            "otgb_mlp_get_normalization", "otgb_mlp_set_params", "otgb_mlp_get_params", "otgb_mlp_grad",
            "otgb_mlp_adam_step", "otgb_mlp_train_step", "otgb_mlp_train_epoch", "otgb_mlp_infer", "otgb_mlp_save",
            "otgb_mlp_load", "sinkhorn_divergence_warm", "sinkhorn_grad_x", "sinkhorn_barycenter", "otgb_flip_fibers",
-           "otgb_select_flips", "otgb_unit_rates"]
+           "otgb_select_flips", "otgb_unit_rates", "otgb_debug_set"]
 
 
 def kernel_launches() -> int:
@@ -166,6 +166,8 @@ def load(build_if_missing: bool = True):
     lib.otgb_unit_rates.argtypes = [vp, C.POINTER(cd), C.POINTER(cd), C.POINTER(cd)]
     lib.otgb_unit_rates.restype = ci
     lib.otgb_select_flips.argtypes = [vp, vp, vp, ci, vp, vp, vp]
+    lib.otgb_debug_set.argtypes = [vp, ci, C.c_longlong]
+    lib.otgb_debug_set.restype = ci
     for name in ("otgb_flip_fibers", "otgb_select_flips", "sinkhorn_grad_x", "sinkhorn_barycenter", "otgb_create", "otgb_destroy", "sinkhorn_divergence",
                  "transport_apply", "cluster_grid",
                  "cluster_kmeans", "otgb_softmin", "otgb_mlp_create", "otgb_mlp_destroy", "otgb_mlp_n_params",
@@ -221,6 +223,10 @@ class Context:
     def check(self, rc):
         if rc != 0:
             raise OtgbError(rc, load().otgb_last_error(self.h).decode())
+
+    def debug_set(self, key, value):
+        """otgb_debug_set: a test hook of this context."""
+        self.check(load().otgb_debug_set(self.h, int(key), int(value)))
 
     def close(self):
         if getattr(self, "h", None):
