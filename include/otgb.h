@@ -51,8 +51,8 @@ typedef enum {
    operand of either form is centred at its cluster's centroid and split once per solve, which holds
    per point of x and of y two copies of 2 x pieces x round_up(round_up(D, 4) + 4, 16) bytes in the
    context's scratch (D = 60: 0.5 KB per point with two pieces, 0.77 KB with three; at most 8192
-   clusters per side).  Where that is more than 8 GB and more than half of the free device memory, the
-   float32 form runs on the CUDA cores instead.
+   clusters per side).  Where that is more than 8 GB and more than half of the free device memory, or
+   where an allocation fails, the float32 form runs on the CUDA cores instead.
    OTGB_FP32_SIMT: float32 on the CUDA cores for every D. */
 typedef enum { OTGB_FP32 = 0, OTGB_TC_BF16X3 = 1, OTGB_FP32_SIMT = 2 } otgb_precision;
 typedef enum { OTGB_CLUSTER_GRID = 0, OTGB_CLUSTER_KMEANS = 1 } otgb_cluster_kind;
@@ -159,8 +159,10 @@ int otgb_create(otgb_ctx **out, int device, void *cuda_stream);
 /* Release the context and all its scratch memory. */
 int otgb_destroy(otgb_ctx *ctx);
 /* Test hooks of a context, all 0 by default.  OTGB_DEBUG_WAIT_PROBE: 1 = an otgb_softmin over all pairs also runs one device
-   wait that runs out (as otgb_params.debug_wait_probe) and returns OTGB_ETIMEOUT. */
-typedef enum { OTGB_DEBUG_WAIT_PROBE = 0, OTGB_DEBUG_KEYS = 1 } otgb_debug_key;
+   wait that runs out (as otgb_params.debug_wait_probe) and returns OTGB_ETIMEOUT.
+   OTGB_DEBUG_SCRATCH_LIMIT: > 0 = device scratch allocations of the context fail once it would hold more bytes than
+   this, as on a device without more free memory. */
+typedef enum { OTGB_DEBUG_WAIT_PROBE = 0, OTGB_DEBUG_SCRATCH_LIMIT = 1, OTGB_DEBUG_KEYS = 2 } otgb_debug_key;
 int otgb_debug_set(otgb_ctx *ctx, int key, long long value);
 /* Last error message of the context (static storage when ctx is NULL). */
 const char *otgb_last_error(const otgb_ctx *ctx);

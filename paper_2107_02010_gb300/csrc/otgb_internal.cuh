@@ -104,7 +104,9 @@ struct Workspace {
     };
     std::vector<Buf> bufs;
     cudaStream_t stream = nullptr;
+    size_t limit = 0;  // test hook: total bytes above which an allocation fails (0: none)
     void *get(const std::string &name, size_t bytes);
+    void release_scratch();  // frees what no caller of a solve keeps (barycenter, warm start, network)
     size_t held(const std::string &name) const;  // bytes of a buffer already there (0: none)
     template <class T> T *get(const std::string &name, size_t count) {
         return static_cast<T *>(get(name, count * sizeof(T) + 16));

@@ -519,10 +519,11 @@ void Solver::fine_step(double sigma) {
 
 using namespace otgb;
 
-int otgb::solve_divergence(otgb_ctx *ctx, const float *x, const float *a, int N, const float *y, const float *b,
-                           int M, int D, const otgb_params *params, double *cost_host, float *f, float *g,
-                           float *a_self, float *b_self, otgb_plan **plan_out, otgb_stats *stats,
-                           const GradRequest *gr) {
+// lean: without the tensor-core forms of D > 3, whose tiles and partial sums are the only scratch that the CUDA-core kernels
+// can do without.
+static int solve_once(otgb_ctx *ctx, const float *x, const float *a, int N, const float *y, const float *b, int M, int D,
+                      const otgb_params *params, double *cost_host, float *f, float *g, float *a_self, float *b_self,
+                      otgb_plan **plan_out, otgb_stats *stats, const GradRequest *gr, bool lean) {
     if (!ctx) return fail(nullptr, Error{OTGB_EINVAL, "sinkhorn_divergence: null context"});
     try {
         ctx_set_device(ctx);
@@ -553,8 +554,8 @@ int otgb::solve_divergence(otgb_ctx *ctx, const float *x, const float *a, int N,
         s.translation = P.translation != 0;
         s.use_tc = P.precision == OTGB_TC_BF16X3 && D >= 16 && P.p == 2;
         s.use_tc3 = P.precision == OTGB_FP32 && D <= 3 && P.p == 2;
-        s.use_xd = P.precision == OTGB_FP32 && P.p == 2 && xd_width(D);
-        s.tcc_pieces = P.p != 2 || D <= 3 ? 0 : (s.use_tc ? 2 : (P.precision == OTGB_FP32 ? 3 : 0));
+        s.use_xd = !lean && P.precision == OTGB_FP32 && P.p == 2 && xd_width(D);
+        s.tcc_pieces = P.p != 2 || D <= 3 ? 0 : (s.use_tc ? 2 : (!lean && P.precision == OTGB_FP32 ? 3 : 0));
         cudaStream_t st = s.st;
         OTGB_CUDA_TRY(cudaEventRecord(ctx_event(ctx, 0), st));
 
@@ -747,6 +748,18 @@ int otgb::solve_divergence(otgb_ctx *ctx, const float *x, const float *a, int N,
     } catch (const Error &e) {
         return fail(ctx, e);
     }
+}
+
+// An allocation that fails leaves inputs and outputs as they were: the solve runs once more in an empty workspace (earlier
+// calls' buffers given back) with the kernels that need the least.
+int otgb::solve_divergence(otgb_ctx *ctx, const float *x, const float *a, int N, const float *y, const float *b,
+                           int M, int D, const otgb_params *params, double *cost_host, float *f, float *g,
+                           float *a_self, float *b_self, otgb_plan **plan_out, otgb_stats *stats,
+                           const GradRequest *gr) {
+    const int rc = solve_once(ctx, x, a, N, y, b, M, D, params, cost_host, f, g, a_self, b_self, plan_out, stats, gr, false);
+    if (rc != OTGB_ENOMEM) return rc;
+    ctx_ws(ctx).release_scratch();
+    return solve_once(ctx, x, a, N, y, b, M, D, params, cost_host, f, g, a_self, b_self, plan_out, stats, gr, true);
 }
 
 extern "C" int sinkhorn_divergence(otgb_ctx *ctx, const float *x, const float *a, int N, const float *y,

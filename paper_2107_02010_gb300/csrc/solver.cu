@@ -47,24 +47,39 @@ int current_device() {
 namespace otgb {
 
 void *Workspace::get(const std::string &name, size_t bytes) {
-    for (auto &b : bufs)
-        if (b.name == name) {
-            if (b.bytes >= bytes) return b.ptr;
-            if (b.ptr) OTGB_CUDA_TRY(cudaFreeAsync(b.ptr, stream));  // null after a growth that failed
-            b.ptr = nullptr;
-            b.bytes = 0;
-            const cudaError_t e = cudaMallocAsync(&b.ptr, bytes, stream);
-            if (e != cudaSuccess) throw Error{OTGB_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes failed"};
-            b.bytes = bytes;
-            return b.ptr;
-        }
-    Buf b;
-    b.name = name;
-    const cudaError_t e = cudaMallocAsync(&b.ptr, bytes, stream);
-    if (e != cudaSuccess) throw Error{OTGB_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes failed"};
-    b.bytes = bytes;
-    bufs.push_back(b);
-    return b.ptr;
+    Buf *b = nullptr;
+    size_t others = 0;
+    for (auto &u : bufs) {
+        if (u.name == name) b = &u;
+        else others += u.bytes;
+    }
+    if (b && b->bytes >= bytes) return b->ptr;
+    if (!b) {
+        bufs.emplace_back();
+        b = &bufs.back();
+        b->name = name;
+    }
+    if (b->ptr) OTGB_CUDA_TRY(cudaFreeAsync(b->ptr, stream));  // null: new, or after a growth that failed
+    b->ptr = nullptr;
+    b->bytes = 0;
+    if ((limit && others + bytes > limit) || cudaMallocAsync(&b->ptr, bytes, stream) != cudaSuccess) {
+        b->ptr = nullptr;
+        cudaGetLastError();  // the next launch check must not see it
+        throw Error{OTGB_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes failed"};
+    }
+    b->bytes = bytes;
+    return b->ptr;
+}
+
+void Workspace::release_scratch() {
+    std::vector<Buf> kept;
+    for (auto &b : bufs) {
+        bool keep = false;
+        for (const char *p : {"bary:", "warm:", "mlp:"}) keep = keep || b.name.compare(0, std::strlen(p), p) == 0;
+        if (keep) kept.push_back(b);
+        else if (b.ptr) cudaFreeAsync(b.ptr, stream);
+    }
+    bufs.swap(kept);
 }
 
 size_t Workspace::held(const std::string &name) const {
@@ -171,6 +186,7 @@ int otgb_debug_set(otgb_ctx *ctx, int key, long long value) {
         return OTGB_EINVAL;
     }
     ctx->debug[key] = value;
+    ctx->ws.limit = (size_t)std::max(ctx->debug[OTGB_DEBUG_SCRATCH_LIMIT], 0ll);
     return OTGB_OK;
 }
 

@@ -1,0 +1,69 @@
+"""Calls that can do with less scratch do so when an allocation fails (here: a limit on the bytes that a context may hold),
+instead of returning ENOMEM: whatever the CUDA-core kernels can solve within a limit, the default forms solve too."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2107_02010_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+LIMIT = 1  # OTGB_DEBUG_SCRATCH_LIMIT
+
+
+def T(v):
+    return torch.from_numpy(np.ascontiguousarray(v)).cuda()
+
+
+def under(limit, call):
+    """call(context) on a fresh context that may hold `limit` bytes; None when it returns ENOMEM."""
+    from paper_2107_02010_gb300 import otgb
+
+    ctx = otgb.Context()
+    ctx.debug_set(LIMIT, limit)
+    try:
+        return call(ctx)
+    except otgb.OtgbError as e:
+        assert e.code == -3, e
+        return None
+    finally:
+        ctx.close()
+
+
+def least(call):
+    """The smallest limit within 3 % under which call succeeds."""
+    lo, hi = 1, 1 << 33
+    assert under(hi, call) is not None
+    while hi > 1.03 * lo:
+        mid = int((lo * hi) ** 0.5) if hi > 2 * lo else (lo + hi) // 2
+        lo, hi = (lo, mid) if under(mid, call) is not None else (mid, hi)
+    return hi
+
+
+@pytest.mark.parametrize("multiscale", [0, 1])
+def test_solve_within_the_scratch_of_the_cuda_core_form(multiscale):
+    from paper_2107_02010_gb300 import otgb
+
+    x, a, _ = synth.fiber_bundles(6000, seed=4, perturb=3.0)
+    y, b, _ = synth.fiber_bundles(5000, seed=5)
+    x, a, y, b = T(x), T(a), T(y), T(b)
+
+    def solve(precision):
+        p = otgb.default_params(blur=2.0, reach=20.0, multiscale=multiscale, cluster=1, k_clusters=40, fixed_iters=3,
+                                precision=precision)
+        return lambda ctx: otgb.sinkhorn_divergence(ctx, x, a, y, b, p)
+
+    limit = least(solve(2))
+    want = under(1 << 33, solve(2))
+    for room in (1.0, 1.05, 1.2, 1.5, 3.0):
+        got = under(int(room * limit), solve(0))
+        assert got is not None, room
+        assert abs(got["S"] - want["S"]) <= 1e-5 * abs(want["S"])
+    # a context that once failed goes on working
+    ctx = otgb.Context()
+    ctx.debug_set(LIMIT, limit // 4)
+    with pytest.raises(otgb.OtgbError) as e:
+        solve(0)(ctx)
+    assert e.value.code == -3
+    ctx.debug_set(LIMIT, 0)
+    assert abs(solve(0)(ctx)["S"] - want["S"]) <= 1e-5 * abs(want["S"])
+    ctx.close()
