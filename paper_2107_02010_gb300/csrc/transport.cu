@@ -374,8 +374,9 @@ void label_order(otgb_ctx *ctx, const int *labels, int M, int L, uint32_t *keys,
 
 using namespace otgb;
 
-extern "C" int transport_apply(otgb_ctx *ctx, const otgb_plan *plan, const float *f, const float *g,
-                               const int32_t *labels, int L, float *scores, int32_t *argmax, float *row_mass) {
+// lean: without the tensor-core path, whose tiles and class-major scores the other kernels do not need
+static int transport_once(otgb_ctx *ctx, const otgb_plan *plan, const float *f, const float *g, const int32_t *labels, int L,
+                          float *scores, int32_t *argmax, float *row_mass, bool lean) {
     if (!ctx) return fail(nullptr, Error{OTGB_EINVAL, "transport_apply: null context"});
     try {
         ctx_set_device(ctx);
@@ -395,7 +396,7 @@ extern "C" int transport_apply(otgb_ctx *ctx, const otgb_plan *plan, const float
         box_centre(box, box + 64, D, d_cen, st);
         // The tensor-core path keeps column tiles and the scores of every row (N x L).  The kernels below need neither: they
         // stay in charge where both would take more than half of the memory that is free (asked only above 8 GB).
-        bool tc_path = xd_width(D) != 0;
+        bool tc_path = !lean && xd_width(D);
         if (tc_path) {
             const size_t need = sizeof(float) * (size_t)N * L + ((size_t)M / 128 + 2049) * tcc_tile_bytes(3, stride);
             const size_t have = ws.held("ta:sct") + ws.held("ta:tiles");
@@ -499,4 +500,13 @@ extern "C" int transport_apply(otgb_ctx *ctx, const otgb_plan *plan, const float
     } catch (const Error &e) {
         return fail(ctx, e);
     }
+}
+
+// An allocation that fails leaves the outputs unwritten: once more in an empty workspace, with the kernels that need less.
+extern "C" int transport_apply(otgb_ctx *ctx, const otgb_plan *plan, const float *f, const float *g,
+                               const int32_t *labels, int L, float *scores, int32_t *argmax, float *row_mass) {
+    const int rc = transport_once(ctx, plan, f, g, labels, L, scores, argmax, row_mass, false);
+    if (rc != OTGB_ENOMEM) return rc;
+    ctx_ws(ctx).release_scratch();
+    return transport_once(ctx, plan, f, g, labels, L, scores, argmax, row_mass, true);
 }

@@ -67,3 +67,29 @@ def test_solve_within_the_scratch_of_the_cuda_core_form(multiscale):
     ctx.debug_set(LIMIT, 0)
     assert abs(solve(0)(ctx)["S"] - want["S"]) <= 1e-5 * abs(want["S"])
     ctx.close()
+
+
+def test_label_transfer_within_the_scratch_of_the_cuda_core_form():
+    from paper_2107_02010_gb300 import otgb
+
+    n, m, L = 6000, 5000, 30
+    x, a, _ = synth.fiber_bundles(n, seed=4, perturb=3.0)
+    y, b, lab = synth.fiber_bundles(m, seed=5)
+    a, b, lab = T(a), T(b), T((lab % L).astype(np.int32))
+    ctx = otgb.Context()
+    p = otgb.default_params(blur=2.0, reach=20.0, multiscale=1, cluster=1, k_clusters=20, fixed_iters=5)
+
+    def transfer(pad):  # 64 coordinates (the last ones 0) take the CUDA-core kernel
+        X, Y = (T(np.pad(v, ((0, 0), (0, pad)))) for v in (x, y))
+        r = otgb.sinkhorn_divergence(ctx, X, a, Y, b, p, want_plan=True)
+        return lambda c: otgb.transport_apply(c, r["plan"], r["f"], r["g"], lab, L, want_scores=False)
+
+    general, call = transfer(4), transfer(0)
+    limit = least(general)
+    _, am, rm = under(1 << 33, general)
+    for room in (1.0, 1.05, 1.2, 1.5, 3.0):
+        got = under(int(room * limit), call)
+        assert got is not None, room
+        assert (got[1] != am).float().mean() < 1e-3
+        assert torch.allclose(got[2], rm, rtol=1e-3)
+    ctx.close()
