@@ -285,8 +285,12 @@ void grad_sparse_run(const Solver &s, double eps, const GradRequest &gr, cudaStr
     if (s.D <= 3 && s.p == 2) {  // the solve's points are in spatial order: every pair that can matter, on the tensor cores
         const float4 *X = reinterpret_cast<const float4 *>(s.X.pts), *Y = reinterpret_cast<const float4 *>(s.Y.pts);
         const Grad3Part part[2] = {{Y, s.pg[s.cur], s.Y.n, 1.f, s.pf[s.cur]}, {X, s.pa[s.cur], s.X.n, -1.f, s.pa[s.cur]}};
-        grad3_run(s.ctx, X, s.X.n, s.D, part, eps, s.X.w, gr.scale, gr.accumulate, s.X.perm, gr.grad, st);
-        return;
+        try {
+            grad3_run(s.ctx, X, s.X.n, s.D, part, eps, s.X.w, gr.scale, gr.accumulate, s.X.perm, gr.grad, st);
+            return;
+        } catch (const Error &e) {  // no room for the partial sums: the kernel below needs none
+            if (e.code != OTGB_ENOMEM) throw;
+        }
     }
     SpGradArgs A;
     std::memset(&A, 0, sizeof(A));
@@ -358,8 +362,13 @@ extern "C" int sinkhorn_grad_x(otgb_ctx *ctx, const float *x, const float *alpha
         // p = 2 in up to three dimensions: sorted, on the tensor cores (sorted3.cu); in small calls the sorts cost more
         // than the pairs (sorted against every pair: 1,000 + 1,000 points 0.28 / 0.19 ms, 2,000 + 2,000 0.29 / 0.35)
         if (D <= 3 && p == 2 && (double)N * ((double)N + M) >= 8e6) {
-            grad3_apply(ctx, x, alpha, N, y, beta, M, D, eps, f, g, a_self, grad);
-            return OTGB_OK;
+            try {
+                grad3_apply(ctx, x, alpha, N, y, beta, M, D, eps, f, g, a_self, grad);
+                return OTGB_OK;
+            } catch (const Error &e) {  // no room for the sorted copies: the other kernel needs none
+                if (e.code != OTGB_ENOMEM) throw;
+                ctx_ws(ctx).release_scratch();
+            }
         }
         grad_launch(grad_args(x, alpha, N, y, beta, M, D, p, eps, a_self, f, g, grad, 1.f, 0), st);
         OTGB_CUDA_TRY(cudaStreamSynchronize(st));

@@ -770,9 +770,9 @@ extern "C" int sinkhorn_divergence(otgb_ctx *ctx, const float *x, const float *a
                             nullptr);
 }
 
-extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const float *p, const float *w,
-                            const float *pot, int n_in, int D, double eps, double lam, const float *old,
-                            double omega, float *out) {
+// lean: without the sorted form and without split columns, whose copies and partial sums a plain sweep does not need
+static int softmin_once(otgb_ctx *ctx, const float *q, int n_out, const float *p, const float *w, const float *pot, int n_in,
+                        int D, double eps, double lam, const float *old, double omega, float *out, bool lean) {
     if (!ctx) return fail(nullptr, Error{OTGB_EINVAL, "otgb_softmin: null context"});
     try {
         ctx_set_device(ctx);
@@ -791,13 +791,13 @@ extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const floa
         // are some twenty launches.  Sorted against dense: 32k x 32k 0.33 / 0.27 ms, 45k x 45k 0.46 / 0.45, 64k x 64k
         // 0.63 / 0.81, 100k x 100k 0.85 / 1.89.  Few rows or columns make large blocks or tiles, which reach everything:
         // 4,200 x 500k 0.93 / 0.48, 500k x 4,200 0.52 / 0.45.
-        if (D <= 3 && n_out >= 32768 && n_in >= 32768 && (double)n_out * n_in >= 2e9) {
+        if (!lean && D <= 3 && n_out >= 32768 && n_in >= 32768 && (double)n_out * n_in >= 2e9) {
             softmin3_sorted(ctx, q, n_out, p, w, pot, n_in, D, eps, lam, old, omega, out, box, d_cen);
             return OTGB_OK;
         }
         // blocks of 128 rows, their columns split so that the launch fills the GPU (tensor-core kernels); the CUDA-core
         // kernel of D > 60 takes whole blocks
-        const bool tc = D <= 3 || xd_width(D);
+        const bool tc = !lean && (D <= 3 || xd_width(D));
         const int nb = (n_out + 127) / 128, sms = ctx_sm_count(ctx);
         const int chunk = tc ? split_chunk({{nb, n_in}}, (D <= 3 ? 4LL : 2LL) * sms) : n_in;
         const int parts = (n_in - 1) / chunk + 1, n_items = nb * parts;
@@ -849,4 +849,13 @@ extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const floa
     } catch (const Error &e) {
         return fail(ctx, e);
     }
+}
+
+// An allocation that fails leaves the output unwritten: once more in an empty workspace, with what needs less.
+extern "C" int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const float *p, const float *w, const float *pot,
+                            int n_in, int D, double eps, double lam, const float *old, double omega, float *out) {
+    const int rc = softmin_once(ctx, q, n_out, p, w, pot, n_in, D, eps, lam, old, omega, out, false);
+    if (rc != OTGB_ENOMEM) return rc;
+    ctx_ws(ctx).release_scratch();
+    return softmin_once(ctx, q, n_out, p, w, pot, n_in, D, eps, lam, old, omega, out, true);
 }

@@ -93,3 +93,33 @@ def test_label_transfer_within_the_scratch_of_the_cuda_core_form():
         assert (got[1] != am).float().mean() < 1e-3
         assert torch.allclose(got[2], rm, rtol=1e-3)
     ctx.close()
+
+
+@pytest.mark.parametrize("D,n,m", [(3, 50_000, 45_000), (60, 300, 20_000)])
+def test_softmin_within_the_scratch_of_a_plain_sweep(D, n, m):
+    from paper_2107_02010_gb300 import otgb
+
+    rng = np.random.default_rng(3)
+    q, p = (T(10.0 * rng.random((k, D), np.float32)) for k in (n, m))
+    w, pot = T(np.full(m, 1.0 / m, np.float32)), T(rng.normal(size=m).astype(np.float32))
+    call = lambda ctx: otgb.softmin(ctx, q, p, w, pot, 0.5)
+    want = under(1 << 33, call)
+    # packed rows and columns with their log weights, a list entry per row, and 150 KB of small buffers
+    limit = 4 * ((D + 3) & ~3) * (n + m) + 16 * (n + 64) + (4 * m if D > 3 else 0) + 150_000
+    got = under(limit, call)
+    assert got is not None
+    assert (got - want).abs().max() <= 1e-5 * (want.abs().max() + 0.5)
+
+
+def test_gradient_within_no_scratch():
+    from paper_2107_02010_gb300 import otgb
+
+    rng = np.random.default_rng(4)
+    n, m = 9000, 8000
+    x, y = (T(10.0 * rng.random((k, 3), np.float32)) for k in (n, m))
+    a, b = (T(np.full(k, 1.0 / k, np.float32)) for k in (n, m))
+    f, g = (T(rng.normal(size=k).astype(np.float32)) for k in (n, m))
+    call = lambda ctx: otgb.sinkhorn_grad_x(ctx, x, a, y, b, 0.5, f, g, f)
+    want, got = under(1 << 33, call), under(4096, call)
+    assert got is not None
+    assert (got - want).abs().max() <= 1e-5 * want.abs().max()
