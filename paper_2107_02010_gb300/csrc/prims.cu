@@ -88,7 +88,7 @@ __global__ void box_centre_kernel(const float *lo, const float *hi, int D, float
 // Box and centre of a small input in one CTA (up to kBoxSmall values: a few microseconds, less than the launches and the
 // partial results of the general form).
 constexpr int kBoxSmall = 32768;
-__global__ void __launch_bounds__(kBoxT) bbox_small_kernel(const float *x, int n, int D, float *c) {
+__global__ void __launch_bounds__(kBoxT) bbox_small_kernel(const float *x, int n, int D, float *c, float *box) {
     __shared__ float red[kBoxT];
     const int G = kBoxT / D, t = threadIdx.x, g = t / D, d = t - g * D;
     float lo = FLT_MAX, hi = -FLT_MAX;
@@ -111,6 +111,7 @@ __global__ void __launch_bounds__(kBoxT) bbox_small_kernel(const float *x, int n
                 const float w = __shfl_xor_sync(0xffffffffu, v, o);
                 v = h ? fmaxf(v, w) : fminf(v, w);
             }
+            if ((t & 31) == 0) box[64 * h + q] = v;
             out[u] = h ? 0.5f * (out[u] + v) : v;
         }
         __syncthreads();
@@ -617,7 +618,7 @@ void box_centre(const float *lo, const float *hi, int D, float *c, cudaStream_t 
 
 void bbox_centre(const float *x, int n, int D, float *d_centre, float *d_box, float *d_part, cudaStream_t st) {
     if ((size_t)n * D <= kBoxSmall) {
-        bbox_small_kernel<<<1, kBoxT, 0, st>>>(x, n, D, d_centre);
+        bbox_small_kernel<<<1, kBoxT, 0, st>>>(x, n, D, d_centre, d_box);
         OTGB_CHECK_LAUNCH();
         return;
     }

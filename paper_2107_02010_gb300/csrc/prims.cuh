@@ -13,7 +13,8 @@ void bbox(const float *x, int n, int D, int stride, float *d_lo, float *d_hi, fl
 // c (64 floats) = middle of the box, 0 beyond D.
 void box_centre(const float *lo, const float *hi, int D, float *c, cudaStream_t st);
 
-// The middle of the bounding box in one call (one launch for small inputs).  d_box: 128 floats, d_part as for bbox.
+// The bounding box and its middle in one call (one launch for small inputs).  d_box: lo, and hi 64 floats on; d_part as for
+// bbox.
 void bbox_centre(const float *x, int n, int D, float *d_centre, float *d_box, float *d_part, cudaStream_t st);
 
 // S of Eq. (6) in double from the four duals (internal order) and the weights;
