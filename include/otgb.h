@@ -295,9 +295,9 @@ int sinkhorn_grad_x(otgb_ctx *ctx, const float *x, const float *alpha, int N, co
  * each gradient computed at the end of a solve of sinkhorn_divergence with
  * *params (after the first step every solve starts at blur from the previous
  * step's four duals).  The gradient is the expression of sinkhorn_grad_x.  In
- * a coarse-to-fine solve with p = 1 or D > 3 it is summed over the kept cluster
+ * a coarse-to-fine solve with p = 1, D > 3 or OTGB_FP32_SIMT it is summed over the kept cluster
  * pairs of the solve's last truncation; each dropped term is below e^-tau of
- * its row's total.  With D <= 3 and p = 2 every pair that float32 can see is
+ * its row's total.  With D <= 3, p = 2 and OTGB_FP32 every pair that float32 can see is
  * summed.  With p = 2, lr = 1 and without the debiasing term, this is the
  * classical fixed-point update x_i <- mean_k of the barycentric projections.
  *   x: N x D device, updated in place; alpha: N device.

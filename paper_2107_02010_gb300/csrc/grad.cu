@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kGR) grad_sparse_kernel(const __grid_constant_
 }
 
 void grad_sparse_run(const Solver &s, double eps, const GradRequest &gr, cudaStream_t st) {
-    if (s.D <= 3 && s.p == 2) {  // the solve's points are in spatial order: every pair that can matter, on the tensor cores
+    if (s.use_tc3) {  // the solve's points are in spatial order: every pair that can matter, on the tensor cores
         const float4 *X = reinterpret_cast<const float4 *>(s.X.pts), *Y = reinterpret_cast<const float4 *>(s.Y.pts);
         const Grad3Part part[2] = {{Y, s.pg[s.cur], s.Y.n, 1.f, s.pf[s.cur]}, {X, s.pa[s.cur], s.X.n, -1.f, s.pa[s.cur]}};
         try {
