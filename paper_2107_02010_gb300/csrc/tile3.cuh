@@ -1,12 +1,18 @@
 // Operands of the D <= 3 tensor-core tiles without a known row shift: K = 32 BF16 slots whose dot product is the whole
 // base-2 exponent of a pair, -s |x - y|^2 / 2 + s (eps log w + pot), at float32 accuracy.
 //
-// Every float operand is split into three BF16 pieces (h + m + l); per coordinate the six products that matter take six
-// slots.  The rows may come as the caller has them, so that |x - c| |y - c| (c the block's centre) is much larger than any
-// exponent that matters; the slots are arranged so that each of the two K = 16 steps is small by itself for such a pair:
-// step 0 holds coordinates 0 and 1 with their own share of the squares (two pieces of -s (y0^2 + y1^2) / 2 against 1, two
-// of -s (x0^2 + x1^2) / 2), step 1 coordinate 2 and everything else (three pieces each).  The tensor cores cut the sum off
-// towards zero after each step, at the size of what it holds.
+// Every float operand is split into three BF16 pieces (h + m + l); six products per coordinate matter (ml, lm and ll are
+// below 2^-24 of hh).  The rows may come as the caller has them, so that |x - c| |y - c| (c the block's centre) and the
+// squares are much larger than any exponent that matters, while their sum is small.  Two things keep that sum's error down:
+//  - The row's pieces hold s (x - c) with what the product loses to rounding.  Without it (T 2^-25 for every pair of the
+//    row, T = s |x - c| |y - c|) the error of a row is that of a single float product.
+//  - A tensor-core step aligns its products and the accumulator to the largest of them and cuts off what lies some 24 bits
+//    below, towards zero.  The first K = 16 step holds hh, hm, mh and the leading pieces of H and R, whose bits lie above
+//    the cut for the larger coordinates; it leaves something small, to which the second step adds hl, mm, lh and the last
+//    pieces of H and R (2^-16 of the others) without losing their bits.
+// otgb_softmin, rms error against FP64, 3,000 x 2,500 points over 30 units in one / two / three dimensions, eps 1:
+// 4.1e-7 / 4.5e-7 / 3.6e-7 (CUDA cores 1.3e-6 / 1.7e-6 / 1.4e-6; without the rounding of s (x - c) and coordinate by
+// coordinate 1.8e-6 / 1.6e-6 / 0.9e-6; small products first 5.3e-7 / 5.4e-7 / 4.2e-7).
 #pragma once
 
 #include "tcgen05.cuh"
@@ -47,55 +53,39 @@ __device__ __forceinline__ void split3x2(float a, float b, uint32_t &H, uint32_t
     L = bf2(ra - hi_val(M), (rb - lo_val(M)) + rest);
 }
 
-// First word (two K slots) of coordinate d.
-__device__ __forceinline__ constexpr int coord_word(int d) { return d == 2 ? 8 : 3 * d; }
-
-// The row operand of centred point x: 16 words of two slots.
+// Words (two K slots each) of one operand.  Slots 0-8: hh, hm, mh of the coordinates; 9, 10: H's leading pieces, 11, 12:
+// R's; slots 16-24: hl, mm, lh; 25: H's last piece, 26: R's.
+//
+// The row operand of centred point x.
 __device__ __forceinline__ void row_words(float x0, float x1, float x2, float s, uint32_t (&w)[16]) {
     const float x[3] = {s * x0, s * x1, s * x2};
+    const float xr[3] = {fmaf(s, x0, -x[0]), fmaf(s, x1, -x[1]), fmaf(s, x2, -x[2])};
+    uint16_t h[3], m[3], l[3], r1, r2, r3;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        uint16_t h, m, l;
-        xt::split3(x[d], 0.f, h, m, l);
-        const int b0 = coord_word(d);  // h h m h l m (against the column's h m h l h m)
-        w[b0] = pk(h, h);
-        w[b0 + 1] = pk(m, h);
-        w[b0 + 2] = pk(l, m);
-    }
-    const double R01 = -0.5 * (double)s * ((double)x0 * x0 + (double)x1 * x1);
-    const uint16_t ra = bfbits((float)R01), rb = bfbits((float)(R01 - (double)bfval(ra)));
-    const double R2 = (R01 - (double)bfval(ra) - (double)bfval(rb)) - 0.5 * (double)s * ((double)x2 * x2);
-    uint16_t r1, r2, r3;
-    xt::split3((float)R2, (float)(R2 - (double)(float)R2), r1, r2, r3);
-    w[6] = pk(kOne, kOne);
-    w[7] = pk(ra, rb);
-    w[11] = pk(kOne, kOne);
-    w[12] = pk(kOne, r1);
-    w[13] = pk(r2, r3);
-    w[14] = w[15] = 0u;
+    for (int d = 0; d < 3; ++d) xt::split3(x[d], xr[d], h[d], m[d], l[d]);
+    const double R = -0.5 * (double)s * ((double)x0 * x0 + (double)x1 * x1 + (double)x2 * x2);
+    xt::split3((float)R, (float)(R - (double)(float)R), r1, r2, r3);
+    w[0] = pk(h[0], h[0]); w[1] = pk(m[0], h[1]); w[2] = pk(h[1], m[1]); w[3] = pk(h[2], h[2]);
+    w[4] = pk(m[2], kOne); w[5] = pk(kOne, r1); w[6] = pk(r2, 0);
+    w[8] = pk(h[0], m[0]); w[9] = pk(l[0], h[1]); w[10] = pk(m[1], l[1]); w[11] = pk(h[2], m[2]);
+    w[12] = pk(l[2], kOne); w[13] = pk(r3, 0);
+    w[7] = w[14] = w[15] = 0u;
 }
 
 // The column operand of centred point y with log weight lw and potential pot; in = false: no column (exponent -1e30).
 __device__ __forceinline__ void col_words(float y0, float y1, float y2, float lw, float pot, float s, float eps, bool in,
                                           uint32_t (&w)[16]) {
-    // |y0|^2 + |y1|^2 with its rounding errors (Knuth's two-sum, products by FMA), times -s/2; two BF16 pieces of it stay
-    // with those coordinates, what they leave joins the rest of H, which is summed with its errors too
+    // H = s (eps lw + pot) - s |y|^2 / 2 with its rounding errors (Knuth's two-sum, products by FMA)
     const float hs = -0.5f * s;
     const float p0 = y0 * y0, p1 = y1 * y1, t01 = p0 + p1, tb = t01 - p0;
     const float te = ((p0 - (t01 - tb)) + (p1 - tb)) + (fmaf(y0, y0, -p0) + fmaf(y1, y1, -p1));
     const float q01 = hs * t01, qe = fmaf(hs, t01, -q01) + hs * te;
-    const uint32_t wa = bf2(0.f, q01);
-    const float qa = q01 - lo_val(wa);
-    const uint32_t wb = bf2(0.f, qa);
-    const float rem = qa - lo_val(wb);
-    w[6] = in ? pk((uint16_t)wa, (uint16_t)wb) : 0u;
-    w[7] = pk(kOne, kOne);
     const float u = fmaf(eps, lw, pot), v = s * u, ve = fmaf(s, u, -v);
     const float z = y2 * y2, g = hs * z, ge = fmaf(hs, z, -g) + hs * fmaf(y2, y2, -z);
     const float S1 = v + g, sb = S1 - v, se = (v - (S1 - sb)) + (g - sb);
-    float H = S1 + rem;
+    float H = S1 + q01;
     const float hb = H - S1;
-    float rest = ((S1 - (H - hb)) + (rem - hb)) + (se + (ve + ge) + qe);
+    float rest = ((S1 - (H - hb)) + (q01 - hb)) + (se + (ve + ge) + qe);
     if (!in || H <= -1e30f) {  // absent, or zero weight (log w = -inf); NaN goes on
         H = -1e30f;
         rest = 0.f;
@@ -106,17 +96,11 @@ __device__ __forceinline__ void col_words(float y0, float y1, float y2, float lw
     const uint16_t h[3] = {(uint16_t)(H01 >> 16), (uint16_t)H01, (uint16_t)(H2h >> 16)};
     const uint16_t m[3] = {(uint16_t)(M01 >> 16), (uint16_t)M01, (uint16_t)(M2h >> 16)};
     const uint16_t l[3] = {(uint16_t)(L01 >> 16), (uint16_t)L01, (uint16_t)(L2h >> 16)};
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const int b0 = coord_word(d);
-        w[b0] = pk(h[d], m[d]);
-        w[b0 + 1] = pk(h[d], l[d]);
-        w[b0 + 2] = pk(h[d], m[d]);
-    }
-    w[11] = pk((uint16_t)H2h, (uint16_t)M2h);
-    w[12] = pk((uint16_t)L2h, kOne);
-    w[13] = pk(kOne, kOne);
-    w[14] = w[15] = 0u;
+    w[0] = pk(h[0], m[0]); w[1] = pk(h[0], h[1]); w[2] = pk(m[1], h[1]); w[3] = pk(h[2], m[2]);
+    w[4] = pk(h[2], (uint16_t)H2h); w[5] = pk((uint16_t)M2h, kOne); w[6] = pk(kOne, 0);
+    w[8] = pk(l[0], m[0]); w[9] = pk(h[0], l[1]); w[10] = pk(m[1], h[1]); w[11] = pk(l[2], m[2]);
+    w[12] = pk(h[2], (uint16_t)L2h); w[13] = pk(kOne, 0);
+    w[7] = w[14] = w[15] = 0u;
 }
 
 __device__ __forceinline__ void store_words(unsigned char *tile, int r, const uint32_t (&w)[16]) {

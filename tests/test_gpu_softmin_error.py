@@ -1,0 +1,42 @@
+"""The tensor-core sweeps are no further from FP64 than the CUDA-core sweep of the same problem (otgb_softmin_noalloc): the
+rms error over all rows, for clouds whose blocks of rows span the whole domain."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def softmin64(q, p, w, pot, eps, lam):
+    q, p, pot, lw = q.double(), p.double(), pot.double(), torch.log(w.double())
+    c = p.mean(0)
+    q, p = q - c, p - c
+    h = lw + (pot - 0.5 * (p * p).sum(1)) / eps
+    out = [-lam * (eps * torch.logsumexp(h + (u @ p.T) / eps, 1) - 0.5 * (u * u).sum(1)) for u in q.split(1000)]
+    return torch.cat(out)
+
+
+def errors(n, m, D, side, eps, seed, cloud):
+    from paper_2107_02010_gb300 import otgb
+
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    q, p = cloud(n, D, side, g), cloud(m, D, side, g)
+    w = torch.rand(m, generator=g, device="cuda") + 0.5
+    w /= w.sum()
+    pot = 3.0 * eps * torch.randn(m, generator=g, device="cuda")
+    want = softmin64(q, p, w, pot, eps, 0.99)
+    ctx = otgb.Context()
+    got = otgb.softmin(ctx, q, p, w, pot, eps, 0.99), otgb.softmin_noalloc(q, p, w, pot, eps, 0.99)
+    ctx.close()
+    return [float((v.double() - want).square().mean().sqrt()) for v in got]
+
+
+def uniform(n, D, side, g):
+    return side * torch.rand(n, D, generator=g, device="cuda")
+
+
+@pytest.mark.parametrize("D", [1, 2, 3])
+@pytest.mark.parametrize("n,m,side,eps", [(3000, 2500, 30.0, 1.0), (500, 60_000, 30.0, 1.0), (3000, 2500, 1.0, 0.0025)])
+def test_dense_sweep_in_up_to_three_dimensions(D, n, m, side, eps):
+    e = [errors(n, m, D, side, eps, seed, uniform) for seed in range(3)]
+    tc, cuda = (sum(v[k] ** 2 for v in e) ** 0.5 for k in (0, 1))
+    assert tc <= cuda, (tc, cuda)
