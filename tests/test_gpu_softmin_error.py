@@ -1,7 +1,10 @@
 """The tensor-core sweeps are no further from FP64 than the CUDA-core sweep of the same problem (otgb_softmin_noalloc): the
 rms error over all rows, for clouds whose blocks of rows span the whole domain."""
+import numpy as np
 import pytest
 import torch
+
+from paper_2107_02010_gb300 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -38,5 +41,18 @@ def uniform(n, D, side, g):
 @pytest.mark.parametrize("n,m,side,eps", [(3000, 2500, 30.0, 1.0), (500, 60_000, 30.0, 1.0), (3000, 2500, 1.0, 0.0025)])
 def test_dense_sweep_in_up_to_three_dimensions(D, n, m, side, eps):
     e = [errors(n, m, D, side, eps, seed, uniform) for seed in range(3)]
+    tc, cuda = (sum(v[k] ** 2 for v in e) ** 0.5 for k in (0, 1))
+    assert tc <= cuda, (tc, cuda)
+
+
+def fibers(n, D, side, g):
+    x = synth.fiber_bundles(n, seed=int(torch.randint(0, 1 << 30, (1,), generator=g, device="cuda")), perturb=3.0)[0]
+    return torch.from_numpy(np.ascontiguousarray(x[:, :D])).cuda()
+
+
+@pytest.mark.parametrize("D,cloud,eps", [(4, uniform, 1.0), (7, uniform, 4.0), (12, uniform, 25.0), (4, fibers, 25.0), (5, fibers, 25.0),
+                                         (13, fibers, 4.0), (24, fibers, 4.0), (45, fibers, 1.0), (60, fibers, 4.0)])
+def test_dense_sweep_in_more_dimensions(D, cloud, eps):
+    e = [errors(3001, 2777, D, 30.0, eps, seed, cloud) for seed in range(3)]
     tc, cuda = (sum(v[k] ** 2 for v in e) ** 0.5 for k in (0, 1))
     assert tc <= cuda, (tc, cuda)
