@@ -40,6 +40,7 @@ template <int K> struct XdSmem {
     float cen[kW];
     float csum[4][kW];
     unsigned long long raw_full[2], b_full, b_empty, acc_full, acc_free, a_ready, drain;
+    float tmax[4];  // largest T of the rows, per warp
     uint32_t tslot;
     int abort;
     int bc[2];
@@ -103,6 +104,7 @@ __global__ void __launch_bounds__(kThreads, 2) softmin_xd_kernel(const __grid_co
             int copied = 0;
             for (; copied < 2 && copied < ntiles; ++copied) copy(copied);
             if (ntiles > 0) ok = xt::wait(&S.a_ready, 0, abort);
+            const bool last = !MAXP && xt::fold_last(S.tmax);  // without old values the rows come as they are
             for (int k = 0; ok && k < ntiles; ++k) {
                 ok = xt::wait(&S.b_full, (uint32_t)(k & 1), abort);
                 if (!ok) break;
@@ -111,7 +113,7 @@ __global__ void __launch_bounds__(kThreads, 2) softmin_xd_kernel(const __grid_co
                 ok = k == 0 || xt::wait(&S.acc_free, (uint32_t)((k - 1) & 1), abort);
                 if (!ok) break;
                 tc::fence_after();
-                xt::issue<3, K>(tmem, tmem + kN, tc::smem_u32(S.b), k & 1);
+                xt::issue<3, K>(tmem, tmem + kN, tc::smem_u32(S.b), last ? xt::kFoldLast : k & 1);
                 tc::commit(&S.b_empty);
                 tc::commit(&S.acc_full);
             }
@@ -170,7 +172,8 @@ __global__ void __launch_bounds__(kThreads, 2) softmin_xd_kernel(const __grid_co
                 x[4 * q + 3] = v.w;
             }
             if (!MAXP && valid) Mi = (float)(-(double)s * (double)I.row_old[r0 + t] / (double)I.lam);
-            xt::stage_row<3, K>(x, D4, S.cen, s, Mi, valid, lanes + kN);
+            const float T = xt::stage_row<3, K>(x, D4, S.cen, s, Mi, valid, lanes + kN);
+            if constexpr (!MAXP) xt::put_t(T, &S.tmax[warp], lane);
         }
         xt::st_wait();
         tc::fence_before();

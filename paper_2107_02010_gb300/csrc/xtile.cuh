@@ -116,15 +116,23 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t db, uint
 // The tensor cores cut the running sum off towards zero after every step, so each step leaves a bias of half a unit
 // in the last place against the sign of what the accumulator holds.  For a pair that matters the cross term is
 // about T = s |x - c|^2 and H + R about -T: the K step with the folded slots goes in the middle, so that the sum
-// passes through about T / 2 and -T / 2 instead of T, and `parity` moves it by one step where the number of steps
-// is even, so that the biases of even and odd tiles have opposite signs.
+// passes through about T / 2 and -T / 2 instead of T, and `parity` 0 / 1 moves it by one step where the number of steps
+// is even, so that the biases of even and odd tiles have opposite signs.  Where T is small beside the exponents (row
+// blocks much smaller than the blur: single-scale solves, above all at the first scales of the schedule) the partial cross
+// terms are what is small: with the folded step last (kFoldLast) a single step is cut off at the size of the exponent.  In
+// the middle the same loss in every step stayed in the slowly contracting modes of f and g (single-scale solve, 60-D,
+// reach 20: f off by 2.5e-7, CUDA cores 1.3e-7; now 1.4e-7; 48-D 1.7e-7, 1.3e-7, now 1.1e-7).  Cluster tiles stay with the
+// middle: T is that of a whole cluster there, and the bundle means of a step are nearer to FP64 with it (2.8e-6 against
+// 4.3e-6 last and 4.5e-6 on the CUDA cores at sigma 4).
+constexpr int kFoldLast = 2;
+constexpr float kFoldT = 4.f;
 template <int NP, int K, int PAR> __device__ __forceinline__ void issue_as(uint32_t d, uint32_t a, uint32_t b) {
     constexpr uint32_t idesc = tc::idesc_bf16(kRows, kCols);
     constexpr int kP = NP == 3 ? 6 : 3, kS = K / 16;
     // (row piece, column piece), smallest products first
     constexpr int rp[6] = {NP == 3 ? 2 : 1, 0, NP == 3 ? 1 : 0, 1, 0, 0};
     constexpr int cp[6] = {0, NP == 3 ? 2 : 1, NP == 3 ? 1 : 0, 0, 1, 0};
-    constexpr int fold = (kS - 1 + PAR) / 2;  // place of the folded step
+    constexpr int fold = PAR == kFoldLast ? kS - 1 : (kS - 1 + PAR) / 2;  // place of the folded step
     uint32_t acc = 0u;
 #pragma unroll
     for (int q = 0; q < kP; ++q)
@@ -137,16 +145,19 @@ template <int NP, int K, int PAR> __device__ __forceinline__ void issue_as(uint3
         }
 }
 template <int NP, int K> __device__ __forceinline__ void issue(uint32_t d, uint32_t a, uint32_t b, int parity) {
-    if (parity) issue_as<NP, K, 1>(d, a, b);
+    if (parity == kFoldLast) issue_as<NP, K, kFoldLast>(d, a, b);
+    else if (parity) issue_as<NP, K, 1>(d, a, b);
     else issue_as<NP, K, 0>(d, a, b);
 }
 
 // The row operand of this thread's row for centre c: s (x - c) in NP pieces, the folded slots, R = -s |x - c|^2 / 2
-// - (M + Mlo).  `a`: tensor-memory column of the row pieces, with the warp's lane quadrant.  Warp-collective.
+// - (M + Mlo).  `a`: tensor-memory column of the row pieces, with the warp's lane quadrant.  Returns T = s |x - c|^2 (0 when
+// not valid).  Warp-collective.
 template <int NP, int K>
-__device__ __forceinline__ void stage_row(const float (&x)[K - 4], int D4, const float *c, float s, float M, bool valid,
+__device__ __forceinline__ float stage_row(const float (&x)[K - 4], int D4, const float *c, float s, float M, bool valid,
                                           uint32_t a, float Mlo = 0.f) {
     const float4 *c4 = reinterpret_cast<const float4 *>(c);
+    float T = 0.f;
     float4 sq = make_float4(0.f, 0.f, 0.f, 0.f);  // four short chains: less rounding than one long one
 #pragma unroll
     for (int kk = 0; kk < K / 16; ++kk) {
@@ -190,6 +201,7 @@ __device__ __forceinline__ void stage_row(const float (&x)[K - 4], int D4, const
             // R = P - M with what the product and the difference lose to rounding (where the finish adds M back its
             // own rounding cancels and Mlo is 0)
             const float hq = 0.5f * ((sq.x + sq.y) + (sq.z + sq.w)), P = -s * hq;
+            if (valid) T = -2.f * P;
             const float R = P - M, bb = P - R;  // two-difference (Knuth)
             const float rest = (fmaf(-s, hq, -P) + ((P - (R + bb)) + (bb - M))) - Mlo;
             uint16_t r1, r2, r3;
@@ -208,6 +220,16 @@ __device__ __forceinline__ void stage_row(const float (&x)[K - 4], int D4, const
 #pragma unroll
         for (int q = 0; q < NP; ++q) st8(a + (uint32_t)(q * (K / 2) + kk * 8), w[q]);
     }
+    return T;
+}
+
+// The largest T of a block from its four row warps: each warp's maximum (T is never negative: its bits order as it does).
+__device__ __forceinline__ void put_t(float T, float *slot, int lane) {
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(T));
+    if (lane == 0) *slot = __uint_as_float(m);
+}
+__device__ __forceinline__ bool fold_last(const volatile float *t) {
+    return fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3])) < kFoldT;
 }
 
 // Column c of a tile: the point y centred at `cen` in NP pieces into `dst` (and `dst2` when non-null); the folded
