@@ -75,13 +75,13 @@ __device__ __forceinline__ float lo_val(uint32_t w) { return __uint_as_float(w <
 
 // the NP pieces of two consecutive slots (k in the low half); rest0, rest1: what the values lost to their own rounding
 // (they reach the third piece)
-template <int NP>
+template <int NP, bool REST = false>
 __device__ __forceinline__ void split2(float v0, float v1, uint32_t (&p)[NP], float rest0 = 0.f, float rest1 = 0.f) {
     p[0] = bf2(v1, v0);
     float r0 = v0 - lo_val(p[0]), r1 = v1 - hi_val(p[0]);
 #pragma unroll
     for (int q = 1; q < NP; ++q) {
-        if (q == 2) {
+        if (REST && q == 2) {
             r0 += rest0;
             r1 += rest1;
         }
@@ -191,7 +191,7 @@ __device__ __forceinline__ float stage_row(const float (&x)[K - 4], int D4, cons
             // otgb_softmin in 4 dimensions 0.95 -> 0.72 of the CUDA cores'); among more coordinates it averages (no difference
             // from 24 on).
             if constexpr (K == 16)
-                split2<NP>(v[2 * j], v[2 * j + 1], p, fmaf(s, d1[2 * j], -v[2 * j]), fmaf(s, d1[2 * j + 1], -v[2 * j + 1]));
+                split2<NP, true>(v[2 * j], v[2 * j + 1], p, fmaf(s, d1[2 * j], -v[2 * j]), fmaf(s, d1[2 * j + 1], -v[2 * j + 1]));
             else
                 split2<NP>(v[2 * j], v[2 * j + 1], p);
 #pragma unroll
