@@ -48,12 +48,12 @@ namespace otgb {
 
 void *Workspace::get(const std::string &name, size_t bytes) {
     Buf *b = nullptr;
-    size_t others = 0;
-    for (auto &u : bufs) {
-        if (u.name == name) b = &u;
-        else others += u.bytes;
-    }
-    if (b && b->bytes >= bytes) return b->ptr;
+    for (auto &u : bufs)
+        if (u.name == name) {
+            if (u.bytes >= bytes) return u.ptr;
+            b = &u;
+            break;
+        }
     if (!b) {
         bufs.emplace_back();
         b = &bufs.back();
@@ -62,7 +62,9 @@ void *Workspace::get(const std::string &name, size_t bytes) {
     if (b->ptr) OTGB_CUDA_TRY(cudaFreeAsync(b->ptr, stream));  // null: new, or after a growth that failed
     b->ptr = nullptr;
     b->bytes = 0;
-    if ((limit && others + bytes > limit) || cudaMallocAsync(&b->ptr, bytes, stream) != cudaSuccess) {
+    size_t total = bytes;
+    for (auto &u : bufs) total += u.bytes;
+    if ((limit && total > limit) || cudaMallocAsync(&b->ptr, bytes, stream) != cudaSuccess) {
         b->ptr = nullptr;
         cudaGetLastError();  // the next launch check must not see it
         throw Error{OTGB_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes failed"};
