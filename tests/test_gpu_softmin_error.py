@@ -45,6 +45,15 @@ def test_dense_sweep_in_up_to_three_dimensions(D, n, m, side, eps):
     assert tc <= cuda, (tc, cuda)
 
 
+@pytest.mark.parametrize("D", [1, 2, 3])
+@pytest.mark.parametrize("side,eps", [(30.0, 1.0), (1.0, 0.0025)])
+def test_sorted_sweep(D, side, eps):
+    """Thousands of columns in a row's sum, most of them small beside it."""
+    e = [errors(46_001, 47_003, D, side, eps, seed, uniform) for seed in range(2)]
+    tc, cuda = (sum(v[k] ** 2 for v in e) ** 0.5 for k in (0, 1))
+    assert tc <= cuda, (tc, cuda)
+
+
 def fibers(n, D, side, g):
     x = synth.fiber_bundles(n, seed=int(torch.randint(0, 1 << 30, (1,), generator=g, device="cuda")), perturb=3.0)[0]
     return torch.from_numpy(np.ascontiguousarray(x[:, :D])).cuda()
