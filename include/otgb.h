@@ -279,8 +279,10 @@ int cluster_kmeans(otgb_ctx *ctx, const float *x, const float *w, int N, int D, 
  * (y, beta, M, x, alpha, N, ..., f := g, g := f, a_self := b_self).
  *   x: N x D, alpha: N, y: M x D, beta: M, f: N, g: M, a_self: N (device);
  *   grad: N x D device output (float32).
- * Dense: every pair is summed (the direct difference form of the cost, FP32,
- * with a running maximum per row), for any 1 <= D <= 64.
+ * The direct difference form of the cost in FP32 with a running maximum per
+ * row, for any 1 <= D <= 64: every pair is summed; with D <= 3 and p = 2 (from
+ * a few thousand points on) every pair whose term reaches 2^-60 of its row's
+ * largest one.
  * Errors: EINVAL for null pointers, sizes < 1, D outside [1, 64], p not in {1, 2}, eps <= 0.
  */
 int sinkhorn_grad_x(otgb_ctx *ctx, const float *x, const float *alpha, int N, const float *y, const float *beta,

@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kGR) grad_sparse_kernel(const __grid_constant_
 }
 
 void grad_sparse_run(const Solver &s, double eps, const GradRequest &gr, cudaStream_t st) {
-    if (s.use_tc3) {  // the solve's points are in spatial order: every pair that can matter, on the tensor cores
+    if (s.use_tc3) {  // the solve's points are in spatial order: every pair that can matter, tile by tile
         const float4 *X = reinterpret_cast<const float4 *>(s.X.pts), *Y = reinterpret_cast<const float4 *>(s.Y.pts);
         const Grad3Part part[2] = {{Y, s.pg[s.cur], s.Y.n, 1.f, s.pf[s.cur]}, {X, s.pa[s.cur], s.X.n, -1.f, s.pa[s.cur]}};
         try {
@@ -359,8 +359,9 @@ extern "C" int sinkhorn_grad_x(otgb_ctx *ctx, const float *x, const float *alpha
         require(p == 1 || p == 2, "sinkhorn_grad_x: p must be 1 or 2");
         require(eps > 0.0 && std::isfinite(eps), "sinkhorn_grad_x: eps must be > 0");
         cudaStream_t st = ctx_stream(ctx);
-        // p = 2 in up to three dimensions: sorted, on the tensor cores (sorted3.cu); in small calls the sorts cost more
-        // than the pairs (sorted against every pair: 1,000 + 1,000 points 0.28 / 0.19 ms, 2,000 + 2,000 0.29 / 0.35)
+        // p = 2 in up to three dimensions: over sorted points (sorted3.cu).  The sorts and their launches are 0.17 ms, what
+        // grad_kernel takes for 1,000 + 1,000 points; at the line, sorted against every pair: 2,000 + 2,000 points 0.17 / 0.35
+        // ms, 500 + 20,000 0.19 / 1.67, at any blur between 0.2 and 4.5 on points spread over 30 units.
         if (D <= 3 && p == 2 && (double)N * ((double)N + M) >= 8e6) {
             try {
                 grad3_apply(ctx, x, alpha, N, y, beta, M, D, eps, f, g, a_self, grad);
