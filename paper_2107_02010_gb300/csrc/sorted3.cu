@@ -621,7 +621,9 @@ __global__ void grad3_finish_kernel(const __grid_constant__ GradFinish F) {
             v[1] = fmaf(f, u.z, v[1]);
             v[2] = fmaf(f, u.w, v[2]);
         }
-        const float em = F.sign[q] * exp2f((float)((double)m + (double)F.s * (double)F.row_pot[q][r]));
+        const float rp = F.row_pot[q][r];
+        if (rp != rp) continue;  // as in grad_kernel: no exponent, no term; at +inf no shift makes the terms finite
+        const float em = rp == INFINITY ? NAN : F.sign[q] * exp2f((float)((double)m + (double)F.s * (double)rp));
         for (int d = 0; d < 3; ++d) out[d] = fmaf(em, v[d], out[d]);
     }
     const size_t i = F.perm ? F.perm[r] : r;
