@@ -45,3 +45,19 @@ def test_gradient(n, m, kind, eps):
          for u, v in ((x, y), tuple(torch.nn.functional.pad(w, (0, 1)).contiguous() for w in (x, y)))]  # 4-D: every pair
     ctx.close()
     assert t[0] <= 1.3 * t[1], t
+
+
+@pytest.mark.parametrize("n,kind,eps,wild", [(46_000, "cloud", 0.01, True), (100_000, "line", 0.01, False), (46_000, "line", 0.01, True),
+                                             (46_000, "outlier", 1.0, False), (46_000, "outlier", 0.05, False)])
+def test_softmin(n, kind, eps, wild):
+    from paper_2107_02010_gb300 import otgb
+
+    g = torch.Generator(device="cuda").manual_seed(2)
+    q, p = points(n, kind, g), points(n, kind, g)
+    w, pot = torch.full((n,), 1.0 / n, device="cuda"), torch.zeros(n, device="cuda")
+    if wild:  # potentials that reach far beyond the neighbours
+        pot = 200.0 * eps * torch.randn(n, generator=g, device="cuda")
+    ctx = otgb.Context()
+    t = best(lambda: otgb.softmin(ctx, q, p, w, pot, eps)), best(lambda: otgb.softmin_noalloc(q, p, w, pot, eps))
+    ctx.close()
+    assert t[0] <= 1.3 * t[1], t
