@@ -36,12 +36,28 @@ struct TransportArgs {
     int4 *fallback;
     int *n_fallback;
     const int *out_perm;   // safe kernel: row -> place in scores / argmax / mass (null: the row itself)
+    // near ties of the tensor-core path (transport_gen_kernel): the classes of each block that are summed (cls_words words per
+    // block; null: all), the rows whose argmax is written, at out_perm[row]
+    const unsigned *cls_bits;
+    const unsigned char *tied;
+    int cls_words;
 };
 
 __device__ __forceinline__ float ex2f_(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+__device__ __forceinline__ unsigned long long pack2_(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2_(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
 }
 
 __global__ void __launch_bounds__(kTT) transport_kernel(const __grid_constant__ TransportArgs A) {
@@ -167,6 +183,12 @@ __global__ void __launch_bounds__(kTG) transport_gen_kernel(const __grid_constan
     const int t = threadIdx.x, b = blockIdx.x;
     const int r0 = blk_row0[b], nr = min(blk_row0[b + 1] - r0, kTBM);
     const float s = A.s;
+    const unsigned *cls = A.cls_bits ? A.cls_bits + (size_t)b * A.cls_words : nullptr;
+    if (cls) {
+        unsigned any = 0u;
+        for (int w = 0; w < A.cls_words; ++w) any |= cls[w];
+        if (!any) return;  // no near tie among the block's rows (uniform)
+    }
     for (int e = t; e < kTBM * D4; e += kTG) {
         const int r = e / D4, k = e - r * D4;
         S.xs[k][r] = (r < nr) ? A.rows[(size_t)(r0 + r) * D4 + k] : 0.f;
@@ -204,6 +226,7 @@ __global__ void __launch_bounds__(kTG) transport_gen_kernel(const __grid_constan
     for (int i = 0; i < 8; ++i) mreg[i] = S.mrow[tr * 8 + i];
     const int D44 = D4 >> 2;
     for (int l = 0; l < A.L; ++l) {
+        if (cls && !(cls[l >> 5] >> (l & 31) & 1u)) continue;  // uniform
         const int lb = lab_off[l], le = lab_off[l + 1];
         float rs[8];
 #pragma unroll
@@ -225,32 +248,44 @@ __global__ void __launch_bounds__(kTG) transport_gen_kernel(const __grid_constan
             if (t < kTBN) {
                 const int j = p0 + t;
                 float acc = 0.f;
+#pragma unroll 20
                 for (int k = 0; k < D4; ++k) acc = fmaf(S.ys[k][t], S.ys[k][t], acc);
                 S.hs[t] = j < le ? s * (fmaf(A.eps, A.col_logw[j], A.g[j]) - 0.5f * acc) : -INFINITY;
             }
             __syncthreads();
-            float acc[8][4];
+            // rows in pairs through packed FMAs (each half is the scalar chain over the coordinates: the same result)
+            unsigned long long acc[4][4];
             const float4 h4 = *reinterpret_cast<const float4 *>(&S.hs[tc * 4]);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                acc[i][0] = h4.x - mreg[i]; acc[i][1] = h4.y - mreg[i];
-                acc[i][2] = h4.z - mreg[i]; acc[i][3] = h4.w - mreg[i];
+            for (int i = 0; i < 4; ++i) {
+                acc[i][0] = pack2_(h4.x - mreg[2 * i], h4.x - mreg[2 * i + 1]);
+                acc[i][1] = pack2_(h4.y - mreg[2 * i], h4.y - mreg[2 * i + 1]);
+                acc[i][2] = pack2_(h4.z - mreg[2 * i], h4.z - mreg[2 * i + 1]);
+                acc[i][3] = pack2_(h4.w - mreg[2 * i], h4.w - mreg[2 * i + 1]);
             }
 #pragma unroll 4
             for (int k = 0; k < D4; ++k) {
-                const float4 xa = *reinterpret_cast<const float4 *>(&S.xs[k][tr * 8]);
-                const float4 xb = *reinterpret_cast<const float4 *>(&S.xs[k][tr * 8 + 4]);
+                const ulonglong2 xa = *reinterpret_cast<const ulonglong2 *>(&S.xs[k][tr * 8]);
+                const ulonglong2 xb = *reinterpret_cast<const ulonglong2 *>(&S.xs[k][tr * 8 + 4]);
                 const float4 yv = *reinterpret_cast<const float4 *>(&S.ys[k][tc * 4]);
-                const float xv[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
-                const float yy[4] = {yv.x, yv.y, yv.z, yv.w};
+                const unsigned long long xv[4] = {xa.x, xa.y, xb.x, xb.y};
+                const unsigned long long yy[4] = {pack2_(yv.x, yv.x), pack2_(yv.y, yv.y), pack2_(yv.z, yv.z), pack2_(yv.w, yv.w)};
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
+                for (int i = 0; i < 4; ++i)
 #pragma unroll
-                    for (int jj = 0; jj < 4; ++jj) acc[i][jj] = fmaf(xv[i], yy[jj], acc[i][jj]);
+                    for (int jj = 0; jj < 4; ++jj) acc[i][jj] = fma2_(xv[i], yy[jj], acc[i][jj]);
             }
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                rs[i] += (ex2f_(acc[i][0]) + ex2f_(acc[i][1])) + (ex2f_(acc[i][2]) + ex2f_(acc[i][3]));
+            for (int i = 0; i < 4; ++i) {
+                float lo[4], hi[4];
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) {
+                    lo[jj] = __uint_as_float((unsigned)acc[i][jj]);
+                    hi[jj] = __uint_as_float((unsigned)(acc[i][jj] >> 32));
+                }
+                rs[2 * i] += (ex2f_(lo[0]) + ex2f_(lo[1])) + (ex2f_(lo[2]) + ex2f_(lo[3]));
+                rs[2 * i + 1] += (ex2f_(hi[0]) + ex2f_(hi[1])) + (ex2f_(hi[2]) + ex2f_(hi[3]));
+            }
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -270,6 +305,10 @@ __global__ void __launch_bounds__(kTG) transport_gen_kernel(const __grid_constan
     __syncthreads();
     if (t < nr) {
         const int r = r0 + t;
+        if (cls) {
+            if (A.tied[r]) A.argmax[A.out_perm[r]] = S.bestl[t];
+            return;
+        }
         const float tot = S.tot[t];
         if (!(tot >= 0x1p-60f && tot <= 0x1p60f) && A.m > 0) {
             const int k = atomicAdd(A.n_fallback, 1);
@@ -357,6 +396,30 @@ __global__ void unpermute_rows_kernel(const float *sc, const int *am, const floa
 }
 
 }  // namespace
+
+namespace {
+void transport_gen_launch(const TransportArgs &A, const int *d_blk, int nblk, const int *lab_off, cudaStream_t st) {
+    static PerDevice<int> attr;
+    attr.get([] {
+        OTGB_CUDA_TRY(cudaFuncSetAttribute(transport_gen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)sizeof(TransportGenSmem)));
+        return 1;
+    });
+    transport_gen_kernel<<<nblk, kTG, sizeof(TransportGenSmem), st>>>(A, d_blk, lab_off, A.stride);
+    OTGB_CHECK_LAUNCH();
+}
+}  // namespace
+
+void transport_gen_ties(const TieBlocks &T, cudaStream_t st) {
+    TransportArgs A;
+    std::memset(&A, 0, sizeof(A));
+    A.rows = T.rows; A.f = T.f; A.cols = T.cols; A.col_logw = T.col_logw; A.g = T.g;
+    A.n = T.n; A.m = T.m; A.D = T.D; A.stride = (T.D + 3) & ~3; A.L = T.L;
+    A.eps = T.eps; A.s = T.s;
+    A.argmax = T.argmax; A.out_perm = T.perm;
+    A.cls_bits = T.cls_bits; A.tied = T.tied; A.cls_words = (T.L + 31) / 32;
+    transport_gen_launch(A, T.blk_row0, T.nblk, T.lab_off, st);
+}
 
 void label_order(otgb_ctx *ctx, const int *labels, int M, int L, uint32_t *keys, int *perm, int *lab_off) {
     cudaStream_t st = ctx_stream(ctx);
@@ -481,14 +544,7 @@ static int transport_once(otgb_ctx *ctx, const otgb_plan *plan, const float *f, 
             pack_points(plan->x, nullptr, kr.perm, N, D, d_cen, Rw, nullptr, nullptr, st);
             permute(f, kr.perm, N, fs, st);
             A.rows = Rw; A.f = fs;
-            static PerDevice<int> attr;
-            attr.get([] {
-                OTGB_CUDA_TRY(cudaFuncSetAttribute(transport_gen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)sizeof(TransportGenSmem)));
-                return 1;
-            });
-            transport_gen_kernel<<<(int)hb.size() - 1, kTG, sizeof(TransportGenSmem), st>>>(A, d_blk, lab_off, stride);
-            OTGB_CHECK_LAUNCH();
+            transport_gen_launch(A, d_blk, (int)hb.size() - 1, lab_off, st);
             OTGB_CUDA_TRY(cudaStreamSynchronize(st));  // hb, off released
         }
         transport_fallback_kernel<<<64, 256, 0, st>>>(A);

@@ -25,6 +25,18 @@ struct TransportFallback {
 };
 // Columns by label (stable; labels outside [0, L) last): sorted keys, order, first position of each class (L + 1).
 void label_order(otgb_ctx *ctx, const int *labels, int M, int L, uint32_t *keys, int *perm, int *lab_off);
+// Near ties in numbers: transport_gen_kernel over the blocks that hold one, the classes marked in cls_bits (per block), writing
+// the argmax of the rows marked in tied.  rows, f: in the order perm of that kernel; cols, col_logw, g: sorted by label.
+struct TieBlocks {
+    const float *rows, *f, *cols, *col_logw, *g;
+    const int *blk_row0, *lab_off, *perm;
+    int nblk, n, m, D, L;
+    float eps, s;
+    const unsigned *cls_bits;
+    const unsigned char *tied;
+    int *argmax;
+};
+void transport_gen_ties(const TieBlocks &T, cudaStream_t st);
 // 3 < D, D4 <= 60.
 TransportFallback transport_xt_apply(otgb_ctx *ctx, const TransportCall &c);
 

@@ -17,7 +17,10 @@
 // Near ties.  A row's label is a whole number and must not depend on which kernel summed its classes, so a row whose two
 // best scores lie within kTie of each other is decided by the arithmetic of the CUDA-core kernel (transport_gen_kernel):
 // the centre of the row's block in that kernel's k-means order, its FMA chains and its order of sums.  That costs the
-// block order (a k-means over all rows) when there is such a row, and nothing otherwise.
+// block order (a k-means over all rows) when there is such a row, and nothing otherwise.  Up to kFewTies rows take a CTA each;
+// more of them (an atlas with two labels on the same fibers ties every row) that kernel itself, over the blocks and classes
+// concerned: 60k x 50k fibers, two such labels, 262 ms with a CTA per row, 20.5 now (transport_gen_kernel alone 24.2, 20 now
+// that its FMAs are packed); a small atlas of ties pays for the sweep that decided nothing (5,000 x 5,000: 1.3 ms, 1.0).
 //
 // Measured (60k x 50k fibers, 60-D, 20 labels that split every bundle; whole call): 24.5 -> 3.2 ms, of which the sweep
 // 0.65 (13 % of the pairs visited; dense at the tensor bound: 1.2), the two k-means and their sorts 0.8, about 20 near
@@ -38,6 +41,7 @@ constexpr int kThreads = 192;
 constexpr int kN = xt::kCols;
 constexpr float kSkip = -130.f;  // base-2 exponents below this are 0 in float32 (2^-126 is the smallest normal number)
 
+constexpr int kFewTies = 256;       // rows that a CTA each decides
 constexpr float kTie = 2e-5f;       // four times the scores' error (measured: at most 5e-6 against the CUDA-core kernel)
 
 struct XferArgs {
@@ -473,6 +477,22 @@ __global__ void __launch_bounds__(256) xfer_tie_kernel(const __grid_constant__ T
     }
 }
 
+// The candidates of the listed rows (the classes within kTie of the best one) into their blocks' class bits, and the rows' marks.
+// label: cluster of a row in the caller's order; blk0: first block of a cluster.
+__global__ void xfer_mark_kernel(const int2 *ties, int n, const float *score, size_t ld, int L, const int *label, const int *off,
+                                 const int *inv, const int *blk0, int words, unsigned *bits, unsigned char *tied) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const int i = ties[k].x, c = label[i], r = inv[i];
+    const float *sc = score + ties[k].y;
+    unsigned *b = bits + (size_t)(blk0[c] + (r - off[c]) / 128) * words;
+    float best = 0.f;
+    for (int l = 0; l < L; ++l) best = fmaxf(best, sc[(size_t)l * ld]);
+    for (int l = 0; l < L; ++l)
+        if (best - sc[(size_t)l * ld] <= kTie * best && !(b[l >> 5] >> (l & 31) & 1u)) atomicOr(b + (l >> 5), 1u << (l & 31));
+    tied[r] = 1;
+}
+
 // sort keys of the columns: cluster, then label (L: ignored)
 __global__ void xfer_keys_kernel(const int *cl, const int *labels, int m, int L, uint32_t *keys) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -615,7 +635,8 @@ TransportFallback transport_xt_apply(otgb_ctx *ctx, const TransportCall &c) {
     if (n_ties <= 0) return out;
 
     // the orders of the CUDA-core kernel: columns by label, rows by a k-means of N / 64 clusters
-    KmeansResult kt = kmeans(ctx, "ta:kt", c.x, nullptr, N, D, std::max(1, std::min(N / 64, 4096)), 4, 12345, nullptr);
+    const int Kt = std::max(1, std::min(N / 64, 4096));
+    KmeansResult kt = kmeans(ctx, "ta:kt", c.x, nullptr, N, D, Kt, 4, 12345, nullptr);
     uint32_t *k2 = ws.get<uint32_t>("ta:keys2", M);
     int *perm2 = ws.get<int>("ta:cperm2", M), *lab_off = ws.get<int>("ta:laboff", L + 1), *inv = ws.get<int>("ta:inv", N);
     float *C2 = ws.get<float>("ta:C2", (size_t)M * D4), *lw2 = ws.get<float>("ta:Clw2", M), *g2 = ws.get<float>("ta:g2", M);
@@ -623,12 +644,40 @@ TransportFallback transport_xt_apply(otgb_ctx *ctx, const TransportCall &c) {
     label_order(ctx, c.labels, M, L, k2, perm2, lab_off);
     pack_points(c.y, c.b, perm2, M, D, c.d_cen, C2, lw2, nullptr, st);
     permute(c.g, perm2, M, g2, st);
-    pack_points(c.x, nullptr, nullptr, N, D, c.d_cen, R2, nullptr, nullptr, st);
     inverse_kernel<<<(N + 255) / 256, 256, 0, st>>>(kt.perm, N, inv);
     OTGB_CHECK_LAUNCH();
-    const TieArgs T{ties, A.score, A.ld, R2, c.f, kt.labels, kt.perm, inv, kt.offsets, C2, lw2, g2, lab_off, D4, L, eps, s, c.argmax};
-    xfer_tie_kernel<<<n_ties, 256, 0, st>>>(T);
+    if (n_ties <= kFewTies) {  // a CTA per row
+        pack_points(c.x, nullptr, nullptr, N, D, c.d_cen, R2, nullptr, nullptr, st);
+        const TieArgs T{ties, A.score, A.ld, R2, c.f, kt.labels, kt.perm, inv, kt.offsets, C2, lw2, g2, lab_off, D4, L, eps, s, c.argmax};
+        xfer_tie_kernel<<<n_ties, 256, 0, st>>>(T);
+        OTGB_CHECK_LAUNCH();
+        return out;
+    }
+    // the kernel itself, over the blocks and classes that are concerned
+    std::vector<int> off(Kt + 1), b0(Kt), rows;
+    OTGB_CUDA_TRY(cudaMemcpyAsync(off.data(), kt.offsets, sizeof(int) * (Kt + 1), cudaMemcpyDeviceToHost, st));
+    pack_points(c.x, nullptr, kt.perm, N, D, c.d_cen, R2, nullptr, nullptr, st);
+    float *f2 = ws.get<float>("ta:f2", N);
+    permute(c.f, kt.perm, N, f2, st);
+    OTGB_CUDA_TRY(cudaStreamSynchronize(st));
+    for (int q = 0; q < Kt; ++q) {
+        b0[q] = (int)rows.size();
+        for (int r = off[q]; r < off[q + 1]; r += 128) rows.push_back(r);
+    }
+    const int nb = (int)rows.size(), words = (L + 31) / 32;
+    rows.push_back(N);
+    rows.insert(rows.end(), b0.begin(), b0.end());
+    int *d_rows = ws.get<int>("ta:blk2", rows.size());
+    unsigned *bits2 = ws.get<unsigned>("ta:cls", (size_t)nb * words);
+    unsigned char *tied = ws.get<unsigned char>("ta:tied", N);
+    OTGB_CUDA_TRY(cudaMemcpyAsync(d_rows, rows.data(), sizeof(int) * rows.size(), cudaMemcpyHostToDevice, st));
+    OTGB_CUDA_TRY(cudaMemsetAsync(bits2, 0, sizeof(unsigned) * nb * words, st));
+    OTGB_CUDA_TRY(cudaMemsetAsync(tied, 0, N, st));
+    xfer_mark_kernel<<<(n_ties + 255) / 256, 256, 0, st>>>(ties, n_ties, A.score, A.ld, L, kt.labels, kt.offsets, inv,
+                                                          d_rows + nb + 1, words, bits2, tied);
     OTGB_CHECK_LAUNCH();
+    transport_gen_ties(TieBlocks{R2, f2, C2, lw2, g2, d_rows, lab_off, kt.perm, nb, N, M, D, L, eps, s, bits2, tied, c.argmax}, st);
+    OTGB_CUDA_TRY(cudaStreamSynchronize(st));  // the host vector goes out of scope
     return out;
 }
 

@@ -1,0 +1,56 @@
+"""Near ties of label transfer: a row's label does not depend on which kernel summed its classes, for few near ties and for an
+atlas that ties every row (two labels on the same fibers), and such an atlas is not slow.  The same points with four more
+coordinates 0 take the CUDA-core kernel, whose sums decide the ties."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2107_02010_gb300 import synth
+from test_gpu_not_slower import best
+
+pytestmark = pytest.mark.gpu
+
+
+def T(v):
+    return torch.from_numpy(np.ascontiguousarray(v)).cuda()
+
+
+def problem(n, m, L, twins, seed=4, blur=2.0, scale=1.0, P=20):
+    """Calls of both widths, (60-D, 64-D): labels carried from an atlas in which every fiber has a twin with another label."""
+    from paper_2107_02010_gb300 import otgb
+
+    x = scale * synth.fiber_bundles(n, seed=seed, P=P, perturb=3.0)[0]
+    y, _, lab = synth.fiber_bundles(m // 2 if twins else m, seed=seed + 1, P=P)
+    y = scale * y
+    rng = np.random.default_rng(seed)
+    if twins:
+        half = max(1, L // 2)
+        y, lab = np.concatenate([y, y]), np.concatenate([lab % half, lab % half + half])
+    else:
+        lab = rng.integers(0, L, m)
+    m = len(y)
+    a, b = T(np.full(n, 1.0 / n, np.float32)), T(np.full(m, 1.0 / m, np.float32))
+    lab = T(lab.astype(np.int32))
+    ctx = otgb.Context()
+    p = otgb.default_params(blur=blur, reach=10.0 * blur, fixed_iters=20, multiscale=1, cluster=1, k_clusters=max(2, n // 1000))
+    calls = []
+    for pad in (0, 64 - 3 * P):
+        X, Y = (T(np.pad(v, ((0, 0), (0, pad)))) for v in (x.astype(np.float32), y.astype(np.float32)))
+        r = otgb.sinkhorn_divergence(ctx, X, a, Y, b, p, want_plan=True)
+        if not calls:
+            f, g = r["f"], r["g"]
+        calls.append(lambda r=r: otgb.transport_apply(ctx, r["plan"], f, g, lab, L, want_scores=False))
+    return calls
+
+
+@pytest.mark.parametrize("n,m,L,twins", [(3000, 2600, 2, True), (700, 900, 40, True), (257, 64, 3, True), (20_000, 9000, 7, False),
+                                         (1500, 4000, 2, False)])
+def test_labels_are_those_of_the_cuda_core_kernel(n, m, L, twins):
+    tc, cuda = (call()[1] for call in problem(n, m, L, twins))
+    assert torch.equal(tc, cuda), int((tc != cuda).sum())
+
+
+def test_an_atlas_of_ties_is_not_slow():
+    tc, cuda = problem(30_000, 20_000, 2, True)
+    t = best(tc), best(cuda)
+    assert t[0] <= 1.3 * t[1], t
