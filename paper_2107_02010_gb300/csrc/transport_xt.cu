@@ -42,7 +42,12 @@ constexpr int kN = xt::kCols;
 constexpr float kSkip = -130.f;  // base-2 exponents below this are 0 in float32 (2^-126 is the smallest normal number)
 
 constexpr int kFewTies = 256;       // rows that a CTA each decides
-constexpr float kTie = 2e-5f;       // four times the scores' error (measured: at most 5e-6 against the CUDA-core kernel)
+// Two scores within this of each other (relative) are a near tie: four times the scores' error at eps 4 (at most 5e-6 against
+// the CUDA-core kernel), and where the exponents are larger what they are rounded at there.  That kernel rounds s u_j (u_j =
+// eps log b_j + g_j), its sum with -s |y - c|^2 / 2 and the product once each and sums the cross term over the coordinates: an
+// exponent is off by up to about 3 2^-24 s |u| + 8 2^-24 s r^2 (r: the row cluster's radius), a score by ln 2 of that, the
+// difference of two by twice as much: 2.5e-7 s |u| + 6.6e-7 s r^2.  A column that matters has u between -|f| and the largest u.
+constexpr float kTie = 2e-5f, kTieRel = 5e-7f;
 
 struct XferArgs {
     const float *rows;  // packed rows, grouped by cluster
@@ -95,7 +100,8 @@ template <int K> __global__ void __launch_bounds__(kN) xfer_tiles_kernel(const _
 
 // Largest f (rows) or eps log w + g (columns) of each cluster, one warp per cluster; NaN counts as +inf, so that the
 // cluster is visited.
-__global__ void xfer_max_kernel(const int *off, int ncl, const float *v, const float *lw, float eps, float *out) {
+// top (optional; zero it first): the largest positive finite value over all of them, as its bits.
+__global__ void xfer_max_kernel(const int *off, int ncl, const float *v, const float *lw, float eps, float *out, unsigned *top) {
     const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (c >= ncl) return;
     float m = -INFINITY;
@@ -104,7 +110,10 @@ __global__ void xfer_max_kernel(const int *off, int ncl, const float *v, const f
         m = u == u ? fmaxf(m, u) : INFINITY;
     }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) out[c] = m;
+    if (lane == 0) {
+        out[c] = m;
+        if (top && m > 0.f && m < INFINITY) atomicMax(top, __float_as_uint(m));
+    }
 }
 
 // Keep bits of row cluster blockIdx.x.  !(bound < kSkip) keeps a pair whose bound is NaN.
@@ -340,10 +349,17 @@ template <int K> __global__ void __launch_bounds__(kThreads, 2) xfer_kernel(cons
     if (warp == 5) tc::tmem_dealloc(tmem, xt::kTmemCols);
 }
 
+// A row whose label is decided again: its place in the caller's order, its row of `score`, the tolerance of its scores.
+struct Tie {
+    int i, r;
+    float tol;
+};
+
 // Row sums, argmax (lowest class on ties) and scores in the caller's order; rows outside the safe range are listed.
-__global__ void xfer_finish_kernel(const float *score, size_t ld, int n, int m, int L, const int *perm, float *sc_out,
-                                   int *am_out, float *ms_out, int4 *fallback, int *n_fallback, int2 *ties,
-                                   int *n_ties) {
+// f, cl: potential and cluster of a row; rad: radius of a cluster; umax: bits of the largest u.
+__global__ void xfer_finish_kernel(const float *score, size_t ld, int n, int L, const int *perm, const float *f, const uint32_t *cl,
+                                   const float *rad, const unsigned *umax, float s, float *sc_out, int *am_out, float *ms_out,
+                                   int4 *fallback, int *n_fallback, Tie *ties, int *n_ties) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const int i = perm[r];
@@ -367,7 +383,8 @@ __global__ void xfer_finish_kernel(const float *score, size_t ld, int n, int m, 
     }
     am_out[i] = bestl;
     if (ms_out) ms_out[i] = tot;
-    if (second > 0.f && best - second <= kTie * best) ties[atomicAdd(n_ties, 1)] = make_int2(i, r);
+    const float rc = rad[cl[r]], tol = fmaxf(kTie, kTieRel * s * (2.f * fabsf(f[r]) + __uint_as_float(*umax) + rc * rc));
+    if (second > 0.f && best - second <= tol * best) ties[atomicAdd(n_ties, 1)] = Tie{i, r, tol};
 }
 
 __global__ void inverse_kernel(const int *perm, int n, int *inv) {
@@ -375,11 +392,11 @@ __global__ void inverse_kernel(const int *perm, int n, int *inv) {
     if (k < n) inv[perm[k]] = k;
 }
 
-// One CTA per listed row: the sums of the classes within kTie of the best one, as transport_gen_kernel forms them, then
+// One CTA per listed row: the sums of the classes within the tolerance of the best one, as transport_gen_kernel forms them, then
 // the argmax.  rows: packed in the caller's order (perm: the k-means order of that kernel); cols, logw, g: sorted by
 // label, lab_off their classes.
 struct TieArgs {
-    const int2 *ties;     // (row in the caller's order, row of `score`)
+    const Tie *ties;
     const float *score;
     size_t ld;
     const float *rows, *f;
@@ -394,14 +411,15 @@ __global__ void __launch_bounds__(256) xfer_tie_kernel(const __grid_constant__ T
     __shared__ float cen[64], X[64], scores[1024], term[256];
     __shared__ int cand[1024], n_cand;
     __shared__ float m_s;
-    const int t = threadIdx.x, D4 = A.D4, i = A.ties[blockIdx.x].x;
+    const Tie tie = A.ties[blockIdx.x];
+    const int t = threadIdx.x, D4 = A.D4, i = tie.i;
     if (t == 0) {  // the candidates in class order
-        const float *sc = A.score + A.ties[blockIdx.x].y;
+        const float *sc = A.score + tie.r;
         float best = 0.f;
         int n = 0;
         for (int l = 0; l < A.L; ++l) best = fmaxf(best, sc[(size_t)l * A.ld]);
         for (int l = 0; l < A.L; ++l)
-            if (best - sc[(size_t)l * A.ld] <= kTie * best) cand[n++] = l;
+            if (best - sc[(size_t)l * A.ld] <= tie.tol * best) cand[n++] = l;
         n_cand = n;
     }
     const float s = A.s;
@@ -477,19 +495,20 @@ __global__ void __launch_bounds__(256) xfer_tie_kernel(const __grid_constant__ T
     }
 }
 
-// The candidates of the listed rows (the classes within kTie of the best one) into their blocks' class bits, and the rows' marks.
+// The candidates of the listed rows (the classes within the tolerance of the best one) into their blocks' class bits, and the rows' marks.
 // label: cluster of a row in the caller's order; blk0: first block of a cluster.
-__global__ void xfer_mark_kernel(const int2 *ties, int n, const float *score, size_t ld, int L, const int *label, const int *off,
+__global__ void xfer_mark_kernel(const Tie *ties, int n, const float *score, size_t ld, int L, const int *label, const int *off,
                                  const int *inv, const int *blk0, int words, unsigned *bits, unsigned char *tied) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
-    const int i = ties[k].x, c = label[i], r = inv[i];
-    const float *sc = score + ties[k].y;
+    const Tie tie = ties[k];
+    const int i = tie.i, c = label[i], r = inv[i];
+    const float *sc = score + tie.r;
     unsigned *b = bits + (size_t)(blk0[c] + (r - off[c]) / 128) * words;
     float best = 0.f;
     for (int l = 0; l < L; ++l) best = fmaxf(best, sc[(size_t)l * ld]);
     for (int l = 0; l < L; ++l)
-        if (best - sc[(size_t)l * ld] <= kTie * best && !(b[l >> 5] >> (l & 31) & 1u)) atomicOr(b + (l >> 5), 1u << (l & 31));
+        if (best - sc[(size_t)l * ld] <= tie.tol * best && !(b[l >> 5] >> (l & 31) & 1u)) atomicOr(b + (l >> 5), 1u << (l & 31));
     tied[r] = 1;
 }
 
@@ -560,9 +579,12 @@ TransportFallback transport_xt_apply(otgb_ctx *ctx, const TransportCall &c) {
     cluster_stats(C, D4, D, Cw, km.offsets, K, cen, D4, mass, rad, nullptr, st);
     cluster_stats(R, D4, D, Rw, ro.offsets, Kr, rcen, D4, mass + K, rrad, nullptr, st);
     const float eps = (float)c.eps, s = (float)(1.4426950408889634 / c.eps);
-    xfer_max_kernel<<<(K + 7) / 8, 256, 0, st>>>(km.offsets, K, gs, Clw, eps, mx);
+    int *nfb = ws.get<int>("ta:nfb", 3);  // fallback rows, near ties, bits of the largest u
+    unsigned *umax = reinterpret_cast<unsigned *>(nfb + 2);
+    OTGB_CUDA_TRY(cudaMemsetAsync(nfb, 0, 3 * sizeof(int), st));
+    xfer_max_kernel<<<(K + 7) / 8, 256, 0, st>>>(km.offsets, K, gs, Clw, eps, mx, umax);
     OTGB_CHECK_LAUNCH();
-    xfer_max_kernel<<<(Kr + 7) / 8, 256, 0, st>>>(ro.offsets, Kr, fs, nullptr, eps, mx + K);
+    xfer_max_kernel<<<(Kr + 7) / 8, 256, 0, st>>>(ro.offsets, Kr, fs, nullptr, eps, mx + K, nullptr);
     OTGB_CHECK_LAUNCH();
     const int nwords = (K + 31) / 32;
     unsigned *kb = ws.get<unsigned>("ta:bits", (size_t)Kr * nwords);
@@ -618,12 +640,10 @@ TransportFallback transport_xt_apply(otgb_ctx *ctx, const TransportCall &c) {
         case 64: sweep<64>(A, nblk, st); break;
         default: throw Error{OTGB_EINTERNAL, "transport_apply: unsupported width"};
     }
-    int *nfb = ws.get<int>("ta:nfb", 2);  // fallback rows, near ties
     int4 *fb = ws.get<int4>("ta:fb", N);
-    int2 *ties = ws.get<int2>("ta:ties", N);
-    OTGB_CUDA_TRY(cudaMemsetAsync(nfb, 0, 2 * sizeof(int), st));
-    xfer_finish_kernel<<<(N + 127) / 128, 128, 0, st>>>(A.score, A.ld, N, M, L, ro.perm, c.scores, c.argmax, c.row_mass, fb,
-                                                        nfb, ties, nfb + 1);
+    Tie *ties = ws.get<Tie>("ta:ties", N);
+    xfer_finish_kernel<<<(N + 127) / 128, 128, 0, st>>>(A.score, A.ld, N, L, ro.perm, fs, ro.sorted_keys, rrad, umax, s, c.scores,
+                                                        c.argmax, c.row_mass, fb, nfb, ties, nfb + 1);
     OTGB_CHECK_LAUNCH();
     int *hp = static_cast<int *>(ctx_pinned(ctx));
     OTGB_CUDA_TRY(cudaMemcpyAsync(hp, nfb + 1, sizeof(int), cudaMemcpyDeviceToHost, st));

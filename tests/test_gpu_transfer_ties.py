@@ -50,6 +50,33 @@ def test_labels_are_those_of_the_cuda_core_kernel(n, m, L, twins):
     assert torch.equal(tc, cuda), int((tc != cuda).sum())
 
 
+@pytest.mark.parametrize("blur", [0.2, 0.05])
+def test_labels_at_a_small_blur(blur):
+    """Exponents of hundreds to thousands, rounded at 1e-4 to 1e-3: twins whose weights differ by that are near ties."""
+    from paper_2107_02010_gb300 import otgb
+
+    n, m, eps = 6000, 2000, blur * blur
+    x = synth.fiber_bundles(n, seed=7, perturb=3.0)[0]
+    y = synth.fiber_bundles(m, seed=8)[0]
+    rng = np.random.default_rng(9)
+    y = np.concatenate([y, y])
+    b = (1.0 + 1e-3 * rng.normal(size=2 * m)) / (2 * m)
+    a, b, g = T(np.full(n, 1.0 / n, np.float32)), T(b.astype(np.float32)), T(np.tile(20.0 + 5.0 * rng.normal(size=m), 2).astype(np.float32))
+    lab = T(np.repeat([0, 1], m).astype(np.int32))
+    ctx = otgb.Context()
+    p = otgb.default_params(blur=blur, fixed_iters=1, sigma_start=blur, multiscale=1, cluster=1, k_clusters=10)
+    out = []
+    for pad in (0, 4):
+        X, Y = (T(np.pad(v, ((0, 0), (0, pad)))) for v in (x, y))
+        if not out:
+            f = otgb.softmin(ctx, X, Y, b, g, eps)  # row sums of about 1
+        plan = otgb.sinkhorn_divergence(ctx, X, a, Y, b, p, want_plan=True)["plan"]
+        out.append(otgb.transport_apply(ctx, plan, f, g, lab, 2, want_scores=False))
+    (_, am, rm), (_, am2, _) = out
+    assert 0.5 < float(rm.min()) and float(rm.max()) < 2.0
+    assert torch.equal(am, am2), int((am != am2).sum())
+
+
 def test_an_atlas_of_ties_is_not_slow():
     tc, cuda = problem(30_000, 20_000, 2, True)
     t = best(tc), best(cuda)
