@@ -5,6 +5,7 @@
 #include <cmath>
 
 #include "prims.cuh"
+#include "threefloat.cuh"
 
 namespace otgb {
 namespace {
@@ -453,102 +454,124 @@ __global__ void finite_kernel(const float *v, int n, int *bad) {
 }
 
 // ------------------------------------------------------ cluster statistics --
-// A sum in two floats (about 48 bits: Knuth's two-sum, Dekker's product by FMA).  The FP64 units of this GPU do two
-// operations per clock and SM, so double sums over all coordinates bounded the kernel (290 us for 100 clusters of 512
-// points); a two-float step is ten FP32 operations.
-struct DF {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float v, float e = 0.f) {
-        const float s = __fadd_rn(hi, v), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(e, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b))));
-        hi = s;
-    }
-    __device__ __forceinline__ void add_product(float a, float b) {
-        const float p = __fmul_rn(a, b);
-        add(p, fmaf(a, b, -p));
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
 // Over sorted positions [off[k], off[k+1]) of the packed points (stride floats per point): mass = sum w, centroid =
-// weighted mean (plain mean when the mass is 0), radius = max distance to the centroid, ssq = sum w |x - c|^2.  Sums to
-// about 48 bits, in a fixed order.
+// weighted mean (plain mean when the mass is 0), radius = max distance to the centroid, ssq = sum w |x - c|^2.  Sums in at
+// least FP64 accuracy, in a fixed order.
 // D > 3: one CTA per cluster, thread (group g, coordinate d): a warp reads along the rows, and the points pass twice (a
-// pass per coordinate with a reduction each took 380 us for 300 clusters of 1000 points).
+// pass per coordinate with a reduction each took 380 us for 300 clusters of 1000 points; sums in FP64 290 us for 100
+// clusters of 512).
 constexpr int kStT = 1024, kStG = kStT / 64, kStW = kStT / 32;
 __global__ void __launch_bounds__(kStT) cluster_stats_kernel(const float *pts, int stride, int D, const float *w_sorted,
                                                             const int *off, int ncl, float *cent, int cstride, float *mass,
                                                             float *radius, float *ssq) {
-    __shared__ double red[kStG][64], mred[kStG];
+    __shared__ float part[3][kStG][64], mpart[3][kStG], wpart[3][kStW];
+    __shared__ double vsum[64], msum;
     __shared__ float c_s[64];
     __shared__ float rmax[kStW];
-    __shared__ double wsum[kStW];
     const int k = blockIdx.x;
     if (k >= ncl) return;
     const int a = off[k], b = off[k + 1];
     const int t = threadIdx.x, g = t >> 6, d = t & 63;
-    DF acc, m;
+    // The groups' sums are combined as they are, and only 65 threads go over to FP64 (1024 of them took a third of the kernel).
+    auto put = [](const ThreeFloat &f, float &hi, float &mid, float &lo) {
+        hi = f.hi;
+        mid = f.mid;
+        lo = f.lo;
+    };
+    auto join = [](ThreeFloat &s, float hi, float mid, float lo) {
+        s.add(hi);
+        s.add_small(mid);
+        s.lo += lo;
+    };
+    auto combine = [&] {  // vsum[d], msum from the groups' sums
+        __syncthreads();
+        ThreeFloat s;
+        if (t < 64) {
+            for (int q = 0; q < kStG; ++q) join(s, part[0][q][t], part[1][q][t], part[2][q][t]);
+            vsum[t] = s.value();
+        } else if (t == 64) {
+            for (int q = 0; q < kStG; ++q) join(s, mpart[0][q], mpart[1][q], mpart[2][q]);
+            msum = s.value();
+        }
+        __syncthreads();
+    };
+    // in double, one thread per coordinate: beyond the float range, or products that lose bits below it (rare)
+    auto in_double = [&](bool weighted) {
+        __syncthreads();
+        double v = 0.0, m = 0.0;
+        if (t < 64) {
+            for (int i = a; i < b; ++i) {
+                const double w = w_sorted[i];
+                m += w;
+                v += (weighted ? w : 1.0) * (t < D ? pts[(size_t)i * stride + t] : 0.f);
+            }
+            vsum[t] = v;
+            if (t == 0) msum = m;
+        }
+        __syncthreads();
+    };
+    ThreeFloat acc, m;
 #pragma unroll 4
     for (int i = a + g; i < b; i += kStG) {
         const float w = w_sorted[i], v = d < D ? pts[(size_t)i * stride + d] : 0.f;
-        m.add(w);
+        if (d == 0) m.add(w);
         acc.add_product(w, v);
     }
-    double accd = acc.value(), md = m.value();
-    if (__syncthreads_or(!isfinite(accd) || !isfinite(md))) {  // beyond the float range: in double
-        accd = md = 0.0;
-        for (int i = a + g; i < b; i += kStG) {
-            const double w = w_sorted[i];
-            md += w;
-            accd += w * (d < D ? pts[(size_t)i * stride + d] : 0.f);
-        }
-    }
-    red[g][d] = accd;
-    if (d == 0) mred[g] = md;
-    __syncthreads();
-    double mass_k = 0.0;
-    for (int q = 0; q < kStG; ++q) mass_k += mred[q];
+    put(acc, part[0][g][d], part[1][g][d], part[2][g][d]);
+    if (d == 0) put(m, mpart[0][g], mpart[1][g], mpart[2][g]);
+    if (__syncthreads_or(!acc.usable() || !m.usable())) in_double(true);
+    else combine();
+    const double mass_k = msum;
     if (!(mass_k > 0.0)) {  // uniform
-        DF plain;
+        ThreeFloat plain;
         for (int i = a + g; i < b; i += kStG) plain.add(d < D ? pts[(size_t)i * stride + d] : 0.f);
-        __syncthreads();
-        red[g][d] = plain.value();
-        __syncthreads();
+        put(plain, part[0][g][d], part[1][g][d], part[2][g][d]);
+        if (__syncthreads_or(!plain.usable())) in_double(false);
+        else combine();
     }
-    if (g == 0) {
-        double v = 0.0;
-        for (int q = 0; q < kStG; ++q) v += red[q][d];
-        c_s[d] = (float)(v / (mass_k > 0.0 ? mass_k : (double)(b - a)));
-    }
+    if (t < 64) c_s[t] = (float)(vsum[t] / (mass_k > 0.0 ? mass_k : (double)(b - a)));
     __syncthreads();
     // distances: a warp per point
     const int warp = t >> 5, lane = t & 31;
     const float c0 = lane < D ? c_s[lane] : 0.f, c1 = lane + 32 < D ? c_s[lane + 32] : 0.f;
     float r2 = 0.f;
-    DF wss;
-#pragma unroll 4
-    for (int i = a + warp; i < b; i += kStW) {
+    ThreeFloat wss;
+    auto square = [&](int i) -> float {
         const float u = lane < D ? pts[(size_t)i * stride + lane] - c0 : 0.f;
         const float v = lane + 32 < D ? pts[(size_t)i * stride + lane + 32] - c1 : 0.f;
         float s2 = fmaf(u, u, v * v);
         for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        return s2;
+    };
+#pragma unroll 4
+    for (int i = a + warp; i < b; i += kStW) {
+        const float s2 = square(i);
         r2 = fmaxf(r2, s2);
-        wss.add_product(w_sorted[i], s2);
+        if (ssq) wss.add_product(w_sorted[i], s2);
     }
     if (lane == 0) {
         rmax[warp] = r2;
-        wsum[warp] = wss.value();
+        put(wss, wpart[0][warp], wpart[1][warp], wpart[2][warp]);
     }
-    __syncthreads();
-    if (t == 0) {
-        double ws = 0.0;
-        for (int q = 0; q < kStW; ++q) {
-            r2 = fmaxf(r2, rmax[q]);
-            ws += wsum[q];
+    const bool bad = __syncthreads_or(!wss.usable()) != 0;
+    if (bad) {  // in double
+        double v = 0.0;
+        for (int i = a + warp; i < b; i += kStW) v += (double)w_sorted[i] * square(i);
+        if (lane == 0) vsum[warp] = v;
+        __syncthreads();
+    }
+    if (warp == 0) {
+        double ws = bad ? vsum[lane] : (double)wpart[0][lane] + ((double)wpart[1][lane] + (double)wpart[2][lane]);
+        float r = rmax[lane];
+        for (int o = 16; o > 0; o >>= 1) {
+            ws += __shfl_xor_sync(0xffffffffu, ws, o);
+            r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
         }
-        mass[k] = (float)mass_k;
-        radius[k] = sqrtf(r2) * (1.0f + 1e-6f) + 1e-30f;
-        if (ssq) ssq[k] = (float)ws;
+        if (lane == 0) {
+            mass[k] = (float)mass_k;
+            radius[k] = sqrtf(r) * (1.0f + 1e-6f) + 1e-30f;
+            if (ssq) ssq[k] = (float)ws;
+        }
     }
     if (t < cstride) cent[(size_t)k * cstride + t] = t < D ? c_s[t] : 0.f;
 }
