@@ -15,8 +15,9 @@
 // tiles: a block across a jump costs two short passes instead of one that visits everything between.  A single part above
 // kSpread (outliers: the dot product's terms would dwarf the exponents) is summed from coordinate differences alone.  Where
 // that comes to more passes than one over all tiles (points so sparse at the blur, or so far from each other's cells of the
-// curve, that every part is loose) the block is one run, as in the dense sweep: 100k points on a line, eps 0.01, 21 -> 0.7 ms
-// (CUDA cores 7.0); 100k points with one outlier that takes the curve's resolution 135 -> 2.3 (7.3).
+// curve, that every part is loose) both limits grow by eights until it does not or a few passes are left, as far as one run
+// for the block, which is what the dense sweep has: 100k points on a line, eps 0.01, 21 -> 0.9 ms (CUDA cores 7.0); 100k points with one outlier that
+// takes the curve's resolution 135 -> 4.2 (7.3).
 // Bound: MUFU, 32 pairs per clock and SM.  otgb_softmin on 100k x 100k voxels 0.86 ms, of it 0.56 the sums; the dense
 // tensor-core sweep 1.89, the CUDA cores 7.0.
 //
@@ -50,7 +51,8 @@ constexpr float kNoTerm = -1e29f;
 constexpr float kReach = 60.f;    // binades below the row's largest term that are visited
 // s (half diagonal)^2 of a run: what the products of the exponent are rounded at (error 7e-8 at 96)
 constexpr float kCompact = 96.f;
-constexpr int kPasses = 12;       // of a block's runs (one outside kSpread counts four): above, the block is one run
+constexpr int kPasses = 12;       // of a block's runs (one outside kSpread counts four): above, they are made larger,
+constexpr int kFewPasses = 6;     // and where together they visit more than every tile once: up to this number by one step only
 constexpr float kSpread = 256.f;  // terms of this size are rounded at 8e-6, as s f + s g - s C is at |s f| = 128
 
 struct S3Part {
@@ -246,6 +248,7 @@ __global__ void __launch_bounds__(kT, 4) softmin3_sorted_kernel(const __grid_con
     float4 rq = make_float4(0.f, 0.f, 0.f, 0.f);
     float rpot = 0.f;
     bool rin = false;
+    float limit = kCompact;
     // The run that starts at part ga: its box; the part after it.
     auto extent = [&](int ga, float (&lo)[3], float (&hi)[3], bool &spread) -> int {
         float hd2 = 0.f;
@@ -255,7 +258,7 @@ __global__ void __launch_bounds__(kT, 4) softmin3_sorted_kernel(const __grid_con
             hi[d] = -M.sub[ga][d + 3];
             hd2 = fmaf(0.25f * (hi[d] - lo[d]), hi[d] - lo[d], hd2);
         }
-        spread = !(s * hd2 <= kSpread);
+        spread = !(s * hd2 <= limit * (kSpread / kCompact));
         int gb = ga + 1;
         for (; gb < 16 && !spread; ++gb) {
             if (M.start[gb] >= M.start[gb + 1]) continue;
@@ -266,7 +269,7 @@ __global__ void __launch_bounds__(kT, 4) softmin3_sorted_kernel(const __grid_con
                 h[d] = fmaxf(hi[d], -M.sub[gb][d + 3]);
                 u = fmaf(0.25f * (h[d] - l[d]), h[d] - l[d], u);
             }
-            if (!(s * u <= kCompact)) break;
+            if (!(s * u <= limit)) break;
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 lo[d] = l[d];
@@ -275,48 +278,38 @@ __global__ void __launch_bounds__(kT, 4) softmin3_sorted_kernel(const __grid_con
         }
         return gb;
     };
-    // What the runs cost, in passes over the tiles; a block that needs many of them, or whose first run visits so many tiles
-    // that all of them would come to more than one pass over everything, is one run instead.
-    int passes = 0;
-    bool whole = false;
-    {
-        float lo[3], hi[3];
-        bool spread, finite = true;
+    // What the runs cost, in passes over the tiles.  Where that is too much the limit grows: larger runs, fewer passes; a block
+    // across a jump of the curve stays cut there as long as any other one.
+    auto count = [&]() -> int {
+        int n = 0;
+        bool finite = true;
         for (int ga = 0; ga < 16;) {
             if (M.start[ga] >= M.start[ga + 1]) {
                 ++ga;
                 continue;
             }
+            float lo[3], hi[3];
+            bool spread;
             ga = extent(ga, lo, hi, spread);
-            passes += spread ? 4 : 1;
+            n += spread ? 4 : 1;
             for (int d = 0; d < 3; ++d) finite = finite && hi[d] - lo[d] <= FLT_MAX;
         }
-        if (!finite) passes = 1;  // the centre of such a block is no number
-        whole = passes > kPasses;
+        return finite ? n : 1;  // no larger runs around a part without a centre
+    };
+    int passes = count();
+    while (passes > kPasses && limit < 1e30f) {
+        limit *= 8.f;
+        passes = count();
     }
     for (int ga = 0, gb; ok && ga < 16; ga = gb) {
     // ---- the run of parts [ga, gb): box, centre, row operand
-    if (!whole && M.start[ga] >= M.start[ga + 1]) {  // an empty part (uniform)
+    if (M.start[ga] >= M.start[ga + 1]) {  // an empty part (uniform)
         gb = ga + 1;
         continue;
     }
     float lo[3], hi[3];
-    bool spread = false;  // uniform
-    if (whole) {
-        gb = 16;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) lo[d] = hi[d] = FLT_MAX;  // hi: negated
-        for (int q = 0; q < 16; ++q)
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                lo[d] = fminf(lo[d], M.sub[q][d]);
-                hi[d] = fminf(hi[d], M.sub[q][d + 3]);
-            }
-#pragma unroll
-        for (int d = 0; d < 3; ++d) hi[d] = -hi[d];
-    } else {
-        gb = extent(ga, lo, hi, spread);
-    }
+    bool spread;  // uniform
+    gb = extent(ga, lo, hi, spread);
     const int ra = M.start[ga], rb = M.start[gb];
     const bool in_run = t >= ra && t < rb;
     const bool warp_on = 32 * warp < rb && 32 * warp + 32 > ra;  // some of the warp's rows are in the run
@@ -450,8 +443,8 @@ __global__ void __launch_bounds__(kT, 4) softmin3_sorted_kernel(const __grid_con
         }
         // the other tiles of this split that can matter, in order (a NaN bound is visited)
         const int n_list = list_tiles(M.v, max(ta - w0, 0), min(tb - w0, nw), bi, thr);
-        if (!whole && passes > 1 && passes * n_list > tb - ta) {
-            whole = restart = true;
+        if (passes > 1 && passes * n_list > tb - ta && limit < (passes > kFewPasses ? 1e30f : kCompact * 8.f)) {
+            restart = true;
             break;
         }
         int k = next_tile(M.v, 0, n_list, thr);
@@ -463,7 +456,11 @@ __global__ void __launch_bounds__(kT, 4) softmin3_sorted_kernel(const __grid_con
         }
         __syncthreads();  // the next window overwrites the bounds
     }
-    if (restart) {
+    if (restart) {  // from the first part, in fewer runs
+        for (const int before = passes; passes == before && limit < (before > kFewPasses ? 1e30f : kCompact * 8.f);) {
+            limit *= 8.f;
+            passes = count();
+        }
         gb = 0;
         continue;
     }
