@@ -43,15 +43,18 @@ typedef enum {
     OTGB_EINTERNAL = -7   /* internal consistency check failed */
 } otgb_status;
 
-/* OTGB_FP32: float32 accuracy; for D <= 3, and in coarse-to-fine solves with k-means clusters for
-   3 < D and round_up(D, 4) <= 60, the exponent of every pair is one tensor-core dot product of
-   three-piece BF16 operands (about 24 significant bits) with FP32 accumulation, elsewhere CUDA-core
-   float32.  OTGB_TC_BF16X3: the reduced-precision tensor-core cross term for D >= 16 (two pieces,
+/* OTGB_FP32: float32 accuracy; for D <= 3 with p = 2, and for 3 < D and round_up(D, 4) <= 60 in dense
+   sweeps (single-scale and coarse solves, the extrapolation) and in coarse-to-fine solves with k-means
+   clusters, the exponent of every pair is one tensor-core dot product of three-piece BF16 operands
+   (about 24 significant bits) with FP32 accumulation, elsewhere CUDA-core float32.  The calls without a
+   precision parameter compute likewise: otgb_softmin as the dense sweeps, transport_apply with
+   three-piece operands for 3 < D and round_up(D, 4) <= 60, gradients and otgb_softmin_noalloc in
+   CUDA-core float32.  OTGB_TC_BF16X3: the reduced-precision tensor-core cross term for D >= 16 (two pieces,
    about 16 bits).  In coarse-to-fine solves with k-means clusters and round_up(D, 4) <= 60 the column
    operand of either form is centred at its cluster's centroid and split once per solve, which holds
    per point of x and of y two copies of 2 x pieces x round_up(round_up(D, 4) + 4, 16) bytes in the
-   context's scratch (D = 60: 0.5 KB per point with two pieces, 0.77 KB with three; at most 8192
-   clusters per side).  Where that is more than 8 GB and more than half of the free device memory, or
+   context's scratch (D = 60, both copies: 0.5 KB per point with two pieces, 0.77 KB with three; at
+   most 8192 clusters per side).  Where that is more than 8 GB and more than half of the free device memory, or
    where an allocation fails, the float32 form runs on the CUDA cores instead.
    OTGB_FP32_SIMT: float32 on the CUDA cores for every D. */
 typedef enum { OTGB_FP32 = 0, OTGB_TC_BF16X3 = 1, OTGB_FP32_SIMT = 2 } otgb_precision;
@@ -203,7 +206,8 @@ int sinkhorn_divergence(otgb_ctx *ctx, const float *x, const float *a, int N, co
  *     -1 when the row is empty), row_mass: N float32 = sum_l Lab_il (optional).
  * A row whose mass is near 0 is an outlier (Section 2, label transfer).
  * The sum runs over all atlas points (dense), for any 1 <= D <= 64.
- * Errors: EINVAL for a null plan, a plan of a p = 1 solve, L < 1 or L > 1024, null f/g/labels/argmax.
+ * Errors: EINVAL for a null plan, a plan of a p = 1 solve, L < 1 or L > 1024, null f/g/labels/argmax; ETIMEOUT
+ * when a bounded device wait gave up (the outputs are then not complete).
  */
 int transport_apply(otgb_ctx *ctx, const otgb_plan *plan, const float *f, const float *g, const int32_t *labels,
                     int L, float *scores, int32_t *argmax, float *row_mass);
@@ -327,8 +331,9 @@ int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const float *p, const
                  int n_in, int D, double eps, double lam, const float *old, double omega, float *out);
 
 /*
- * otgb_softmin_noalloc: the same sweep as otgb_softmin, for callers that may
- * not allocate device memory.  The paper has no counterpart: this entry point
+ * otgb_softmin_noalloc: the sum of otgb_softmin, for callers that may not
+ * allocate device memory (in two passes on the CUDA cores: the results of the
+ * two calls differ in float32 rounding, and large sweeps take longer here).  The paper has no counterpart: this entry point
  * exists for integration only.
  *
  * Who needs it: code that runs where a device allocation is not allowed or
@@ -343,7 +348,7 @@ int otgb_softmin(otgb_ctx *ctx, const float *q, int n_out, const float *p, const
  *
  *   q: n_out x D rows, p: n_in x D columns, w: n_in weights, pot: n_in
  *   potential, old (optional), out: n_out -- device pointers owned by the
- *   caller, as in otgb_softmin (same arguments, same result).
+ *   caller, with the meaning that they have in otgb_softmin.
  *   cuda_stream: the cudaStream_t to run on (NULL: the legacy default stream).
  *   The call returns when the result is complete on that stream.
  * Limits and errors: EINVAL when the scratch of the problem exceeds 16 MiB --

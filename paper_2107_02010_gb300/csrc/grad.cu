@@ -10,6 +10,8 @@
 // enters that term twice).  The barycenter ("Track density atlas" of Section 2)
 // moves the support of alpha down the mean gradient of S(alpha, beta_k).
 //
+// For D <= 3 and p = 2 sorted3.cu sums over sorted points (large calls, and the
+// barycenter's steps with OTGB_FP32); the kernels here do the rest.
 // Each CTA owns 128 rows (one per thread, the row's point and its gradient in
 // registers); column tiles are staged in shared memory and read as broadcasts.
 // Two forms: every pair (sinkhorn_grad_x, from the caller's points and duals),

@@ -600,7 +600,7 @@ void Multiscale::setup_tcc(Solver &s) {
     cudaStream_t st = s.st;
     Workspace &ws = *s.ws;
     // The float32 form has the CUDA-core kernel to go back to, which needs no tiles: it stays in charge where the
-    // tiles would take more than half of the memory that is free (0.77 KB per point of 60 coordinates and copy).
+    // tiles would take more than half of the memory that is free (both copies 0.77 KB per point of 60 coordinates).
     // Asked only above 8 GB of new memory (some 5 million points per side), so that ordinary solves pay nothing.
     if (np == 3) {
         size_t need = 0, have = 0, free_b = 0, total_b = 0;

@@ -282,8 +282,7 @@ void Solver::set_work(const std::vector<std::vector<int>> &ncols, bool allow_spl
             const int n = ncols[k][b];
             const int first = (int)items.size();
             if (n <= CH) items.push_back(make_int4(k, b, 0, n));
-            else
-{
+            else {
                 // equal pieces of whole tiles
                 const int parts = (n + CH - 1) / CH, len = ((n + parts - 1) / parts + 127) / 128 * 128;
                 for (int c = 0; c < n; c += len) items.push_back(make_int4(k, b, c, std::min(n, c + len)));
@@ -788,9 +787,10 @@ static int softmin_once(otgb_ctx *ctx, const float *q, int n_out, const float *p
         float *box = ws.get<float>("box", 4 * 64);
         bbox_centre(p, n_in, D, d_cen, box, ws.get<float>("bpart", 64 * 2 * 64), st);
         // Large 3-D sweeps sort their points and visit the tiles that can matter (sorted3.cu); the sorts and permutations
-        // are some twenty launches.  Sorted against dense: 32k x 32k 0.33 / 0.27 ms, 45k x 45k 0.46 / 0.45, 64k x 64k
-        // 0.63 / 0.81, 100k x 100k 0.85 / 1.89.  Few rows or columns make large blocks or tiles, which reach everything:
-        // 4,200 x 500k 0.93 / 0.48, 500k x 4,200 0.52 / 0.45.
+        // are some twenty launches.  Sorted against dense, points uniform in a cube of side 30, eps 1: 32k x 32k 0.33 / 0.26 ms,
+        // 45k x 45k 0.46 / 0.44, 64k x 64k 0.63 / 0.80, 100k x 100k 1.01 / 1.87; at eps 0.05 0.30, 0.45, 0.60 and 0.81, at
+        // eps 20, where more tiles reach, 0.43, 0.66, 1.05 and 2.26 (voxels of a density map at eps 1: 0.83).  Few rows or columns make large blocks or
+        // tiles, which reach everything: 4,200 x 500k 0.69 / 0.47, 500k x 4,200 0.53 / 0.43.
         if (!lean && D <= 3 && n_out >= 32768 && n_in >= 32768 && (double)n_out * n_in >= 2e9) {
             softmin3_sorted(ctx, q, n_out, p, w, pot, n_in, D, eps, lam, old, omega, out, box, d_cen);
             return OTGB_OK;

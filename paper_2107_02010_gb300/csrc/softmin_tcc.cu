@@ -17,7 +17,7 @@
 // CUDA-core form (softmin_gen_kernel) needs D + 2 FP32 operations at a fiftieth of the rate.
 // Bound: the tensor pipe, 1910.7 TFLOP/s (measured) / (2 K x products) = 2.49e12 (NP = 3) and 4.98e12 (NP = 2)
 // pairs/s at K = 64.  Measured on the 60-D fiber bundles (300k and 1M per side): NP = 3 2.30e12 pairs/s = 92 %, where
-// softmin_gen_kernel has 3.9e11 (a solve of 300k per side 379 -> 76 ms); NP = 2 3.76e12 = 75 %, where the form with
+// softmin_gen_kernel has 3.9e11 (a solve of 300k per side 379 -> 71 ms); NP = 2 3.76e12 = 75 %, where the form with
 // the row operand in shared memory, one warp group for everything and two accumulators had 2.9e12.  Error of one
 // step of NP = 3 against FP64, geometric mean over D = 5 .. 60: 1.07e-7 of the duals, softmin_gen_kernel 1.28e-7.
 //

@@ -15,8 +15,8 @@
 // holds one column operand and one accumulator.
 //
 // Bound: the tensor pipe, six products, 2.49e12 pairs/s at K = 64 (4e8 pairs: 0.16 ms).  Measured, otgb_softmin of
-// 20k x 20k fibers (60-D): 5.42 -> 0.46 ms for the whole call (softmin_gen_kernel: two sweeps, 157 CTAs for 304
-// slots); error against FP64 6.3e-6 -> 3.4e-6 of the result.  Extrapolation at 300k per side: 4.5 -> 2.3 ms.
+// 20k x 20k fibers (60-D): 5.42 -> 0.375 ms for the whole call, 0.32 of it this kernel (softmin_gen_kernel: two sweeps,
+// 157 CTAs for 304 slots); error against FP64 (rms, of the largest result) 1.3e-6 -> 0.7e-6.  Extrapolation at 300k per side: 4.5 -> 2.3 ms.
 //
 // Columns of a block may be split over several items (SoftminLaunch::part: shift and sum per row, combined in item
 // order by the CTA that completes the block's last item).

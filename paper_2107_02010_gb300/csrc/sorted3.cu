@@ -18,8 +18,8 @@
 // curve, that every part is loose) both limits grow by eights until it does not or a few passes are left, as far as one run
 // for the block, which is what the dense sweep has: 100k points on a line, eps 0.01, 21 -> 0.9 ms (CUDA cores 7.0); 100k points with one outlier that
 // takes the curve's resolution 135 -> 4.2 (7.3).
-// Bound: MUFU, 32 pairs per clock and SM.  otgb_softmin on 100k x 100k voxels 0.86 ms, of it 0.56 the sums; the dense
-// tensor-core sweep 1.89, the CUDA cores 7.0.
+// Bound: MUFU, 32 pairs per clock and SM.  otgb_softmin on 100k x 100k voxels 0.83 ms, of it 0.55 the sums (ex2 at 51 % of the
+// MUFU, issue 66 % of the active clocks); the dense tensor-core sweep 1.87, the CUDA cores 7.0.
 //
 // grad3_sorted_kernel: the whole block in one run, in coordinate differences (two columns per packed f32x2 operation, a
 // running shift per row, the tile's coordinates read as broadcasts).  The gradient is a small difference of two large sums:
@@ -27,9 +27,10 @@
 // up to sixteen passes a block, and was slower than grad_kernel where blocks are loose (2,000 + 2,000 points 0.53 against
 // 0.35 ms, 20,000 + 20,000 with one far outlier, which takes the curve's whole resolution, 14 against 3.4).  Differences
 // need no compact runs, and a block that is loose only visits more tiles.
-// Bound: issue, about 9 instructions per pair (1.5 differences, 2 for the exponent, 1 maximum, 0.5 shift, ex2, 1.5 sums, 1
-// shared load).  sinkhorn_grad_x on 50k + 50k voxels 2.17 -> 1.24 ms (grad_kernel 8.6), error 9.7e-7 -> 4.6e-7; 2,000 +
-// 2,000 points 0.53 -> 0.17; every pair of 50k + 50k points (far outlier) 76 -> 2.5.
+// Bound: the FP32 pipe, 11 operations per pair (3 differences, 4 for the exponent, 1 shift, 3 sums; ex2 takes 4 of its
+// clocks): 3.7e12 pairs/s.  Every pair of 50k + 50k points (far outlier) 76 -> 2.5 ms = 2.0e12; the FP32 pipe and
+// fixed-latency waits are the largest stalls.  sinkhorn_grad_x on 50k + 50k voxels 2.17 -> 1.24 ms, of it 1.01 the sums
+// (grad_kernel 8.6), error 9.7e-7 -> 4.6e-7; 2,000 + 2,000 points 0.53 -> 0.17.
 //
 // Each (block, split, part) writes its shift and sums; a finish kernel combines the splits in order, so the result does
 // not depend on scheduling.

@@ -22,9 +22,9 @@
 // concerned: 60k x 50k fibers, two such labels, 262 ms with a CTA per row, 20.5 now (transport_gen_kernel alone 24.2, 20 now
 // that its FMAs are packed); a small atlas of ties pays for the sweep that decided nothing (5,000 x 5,000: 1.3 ms, 1.0).
 //
-// Measured (60k x 50k fibers, 60-D, 20 labels that split every bundle; whole call): 24.5 -> 3.2 ms, of which the sweep
-// 0.65 (13 % of the pairs visited; dense at the tensor bound: 1.2), the two k-means and their sorts 0.8, about 20 near
-// ties 1.5.  transport_gen_kernel alone took 22 ms.  Error of the scores against FP64 8.1e-7 - 9.1e-7 -> 3.6e-7 - 7.1e-7.
+// Measured (60k x 50k fibers, 60-D, 20 labels that split every bundle; whole call): 24.5 -> 3.1 ms, of which the sweep
+// 0.66 (13 % of the pairs visited; dense at the tensor bound: 1.2), the two k-means and their sorts 0.8, about 20 near
+// ties 1.4 (the k-means over all rows 1.28, their sums 0.15).  transport_gen_kernel alone took 22 ms.  Error of the scores against FP64 8.1e-7 - 9.1e-7 -> 3.6e-7 - 7.1e-7.
 #include <cmath>
 #include <cstring>
 
