@@ -871,11 +871,11 @@ __global__ void __launch_bounds__(kFbThreads) softmin_fallback_kernel(const __gr
                 }
                 lw = I.col_logw[j];
             }
-            return s * (fmaf(eps, lw, I.col_pot[j]) - 0.5f * d2);
+            return fmaf(eps, lw, I.col_pot[j]) - 0.5f * d2;
         };
         float m = -INFINITY;
         walk.start(I, blk, t);
-        for (int p = t; p < n; p += kFbThreads) m = fmaxf(m, term(p));
+        for (int p = t; p < n; p += kFbThreads) m = fmaxf(m, s * term(p));
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (lane == 0) redf[wid] = m;
         __syncthreads();
@@ -884,8 +884,14 @@ __global__ void __launch_bounds__(kFbThreads) softmin_fallback_kernel(const __gr
         for (int k = 1; k < kFbThreads / 32; ++k) m = fmaxf(m, redf[k]);
         double acc = 0.0;
         walk.start(I, blk, t);
+        // s u - m in one rounding, except where m itself is rounded by more than an ex2 can hold (64 and more): there the best
+        // column has to come to 2^0 (every potential at -1e30, say: 2^inf or 2^-inf otherwise)
+        const bool large = fabsf(m) > 0x1p30f;
         if (m > -INFINITY)
-            for (int p = t; p < n; p += kFbThreads) acc += (double)exp2f(term(p) - m);
+            for (int p = t; p < n; p += kFbThreads) {
+                const float u = term(p);
+                acc += (double)exp2f(large ? __fsub_rn(__fmul_rn(s, u), m) : fmaf(s, u, -m));
+            }
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) redd[wid] = acc;
         __syncthreads();
