@@ -197,6 +197,7 @@ __global__ void __launch_bounds__(kThreads, 4) softmin3_tc_kernel(const __grid_c
     }
     const float x0 = valid ? p.x - c[0] : 0.f, x1 = valid ? p.y - c[1] : 0.f, x2 = valid ? p.z - c[2] : 0.f;
     const double hx = 0.5 * ((double)x0 * x0 + (double)x1 * x1 + (double)x2 * x2);
+    const bool far_row = MAXP && valid && hx > 0.5 * (double)xt::kFarRow / (double)s;
     float m = -INFINITY;
     if (!MAXP && valid) m = (float)((double)s * (hx - (double)I.row_old[r0 + t] / (double)I.lam));
     float Cb = 0.f;
@@ -368,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, 4) softmin3_tc_kernel(const __grid_c
     float dmax = 0.f;
     if (valid) {
         const int r = r0 + t;
-        if (!(tot >= 0x1p-60f && tot <= 0x1p60f)) {
+        if (!(tot >= 0x1p-60f && tot <= 0x1p60f) || far_row) {
             const int k = atomicAdd(L.n_fallback, 1);
             if (k < L.fallback_cap) L.fallback[k] = make_int4(item.x, r, blk, 0);
         } else {

@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(kThreads, 2) softmin_xd_kernel(const __grid_co
     __syncthreads();
 
     float tot = 0.f, sh = kNoTerm, Mi = 0.f;
+    bool far_row = false;
     if (warp == 8) {
         if (lane == 0) {
             bool ok = true;
@@ -174,6 +175,7 @@ __global__ void __launch_bounds__(kThreads, 2) softmin_xd_kernel(const __grid_co
             if (!MAXP && valid) Mi = (float)(-(double)s * (double)I.row_old[r0 + t] / (double)I.lam);
             const float T = xt::stage_row<3, K>(x, D4, S.cen, s, Mi, valid, lanes + kN);
             if constexpr (!MAXP) xt::put_t(T, &S.tmax[warp], lane);
+            else far_row = T > xt::kFarRow;
         }
         xt::st_wait();
         tc::fence_before();
@@ -231,7 +233,7 @@ __global__ void __launch_bounds__(kThreads, 2) softmin_xd_kernel(const __grid_co
     float dmax = 0.f;
     if (t < nr) {
         const int r = r0 + t;
-        if (!(tot >= 0x1p-60f && tot <= 0x1p60f)) {
+        if (!(tot >= 0x1p-60f && tot <= 0x1p60f) || far_row) {
             const int q = atomicAdd(L.n_fallback, 1);
             if (q < L.fallback_cap) L.fallback[q] = make_int4(item.x, r, blk, 0);
         } else {

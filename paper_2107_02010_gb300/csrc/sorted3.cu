@@ -465,7 +465,11 @@ __global__ void __launch_bounds__(kT, 4) softmin3_sorted_kernel(const __grid_con
         gb = 0;
         continue;
     }
-    if (in_run) A.out[(size_t)blockIdx.y * A.n_rows + r0 + t] = make_float4(sh, S - Slost, 0.f, 0.f);
+    if (in_run) {
+        const float x0 = p.x - c[0], x1 = p.y - c[1], x2 = p.z - c[2];
+        const bool far_row = !spread && s * fmaf(x0, x0, fmaf(x1, x1, x2 * x2)) > xt::kFarRow;  // NaN: the safe kernel's row
+        A.out[(size_t)blockIdx.y * A.n_rows + r0 + t] = make_float4(sh, far_row ? NAN : S - Slost, 0.f, 0.f);
+    }
     }
     tc::fence_before();
     __syncthreads();

@@ -28,6 +28,11 @@ namespace otgb {
 namespace xt {
 
 constexpr int kRows = 128, kCols = 128;
+// Rows with T = s |x - c|^2 above this (c: the centre of the row's block) are left to the safe kernel by the forms with a
+// running shift.  A pair near such a row is a difference of numbers as large as T, rounded at 64 binades and more; a shift
+// from old values shows that by a sum out of range, a running shift follows the wrong maximum (one row at 1e5 among points
+// at 0 to 4, eps 0.09: every row of its block off by 70 to 150).
+constexpr float kFarRow = 0x1p30f;
 constexpr uint32_t kTmemCols = 256;  // accumulator (128) and the row operand(s)
 
 // K slots of a point of D4 coordinates: the coordinates and the four (NP = 2) or two (NP = 3) folded slots, rounded
